@@ -614,8 +614,8 @@ static int forward_rows(cl_ctx *c, const int *tok, int T, int row0, const uint8_
 
 // The prompt pass over M <= CL_WIDE_MAX_M rows at positions ctx .. ctx + M - 1 (bf16 models): every matrix is one wide
 // tensor-core GEMM whose product a small kernel consumes (rotary + cache append, residual add + RMSNorm, SiLU).
-// Fills the KV cache and, when asked, the hidden taps; computes no logits (the caller runs the last prompt token
-// through the T-row pass for those).
+// Fills the KV cache and, when asked, the hidden taps; computes no logits (the caller runs
+// the LM head on the last row of w_x).
 static int forward_wide(cl_ctx *c, const int *tok, int M, int tap) {
     const cl_model_cfg &g = c->cfg;
     const int d = g.d_model, F = g.d_ffn, L = g.n_layers, qkv_rows = d + 2 * g.n_kv_heads * g.head_dim;
@@ -771,12 +771,21 @@ extern "C" int cl_prefill(cl_ctx *c, const int32_t *tokens, int n, int tap_hidde
     if ((rc = poke(c, p))) return rc;
     int c0 = 0;
     if (c->use_wide && n > 2 * CL_PREFILL_CHUNK) {
-        // all prompt rows but the last go through the wide GEMMs; the last one takes the T-row pass, which has the LM head
-        while (c0 < n - 1) {
-            const int M = (n - 1 - c0 < CL_WIDE_MAX_M) ? n - 1 - c0 : CL_WIDE_MAX_M;
+        // Every prompt row goes through the wide GEMMs, in passes of equal size (a last pass of a row or two would stream all
+        // weights for them); then only the last row needs the LM head, whose weights are all that is read again.
+        const int n_pass = (n + CL_WIDE_MAX_M - 1) / CL_WIDE_MAX_M;
+        for (int i = 0; i < n_pass; ++i) {
+            const int M = (int)((long long)n * (i + 1) / n_pass) - c0;
             if ((rc = forward_wide(c, c->prompt_dev + c0, M, tap_hidden))) return rc;
-            KL(cl_launch_advance(c->st, M, 0, c->stream));
             c0 += M;
+            if (c0 < n) KL(cl_launch_advance(c->st, M, -1, c->stream));
+            else {
+                KL(cl_launch_rmsnorm(c->w_x + (size_t)(M - 1) * c->cfg.d_model, c->final_norm, 1, c->cfg.d_model, c->cfg.rms_eps,
+                                     c->xn, c->st, c->stream));
+                if ((rc = head(c, 1, c->xn, c->st, ST_FIELD(c, int, tgt_tok), ST_FIELD(c, float, v_pmax), ST_FIELD(c, float, v_conf),
+                               nullptr))) return rc;
+                KL(cl_launch_advance(c->st, M, 0, c->stream));
+            }
         }
     }
     for (; c0 < n; c0 += CL_PREFILL_CHUNK) {
@@ -785,7 +794,7 @@ extern "C" int cl_prefill(cl_ctx *c, const int32_t *tokens, int n, int tap_hidde
         rc = forward_rows(c, c->prompt_dev + c0, T, 0, nullptr, tap_hidden, last, ST_FIELD(c, int, tgt_tok),
                           ST_FIELD(c, float, v_pmax), ST_FIELD(c, float, v_conf), nullptr);
         if (rc) return rc;
-        KL(cl_launch_advance(c->st, T, last ? 1 : 0, c->stream));
+        KL(cl_launch_advance(c->st, T, last ? T - 1 : -1, c->stream));
     }
     if ((rc = sync_state(c))) return rc;
     if ((rc = check_device_err(c, "cl_prefill"))) {

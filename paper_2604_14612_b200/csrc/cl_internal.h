@@ -173,7 +173,7 @@ cudaError_t cl_launch_attn(int wdtype, int T, const ClAttnArgs &a, cudaStream_t 
 cudaError_t cl_launch_tap(int wdtype, const float *x, int T, int row0, int d, void *ring_layer, int P,
                           const ClDevState *st, cudaStream_t s);
 cudaError_t cl_launch_accept(ClDevState *st, int K, int *out_tokens, cudaStream_t s);
-cudaError_t cl_launch_advance(ClDevState *st, int n, int set_pending_from_tgt, cudaStream_t s);
+cudaError_t cl_launch_advance(ClDevState *st, int n, int pending, cudaStream_t s);
 // epilogues of the tensor-core GEMMs of the T-row pass
 enum { CL_VEPI_STORE = 0, CL_VEPI_RESID = 1, CL_VEPI_SILU = 2, CL_VEPI_HEAD = 3 };
 

@@ -249,10 +249,11 @@ __global__ void k_accept(ClDevState *st, int K, int *out_tokens) {
     st->emitted_total += (unsigned long long)(n + 1);
 }
 
-__global__ void k_advance(ClDevState *st, int n, int set_pending_from_tgt) {
+// ctx += n; pending >= 0: the greedy token after row `pending` of the pass becomes the pending token.
+__global__ void k_advance(ClDevState *st, int n, int pending) {
     if (threadIdx.x != 0) return;
     st->ctx += n;
-    if (set_pending_from_tgt) st->cyc_tok[0] = st->tgt_tok[n - 1];
+    if (pending >= 0) st->cyc_tok[0] = st->tgt_tok[pending];
 }
 
 // ---- c_layer[r] = mean over P positions of conf_rows[r, :] (fixed order, double) -------------
@@ -459,8 +460,8 @@ cudaError_t cl_launch_accept(ClDevState *st, int K, int *out_tokens, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t cl_launch_advance(ClDevState *st, int n, int set_pending_from_tgt, cudaStream_t s) {
-    k_advance<<<1, 32, 0, s>>>(st, n, set_pending_from_tgt);
+cudaError_t cl_launch_advance(ClDevState *st, int n, int pending, cudaStream_t s) {
+    k_advance<<<1, 32, 0, s>>>(st, n, pending);
     return cudaGetLastError();
 }
 
