@@ -413,7 +413,7 @@ extern "C" int cl_load(cl_ctx *c, const cl_weights *w) {
                     CU(cudaMemsetAsync(c->w_aatt, 0, 2 * Mw * d * 2, c->stream));
                     CU(cudaMemsetAsync(c->w_ah, 0, 2 * Mw * F * 2, c->stream));
                     DM(c->w_x, Mw * d * 4);
-                    c->w_P_floats = 2 * Mw * widest;
+                    c->w_P_floats = 3 * Mw * widest;   // (the widest product in two parts, four where a half tile follows a full one)
                     DM(c->w_P, c->w_P_floats * 4);
                     if (!(cl_make_tensor_map(&c->map_wx, c->w_ax, (int)(2 * Mw), (int)d, 128, f16) &&
                           cl_make_tensor_map(&c->map_watt, c->w_aatt, (int)(2 * Mw), (int)d, 128, f16) &&
@@ -619,14 +619,11 @@ static int forward_rows(cl_ctx *c, const int *tok, int T, int row0, const uint8_
 static int forward_wide(cl_ctx *c, const int *tok, int M, int tap) {
     const cl_model_cfg &g = c->cfg;
     const int d = g.d_model, F = g.d_ffn, L = g.n_layers, qkv_rows = d + 2 * g.n_kv_heads * g.head_dim;
-    const int KBd = (d + 63) / 64, KBf = (F + 63) / 64, MT = (M + 127) / 128, lo0 = CL_WIDE_MAX_M;
+    const int KBd = (d + 63) / 64, KBf = (F + 63) / 64, lo0 = CL_WIDE_MAX_M;
     const int f16 = g.weight_dtype == 2;
-    auto gemm = [&](const ClTensorMap &mapA, const ClTensorMap &mapB, int rows, int KB, int *splits) -> int {
-        ClWideArgs a;
-        a.M = M; a.rows = rows; a.KB = KB; a.MT = MT; a.NT = (rows + 255) / 256;
-        a.splits = *splits = cl_wide_splits(M, rows, KB, c->n_sm, c->w_P_floats);
-        a.lo_row0 = lo0; a.P = c->w_P; a.err = &c->st->err; a.f16 = f16;
-        KL(cl_launch_wide(mapA, mapB, a, c->stream));
+    auto gemm = [&](const ClTensorMap &mapA, const ClTensorMap &mapB, int rows, int KB, ClWideParts *p) -> int {
+        *p = cl_wide_plan(M, rows, KB, c->n_sm, c->w_P, c->w_P_floats);
+        KL(cl_launch_wide(mapA, mapB, *p, lo0, &c->st->err, f16, c->stream));
         return CL_OK;
     };
     ClWideNormArgs nb;
@@ -638,24 +635,25 @@ static int forward_wide(cl_ctx *c, const int *tok, int M, int tap) {
         n.embed = c->embed; n.tok = tok; n.g = L ? c->layers[0].n1 : nullptr;
         KL(cl_launch_wide_norm(n, c->stream));
     }
-    int rc, sp;
+    int rc;
+    ClWideParts p;
     for (int l = 0; l < L; ++l) {
         const ClLayer &y = c->layers[l];
-        if ((rc = gemm(c->map_wx, c->map_qkv[l], qkv_rows, KBd, &sp))) return rc;
-        KL(cl_launch_wide_rope_append(c->w_P, sp, M, g.n_heads, g.n_kv_heads, g.head_dim, d, c->rope_cs, y.kc, y.vc, g.max_seq,
-                                      c->st, f16, c->stream));
+        if ((rc = gemm(c->map_wx, c->map_qkv[l], qkv_rows, KBd, &p))) return rc;
+        KL(cl_launch_wide_rope_append(p, g.n_heads, g.n_kv_heads, g.head_dim, d, c->rope_cs, y.kc, y.vc, g.max_seq, c->st, f16,
+                                      c->stream));
         KL(cl_launch_attn_wide(c->w_P, qkv_rows, y.kc, y.vc, c->w_aatt, lo0, M, d, g.n_heads, g.n_kv_heads, g.head_dim,
                                g.max_seq, c->st, f16, c->stream));
-        if ((rc = gemm(c->map_watt, c->map_o[l], d, KBd, &sp))) return rc;
+        if ((rc = gemm(c->map_watt, c->map_o[l], d, KBd, &p))) return rc;
         ClWideNormArgs n = nb;
-        n.P = c->w_P; n.splits = sp; n.g = y.n2;
+        n.parts = p; n.g = y.n2;
         if (tap) n.tap = ring_slot(c, l, 0);
         KL(cl_launch_wide_norm(n, c->stream));
-        if ((rc = gemm(c->map_wx, c->map_gu[l], 2 * F, KBd, &sp))) return rc;
-        KL(cl_launch_wide_silu(c->w_P, sp, M, F, c->w_ah, lo0, f16, c->stream));
-        if ((rc = gemm(c->map_wh, c->map_d[l], d, KBf, &sp))) return rc;
+        if ((rc = gemm(c->map_wx, c->map_gu[l], 2 * F, KBd, &p))) return rc;
+        KL(cl_launch_wide_silu(p, F, c->w_ah, lo0, f16, c->stream));
+        if ((rc = gemm(c->map_wh, c->map_d[l], d, KBf, &p))) return rc;
         n = nb;
-        n.P = c->w_P; n.splits = sp; n.g = (l + 1 < L) ? c->layers[l + 1].n1 : nullptr;
+        n.parts = p; n.g = (l + 1 < L) ? c->layers[l + 1].n1 : nullptr;
         if (tap) n.tap = ring_slot(c, l, 1);
         KL(cl_launch_wide_norm(n, c->stream));
     }

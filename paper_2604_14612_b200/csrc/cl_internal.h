@@ -232,18 +232,37 @@ cudaError_t cl_launch_rows_pass(int wdtype, int head_dim, const ClRowsArgs &a, i
 
 // ---- wide tensor-core GEMM of the prompt pass (bf16 models): up to CL_WIDE_MAX_M prompt rows at a time ----
 #define CL_WIDE_MAX_M 512
+struct ClWideParts {                  // a GEMM's product as its consumer sees it: parts of [M, rows] floats, added in order
+    float *P;
+    int M, rows, KB;                  // operand rows, weight rows, K blocks of 64
+    int MT, half, NT, G;              // full tiles of 256 operand rows, a half tile after them (0 / 1), tiles of 256 weight rows, CTA pairs
+};
 struct ClWideArgs {
-    int M, rows, KB;                  // token rows of the pass, weight rows, K blocks of 64
-    int MT, NT, splits;               // 128-row token tiles, 256-row weight tiles, parts the K range is cut into
+    ClWideParts p;
+    int chain;                        // K blocks per accumulation chain
     int lo_row0;                      // first row of the lo parts in the activation buffer (hi parts start at row 0)
-    float *P;                         // [splits, M, rows] partial products (a later kernel adds the splits in order)
     int *err;
     int f16;                          // the model's 16-bit type: 0 bf16, 1 fp16
 };
+// The K blocks of all tiles are one sequence: weight tile by weight tile, within it the operand tiles, a block of a full
+// tile costing 2 and one of a half tile 1.  Of the total cost T, pair p takes the blocks that begin at a cost in
+// [floor(T p / G), floor(T (p + 1) / G)).
+#ifdef __CUDACC__
+#define CL_HD __host__ __device__ __forceinline__
+#else
+#define CL_HD static inline
+#endif
+CL_HD int cl_wide_col_cost(const ClWideParts &p) { return p.KB * (2 * p.MT + p.half); }
+CL_HD int cl_wide_cost(const ClWideParts &p) { return p.NT * cl_wide_col_cost(p); }
+// The pair that has K block kb of tile (nt, mt).
+CL_HD int cl_wide_owner(const ClWideParts &p, int nt, int mt, int kb) {
+    const unsigned c = (unsigned)(nt * cl_wide_col_cost(p) + 2 * mt * p.KB + (mt < p.MT ? 2 * kb : kb));
+    return (int)(((c + 1u) * (unsigned)p.G - 1u) / (unsigned)cl_wide_cost(p));
+}
 struct ClWideNormArgs {
     float *x;                         // [M, d] residual stream of the pass
-    int M, d, splits;
-    const float *P;                   // [splits, M, d] products to add to x, or null
+    int M, d;
+    ClWideParts parts;                // product to add to x
     const void *embed;                // with tok: x = E[tok[t]] instead (start of the pass)
     const int *tok;
     const float *g;                   // gain of the RMSNorm that follows, or null (no normalised rows are written)
@@ -255,17 +274,18 @@ struct ClWideNormArgs {
     const ClDevState *st;
     int f16;                          // the model's 16-bit type: 0 bf16, 1 fp16 (embedding, taps, normalised rows)
 };
-int cl_wide_splits(int M, int rows, int KB, int n_sm, size_t ws_floats);
-cudaError_t cl_launch_wide(const ClTensorMap &mapA, const ClTensorMap &mapB, const ClWideArgs &a, cudaStream_t s);
+ClWideParts cl_wide_plan(int M, int rows, int KB, int n_sm, float *P, size_t ws_floats);
+cudaError_t cl_launch_wide(const ClTensorMap &mapA, const ClTensorMap &mapB, const ClWideParts &p, int lo_row0, int *err, int f16,
+                           cudaStream_t s);
 cudaError_t cl_launch_wide_norm(const ClWideNormArgs &a, cudaStream_t s);
-cudaError_t cl_launch_wide_rope_append(float *P, int splits, int M, int H, int Hkv, int hd, int d, const float2 *rope_cs,
-                                       void *kcache, void *vcache, int max_seq, const ClDevState *st, int f16, cudaStream_t s);
+cudaError_t cl_launch_wide_rope_append(const ClWideParts &p, int H, int Hkv, int hd, int d, const float2 *rope_cs, void *kcache,
+                                       void *vcache, int max_seq, const ClDevState *st, int f16, cudaStream_t s);
 // causal attention of the M rows of the pass (positions ctx ..) over the cache; q: fp32 rows [M, ld_q], rotary applied;
 // the output goes out as bf16 hi (row t) and lo (row lo_row0 + t) parts [.., d]
 cudaError_t cl_launch_attn_wide(const float *q, int ld_q, const void *kcache, const void *vcache, __nv_bfloat16 *out_b,
                                 int lo_row0, int M, int d, int H, int Hkv, int hd, int max_seq, const ClDevState *st,
                                 int f16, cudaStream_t s);
-cudaError_t cl_launch_wide_silu(const float *P, int splits, int M, int F, __nv_bfloat16 *A, int lo_row0, int f16, cudaStream_t s);
+cudaError_t cl_launch_wide_silu(const ClWideParts &p, int F, __nv_bfloat16 *A, int lo_row0, int f16, cudaStream_t s);
 
 // tensor-core scoring (bf16 / fp16 LM head): normalise to the 16-bit type, contraction fused with the softmax statistics, finalize
 int cl_score_tc_ranges(int R, int n_sm);

@@ -2,159 +2,279 @@
 // Section 3 over up to 512 prompt rows at a time, so that the weights stream from HBM once per 512 tokens instead
 // of once per 8.
 //
-//   P[ks, t, r] = sum_{k in part ks} a[t, k] * W[r, k]        a: M activation rows, W: [rows, K] 16-bit weights
+//   sum over parts of P[part, t, r] = sum_k a[t, k] * W[r, k]        a: M activation rows, W: [rows, K] 16-bit weights
 //
-// Here the token rows are the M = 128 operand of tcgen05.mma (one tensor-memory lane per token) and 256 weight rows
-// are N.  Activations are fp32 everywhere else; each row enters as hi = round16(v) and lo = round16(v - hi) in the
-// weights' type and both products accumulate into the same fp32 accumulator, so the product keeps about 16 (bf16)
-// or 22 (fp16) mantissa bits of the activation.
-// One CTA computes one (token tile, weight tile, K part): the K range is cut into `splits` parts only to fill the
-// 148 SMs when a matrix has few output tiles (4096 outputs are 16 tiles), and the parts are added in a fixed order
-// by the small kernel that consumes the product:
+// Activations are fp32 everywhere else; each row enters as hi = round16(v) and lo = round16(v - hi) in the weights' type
+// and both products count, so the product keeps about 16 (bf16) or 22 (fp16) mantissa bits of the activation.
+//   k_wide               the GEMM; its product parts are added in a fixed order by the kernel that consumes them:
 //   k_wide_rope_append   q, k, v: rotary embedding at the row's position, cache append, q left in place
 //   k_attn_wide          causal attention of the pass's rows over the cache -> hi/lo rows of the output projection
 //   k_wide_norm          x += product (or x = E[token]); hidden tap; RMSNorm -> hi/lo rows of the next GEMM
 //   k_wide_silu          h = silu(gate) * up on the interleaved gate/up product -> hi/lo rows of the down projection
-// Warp roles: warp 0 TMA producer (A hi 128 x 64, A lo 128 x 64, B 256 x 64 as two 128-row boxes, 128-byte swizzle,
-// 3-stage ring of 64 KB), warp 1 tensor-memory allocation and MMA issue, warps 2-5 store the accumulator (thread =
-// token row, 256 consecutive outputs).  CTAs that share a weight tile are neighbours in the grid, so the tile comes
-// from HBM once and from L2 for the other token tiles.  Every wait is bounded in time.
+// The launches of a pass are chained by programmatic dependent launch: a kernel lets its successor start at once and the
+// successor waits (griddepcontrol.wait) before it touches anything another kernel writes; only weights are read earlier.
+// Every wait is bounded in time.
 #include <math.h>
+
+#include <algorithm>
 
 #include "tc_common.cuh"
 
 namespace {
 
-constexpr int WM = 128, WN = 256, WSTAGES = 3;
-constexpr int WA_BYTES = WM * TC_BK * 2, WB_BYTES = WN * TC_BK * 2, WSTAGE_BYTES = 2 * WA_BYTES + WB_BYTES;   // 64 KB
-constexpr int WTHREADS = 192;
+// ---- the GEMM ------------------------------------------------------------------------------------------------
+// One CTA pair (cluster of 2, tcgen05 cta_group::2) computes tiles of 256 operand rows x 256 weight rows: each CTA holds
+// 128 operand rows and half of the weight rows in its shared memory and the accumulator rows of its 128 operand rows
+// (tensor-memory lanes) over all 256 columns.
+// Bound: the tensor pipe for M > 128.  A single-CTA 128 x 256 tile has to fill 64 KB of shared memory per 64 elements of K
+// and read 96 bytes of it per cycle for the multiply-adds, which held it at 1.06 PFLOP/s; the pair splits the weight rows,
+// so a CTA fills 48 KB and reads 64 bytes per cycle.
+//   full tile  256 token rows; per K block two products (hi, lo) into the same accumulator
+//   half tile  128 token rows or fewer (the rest of M, if there is one of that size): their hi parts are the rows of CTA 0,
+//              their lo parts those of CTA 1, one product per K block; the two halves of the sum are separate parts.  Half the
+//              multiply-adds of a full tile, and with M <= 128, where the pass is bound by the weight stream, each SM fills
+//              32 KB per K block, half of it weights.
+// Work is cut evenly: the K blocks of all tiles, in tile order, are one sequence (cost 2 per block of a full tile, 1 of a
+// half tile) of which every pair takes an equal contiguous share.  A share may end inside a tile: a tile's product comes in
+// as many parts as pairs touched it, part = pair - first pair of the tile.  Equal shares matter: 4096 x 4096 outputs at
+// M = 512 are 32 tiles for 74 pairs.
+// The accumulator is double-buffered (2 x 256 columns): the store of one piece overlaps the multiply-adds of the next.  A
+// piece is at most `chain` K blocks of one tile (a longer accumulation chain in tensor memory loses accuracy); later pieces
+// of a share are added to the part's memory.
+// Roles per CTA: warp 0 TMA producer (the weights of the first stages are requested before the wait for the previous
+// kernel), warp 1 tensor memory and, in CTA 0, the multiply-adds, warps 2-5 store (thread = operand row, 32 bytes per
+// store instruction).
+constexpr int WN = 256, WTHREADS = 192, W_TILE = 128 * TC_BK * 2;   // 16 KB: 128 rows x 64 elements
+constexpr int W_SMEM_TILES = 12;                                     // 192 KB ring: 4 stages of 3 tiles, or 6 of 2 (half tiles only)
+constexpr int W_MAX_STAGES = 6;
+constexpr int W_CHAIN = 32;   // K blocks (of 64 elements) per accumulation chain
 
 struct WSmem {
-    unsigned long long full[WSTAGES], empty[WSTAGES], tfull;
+    unsigned long long full[W_MAX_STAGES], empty[W_MAX_STAGES], tfull[2], tempty[2];
     unsigned tmem_base;
     int abort;
 };
 
+// The share of a pair, walked piece by piece.
+struct WPiece {
+    int nt, mt, kb0, kb1;   // tile and its K blocks
+    bool half, first;       // first piece of this share in the tile: stores, later ones add
+};
+struct WWalk {
+    const ClWideParts &p;
+    int chain, nt, mt, kb, c, c1;   // next K block; cost of all blocks before it; end of the share
+    bool fresh;
+    __device__ WWalk(const ClWideParts &parts, int pair, int chain_) : p(parts), chain(chain_), fresh(true) {
+        const int T = cl_wide_cost(p), W = cl_wide_col_cost(p), c0 = (int)((long long)T * pair / p.G);
+        c1 = (int)((long long)T * (pair + 1) / p.G);
+        nt = c0 / W;
+        const int rem = c0 - nt * W, full = 2 * p.KB * p.MT;
+        if (rem < full) {
+            mt = rem / (2 * p.KB);
+            kb = (rem - mt * 2 * p.KB + 1) >> 1;   // a boundary inside a block of cost 2 belongs to the pair before it
+        } else {
+            mt = p.MT;
+            kb = rem - full;
+        }
+        c = nt * W + (mt < p.MT ? 2 * (mt * p.KB + kb) : full + kb);
+        if (kb == p.KB) step();
+    }
+    __device__ void step() {   // to the next tile
+        kb = 0;
+        if (++mt == p.MT + p.half) { mt = 0; ++nt; }
+    }
+    __device__ bool next(WPiece &o) {
+        if (c >= c1) return false;
+        o.nt = nt; o.mt = mt; o.half = mt == p.MT;
+        o.kb0 = kb;
+        const int left = o.half ? c1 - c : (c1 - c + 1) >> 1;
+        o.kb1 = min(min(p.KB, kb + chain), kb + left);
+        o.first = fresh || kb == 0;
+        fresh = false;
+        c += (o.kb1 - kb) * (o.half ? 1 : 2);
+        kb = o.kb1;
+        if (kb == p.KB) step();
+        return true;
+    }
+};
+
 __global__ void __launch_bounds__(WTHREADS, 1)
-k_wide(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, ClWideArgs a) {
+k_wide(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const __grid_constant__ ClWideArgs a) {
+    const int stage_tiles = a.p.MT ? 3 : 2, stages = W_SMEM_TILES / stage_tiles, stage_bytes = stage_tiles * W_TILE;
     extern __shared__ unsigned char smem_dyn[];
     unsigned char *tiles = (unsigned char *)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
-    WSmem *sm = (WSmem *)(tiles + (size_t)WSTAGES * WSTAGE_BYTES);
+    WSmem *sm = (WSmem *)(tiles + (size_t)W_SMEM_TILES * W_TILE);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int cta = blockIdx.x;
-    if (cta >= a.MT * a.NT * a.splits) return;   // whole CTA leaves before anything is set up
-    const int mt = cta % a.MT, nt = (cta / a.MT) % a.NT, ks = cta / (a.MT * a.NT);
-    const int kb0 = (int)((long long)a.KB * ks / a.splits), kb1 = (int)((long long)a.KB * (ks + 1) / a.splits);
+    const int rank = (int)cluster_rank(), pair = blockIdx.x >> 1;
 
     if (tid == 0) {
-        for (int i = 0; i < WSTAGES; ++i) {
+        for (int i = 0; i < W_MAX_STAGES; ++i) {
             bar_init(&sm->full[i], 1);
             bar_init(&sm->empty[i], 1);
         }
-        bar_init(&sm->tfull, 1);
+        for (int i = 0; i < 2; ++i) {
+            bar_init(&sm->tfull[i], 1);
+            bar_init(&sm->tempty[i], 8);   // the store warps of both CTAs
+        }
         sm->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(s_u32(&sm->tmem_base)) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s_u32(&sm->tmem_base)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    cluster_sync();   // the peer's barriers exist before anything signals them
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    pdl_launch_dependents();
     const unsigned tmem = *(volatile unsigned *)&sm->tmem_base;
 
+    WWalk walk(a.p, pair, a.chain);
+    WPiece pc;
     if (warp == 0) {
-        // ---------------- TMA producer ----------------
+        // ---------------- TMA producer: this CTA's operand rows and its half of the weight rows ----------------
         if (lane == 0) {
-            unsigned stage = 0, par = 0, issued[WSTAGES];
-            for (int i = 0; i < WSTAGES; ++i) issued[i] = 2u;
-            bool ok = true;
-            for (int kb = kb0; kb < kb1; ++kb) {
-                if (!bar_wait(&sm->empty[stage], par ^ 1u, &sm->abort, a.err)) { ok = false; break; }
-                unsigned char *dst = tiles + (size_t)stage * WSTAGE_BYTES;
-                bar_expect(&sm->full[stage], WSTAGE_BYTES);
-                tma_load_2d(dst, &mapA, kb * TC_BK, mt * WM, &sm->full[stage]);
-                tma_load_2d(dst + WA_BYTES, &mapA, kb * TC_BK, a.lo_row0 + mt * WM, &sm->full[stage]);
-                tma_load_2d(dst + 2 * WA_BYTES, &mapB, kb * TC_BK, nt * WN, &sm->full[stage]);
-                tma_load_2d(dst + 2 * WA_BYTES + WB_BYTES / 2, &mapB, kb * TC_BK, nt * WN + WN / 2, &sm->full[stage]);
-                issued[stage] = par;
-                if (++stage == WSTAGES) { stage = 0; par ^= 1u; }
-            }
-            if (!ok) {   // gave up: still let the copies in flight land before the CTA may exit (bounded)
-                for (int i = 0; i < WSTAGES; ++i) {
-                    if (issued[i] < 2u) {
-                        const unsigned long long t0 = gtime_ns();
-                        while (!bar_try(&sm->full[i], issued[i]))
-                            if (gtime_ns() - t0 > WAIT_NS) break;
-                    }
+            auto load_b = [&](const WPiece &t, int kb, int s) {
+                if (rank == 0) bar_expect(&sm->full[s], 2 * (t.half ? 2 : 3) * W_TILE);   // both CTAs' copies count on CTA 0's barrier
+                tma_load_2d_pair(tiles + (size_t)s * stage_bytes + (stage_tiles - 1) * W_TILE, &mapB, kb * TC_BK,
+                                 t.nt * WN + rank * 128, &sm->full[s]);
+            };
+            auto load_a = [&](const WPiece &t, int kb, int s) {
+                unsigned char *dst = tiles + (size_t)s * stage_bytes;
+                if (t.half) {
+                    tma_load_2d_pair(dst, &mapA, kb * TC_BK, t.mt * 256 + rank * a.lo_row0, &sm->full[s]);
+                } else {
+                    tma_load_2d_pair(dst, &mapA, kb * TC_BK, t.mt * 256 + rank * 128, &sm->full[s]);
+                    tma_load_2d_pair(dst + W_TILE, &mapA, kb * TC_BK, a.lo_row0 + t.mt * 256 + rank * 128, &sm->full[s]);
                 }
+            };
+            // the weights of the first stages before the operand rows, which come from the previous kernel
+            int n_pre = 0;
+            {
+                WWalk w(walk);
+                while (n_pre < stages && w.next(pc))
+                    for (int kb = pc.kb0; kb < pc.kb1 && n_pre < stages; ++kb) load_b(pc, kb, n_pre++);
+            }
+            pdl_wait();
+            bool ok = true;
+            int s = 0, i = 0;
+            unsigned par = 1u;
+            while (ok && walk.next(pc)) {
+                for (int kb = pc.kb0; kb < pc.kb1; ++kb, ++i) {
+                    if (i >= n_pre) {
+                        if (!bar_wait(&sm->empty[s], par, &sm->abort, a.err)) { ok = false; break; }
+                        load_b(pc, kb, s);
+                    }
+                    load_a(pc, kb, s);
+                    if (++s == stages) { s = 0; par ^= 1u; }
+                }
+            }
+            if (!ok) {   // gave up: let the copies in flight land (they signal CTA 0, so this CTA can only give them time)
+                const unsigned long long t0 = gtime_ns();
+                while (gtime_ns() - t0 < 2000000ull) {}
             }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            const unsigned idesc = umma_idesc(WM, WN, a.f16);
-            unsigned stage = 0, par = 0;
+        // ---------------- MMA issuer (CTA 0, for both) ----------------
+        if (lane == 0 && rank == 0) {
+            const unsigned idesc = umma_idesc(256, WN, a.f16);
+            int s = 0, n = 0;
+            unsigned par = 0u;
             bool ok = true;
-            for (int kb = kb0; kb < kb1; ++kb) {
-                if (!bar_wait(&sm->full[stage], par, &sm->abort, a.err)) { ok = false; break; }
+            while (ok && walk.next(pc)) {
+                const unsigned b = (unsigned)n & 1u, acc = tmem + b * WN;
+                if (!bar_wait(&sm->tempty[b], ((unsigned)(n >> 1) & 1u) ^ 1u, &sm->abort, a.err)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const unsigned hi_addr = s_u32(tiles + (size_t)stage * WSTAGE_BYTES), lo_addr = hi_addr + WA_BYTES,
-                               b_addr = hi_addr + 2 * WA_BYTES;
+                for (int kb = pc.kb0; kb < pc.kb1; ++kb) {
+                    if (!bar_wait(&sm->full[s], par, &sm->abort, a.err)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const unsigned hi_addr = s_u32(tiles + (size_t)s * stage_bytes), b_addr = hi_addr + (stage_tiles - 1) * W_TILE;
 #pragma unroll
-                for (int k = 0; k < TC_BK / 16; ++k) {
-                    umma_bf16(tmem, umma_desc(hi_addr + k * 32), umma_desc(b_addr + k * 32), idesc, (unsigned)((kb - kb0) | k));
-                    umma_bf16(tmem, umma_desc(lo_addr + k * 32), umma_desc(b_addr + k * 32), idesc, 1u);
+                    for (int k = 0; k < TC_BK / 16; ++k) {
+                        umma_pair(acc, umma_desc(hi_addr + k * 32), umma_desc(b_addr + k * 32), idesc, (unsigned)((kb - pc.kb0) | k));
+                        if (!pc.half) umma_pair(acc, umma_desc(hi_addr + W_TILE + k * 32), umma_desc(b_addr + k * 32), idesc, 1u);
+                    }
+                    umma_commit_pair(&sm->empty[s]);   // free in both CTAs once these multiply-adds have read it
+                    if (++s == stages) { s = 0; par ^= 1u; }
                 }
-                umma_commit(&sm->empty[stage]);   // the stage is free once these multiply-adds have read it
-                if (++stage == WSTAGES) { stage = 0; par ^= 1u; }
+                if (ok) umma_commit_pair(&sm->tfull[b]);
+                ++n;
             }
-            if (ok) umma_commit(&sm->tfull);
         }
     } else {
-        // ---------------- store: one thread per token row ----------------
+        // ---------------- store: one thread per operand row ----------------
         const int q = warp & 3;                        // the tensor-memory lane quadrant this warp may read
-        const int t = mt * WM + q * 32 + lane;
-        if (bar_wait(&sm->tfull, 0u, &sm->abort, a.err)) {
+        pdl_wait();   // the previous kernel may still read the product buffer
+        for (int n = 0; walk.next(pc); ++n) {
+            const unsigned b = (unsigned)n & 1u;
+            if (!bar_wait(&sm->tfull[b], (unsigned)(n >> 1) & 1u, &sm->abort, a.err)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float *dst = a.P + ((size_t)ks * a.M + (size_t)min(t, a.M - 1)) * a.rows;
+            int part = pair - cl_wide_owner(a.p, pc.nt, pc.mt, 0);
+            int t = pc.mt * 256 + q * 32 + lane;
+            if (pc.half) part = 2 * part + rank;
+            else t += rank * 128;
+            float *dst = a.p.P + ((size_t)part * a.p.M + (size_t)min(t, a.p.M - 1)) * a.p.rows;
 #pragma unroll 1
             for (int cb = 0; cb < WN / 32; ++cb) {
                 float v[32];
-                tmem_ld32(tmem + ((unsigned)(q * 32) << 16) + (unsigned)(cb * 32), v);   // (whole warp, also for rows past M)
-                const int col0 = nt * WN + cb * 32;
-                if (t < a.M) {
+                tmem_ld32(tmem + b * WN + ((unsigned)(q * 32) << 16) + (unsigned)(cb * 32), v);   // (whole warp, also rows past M)
+                const int col0 = pc.nt * WN + cb * 32;
+                if (t < a.p.M) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (col0 + 4 * i + 4 <= a.rows)
-                            *(float4 *)(dst + col0 + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                    for (int i = 0; i < 4; ++i) {
+                        if (col0 + 8 * i + 8 <= a.p.rows) {
+                            if (pc.first) st_global_v8(dst + col0 + 8 * i, v + 8 * i);
+                            else red_add_v8(dst + col0 + 8 * i, v + 8 * i);
+                        }
+                    }
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) bar_arrive_rank0(&sm->tempty[b]);
         }
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    cluster_sync();   // CTA 0's multiply-adds read CTA 1's shared memory, and both signal each other's barriers
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
 }
 
+// Number of product parts at (row t, column col): the pairs that share the tile, twice in a half tile.
+__device__ __forceinline__ int wide_parts(const ClWideParts &p, int t, int col) {
+    const int nt = col >> 8, mt = t >> 8;
+    return (cl_wide_owner(p, nt, mt, p.KB - 1) - cl_wide_owner(p, nt, mt, 0) + 1) << (mt == p.MT);
+}
+
 // One CTA per token row: x[t] = E[token] or x[t] += product parts (added in part order); the optional hidden tap;
-// then the rows of the next GEMM: hi/lo(x * rsqrt(mean x^2 + eps) * g).
-__global__ void __launch_bounds__(256) k_wide_norm(ClWideNormArgs a) {
-    __shared__ float red[8];
-    const int t = blockIdx.x, tid = threadIdx.x, d = a.d;
+// then the rows of the next GEMM: hi/lo(x * rsqrt(mean x^2 + eps) * g).  A thread's elements stay in registers between
+// the two passes (up to two chunks of 4; the rest is read again).  As many threads as there are chunks of 4, up to 1024: with few
+// rows the loads in flight per SM are what bounds it.
+__global__ void __launch_bounds__(1024) k_wide_norm(ClWideNormArgs a) {
+    __shared__ float red[32];
+    constexpr int KEEP = 2;
+    pdl_launch_dependents();
+    const int t = blockIdx.x, tid = threadIdx.x, d = a.d, span = 4 * blockDim.x;   // columns per round of the CTA
     float *xr = a.x + (size_t)t * d;
+    float4 keep[KEEP], gain[KEEP];
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k) {   // (gains are weights: read ahead of the wait)
+        const int i = tid * 4 + k * span;
+        gain[k] = (a.g && i < d) ? __ldg((const float4 *)(a.g + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    pdl_wait();
     const unsigned short *er = a.tok ? (const unsigned short *)a.embed + (size_t)a.tok[t] * d : nullptr;
     // only the last tap_P rows of the pass reach the ring: an earlier row of the same slot would be overwritten anyway
     unsigned short *tap = nullptr;
     if (a.tap && t >= a.M - a.tap_P) tap = (unsigned short *)a.tap + (size_t)((a.st->ctx + t) % a.tap_P) * d;
+    const size_t plane = (size_t)a.M * d;
     float ss = 0.f;
-    for (int i = tid * 4; i < d; i += 1024) {
+    auto element = [&](int i) -> float4 {   // the updated stream at columns i .. i + 3
         float4 v;
         if (er) {
             const uint2 u = *(const uint2 *)(er + i);
@@ -162,330 +282,418 @@ __global__ void __launch_bounds__(256) k_wide_norm(ClWideNormArgs a) {
             pair16_to_f32(u.y, a.f16, v.z, v.w);
         } else {
             v = *(const float4 *)(xr + i);
-            for (int s = 0; s < a.splits; ++s) {
-                const float4 p = __ldcg((const float4 *)(a.P + ((size_t)s * a.M + t) * d + i));
+            const int n = wide_parts(a.parts, t, i);
+            const float *p0 = a.parts.P + (size_t)t * d + i;
+#pragma unroll 4
+            for (int s = 0; s < n; ++s) {
+                const float4 p = __ldcg((const float4 *)(p0 + (size_t)s * plane));
                 v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
             }
         }
         *(float4 *)(xr + i) = v;
         if (tap) {
-            tap[i] = f32_to_b16(v.x, a.f16); tap[i + 1] = f32_to_b16(v.y, a.f16);
-            tap[i + 2] = f32_to_b16(v.z, a.f16); tap[i + 3] = f32_to_b16(v.w, a.f16);
+            const unsigned lo2 = (unsigned)f32_to_b16(v.x, a.f16) | ((unsigned)f32_to_b16(v.y, a.f16) << 16);
+            const unsigned hi2 = (unsigned)f32_to_b16(v.z, a.f16) | ((unsigned)f32_to_b16(v.w, a.f16) << 16);
+            *(uint2 *)(tap + i) = make_uint2(lo2, hi2);
         }
         ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
+        return v;
+    };
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k) {
+        const int i = tid * 4 + k * span;
+        if (i < d) keep[k] = element(i);
     }
+    for (int i = tid * 4 + KEEP * span; i < d; i += span) element(i);
     if (!a.g) return;   // uniform
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
     if ((tid & 31) == 0) red[tid >> 5] = ss;
     __syncthreads();
     float tot = 0.f;
-    for (int w = 0; w < 8; ++w) tot += red[w];   // fixed order
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];   // fixed order
     const float sc = 1.0f / sqrtf(tot / (float)d + a.eps);
     __nv_bfloat16 *hi = a.A + (size_t)t * d, *lo = a.A + (size_t)(a.lo_row0 + t) * d;
-    for (int i = tid * 4; i < d; i += 1024) {
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k) {
+        const int i = tid * 4 + k * span;
+        if (i < d) store_split4(hi + i, lo + i, keep[k].x * sc * gain[k].x, keep[k].y * sc * gain[k].y, keep[k].z * sc * gain[k].z,
+                                keep[k].w * sc * gain[k].w, a.f16);
+    }
+    for (int i = tid * 4 + KEEP * span; i < d; i += span) {
         const float4 v = *(const float4 *)(xr + i);   // this thread's own writes
         const float4 g = *(const float4 *)(a.g + i);
-        store_split(hi + i, lo + i, v.x * sc * g.x, a.f16);
-        store_split(hi + i + 1, lo + i + 1, v.y * sc * g.y, a.f16);
-        store_split(hi + i + 2, lo + i + 2, v.z * sc * g.z, a.f16);
-        store_split(hi + i + 3, lo + i + 3, v.w * sc * g.w, a.f16);
+        store_split4(hi + i, lo + i, v.x * sc * g.x, v.y * sc * g.y, v.z * sc * g.z, v.w * sc * g.w, a.f16);
     }
 }
 
-// grid (M, H), hd / 2 threads: q, k, v of row t and head h from the QKV product parts; rotary embedding at position
-// ctx + t; q goes back in place (part 0), k and v (the first Hkv heads) go to the cache [kv head][position][hd].
-__global__ void k_wide_rope_append(float *P, int splits, int M, int hd, int d, int Hkv, const float2 *rope_cs,
-                                   unsigned short *kcache, unsigned short *vcache, int max_seq, const ClDevState *st, int f16) {
-    const int t = blockIdx.x, h = blockIdx.y, i = threadIdx.x, half = hd >> 1;
+// One item = the four rotary pairs (i .. i + 3, + hd / 2) of one head of one row: q heads first, then k heads, then the
+// same shape over v (no rotation).  Rotary embedding at position ctx + t; q goes back in place (part 0), k and v go to the
+// cache [kv head][position][hd].  grid (M, ceil(items / 256)).
+__global__ void __launch_bounds__(256) k_wide_rope_append(ClWideParts p, int hd, int d, int Hkv, const float2 *rope_cs,
+                                                          unsigned short *kcache, unsigned short *vcache, int max_seq,
+                                                          const ClDevState *st, int f16) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int t = blockIdx.x, half = hd >> 1, per_head = half >> 2, H = d / hd;
+    const int item = blockIdx.y * 256 + threadIdx.x;
+    const int head = item / per_head, i = (item - head * per_head) * 4;
     const int pos = st->ctx + t;
-    if (pos >= max_seq) return;
-    const int kvd = Hkv * hd, ld = d + 2 * kvd;
-    const size_t part = (size_t)M * ld;
-    float *row = P + (size_t)t * ld;
-    auto total = [&](int col) {
-        float v = row[col];
-        for (int s = 1; s < splits; ++s) v += __ldcg(row + (size_t)s * part + col);
+    if (head >= H + 2 * Hkv || pos >= max_seq) return;
+    const int ld = p.rows, col = head * hd + i;   // [q heads | k heads | v heads]
+    const size_t plane = (size_t)p.M * ld;
+    float *row = p.P + (size_t)t * ld;
+    auto total = [&](int c) {
+        const int n = wide_parts(p, t, c);
+        float4 v = __ldcg((const float4 *)(row + c));
+#pragma unroll 2
+        for (int s = 1; s < n; ++s) {
+            const float4 w = __ldcg((const float4 *)(row + (size_t)s * plane + c));
+            v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+        }
         return v;
     };
-    const float2 cs = rope_cs[(size_t)pos * half + i];
-    const float qa = total(h * hd + i), qb = total(h * hd + i + half);
-    row[h * hd + i] = qa * cs.x - qb * cs.y;
-    row[h * hd + i + half] = qb * cs.x + qa * cs.y;
-    if (h >= Hkv) return;
-    const float ka = total(d + h * hd + i), kb = total(d + h * hd + i + half);
-    unsigned short *kc = kcache + ((size_t)h * max_seq + pos) * hd, *vc = vcache + ((size_t)h * max_seq + pos) * hd;
-    kc[i] = f32_to_b16(ka * cs.x - kb * cs.y, f16);
-    kc[i + half] = f32_to_b16(kb * cs.x + ka * cs.y, f16);
-    vc[i] = f32_to_b16(total(d + kvd + h * hd + i), f16);
-    vc[i + half] = f32_to_b16(total(d + kvd + h * hd + i + half), f16);
+    float4 x = total(col), y = total(col + half);
+    if (head < H + Hkv) {
+        const float4 c01 = *(const float4 *)(rope_cs + (size_t)pos * half + i), c23 = *(const float4 *)(rope_cs + (size_t)pos * half + i + 2);
+        const float4 a = x, b = y;
+        x = make_float4(a.x * c01.x - b.x * c01.y, a.y * c01.z - b.y * c01.w, a.z * c23.x - b.z * c23.y, a.w * c23.z - b.w * c23.w);
+        y = make_float4(b.x * c01.x + a.x * c01.y, b.y * c01.z + a.y * c01.w, b.z * c23.x + a.z * c23.y, b.w * c23.z + a.w * c23.w);
+    }
+    if (head < H) {
+        *(float4 *)(row + col) = x;
+        *(float4 *)(row + col + half) = y;
+        return;
+    }
+    unsigned short *dst = (head < H + Hkv ? kcache + ((size_t)(head - H) * max_seq + pos) * hd
+                                          : vcache + ((size_t)(head - H - Hkv) * max_seq + pos) * hd) + i;
+    auto pack = [&](const float4 &v) {
+        return make_uint2((unsigned)f32_to_b16(v.x, f16) | ((unsigned)f32_to_b16(v.y, f16) << 16),
+                          (unsigned)f32_to_b16(v.z, f16) | ((unsigned)f32_to_b16(v.w, f16) << 16));
+    };
+    *(uint2 *)dst = pack(x);
+    *(uint2 *)(dst + half) = pack(y);
 }
 
 // ---- causal attention of the rows of the pass over the cache -------------------------------------------------
-// grid (H, blocks of 64 rows), 256 threads.  Row t sits at position ctx + t and attends to the keys 0 .. ctx + t
-// (its own key is already in the cache).  The keys are walked 64 at a time; per tile the 64 x 64 scores
-// S = Q K^T and the update O += P V are register-tiled fp32 products out of shared memory (thread (ty, tx): rows
-// 4 ty .. 4 ty + 3; keys 4 tx .. 4 tx + 3 of S; columns tx * 4 + 64 v .. of O), with the usual running maximum and
-// sum per row.  The 16 threads of a row group are half a warp, so row reductions are four shuffles.  Blocks of
-// late rows see the most keys and are scheduled first.
-constexpr int AQ = 64, AK = 64, APS = 68;   // rows per CTA, keys per tile, row stride of the probability tile
+// grid (H, blocks of 64 rows), 4 warps of 16 rows each.  Row t sits at position ctx + t and attends to the keys 0 .. ctx + t
+// (its own key is already in the cache).  Keys and values are walked 64 at a time through two shared-memory buffers
+// (cp.async, 16-byte pieces permuted by row & 7), with the usual running maximum and sum per row.
+// Both products run on the tensor cores although the queries and the probabilities are fp32: each enters as three parts
+// of the storage type (v = p0 + p1 + p2 holds 24 bits of it; keys and values are of that type already), so the products are
+// as exact as fp32 ones.  A query row is scaled by a power of two to [1, 2) first, so that the parts of fp16 neither
+// overflow nor underflow.  Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile), 2 % of the
+// pass; the register-tiled fp32 products on the CUDA cores that it replaces took 122 us per layer at 512 rows of 32 heads
+// against 393 us of GEMMs and other kernels.  Blocks of late rows see the most keys and are scheduled first.
+constexpr int AQ = 64, AK = 64;   // rows per CTA, keys per tile
 
 template <int HD>
-__global__ void __launch_bounds__(256, 2)
-k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsigned short *vcache, __nv_bfloat16 *out_b,
-            int lo_row0, int M, int d, int H, int Hkv, int max_seq, const ClDevState *st, int f16) {
-    constexpr int NV = HD / 64;                       // float4 column groups of O per thread
-    constexpr int KP = (HD * AK > AQ * APS) ? HD * AK : AQ * APS;
-    extern __shared__ __align__(16) float asm_[];
-    float *Qt = asm_;              // [HD][AQ]   queries, transposed, scaled by 1 / sqrt(hd)
-    float *Kt = Qt + HD * AQ;      // [HD][AK]   keys of the tile, transposed; reused as Ps [AQ][APS] (probabilities)
-    float *Vs = Kt + KP;           // [AK][HD]   values of the tile
-    float *Ps = Kt;
-    const int h = blockIdx.x, qb = (int)gridDim.y - 1 - (int)blockIdx.y;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int ctx = st->ctx, r0 = qb * AQ;
-    const int rlast = min(r0 + AQ, M) - 1;            // last live row of this block
-    const int nkeys = min(ctx + rlast + 1, max_seq);
-    const int kvh = h / (H / Hkv);
-    const unsigned short *Kc = kcache + (size_t)kvh * max_seq * HD, *Vc = vcache + (size_t)kvh * max_seq * HD;
-    const float scale = rsqrtf((float)HD);
+constexpr size_t attn_wide_smem() { return (size_t)(3 * AQ + 4 * AK) * HD * 2 + AQ * 4; }
 
-    for (int i = tid; i < AQ * HD / 4; i += 256) {
-        const int row = i % AQ, c4 = i / AQ;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r0 + row < M) v = *(const float4 *)(q + (size_t)(r0 + row) * ld_q + h * HD + c4 * 4);
-        Qt[(c4 * 4 + 0) * AQ + row] = v.x * scale;
-        Qt[(c4 * 4 + 1) * AQ + row] = v.y * scale;
-        Qt[(c4 * 4 + 2) * AQ + row] = v.z * scale;
-        Qt[(c4 * 4 + 3) * AQ + row] = v.w * scale;
-    }
-    float m_run[4], l_run[4], o[4][NV][4];
+__device__ __forceinline__ void ldsm4(unsigned (&r)[4], unsigned addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(unsigned (&r)[4], unsigned addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+template <int F16>
+__device__ __forceinline__ void mma16816(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+    if (F16)
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+    else
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Two values -> three packed pairs of the 16-bit type whose sums are the values to 24 bits.
+template <int F16>
+__device__ __forceinline__ void split3(float x, float y, unsigned (&o)[3]) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        m_run[i] = -INFINITY;
-        l_run[i] = 0.f;
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) o[i][v][e] = 0.f;
-    }
-
-    for (int k0 = 0; k0 < nkeys; k0 += AK) {
-        __syncthreads();   // the previous tile's reads of Ps and Vs are over (and Qt is written, first time round)
-        // keys: thread -> (key, 8 head-dim elements); transposed to Kt.  values: natural layout.
-        for (int i = tid; i < AK * HD / 8; i += 256) {
-            const int key = i % AK, c8 = i / AK;
-            uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-            if (k0 + key < nkeys) raw = *(const uint4 *)(Kc + (size_t)(k0 + key) * HD + c8 * 8);
-            const unsigned u[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                pair16_to_f32(u[e], f16, Kt[(c8 * 8 + 2 * e) * AK + key], Kt[(c8 * 8 + 2 * e + 1) * AK + key]);
-            }
-        }
-        for (int i = tid; i < AK * HD / 8; i += 256) {
-            const int key = i / (HD / 8), c8 = i % (HD / 8);
-            uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-            if (k0 + key < nkeys) raw = *(const uint4 *)(Vc + (size_t)(k0 + key) * HD + c8 * 8);
-            float4 *dst = (float4 *)(Vs + key * HD + c8 * 8);
-            float4 lo4, hi4;
-            pair16_to_f32(raw.x, f16, lo4.x, lo4.y);
-            pair16_to_f32(raw.y, f16, lo4.z, lo4.w);
-            pair16_to_f32(raw.z, f16, hi4.x, hi4.y);
-            pair16_to_f32(raw.w, f16, hi4.z, hi4.w);
-            dst[0] = lo4;
-            dst[1] = hi4;
-        }
-        __syncthreads();
-        float sc[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) sc[i][j] = 0.f;
-#pragma unroll 8
-        for (int k = 0; k < HD; ++k) {
-            const float4 qv = *(const float4 *)(Qt + k * AQ + 4 * ty);
-            const float4 kv = *(const float4 *)(Kt + k * AK + 4 * tx);
-            const float qa[4] = {qv.x, qv.y, qv.z, qv.w}, ka[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) sc[i][j] = fmaf(qa[i], ka[j], sc[i][j]);
-        }
-        __syncthreads();   // everyone is done with Kt: it becomes Ps
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int pos = ctx + r0 + 4 * ty + i;   // causal limit of this row
-            const bool live = r0 + 4 * ty + i < M;
-            float mx = -INFINITY;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (!(live && k0 + 4 * tx + j <= pos)) sc[i][j] = -INFINITY;
-                mx = fmaxf(mx, sc[i][j]);
-            }
-#pragma unroll
-            for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-            const float m_new = fmaxf(m_run[i], mx);
-            float p[4] = {0.f, 0.f, 0.f, 0.f}, ps = 0.f, resc = 1.f;
-            if (m_new > -INFINITY) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    p[j] = (sc[i][j] > -INFINITY) ? expf(sc[i][j] - m_new) : 0.f;
-                    ps += p[j];
-                }
-                resc = (m_run[i] > -INFINITY) ? expf(m_run[i] - m_new) : 0.f;
-                m_run[i] = m_new;
-            }
-#pragma unroll
-            for (int w = 8; w > 0; w >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, w);
-            l_run[i] = fmaf(l_run[i], resc, ps);
-#pragma unroll
-            for (int v = 0; v < NV; ++v)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) o[i][v][e] *= resc;
-            *(float4 *)(Ps + (4 * ty + i) * APS + 4 * tx) = make_float4(p[0], p[1], p[2], p[3]);
-        }
-        __syncthreads();
-#pragma unroll 2
-        for (int kk = 0; kk < AK; kk += 4) {
-            float pr[4][4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float4 t4 = *(const float4 *)(Ps + (4 * ty + i) * APS + kk);
-                pr[i][0] = t4.x; pr[i][1] = t4.y; pr[i][2] = t4.z; pr[i][3] = t4.w;
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    const float4 vv = *(const float4 *)(Vs + (kk + j) * HD + v * 64 + tx * 4);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        o[i][v][0] = fmaf(pr[i][j], vv.x, o[i][v][0]);
-                        o[i][v][1] = fmaf(pr[i][j], vv.y, o[i][v][1]);
-                        o[i][v][2] = fmaf(pr[i][j], vv.z, o[i][v][2]);
-                        o[i][v][3] = fmaf(pr[i][j], vv.w, o[i][v][3]);
-                    }
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int row = r0 + 4 * ty + i;
-        if (row >= M || !(l_run[i] > 0.f)) continue;
-        const float inv = 1.f / l_run[i];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const size_t col = (size_t)h * HD + v * 64 + tx * 4;
-            unsigned hi[4], lo[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                unsigned short bh, bl;
-                split_b16(o[i][v][e] * inv, f16, bh, bl);
-                hi[e] = bh;
-                lo[e] = bl;
-            }
-            *(uint2 *)(out_b + (size_t)row * d + col) = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
-            *(uint2 *)(out_b + (size_t)(lo_row0 + row) * d + col) = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
-        }
+    for (int i = 0; i < 3; ++i) {
+        const unsigned short a = f32_to_b16(x, F16), b = f32_to_b16(y, F16);
+        o[i] = (unsigned)a | ((unsigned)b << 16);
+        x -= b16_to_f32(a, F16);
+        y -= b16_to_f32(b, F16);
     }
 }
 
-// grid (M, ceil(F / 256)): the gate/up product has rows interleaved (2 i = gate_i, 2 i + 1 = up_i).
-__global__ void __launch_bounds__(256) k_wide_silu(const float *P, int splits, int M, int F, __nv_bfloat16 *A, int lo_row0, int f16) {
-    const int t = blockIdx.x, i = blockIdx.y * 256 + threadIdx.x;
-    if (i >= F) return;
-    float g = 0.f, u = 0.f;
-    for (int s = 0; s < splits; ++s) {
-        const float2 p = __ldcg((const float2 *)(P + ((size_t)s * M + t) * 2 * F) + i);
-        g += p.x;
-        u += p.y;
+template <int HD, int F16>
+__global__ void __launch_bounds__(128, 2)
+k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsigned short *vcache, __nv_bfloat16 *out_b,
+            int lo_row0, int M, int d, int H, int Hkv, int max_seq, const ClDevState *st) {
+    constexpr int RB = HD * 2, NC = HD / 8;           // bytes and 16-byte pieces per row
+    extern __shared__ __align__(128) unsigned char asm_[];
+    unsigned char *Qs = asm_;                          // [3][AQ][RB] parts of the scaled queries
+    float *rs = (float *)(asm_ + (3 * AQ + 4 * AK) * RB);   // [AQ] what a row's scores are multiplied by
+    const unsigned q_addr = s_u32(Qs), kv_addr = q_addr + 3 * AQ * RB;   // [2 buffers][keys | values][AK][RB]
+    pdl_launch_dependents();
+    pdl_wait();
+    const int h = blockIdx.x, r0 = ((int)gridDim.y - 1 - (int)blockIdx.y) * AQ;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int ctx = st->ctx;
+    const int nkeys = min(ctx + min(r0 + AQ, M), max_seq), ntiles = (nkeys + AK - 1) / AK;
+    const int kvh = h / (H / Hkv);
+    const unsigned short *Kc = kcache + (size_t)kvh * max_seq * HD, *Vc = vcache + (size_t)kvh * max_seq * HD;
+
+    auto load_tile = [&](int tile) {
+        const unsigned base = kv_addr + (unsigned)(tile & 1) * 2 * AK * RB;
+        for (int i = tid; i < AK * NC; i += 128) {
+            const int key = i / NC, c = i % NC, src = min(tile * AK + key, nkeys - 1);
+            const unsigned dst = base + key * RB + ((c ^ (key & 7)) << 4), n = tile * AK + key < nkeys ? 16u : 0u;   // (zeros past the end)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(Kc + (size_t)src * HD + c * 8), "r"(n) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + AK * RB), "l"(Vc + (size_t)src * HD + c * 8), "r"(n) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    load_tile(0);
+
+    // this warp's 16 query rows: scaled to [1, 2) by a power of two, split, stored; nobody else reads them
+    constexpr int EL = HD / 32;
+#pragma unroll 4
+    for (int rr = 0; rr < 16; ++rr) {
+        const int row = warp * 16 + rr;
+        float v[EL], amax = 0.f;
+#pragma unroll
+        for (int e = 0; e < EL; ++e) v[e] = r0 + row < M ? __ldcg(q + (size_t)(r0 + row) * ld_q + h * HD + lane * EL + e) : 0.f;
+#pragma unroll
+        for (int e = 0; e < EL; ++e) amax = fmaxf(amax, fabsf(v[e]));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        const unsigned ex = min(max(__float_as_uint(amax) >> 23, 1u), 253u);
+        const float inv = __uint_as_float((254u - ex) << 23);
+#pragma unroll
+        for (int e = 0; e < EL; e += 2) {
+            unsigned s3[3];
+            split3<F16>(v[e] * inv, v[e + 1] * inv, s3);
+            const int byte = (lane * EL + e) * 2;
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+                *(unsigned *)(Qs + (size_t)(p * AQ + row) * RB + (((byte >> 4) ^ (row & 7)) << 4) + (byte & 15)) = s3[p];
+        }
+        if (lane == 0) rs[row] = __uint_as_float(ex << 23) * rsqrtf((float)HD);
     }
-    const float h = g / (1.f + expf(-g)) * u;
-    store_split(A + (size_t)t * F + i, A + (size_t)(lo_row0 + t) * F + i, h, f16);
+    __syncwarp();
+
+    const int lr = lane >> 2, lc = (lane & 3) * 2;     // accumulator: rows lr and lr + 8, columns lc and lc + 1 of a tile of 8
+    const int mrow = lane & 7, mi = lane >> 3;         // ldmatrix: this lane's row and matrix
+    const int row_a = r0 + warp * 16 + lr, pos_a = row_a < M ? ctx + row_a : -1, pos_b = row_a + 8 < M ? ctx + row_a + 8 : -1;
+    const float rs_a = rs[warp * 16 + lr], rs_b = rs[warp * 16 + lr + 8];
+    float o[HD / 8][4], m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
+#pragma unroll
+    for (int n = 0; n < HD / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
+
+    for (int t = 0; t < ntiles; ++t) {
+        if (t + 1 < ntiles) {
+            load_tile(t + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const int k0 = t * AK;
+        const unsigned ka = kv_addr + (unsigned)(t & 1) * 2 * AK * RB, va = ka + AK * RB;
+        float s[AK / 8][4];
+#pragma unroll
+        for (int n = 0; n < AK / 8; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < HD / 16; ++ks) {
+            unsigned qa[3][4];
+            const int qr = warp * 16 + (mi & 1) * 8 + mrow, qc = ks * 2 + (mi >> 1);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) ldsm4(qa[p], q_addr + (p * AQ + qr) * RB + ((qc ^ (qr & 7)) << 4));
+#pragma unroll
+            for (int np = 0; np < AK / 16; ++np) {
+                unsigned kb[4];
+                const int kr = np * 16 + (mi >> 1) * 8 + mrow, kc = ks * 2 + (mi & 1);
+                ldsm4(kb, ka + kr * RB + ((kc ^ (kr & 7)) << 4));
+#pragma unroll
+                for (int p = 2; p >= 0; --p) {
+                    mma16816<F16>(s[2 * np], qa[p], kb[0], kb[1]);
+                    mma16816<F16>(s[2 * np + 1], qa[p], kb[2], kb[3]);
+                }
+            }
+        }
+        float mx_a = m_a, mx_b = m_b;
+#pragma unroll
+        for (int n = 0; n < AK / 8; ++n) {
+            const int key = k0 + n * 8 + lc;
+            s[n][0] = key <= pos_a ? s[n][0] * rs_a : -INFINITY;
+            s[n][1] = key + 1 <= pos_a ? s[n][1] * rs_a : -INFINITY;
+            s[n][2] = key <= pos_b ? s[n][2] * rs_b : -INFINITY;
+            s[n][3] = key + 1 <= pos_b ? s[n][3] * rs_b : -INFINITY;
+            mx_a = fmaxf(mx_a, fmaxf(s[n][0], s[n][1]));
+            mx_b = fmaxf(mx_b, fmaxf(s[n][2], s[n][3]));
+        }
+#pragma unroll
+        for (int w = 1; w <= 2; w <<= 1) {
+            mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, w));
+            mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, w));
+        }
+        // (a row past M, or one whose scores are all -inf so far, keeps weights of 0)
+        const float ba = mx_a > -INFINITY ? mx_a : 0.f, bb = mx_b > -INFINITY ? mx_b : 0.f;
+        const float ra = expf(m_a - ba), rb = expf(m_b - bb);   // (0 while the maximum is -inf)
+        m_a = mx_a;
+        m_b = mx_b;
+        float sa = 0.f, sb = 0.f;
+#pragma unroll
+        for (int n = 0; n < AK / 8; ++n) {
+            s[n][0] = expf(s[n][0] - ba); s[n][1] = expf(s[n][1] - ba);
+            s[n][2] = expf(s[n][2] - bb); s[n][3] = expf(s[n][3] - bb);
+            sa += s[n][0] + s[n][1];
+            sb += s[n][2] + s[n][3];
+        }
+        l_a = fmaf(l_a, ra, sa);   // (this lane's columns; added over the four lanes of a row at the end)
+        l_b = fmaf(l_b, rb, sb);
+#pragma unroll
+        for (int n = 0; n < HD / 8; ++n) {
+            o[n][0] *= ra; o[n][1] *= ra;
+            o[n][2] *= rb; o[n][3] *= rb;
+        }
+#pragma unroll
+        for (int ks = 0; ks < AK / 16; ++ks) {
+            unsigned pa[3][4], s3[3];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                split3<F16>(s[2 * ks + (e >> 1)][(e & 1) * 2], s[2 * ks + (e >> 1)][(e & 1) * 2 + 1], s3);
+                pa[0][e] = s3[0]; pa[1][e] = s3[1]; pa[2][e] = s3[2];
+            }
+#pragma unroll
+            for (int np = 0; np < HD / 16; ++np) {
+                unsigned vb[4];
+                const int vr = ks * 16 + (mi & 1) * 8 + mrow, vc = np * 2 + (mi >> 1);
+                ldsm4_t(vb, va + vr * RB + ((vc ^ (vr & 7)) << 4));
+#pragma unroll
+                for (int p = 2; p >= 0; --p) {
+                    mma16816<F16>(o[2 * np], pa[p], vb[0], vb[1]);
+                    mma16816<F16>(o[2 * np + 1], pa[p], vb[2], vb[3]);
+                }
+            }
+        }
+        __syncthreads();   // everyone is done with this buffer: the load after next may overwrite it
+    }
+#pragma unroll
+    for (int w = 1; w <= 2; w <<= 1) {
+        l_a += __shfl_xor_sync(0xffffffffu, l_a, w);
+        l_b += __shfl_xor_sync(0xffffffffu, l_b, w);
+    }
+    const float ia = 1.f / l_a, ib = 1.f / l_b;
+#pragma unroll
+    for (int n = 0; n < HD / 8; ++n) {
+        const size_t col = (size_t)h * HD + n * 8 + lc;
+        auto put = [&](int row, float x, float y) {
+            unsigned short xh, xl, yh, yl;
+            split_b16(x, F16, xh, xl);
+            split_b16(y, F16, yh, yl);
+            *(unsigned *)(out_b + (size_t)row * d + col) = (unsigned)xh | ((unsigned)yh << 16);
+            *(unsigned *)(out_b + (size_t)(lo_row0 + row) * d + col) = (unsigned)xl | ((unsigned)yl << 16);
+        };
+        if (row_a < M) put(row_a, o[n][0] * ia, o[n][1] * ia);
+        if (row_a + 8 < M) put(row_a + 8, o[n][2] * ib, o[n][3] * ib);
+    }
+}
+
+// grid (M, ceil(F / 1024)): the gate/up product has rows interleaved (2 i = gate_i, 2 i + 1 = up_i); a thread takes four.
+__global__ void __launch_bounds__(256) k_wide_silu(ClWideParts p, int F, __nv_bfloat16 *A, int lo_row0, int f16) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int t = blockIdx.x, i = (blockIdx.y * 256 + threadIdx.x) * 4;
+    if (i >= F) return;   // (F is a multiple of 8)
+    const int n = wide_parts(p, t, 2 * i);   // (eight consecutive columns lie in one tile)
+    const size_t plane = (size_t)p.M * 2 * F;
+    const float *src = p.P + (size_t)t * 2 * F + 2 * i;
+    float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+#pragma unroll 2
+    for (int s = 0; s < n; ++s) {
+        const float4 x = __ldcg((const float4 *)(src + (size_t)s * plane)), y = __ldcg((const float4 *)(src + (size_t)s * plane) + 1);
+        u.x += x.x; u.y += x.y; u.z += x.z; u.w += x.w;
+        v.x += y.x; v.y += y.y; v.z += y.z; v.w += y.w;
+    }
+    auto h = [](float g, float up) { return g / (1.f + expf(-g)) * up; };
+    store_split4(A + (size_t)t * F + i, A + (size_t)(lo_row0 + t) * F + i, h(u.x, u.y), h(u.z, u.w), h(v.x, v.y), h(v.z, v.w), f16);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cluster > 1) {
+        at[1].id = cudaLaunchAttributeClusterDimension;
+        at[1].val.clusterDim.x = cluster;
+        at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+    }
+    return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
 }  // namespace
 
-// Parts to cut the K range into: the fewest that fill at least 90 % of the last wave of CTAs (else the best found),
-// with at least 8 K blocks per part and the partial products inside the workspace.
-int cl_wide_splits(int M, int rows, int KB, int n_sm, size_t ws_floats) {
-    const long long tiles = (long long)((M + WM - 1) / WM) * ((rows + WN - 1) / WN);
-    int best = 1;
-    double best_eff = 0.0;
-    for (int s = 1; s <= 16; ++s) {
-        if (s > 1 && (KB / s < 8 || (size_t)s * M * rows > ws_floats)) break;
-        const long long n = tiles * s, waves = (n + n_sm - 1) / n_sm;
-        const double eff = (double)n / (double)(waves * n_sm);
-        if (eff > best_eff + 1e-9) {
-            best_eff = eff;
-            best = s;
-        }
-        if (eff >= 0.9) break;
-    }
-    return best;
+// How a GEMM of M operand rows is cut: one CTA pair per two SMs, fewer when there is so little work that a pair would
+// have less than two K blocks, or when the product parts would not fit the workspace.
+ClWideParts cl_wide_plan(int M, int rows, int KB, int n_sm, float *P, size_t ws_floats) {
+    ClWideParts p;
+    p.P = P; p.M = M; p.rows = rows; p.KB = KB;
+    const int rest = M % 256;
+    p.MT = M / 256 + (rest > 128);
+    p.half = rest > 0 && rest <= 128;
+    p.NT = (rows + WN - 1) / WN;
+    p.G = std::max(1, std::min(n_sm / 2, cl_wide_cost(p) / 4));
+    auto max_parts = [&]() {
+        int m = 0;
+        for (int nt = 0; nt < p.NT; ++nt)
+            for (int mt = 0; mt < p.MT + p.half; ++mt)
+                m = std::max(m, (cl_wide_owner(p, nt, mt, KB - 1) - cl_wide_owner(p, nt, mt, 0) + 1) << (mt == p.MT));
+        return m;
+    };
+    while (p.G > 1 && (size_t)max_parts() * M * rows > ws_floats) --p.G;
+    return p;
 }
 
-cudaError_t cl_launch_wide(const ClTensorMap &mapA, const ClTensorMap &mapB, const ClWideArgs &a, cudaStream_t s) {
-    const size_t smem = (size_t)WSTAGES * WSTAGE_BYTES + sizeof(WSmem) + 1024;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    if (a.rows % 4 || a.M < 1 || a.M > CL_WIDE_MAX_M) return cudaErrorInvalidValue;
-    k_wide<<<a.MT * a.NT * a.splits, WTHREADS, smem, s>>>(*(const CUtensorMap *)mapA.bytes, *(const CUtensorMap *)mapB.bytes, a);
-    return cudaGetLastError();
+cudaError_t cl_launch_wide(const ClTensorMap &mapA, const ClTensorMap &mapB, const ClWideParts &p, int lo_row0, int *err, int f16,
+                           cudaStream_t s) {
+    const size_t smem = (size_t)W_SMEM_TILES * W_TILE + sizeof(WSmem) + 1024;
+    ClWideArgs a;
+    a.p = p; a.lo_row0 = lo_row0; a.err = err; a.f16 = f16; a.chain = W_CHAIN;
+    if (p.rows % 8 || p.M < 1 || p.M > CL_WIDE_MAX_M) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(k_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_chained(k_wide, dim3(2 * p.G), WTHREADS, smem, 2, s, *(const CUtensorMap *)mapA.bytes, *(const CUtensorMap *)mapB.bytes, a);
 }
 
 cudaError_t cl_launch_wide_norm(const ClWideNormArgs &a, cudaStream_t s) {
     if (a.d % 4) return cudaErrorInvalidValue;
-    k_wide_norm<<<a.M, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    const int chunks = a.d / 4, rounds = (chunks + 1023) / 1024, threads = ((chunks + rounds - 1) / rounds + 31) / 32 * 32;
+    return launch_chained(k_wide_norm, dim3(a.M), threads, 0, 1, s, a);
 }
 
-cudaError_t cl_launch_wide_rope_append(float *P, int splits, int M, int H, int Hkv, int hd, int d, const float2 *rope_cs,
-                                       void *kcache, void *vcache, int max_seq, const ClDevState *st, int f16, cudaStream_t s) {
-    k_wide_rope_append<<<dim3(M, H), hd / 2, 0, s>>>(P, splits, M, hd, d, Hkv, rope_cs, (unsigned short *)kcache,
-                                                     (unsigned short *)vcache, max_seq, st, f16);
-    return cudaGetLastError();
+cudaError_t cl_launch_wide_rope_append(const ClWideParts &p, int H, int Hkv, int hd, int d, const float2 *rope_cs, void *kcache,
+                                       void *vcache, int max_seq, const ClDevState *st, int f16, cudaStream_t s) {
+    const int items = (H + 2 * Hkv) * (hd / 8);
+    return launch_chained(k_wide_rope_append, dim3(p.M, (items + 255) / 256), 256, 0, 1, s, p, hd, d, Hkv, rope_cs,
+                          (unsigned short *)kcache, (unsigned short *)vcache, max_seq, st, f16);
 }
 
-cudaError_t cl_launch_wide_silu(const float *P, int splits, int M, int F, __nv_bfloat16 *A, int lo_row0, int f16, cudaStream_t s) {
-    k_wide_silu<<<dim3(M, (F + 255) / 256), 256, 0, s>>>(P, splits, M, F, A, lo_row0, f16);
-    return cudaGetLastError();
+cudaError_t cl_launch_wide_silu(const ClWideParts &p, int F, __nv_bfloat16 *A, int lo_row0, int f16, cudaStream_t s) {
+    return launch_chained(k_wide_silu, dim3(p.M, (F + 1023) / 1024), 256, 0, 1, s, p, F, A, lo_row0, f16);
 }
 
 cudaError_t cl_launch_attn_wide(const float *q, int ld_q, const void *kcache, const void *vcache, __nv_bfloat16 *out_b,
                                 int lo_row0, int M, int d, int H, int Hkv, int hd, int max_seq, const ClDevState *st,
                                 int f16, cudaStream_t s) {
-    const dim3 grid(H, (M + AQ - 1) / AQ);
-    const int kp = (hd * AK > AQ * APS) ? hd * AK : AQ * APS;
-    const size_t smem = (size_t)(hd * AQ + kp + AK * hd) * sizeof(float);
-    if (hd == 128) {
-        static bool set128 = false;
-        if (!set128) {
-            cudaError_t e = cudaFuncSetAttribute(k_attn_wide<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            set128 = true;
-        }
-        k_attn_wide<128><<<grid, 256, smem, s>>>(q, ld_q, (const unsigned short *)kcache, (const unsigned short *)vcache, out_b,
-                                                 lo_row0, M, d, H, Hkv, max_seq, st, f16);
-    } else if (hd == 64) {
-        static bool set64 = false;
-        if (!set64) {
-            cudaError_t e = cudaFuncSetAttribute(k_attn_wide<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            set64 = true;
-        }
-        k_attn_wide<64><<<grid, 256, smem, s>>>(q, ld_q, (const unsigned short *)kcache, (const unsigned short *)vcache, out_b,
-                                                lo_row0, M, d, H, Hkv, max_seq, st, f16);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    if (hd != 128 && hd != 64) return cudaErrorInvalidValue;
+    const size_t smem = hd == 128 ? attn_wide_smem<128>() : attn_wide_smem<64>();
+    auto kern = hd == 128 ? (f16 ? k_attn_wide<128, 1> : k_attn_wide<128, 0>) : (f16 ? k_attn_wide<64, 1> : k_attn_wide<64, 0>);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_chained(kern, dim3(H, (M + AQ - 1) / AQ), 128, smem, 1, s, q, ld_q, (const unsigned short *)kcache,
+                          (const unsigned short *)vcache, out_b, lo_row0, M, d, H, Hkv, max_seq, st);
 }
 
 bool cl_make_tensor_map(ClTensorMap *m, const void *base, int rows, int cols, int box_rows, int f16) {

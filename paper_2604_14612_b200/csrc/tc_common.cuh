@@ -102,6 +102,63 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
         : "memory");
 }
 
+// ---- CTA pairs (clusters of 2) ----
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+// The address of the same shared-memory object in CTA 0 of the pair.
+__device__ __forceinline__ unsigned rank0_addr(const void *p) {
+    unsigned r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(s_u32(p)));
+    return r;
+}
+__device__ __forceinline__ void bar_arrive_rank0(unsigned long long *b) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rank0_addr(b)) : "memory");
+}
+// TMA tile load into this CTA's shared memory whose bytes count on CTA 0's barrier.
+__device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *map, int c0, int c1, unsigned long long *bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
+            s_u32(dst)),
+        "l"(map), "r"(rank0_addr(bar)), "r"(c0), "r"(c1)
+        : "memory");
+}
+// Multiply-add of the pair (issued by CTA 0): A rows and B rows are split between the CTAs at the same offsets.
+__device__ __forceinline__ void umma_pair(unsigned tmem_d, unsigned long long adesc, unsigned long long bdesc, unsigned idesc,
+                                          unsigned accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// Arrives on the barrier at this offset in both CTAs once the multiply-adds issued so far have finished.
+__device__ __forceinline__ void umma_commit_pair(unsigned long long *bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(s_u32(bar)),
+                 "h"((unsigned short)3)
+                 : "memory");
+}
+
+// ---- programmatic dependent launch ----
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// 32-byte global accesses (32-byte aligned).
+__device__ __forceinline__ void st_global_v8(float *p, const float *v) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]),
+                 "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void red_add_v8(float *p, const float *v) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+    asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(p + 4), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+}
+
 // Shared-memory matrix descriptor of a K-major bf16 tile written by TMA with the 128-byte swizzle: rows of 128
 // bytes, groups of 8 rows 1024 bytes apart (stride byte offset), descriptor version 1, layout type 2 (128B swizzle).
 __device__ __forceinline__ unsigned long long umma_desc(unsigned smem_addr) {
@@ -142,6 +199,16 @@ __device__ __forceinline__ void store_split(__nv_bfloat16 *hi_p, __nv_bfloat16 *
     split_b16(v, f16, hi, lo);
     *reinterpret_cast<unsigned short *>(hi_p) = hi;
     *reinterpret_cast<unsigned short *>(lo_p) = lo;
+}
+// Four consecutive values -> their hi and lo parts, 8 bytes each (8-byte aligned).
+__device__ __forceinline__ void store_split4(__nv_bfloat16 *hi_p, __nv_bfloat16 *lo_p, float v0, float v1, float v2, float v3, int f16) {
+    unsigned short h0, h1, h2, h3, l0, l1, l2, l3;
+    split_b16(v0, f16, h0, l0);
+    split_b16(v1, f16, h1, l1);
+    split_b16(v2, f16, h2, l2);
+    split_b16(v3, f16, h3, l3);
+    *(uint2 *)hi_p = make_uint2((unsigned)h0 | ((unsigned)h1 << 16), (unsigned)h2 | ((unsigned)h3 << 16));
+    *(uint2 *)lo_p = make_uint2((unsigned)l0 | ((unsigned)l1 << 16), (unsigned)l2 | ((unsigned)l3 << 16));
 }
 __device__ __forceinline__ void umma_bf16(unsigned tmem_d, unsigned long long adesc, unsigned long long bdesc, unsigned idesc,
                                           unsigned accumulate) {
