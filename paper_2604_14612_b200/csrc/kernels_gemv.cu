@@ -240,15 +240,22 @@ cudaError_t cl_launch_gemv(int wdtype, int T, int epi, const ClGemvArgs &a, int 
 // ---- confidence scoring without any allocation ------------------------------------------------------
 // Scratch of cl_layer_confidences_static(): one file-scope array that every GPU loading this library holds until
 // the process exits.  Layout (bytes): [0, 256) the LM-head kernel's ticket counter; then the normalised rows
-// xn [SC_CHUNK, CL_STATIC_MAX_D] fp32; the per-block softmax partials [SC_MAX_GRID, SC_CHUNK]; and the three
+// xn [SC_CHUNK, CL_STATIC_MAX_D] fp32; the softmax partials of either path; the rows' normalisation factors and the three
 // per-row results (confidence, top-1 probability, greedy token) [CL_STATIC_MAX_ROWS] each.
+// Up to SC_GEMV_ROWS rows take passes of the streaming GEMV, more take the tiled kernel of kernels_headrows.cu, whose cost
+// hardly depends on the rows of a tile up to 64 (bf16 heads, whole call, 9 / 16 / 21 / 48 / 100 rows: 32000 x 4096 GEMV
+// 417 / 633 / 761 / 1746 / 3550 us, tiled 479 / 479 / 502 / 564 / 1059; 128256 x 4096 GEMV 1089 / 1752 / 2152 / 5119 / 10622,
+// tiled 1657 / 1662 / 1742 / 2021 / 3773; 5003 x 768 GEMV 114 / 150 / 178 / 331 / 625, tiled 118 / 118 / 121 / 125 / 180).
 namespace {
 
 constexpr int SC_MAX_GRID = 1024;
-constexpr int SC_CHUNK = 8;   // rows per LM-head pass
+constexpr int SC_CHUNK = 8;   // rows per LM-head pass of the GEMV
+constexpr int SC_GEMV_ROWS = 16;   // most rows that take those passes
 constexpr size_t SC_OFF_XN = 256;
 constexpr size_t SC_OFF_PART = SC_OFF_XN + (size_t)SC_CHUNK * CL_STATIC_MAX_D * sizeof(float);
-constexpr size_t SC_OFF_CONF = SC_OFF_PART + (size_t)SC_MAX_GRID * SC_CHUNK * sizeof(ClHeadPartial);
+constexpr size_t SC_PARTIALS = SC_MAX_GRID * SC_CHUNK > CL_HEAD_ROWS_PARTIALS ? SC_MAX_GRID * SC_CHUNK : CL_HEAD_ROWS_PARTIALS;
+constexpr size_t SC_OFF_SCALE = SC_OFF_PART + SC_PARTIALS * sizeof(ClHeadPartial);
+constexpr size_t SC_OFF_CONF = SC_OFF_SCALE + (size_t)CL_STATIC_MAX_ROWS * sizeof(float);
 constexpr size_t SC_OFF_PMAX = SC_OFF_CONF + (size_t)CL_STATIC_MAX_ROWS * sizeof(float);
 constexpr size_t SC_OFF_ARG = SC_OFF_PMAX + (size_t)CL_STATIC_MAX_ROWS * sizeof(float);
 constexpr size_t SC_BYTES = SC_OFF_ARG + (size_t)CL_STATIC_MAX_ROWS * sizeof(int);
@@ -331,7 +338,6 @@ extern "C" int cl_layer_confidences_static(const void *lm_head, const float *fin
     float *xn = (float *)(sc + SC_OFF_XN);
     float *d_conf = (float *)(sc + SC_OFF_CONF), *d_pmax = (float *)(sc + SC_OFF_PMAX);
     int *d_arg = (int *)(sc + SC_OFF_ARG);
-    const size_t es = weight_dtype == 1 ? 2 : 4;
     cudaError_t e = cudaMemsetAsync(sc, 0, SC_OFF_XN, s);   // the ticket must start at zero whatever the last call left
     ClGemvArgs a;
     memset(&a, 0, sizeof(a));
@@ -342,13 +348,19 @@ extern "C" int cl_layer_confidences_static(const void *lm_head, const float *fin
     int grid = ((vocab + 1) / 2 + 7) / 8;
     if (grid > n_sm * 4) grid = n_sm * 4;
     if (grid > SC_MAX_GRID) grid = SC_MAX_GRID;
-    for (int r0 = 0; r0 < n_rows && e == cudaSuccess; r0 += SC_CHUNK) {
-        const int T = n_rows - r0 < SC_CHUNK ? n_rows - r0 : SC_CHUNK;
-        e = cl_launch_rmsnorm_rows(weight_dtype, (const char *)hidden + (size_t)r0 * d_model * es, final_norm, T, d_model, rms_eps,
-                                   xn, s);
-        if (e != cudaSuccess) break;
-        a.out_tok = d_arg + r0; a.out_pmax = d_pmax + r0; a.out_conf = d_conf + r0;
-        e = cl_launch_gemv(weight_dtype, T, CL_EPI_HEAD, a, grid, s);
+    if (e == cudaSuccess && n_rows > SC_GEMV_ROWS) {
+        e = cl_launch_head_rows(weight_dtype, lm_head, hidden, final_norm, n_rows, vocab, d_model, rms_eps, n_sm,
+                                (float *)(sc + SC_OFF_SCALE), a.partials, d_conf, d_pmax, d_arg, s);
+    } else {
+        const size_t es = weight_dtype == 1 ? 2 : 4;
+        for (int r0 = 0; r0 < n_rows && e == cudaSuccess; r0 += SC_CHUNK) {
+            const int T = n_rows - r0 < SC_CHUNK ? n_rows - r0 : SC_CHUNK;
+            e = cl_launch_rmsnorm_rows(weight_dtype, (const char *)hidden + (size_t)r0 * d_model * es, final_norm, T, d_model,
+                                       rms_eps, xn, s);
+            if (e != cudaSuccess) break;
+            a.out_tok = d_arg + r0; a.out_pmax = d_pmax + r0; a.out_conf = d_conf + r0;
+            e = cl_launch_gemv(weight_dtype, T, CL_EPI_HEAD, a, grid, s);
+        }
     }
     if (e == cudaSuccess && conf) e = cudaMemcpyAsync(conf, d_conf, (size_t)n_rows * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && p_max) e = cudaMemcpyAsync(p_max, d_pmax, (size_t)n_rows * 4, cudaMemcpyDeviceToHost, s);

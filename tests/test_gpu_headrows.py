@@ -1,0 +1,38 @@
+"""The tiled LM-head kernel behind the allocation-free scoring call, at the edges of its tiles (run on a B200).
+
+Row tiles hold 16 TM rows (TM = 1 .. 8), weight tiles 128 rows, steps of K 32 elements; the largest call has 4096 rows.
+"""
+import numpy as np
+import pytest
+import torch
+
+import paper_2604_14612_b200 as cl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,V,d,n", [("bf16", 130, 40, 17), ("bf16", 1000, 768, 33), ("bf16", 5003, 1024, 100), ("bf16", 4097, 264, 128),
+                                         ("bf16", 32000, 512, 129), ("fp32", 1024, 256, 65), ("fp32", 301, 72, 50), ("bf16", 300, 64, 4096),
+                                         ("bf16", 200, 8192, 112), ("bf16", 2, 64, 300)])
+def test_tiled_scoring_against_fp64(dtype, V, d, n):
+    """Confidence and top-1 probability against fp64 arithmetic on the same stored values.  A logit is a sum of d products of
+    fp32 activations in chains of 64: its error is below 2^-24 (64 + 3) times the sum of the products' magnitudes, about
+    1e-5 here; the probability and the confidence move by at most twice that."""
+    dt = {"bf16": torch.bfloat16, "fp32": torch.float32}[dtype]
+    g = torch.Generator(device="cuda").manual_seed(V + n)
+    head = (torch.randn((V, d), generator=g, device="cuda") * 2 / d ** 0.5).to(dt)
+    gain = 1.0 + 0.1 * torch.randn((d,), generator=g, device="cuda")
+    hidden = (3 * torch.randn((n, d), generator=g, device="cuda")).to(dt)
+    hidden[0] = 0                                        # a row of zeros: the uniform distribution, lowest index
+    for _ in range(2):                                   # the second call meets the first one's scratch contents
+        got = cl.cl_layer_confidences_static(head, gain, hidden, rms_eps=1e-5)
+        x = hidden.double()
+        lg = (x * torch.rsqrt((x * x).mean(-1, keepdim=True) + 1e-5) * gain.double()) @ head.double().T
+        lp = torch.log_softmax(lg, -1)
+        conf = (1 + (lp.exp() * lp).sum(-1) / np.log(V)).cpu().numpy()
+        assert np.abs(got["conf"] - conf).max() <= 2e-5
+        assert np.abs(got["p_max"] - lp.max(-1).values.exp().cpu().numpy()).max() <= 2e-5
+        top = torch.topk(lg, 2).values
+        clear = ((top[:, 0] - top[:, 1]) > 1e-4).cpu().numpy()
+        assert np.array_equal(got["argmax"][clear], lg.argmax(-1).cpu().numpy()[clear])
+        assert got["argmax"][0] == 0 and abs(got["p_max"][0] - 1 / V) <= 1e-6
