@@ -25,14 +25,18 @@ constexpr int SLOT_BYTES = 32768;      // ring slot: as many whole weight rows a
 constexpr int NSLOT = 6;               // 192 KB in flight per SM
 constexpr int MAXIT = 4;               // 16-byte chunks per thread per row: rows up to 32 KB (C <= 16384 bf16)
 constexpr int RB = 256;                // rows per epilogue block
+constexpr int PST = NCW + 1;           // row stride of the table of partial sums: odd, since threads read whole rows side by side
+                                       // (stride 16: 16-way bank conflicts, 2.3 % of a step at width 4096)
+constexpr int SHORT_CHUNKS = 256;      // rows of up to this many 16-byte chunks are short (see consume_short_rows)
 // (every single wait is bounded by ClStepArgs::wait_ns, 2 s unless a diagnostic lowered it)
 
 struct Smem {
     unsigned long long full[NSLOT];
     unsigned long long empty[NSLOT];
-    float partial[RB * NCW];
+    float partial[RB * PST];
     float red[NCW];
-    ClHeadPartial hp[NCT];
+    ClHeadPartial hp[NCW];
+    float xs[SHORT_CHUNKS * 8];   // input vector of a phase with short rows
     int abort;
     int halt;                     // set by the consumers when drafting stops early: the producer issues no more copies
     unsigned long long wait_ns;   // bound on any single wait (copied from the launch arguments)
@@ -454,7 +458,7 @@ __device__ __forceinline__ void consume_rows(int r0, int r1, int nchunks, int rp
                 }
                 warp_reduce_rows<R>(acc, lane);
                 const int row = sr + g + ((lane >> SH) & (R - 1));
-                if ((lane & ((1 << SH) - 1)) == 0 && row < sr + ns) sm->partial[row * NCW + warp] = acc[0];
+                if ((lane & ((1 << SH) - 1)) == 0 && row < sr + ns) sm->partial[row * PST + warp] = acc[0];
             }
             rg.advance();
         }
@@ -464,7 +468,64 @@ __device__ __forceinline__ void consume_rows(int r0, int r1, int nchunks, int rp
     }
 }
 
-template <typename WT, typename Epi>
+// Short rows (d_model = 768, d_ffn = 2048): spread over all warps, a row of 96 chunks would leave 13 of 16 warps multiplying
+// padding, and the phase would be bound by issue slots (cycle of four steps and a verify pass, 12 layers of width 768: 1.99 ms, this way 1.85).  Here a row
+// belongs to a group of G warps (G = 1 up to 128 chunks, 2 up to 256), a group takes every (NCW / G)-th row of a slot, and the
+// input vector goes through shared memory, from which each warp takes its columns.
+template <typename WT, int G, typename Epi>
+__device__ __forceinline__ void consume_short_rows(int r0, int r1, int nchunks, int rps, const float (&x0)[Chunk<WT>::EPC], Ring &rg,
+                                                   const unsigned char *ring, Smem *sm, ClDevState *st, Epi epi) {
+    constexpr int EPC = Chunk<WT>::EPC, NG = NCW / G, NIT = 4;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = warp / G, wg = warp % G;
+    const unsigned rowbytes = (unsigned)nchunks * 16u, ring_addr = s_u32(ring);
+    if (tid < nchunks) {
+#pragma unroll
+        for (int e = 0; e < EPC; e += 4) *(float4 *)&sm->xs[tid * EPC + e] = make_float4(x0[e], x0[e + 1], x0[e + 2], x0[e + 3]);
+    }
+    consumer_sync();
+    float xr[NIT][EPC];
+    unsigned coff[NIT];
+#pragma unroll
+    for (int it = 0; it < NIT; ++it) {
+        const int ch = (it * G + wg) * 32 + lane;
+        coff[it] = (unsigned)min(ch, nchunks - 1) * 16u;
+#pragma unroll
+        for (int e = 0; e < EPC; e += 4) {
+            const float4 v = ch < nchunks ? *(const float4 *)&sm->xs[ch * EPC + e] : make_float4(0.f, 0.f, 0.f, 0.f);
+            xr[it][e] = v.x; xr[it][e + 1] = v.y; xr[it][e + 2] = v.z; xr[it][e + 3] = v.w;
+        }
+    }
+    const int blockrows = max(1, RB / rps) * rps;
+    for (int rb0 = r0; rb0 < r1; rb0 += blockrows) {
+        const int nrb = min(blockrows, r1 - rb0);
+        for (int sr = 0; sr < nrb; sr += rps) {
+            const int ns = min(rps, nrb - sr);   // rows in this slot
+            mbar_wait(&sm->full[rg.slot], rg.par, sm, st);
+            const unsigned base = ring_addr + rg.slot * (unsigned)SLOT_BYTES;
+            for (int g = grp; g < ns; g += NG) {
+                uint4 w[NIT];
+#pragma unroll
+                for (int it = 0; it < NIT; ++it) w[it] = lds128(base + (unsigned)g * rowbytes + coff[it]);
+                float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+                for (int it = 0; it < NIT; ++it) {
+                    if (it & 1) a1 = Chunk<WT>::dot(w[it], xr[it], a1);
+                    else a0 = Chunk<WT>::dot(w[it], xr[it], a0);
+                }
+                const float v = warp_sum(a0 + a1);
+                if (lane == 0) sm->partial[(sr + g) * PST + wg] = v;
+            }
+            __syncwarp();
+            if (lane == 0) bar_arrive(&sm->empty[rg.slot]);
+            rg.advance();
+        }
+        consumer_sync();
+        epi(rb0, nrb);
+        consumer_sync();
+    }
+}
+
+template <typename WT, bool SHORT, typename Epi>
 __device__ __forceinline__ void consume_matrix(int rows, int cols, int unit, const float (&xr)[MAXIT][Chunk<WT>::EPC],
                                                Ring &rg, const unsigned char *ring, Smem *sm, ClDevState *st, Epi epi,
                                                const float *cum_w, unsigned long long *busy) {
@@ -475,17 +536,29 @@ __device__ __forceinline__ void consume_matrix(int rows, int cols, int unit, con
     const int nchunks = cols / EPC;
     const int rps = rows_per_slot((size_t)nchunks * 16, unit);
     const int nit = (nchunks + NCT - 1) / NCT;   // uniform over the grid
-    if (nit <= 1) consume_rows<WT, 1, 4>(r0, r1, nchunks, rps, xr, rg, ring, sm, st, epi);
-    else if (nit <= 2) consume_rows<WT, 2, 2>(r0, r1, nchunks, rps, xr, rg, ring, sm, st, epi);
-    else consume_rows<WT, 4, 1>(r0, r1, nchunks, rps, xr, rg, ring, sm, st, epi);
+    if constexpr (SHORT) {
+        if (nchunks <= 128) consume_short_rows<WT, 1>(r0, r1, nchunks, rps, xr[0], rg, ring, sm, st, [&](int rb0, int nrb) { epi(rb0, nrb, 1); });
+        else consume_short_rows<WT, 2>(r0, r1, nchunks, rps, xr[0], rg, ring, sm, st, [&](int rb0, int nrb) { epi(rb0, nrb, 2); });
+        if (busy) *busy += gtime_ns() - t_start;
+        return;
+    }
+    const auto all = [&](int rb0, int nrb) { epi(rb0, nrb, NCW); };
+    if (nit <= 1) consume_rows<WT, 1, 4>(r0, r1, nchunks, rps, xr, rg, ring, sm, st, all);
+    else if (nit <= 2) consume_rows<WT, 2, 2>(r0, r1, nchunks, rps, xr, rg, ring, sm, st, all);
+    else consume_rows<WT, 4, 1>(r0, r1, nchunks, rps, xr, rg, ring, sm, st, all);
     if (busy) *busy += gtime_ns() - t_start;
 }
 
-__device__ __forceinline__ float row_sum(const Smem *sm, int r) {
-    const float *p = sm->partial + r * NCW;
+// The total of row r of a block out of its `n` partial sums (1, 2 or one per warp).
+__device__ __forceinline__ float row_sum(const Smem *sm, int r, int n) {
+    const float *p = sm->partial + r * PST;
     float s = p[0];
+    if (n == NCW) {
 #pragma unroll
-    for (int w = 1; w < NCW; ++w) s += p[w];
+        for (int w = 1; w < NCW; ++w) s += p[w];
+    } else if (n > 1) {
+        s += p[1];
+    }
     return s;
 }
 
@@ -847,7 +920,8 @@ __device__ __forceinline__ void load_att_merged(const ClStepArgs &a, float (&xr)
 }
 
 // ---- the kernel ----------------------------------------------------------------------------------------
-template <typename WT, int HD>
+// SHORT: the rows of d_model and of d_ffn elements are short
+template <typename WT, int HD, bool SHORT>
 __global__ void __launch_bounds__(NCT + 32, 1) k_token_steps(ClStepArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *ring = smem_raw;
@@ -902,33 +976,33 @@ __global__ void __launch_bounds__(NCT + 32, 1) k_token_steps(ClStepArgs a) {
             // a matrix phase early, measured slower: whichever thread issues the request, consumer warp or producer,
             // stalls about 1.5 us on it, more than the attention phase gains.)
             load_x_rmsnorm<EPC>(a.x, L.n1, d, a.eps, xr, sm);
-            consume_matrix<WT>(d + 2 * a.Hkv * HD, d, 1, xr, rg, ring, sm, st, [&](int rb0, int nrb) {
-                for (int r = tid; r < nrb; r += NCT) a.qkv[rb0 + r] = row_sum(sm, r);
+            consume_matrix<WT, SHORT>(d + 2 * a.Hkv * HD, d, 1, xr, rg, ring, sm, st, [&](int rb0, int nrb, int np) {
+                for (int r = tid; r < nrb; r += NCT) a.qkv[rb0 + r] = row_sum(sm, r, np);
             }, a.cum_w, busy_p);
             grid_barrier(a.bar, bar_target, a.bar_arrivals, sm, st);
             attention_phase<WT, HD>(a, L, pos, sm, att_first);
             grid_barrier(a.bar, bar_target, a.bar_arrivals, sm, st);
             // attention output projection + residual
             load_att_merged<EPC, HD>(a, xr);
-            consume_matrix<WT>(d, d, 1, xr, rg, ring, sm, st, [&](int rb0, int nrb) {
-                for (int r = tid; r < nrb; r += NCT) a.x[rb0 + r] = ldcg_f(a.x + rb0 + r) + row_sum(sm, r);
+            consume_matrix<WT, SHORT>(d, d, 1, xr, rg, ring, sm, st, [&](int rb0, int nrb, int np) {
+                for (int r = tid; r < nrb; r += NCT) a.x[rb0 + r] = ldcg_f(a.x + rb0 + r) + row_sum(sm, r, np);
             }, a.cum_w, busy_p);
             grid_barrier(a.bar, bar_target, a.bar_arrivals, sm, st);
             }
             if (!(fl & 2)) {
             // gate/up projections (rows interleaved) + SiLU(gate) * up
             load_x_rmsnorm<EPC>(a.x, L.n2, d, a.eps, xr, sm);
-            consume_matrix<WT>(2 * F, d, 2, xr, rg, ring, sm, st, [&](int rb0, int nrb) {
+            consume_matrix<WT, SHORT>(2 * F, d, 2, xr, rg, ring, sm, st, [&](int rb0, int nrb, int np) {
                 for (int pr = tid; pr < nrb / 2; pr += NCT) {
-                    const float gt = row_sum(sm, 2 * pr), up = row_sum(sm, 2 * pr + 1);
+                    const float gt = row_sum(sm, 2 * pr, np), up = row_sum(sm, 2 * pr + 1, np);
                     a.hff[rb0 / 2 + pr] = gt / (1.f + expf(-gt)) * up;
                 }
             }, a.cum_w, busy_p);
             grid_barrier(a.bar, bar_target, a.bar_arrivals, sm, st);
             // down projection + residual
             load_x<EPC>(a.hff, F, xr);
-            consume_matrix<WT>(d, F, 1, xr, rg, ring, sm, st, [&](int rb0, int nrb) {
-                for (int r = tid; r < nrb; r += NCT) a.x[rb0 + r] = ldcg_f(a.x + rb0 + r) + row_sum(sm, r);
+            consume_matrix<WT, SHORT>(d, F, 1, xr, rg, ring, sm, st, [&](int rb0, int nrb, int np) {
+                for (int r = tid; r < nrb; r += NCT) a.x[rb0 + r] = ldcg_f(a.x + rb0 + r) + row_sum(sm, r, np);
             }, a.cum_w, busy_p);
             grid_barrier(a.bar, bar_target, a.bar_arrivals, sm, st);
             }
@@ -937,9 +1011,9 @@ __global__ void __launch_bounds__(NCT + 32, 1) k_token_steps(ClStepArgs a) {
         load_x_rmsnorm<EPC>(a.x, a.final_norm, d, a.eps, xr, sm);
         ClHeadPartial run{0.f, 0.f, 0.f, 0x7fffffff};
         float *lg = a.logits ? a.logits + (size_t)step * V : nullptr;
-        consume_matrix<WT>(V, d, 1, xr, rg, ring, sm, st, [&](int rb0, int nrb) {
+        consume_matrix<WT, SHORT>(V, d, 1, xr, rg, ring, sm, st, [&](int rb0, int nrb, int np) {
             for (int r = tid; r < nrb; r += NCT) {
-                const float l = fminf(fmaxf(row_sum(sm, r), -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP);
+                const float l = fminf(fmaxf(row_sum(sm, r, np), -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP);
                 if (lg) lg[rb0 + r] = l;
                 run = cl_hp_merge(run, ClHeadPartial{l, 1.f, 0.f, rb0 + r});
             }
@@ -999,15 +1073,19 @@ size_t cl_step_smem_bytes() { return (size_t)NSLOT * SLOT_BYTES + sizeof(Smem); 
 
 int cl_step_max_cols(int wdtype) { return MAXIT * NCT * (wdtype != 0 ? 8 : 4); }
 
+template <typename WT>
+static const void *step_kernel(bool h64, bool sh) {
+    if (sh) return h64 ? (const void *)k_token_steps<WT, 64, true> : (const void *)k_token_steps<WT, 128, true>;
+    return h64 ? (const void *)k_token_steps<WT, 64, false> : (const void *)k_token_steps<WT, 128, false>;
+}
+
 cudaError_t cl_launch_token_steps(int wdtype, int head_dim, const ClStepArgs &a, int grid, cudaStream_t s) {
-    const void *fn = nullptr;
-    if (wdtype == 1 && head_dim == 64) fn = (const void *)k_token_steps<__nv_bfloat16, 64>;
-    else if (wdtype == 1 && head_dim == 128) fn = (const void *)k_token_steps<__nv_bfloat16, 128>;
-    else if (wdtype == 2 && head_dim == 64) fn = (const void *)k_token_steps<__half, 64>;
-    else if (wdtype == 2 && head_dim == 128) fn = (const void *)k_token_steps<__half, 128>;
-    else if (wdtype == 0 && head_dim == 64) fn = (const void *)k_token_steps<float, 64>;
-    else if (wdtype == 0 && head_dim == 128) fn = (const void *)k_token_steps<float, 128>;
-    else return cudaErrorInvalidValue;
+    if (head_dim != 64 && head_dim != 128) return cudaErrorInvalidValue;
+    const int epc = wdtype ? 8 : 4;
+    const bool sh = a.d / epc <= SHORT_CHUNKS && a.F / epc <= SHORT_CHUNKS, h64 = head_dim == 64;
+    const void *fn = wdtype == 1   ? step_kernel<__nv_bfloat16>(h64, sh)
+                     : wdtype == 2 ? step_kernel<__half>(h64, sh)
+                                   : step_kernel<float>(h64, sh);
     const size_t smem = cl_step_smem_bytes();
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -1,0 +1,39 @@
+"""Edges of the token-step kernel's row lengths (run on a B200)."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import paper_2604_14612_b200 as cl
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("wd,d,heads,ffn", [("bf16", 128, 2, 192), ("bf16", 1024, 8, 1024), ("bf16", 1088, 17, 2048), ("bf16", 2048, 16, 2056),
+                                            ("bf16", 2176, 17, 1000), ("fp16", 768, 12, 2048), ("fp32", 512, 4, 520), ("fp32", 1024, 8, 1024),
+                                            ("fp32", 1088, 17, 1032)])
+def test_step_kernel_at_short_row_edges(monkeypatch, wd, d, heads, ffn):
+    """Rows of up to 128 16-byte chunks belong to one warp, up to 256 to two, longer ones to all; every case against the
+    per-matrix kernels, which share none of that.  Both compute in fp32 and round cached keys and values once to the storage
+    type, where a value at a rounding boundary may go either way: the first step's logits agree to half of the 1e-2 that a
+    model of this depth is allowed against the oracle."""
+    sh = dataclasses.replace(synth.WORKLOADS["C2"].shape, n_layers=2, d_model=d, n_heads=heads, d_ffn=ffn, vocab=1500, max_seq=64,
+                             weight_dtype=wd)
+    W = synth.make_weights(sh, 41, device="cuda")
+    prompt = synth.make_prompt(41, 12, sh.vocab)
+    out = []
+    for off in ("0", "1"):
+        monkeypatch.setenv("CL_DISABLE_STEP_KERNEL", off)
+        ctx = cl.Context.from_shape(sh)
+        ctx.cl_load(W)
+        ctx.cl_prefill(prompt)
+        ctx.cl_rollback(12, 5)
+        ctx.cl_set_skip_set([0, 3])
+        rows = [ctx.cl_draft(1, want_logits=True)["logits"][0]]
+        ctx.cl_set_skip_set([0, 0])
+        rows.append(ctx.cl_draft(4, want_logits=True)["logits"][0])
+        out.append(rows)
+        ctx.close()
+    for a, b in zip(*out):
+        assert np.isfinite(a).all() and np.abs(a - b).max() <= 5e-3
