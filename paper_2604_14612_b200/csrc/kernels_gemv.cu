@@ -15,6 +15,7 @@
 #include <mutex>
 
 #include "cl_internal.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -80,6 +81,8 @@ __device__ __forceinline__ float silu_f(float x) { return x / (1.f + expf(-x)); 
 
 template <typename WT, int T, int EPI>
 __global__ void __launch_bounds__(256) k_gemv(ClGemvArgs a) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (a.st && a.st->done) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int gw = blockIdx.x * nw + warp, tw = gridDim.x * nw;
@@ -204,13 +207,12 @@ __global__ void __launch_bounds__(256) k_gemv(ClGemvArgs a) {
 template <typename WT, int T>
 cudaError_t launch_t(int epi, const ClGemvArgs &a, int grid, cudaStream_t s) {
     switch (epi) {
-        case CL_EPI_STORE: k_gemv<WT, T, CL_EPI_STORE><<<grid, 256, 0, s>>>(a); break;
-        case CL_EPI_RESID: k_gemv<WT, T, CL_EPI_RESID><<<grid, 256, 0, s>>>(a); break;
-        case CL_EPI_SILU: k_gemv<WT, T, CL_EPI_SILU><<<grid, 256, 0, s>>>(a); break;
-        case CL_EPI_HEAD: k_gemv<WT, T, CL_EPI_HEAD><<<grid, 256, 0, s>>>(a); break;
+        case CL_EPI_STORE: return launch_chained(k_gemv<WT, T, CL_EPI_STORE>, dim3(grid), 256, 0, 1, s, a);
+        case CL_EPI_RESID: return launch_chained(k_gemv<WT, T, CL_EPI_RESID>, dim3(grid), 256, 0, 1, s, a);
+        case CL_EPI_SILU: return launch_chained(k_gemv<WT, T, CL_EPI_SILU>, dim3(grid), 256, 0, 1, s, a);
+        case CL_EPI_HEAD: return launch_chained(k_gemv<WT, T, CL_EPI_HEAD>, dim3(grid), 256, 0, 1, s, a);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 template <typename WT>

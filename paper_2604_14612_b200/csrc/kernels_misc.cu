@@ -4,6 +4,7 @@
 #include <math.h>
 
 #include "cl_internal.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -41,6 +42,8 @@ __device__ __forceinline__ float block_sum(float v, float *sm) {
 // ---- embedding gather: x[t] = E[token[t]] -------------------------------------------------
 template <typename ST>
 __global__ void k_embed(const ST *embed, const int *tok, int d, float *x, const ClDevState *st) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (st->done) return;
     const int t = blockIdx.x;
     const ST *row = embed + (size_t)tok[t] * d;
@@ -63,6 +66,8 @@ __device__ __forceinline__ float4 load4(const ST *p, bool aligned) {
 
 template <typename ST>
 __global__ void __launch_bounds__(1024) k_rmsnorm(const ST *x, const float *g, int d, float eps, float *out, const ClDevState *st) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (st && st->done) return;
     __shared__ float sm[32];
     const int t = blockIdx.x, span = 4 * blockDim.x;
@@ -91,6 +96,8 @@ static int norm_threads(int d) { return d / 4 >= 1024 ? 1024 : (d / 4 + 31) / 32
 template <typename ST>
 __global__ void k_rope_append(float *qkv, int row0, int hd, int d, int Hkv, const float2 *rope_cs, ST *kcache, ST *vcache,
                               int max_seq, const ClDevState *st) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (st->done) return;
     const int t = blockIdx.x, h = blockIdx.y, i = threadIdx.x, half = hd >> 1;
     const int pos = st->ctx + row0 + t;
@@ -119,6 +126,8 @@ __global__ void k_rope_append(float *qkv, int row0, int hd, int d, int Hkv, cons
 // the last block of a (t, h) to finish merges the slices in order.
 template <typename ST, int HD>
 __global__ void __launch_bounds__(128) k_attn(ClAttnArgs a) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (a.st->done) return;
     extern __shared__ float smem[];
     float *sq = smem;               // [HD]
@@ -237,6 +246,8 @@ __global__ void __launch_bounds__(128) k_attn(ClAttnArgs a) {
 // ---- hidden-state tap: ring[pos % P] = storage-type(x[t]) ----------------------------------
 template <typename ST>
 __global__ void k_tap(const float *x, int row0, int d, ST *ring_layer, int P, const ClDevState *st) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (st->done) return;
     const int t = blockIdx.x;
     const int pos = st->ctx + row0 + t;
@@ -247,6 +258,8 @@ __global__ void k_tap(const float *x, int row0, int d, ST *ring_layer, int P, co
 // ---- greedy acceptance (Section 3, Figure 2) ------------------------------------------------
 // drafts d_j = cyc_tok[j] (j = 1..K), target g_j = tgt_tok[j-1].  n = longest matching prefix.
 __global__ void k_accept(ClDevState *st, int K, int *out_tokens) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (threadIdx.x != 0 || st->done) return;
     const int nd = (K < 0) ? st->n_drafted : K;
     int n = 0;
@@ -271,6 +284,8 @@ __global__ void k_accept(ClDevState *st, int K, int *out_tokens) {
 
 // ctx += n; pending >= 0: the greedy token after row `pending` of the pass becomes the pending token.
 __global__ void k_advance(ClDevState *st, int n, int pending) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (threadIdx.x != 0) return;
     st->ctx += n;
     if (pending >= 0) st->cyc_tok[0] = st->tgt_tok[pending];
@@ -278,6 +293,8 @@ __global__ void k_advance(ClDevState *st, int n, int pending) {
 
 // ---- c_layer[r] = mean over P positions of conf_rows[r, :] (fixed order, double) -------------
 __global__ void k_mean_rows(const float *conf_rows, int rows, int P, float *c_layer) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= rows) return;
     double s = 0.0;
@@ -318,6 +335,8 @@ __device__ __forceinline__ double sel_gradient_at(const double *x, int i, int n)
 // bit for bit; the layers themselves (lane i takes layers i, i + 32, ...) run side by side, and the sequential
 // selection of the smallest margins becomes a rank by counting (ties -> lower layer index, as picking minima does).
 __global__ void k_select(cl_select_cfg cfg, int L, const float *c_layer, uint8_t *mask, double *margins) {
+    pdl_launch_dependents();
+    pdl_wait();
     if (blockIdx.x != 0 || threadIdx.x >= 32) return;
     __shared__ double c[CL_SEL_MAX], chat[CL_SEL_MAX], g[CL_SEL_MAX], tmp[CL_SEL_MAX], mg[CL_SEL_MAX];
     const int lane = threadIdx.x;
@@ -432,69 +451,55 @@ __global__ void k_select(cl_select_cfg cfg, int L, const float *c_layer, uint8_t
 
 cudaError_t cl_launch_embed(int wdtype, const void *embed, const int *tok, int T, int d, float *x, const ClDevState *st,
                             cudaStream_t s) {
-    CL_DISPATCH_ST(wdtype, (k_embed<ST><<<T, 256, 0, s>>>((const ST *)embed, tok, d, x, st)));
-    return cudaGetLastError();
+    CL_DISPATCH_ST(wdtype, return launch_chained(k_embed<ST>, dim3(T), 256, 0, 1, s, (const ST *)embed, tok, d, x, st));
 }
 
 cudaError_t cl_launch_rmsnorm(const float *x, const float *g, int T, int d, float eps, float *out, const ClDevState *st,
                               cudaStream_t s) {
-    k_rmsnorm<float><<<T, norm_threads(d), 0, s>>>(x, g, d, eps, out, st);
-    return cudaGetLastError();
+    return launch_chained(k_rmsnorm<float>, dim3(T), norm_threads(d), 0, 1, s, x, g, d, eps, out, st);
 }
 
 cudaError_t cl_launch_rmsnorm_rows(int in_dtype, const void *x, const float *g, int T, int d, float eps, float *out,
                                    cudaStream_t s) {
-    CL_DISPATCH_ST(in_dtype, (k_rmsnorm<ST><<<T, norm_threads(d), 0, s>>>((const ST *)x, g, d, eps, out, nullptr)));
-    return cudaGetLastError();
+    CL_DISPATCH_ST(in_dtype, return launch_chained(k_rmsnorm<ST>, dim3(T), norm_threads(d), 0, 1, s, (const ST *)x, g, d, eps, out, (const ClDevState *)nullptr));
 }
 
 cudaError_t cl_launch_rope_append(int wdtype, float *qkv, int T, int row0, int H, int Hkv, int hd, int d, const float2 *rope_cs,
                                   void *kcache, void *vcache, int max_seq, const ClDevState *st, cudaStream_t s) {
     dim3 grid(T, H);
-    CL_DISPATCH_ST(wdtype, (k_rope_append<ST><<<grid, hd / 2, 0, s>>>(qkv, row0, hd, d, Hkv, rope_cs, (ST *)kcache, (ST *)vcache,
-                                                                      max_seq, st)));
-    return cudaGetLastError();
+    CL_DISPATCH_ST(wdtype, return launch_chained(k_rope_append<ST>, grid, hd / 2, 0, 1, s, qkv, row0, hd, d, Hkv, rope_cs, (ST *)kcache,
+                                                 (ST *)vcache, max_seq, st));
 }
 
 cudaError_t cl_launch_attn(int wdtype, int T, const ClAttnArgs &a, cudaStream_t s) {
     dim3 grid(a.n_heads, T, a.nsplit);
     const size_t smem = (size_t)(3 * a.head_dim + 32 + a.per_max) * sizeof(float);
-    if (a.head_dim == 64) {
-        CL_DISPATCH_ST(wdtype, (k_attn<ST, 64><<<grid, 128, smem, s>>>(a)));
-    } else if (a.head_dim == 128) {
-        CL_DISPATCH_ST(wdtype, (k_attn<ST, 128><<<grid, 128, smem, s>>>(a)));
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    if (a.head_dim == 64) CL_DISPATCH_ST(wdtype, return launch_chained(k_attn<ST, 64>, grid, 128, smem, 1, s, a));
+    if (a.head_dim == 128) CL_DISPATCH_ST(wdtype, return launch_chained(k_attn<ST, 128>, grid, 128, smem, 1, s, a));
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t cl_launch_tap(int wdtype, const float *x, int T, int row0, int d, void *ring_layer, int P,
                           const ClDevState *st, cudaStream_t s) {
-    CL_DISPATCH_ST(wdtype, (k_tap<ST><<<T, 256, 0, s>>>(x, row0, d, (ST *)ring_layer, P, st)));
-    return cudaGetLastError();
+    CL_DISPATCH_ST(wdtype, return launch_chained(k_tap<ST>, dim3(T), 256, 0, 1, s, x, row0, d, (ST *)ring_layer, P, st));
 }
 
 cudaError_t cl_launch_accept(ClDevState *st, int K, int *out_tokens, cudaStream_t s) {
-    k_accept<<<1, 32, 0, s>>>(st, K, out_tokens);
-    return cudaGetLastError();
+    return launch_chained(k_accept, dim3(1), 32, 0, 1, s, st, K, out_tokens);
 }
 
 cudaError_t cl_launch_advance(ClDevState *st, int n, int pending, cudaStream_t s) {
-    k_advance<<<1, 32, 0, s>>>(st, n, pending);
-    return cudaGetLastError();
+    return launch_chained(k_advance, dim3(1), 32, 0, 1, s, st, n, pending);
 }
 
 cudaError_t cl_launch_mean_rows(const float *conf_rows, int rows, int P, float *c_layer, cudaStream_t s) {
-    k_mean_rows<<<(rows + 127) / 128, 128, 0, s>>>(conf_rows, rows, P, c_layer);
-    return cudaGetLastError();
+    return launch_chained(k_mean_rows, dim3((rows + 127) / 128), 128, 0, 1, s, conf_rows, rows, P, c_layer);
 }
 
 cudaError_t cl_launch_select(const cl_select_cfg &cfg, int n_layers, const float *c_layer, uint8_t *mask, double *margins,
                              cudaStream_t s) {
     if (cfg.hi - cfg.lo + 1 > CL_SEL_MAX) return cudaErrorInvalidValue;
-    k_select<<<1, 32, 0, s>>>(cfg, n_layers, c_layer, mask, margins);
-    return cudaGetLastError();
+    return launch_chained(k_select, dim3(1), 32, 0, 1, s, cfg, n_layers, c_layer, mask, margins);
 }
 
 cudaError_t cl_launch_interleave(int wdtype, const void *wg, const void *wu, void *dst, int F, int d, cudaStream_t s) {

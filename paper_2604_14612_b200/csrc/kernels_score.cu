@@ -71,6 +71,8 @@ k_score(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *(volatile unsigned *)&sm->tmem_base;
+    pdl_launch_dependents();
+    pdl_wait();   // the rows come from the previous kernel, and the statistics of the last round may still be read
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
@@ -191,6 +193,8 @@ k_score(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
 // Merge the per-range statistics of every row in a fixed order and evaluate Eq. 2-4.
 __global__ void k_score_finalize(const ClHeadPartial *partials, int NCG, int R, float inv_log_v, float *conf, float *pmax,
                                  int *arg) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= R) return;
     ClHeadPartial f{0.f, 0.f, 0.f, 0x7fffffff};
@@ -221,6 +225,8 @@ __device__ __forceinline__ void load8(const ST *p, float (&v)[8]) {
 // passes; the sum of squares is added in a fixed order (per thread, shuffle tree, warps in order).
 template <typename ST>
 __global__ void k_rmsnorm_to_bf16(const ST *x, const float *g, int d, float eps, unsigned short *out, int f16) {
+    pdl_launch_dependents();
+    pdl_wait();
     __shared__ float red[32];
     constexpr int KEEP = 2;
     const ST *xr = x + (size_t)blockIdx.x * d;
@@ -277,13 +283,10 @@ size_t cl_score_tc_partials(int R, int n_sm) {
 
 cudaError_t cl_launch_rmsnorm_bf16(int in_dtype, const void *x, const float *g, int rows, int d, float eps, void *out,
                                    int f16, cudaStream_t s) {
-    if (in_dtype == 1)
-        k_rmsnorm_to_bf16<__nv_bfloat16><<<rows, 256, 0, s>>>((const __nv_bfloat16 *)x, g, d, eps, (unsigned short *)out, f16);
-    else if (in_dtype == 2)
-        k_rmsnorm_to_bf16<__half><<<rows, 256, 0, s>>>((const __half *)x, g, d, eps, (unsigned short *)out, f16);
-    else
-        k_rmsnorm_to_bf16<float><<<rows, 256, 0, s>>>((const float *)x, g, d, eps, (unsigned short *)out, f16);
-    return cudaGetLastError();
+    unsigned short *o = (unsigned short *)out;
+    if (in_dtype == 1) return launch_chained(k_rmsnorm_to_bf16<__nv_bfloat16>, dim3(rows), 256, 0, 1, s, (const __nv_bfloat16 *)x, g, d, eps, o, f16);
+    if (in_dtype == 2) return launch_chained(k_rmsnorm_to_bf16<__half>, dim3(rows), 256, 0, 1, s, (const __half *)x, g, d, eps, o, f16);
+    return launch_chained(k_rmsnorm_to_bf16<float>, dim3(rows), 256, 0, 1, s, (const float *)x, g, d, eps, o, f16);
 }
 
 // xn: [R, d] bf16 normalised rows; lm_head: [V, d] bf16.  Needs d % 8 == 0 and 16-byte aligned bases.
@@ -303,9 +306,7 @@ cudaError_t cl_launch_score_tc(const void *xn, const void *lm_head, int R, int V
     cudaError_t e = cudaFuncSetAttribute(k_score, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // row blocks beyond n_sm CTAs are handled in waves of whole column ranges
-    k_score<<<a.MT * a.NCG, NTHREADS, smem, s>>>(mapA, mapB, a);
-    e = cudaGetLastError();
+    e = launch_chained(k_score, dim3(a.MT * a.NCG), NTHREADS, smem, 1, s, mapA, mapB, a);
     if (e != cudaSuccess) return e;
-    k_score_finalize<<<(R + 127) / 128, 128, 0, s>>>(partials, a.NCG, R, (float)(1.0 / log((double)V)), conf, pmax, arg);
-    return cudaGetLastError();
+    return launch_chained(k_score_finalize, dim3((R + 127) / 128), 128, 0, 1, s, partials, a.NCG, R, (float)(1.0 / log((double)V)), conf, pmax, arg);
 }

@@ -612,27 +612,6 @@ __global__ void __launch_bounds__(256) k_wide_silu(ClWideParts p, int F, __nv_bf
     store_split4(A + (size_t)t * F + i, A + (size_t)(lo_row0 + t) * F + i, h(u.x, u.y), h(u.z, u.w), h(v.x, v.y), h(v.z, v.w), f16);
 }
 
-template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (cluster > 1) {
-        at[1].id = cudaLaunchAttributeClusterDimension;
-        at[1].val.clusterDim.x = cluster;
-        at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
-        cfg.numAttrs = 2;
-    }
-    return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
-}
-
 }  // namespace
 
 // How a GEMM of M operand rows is cut: one CTA pair per two SMs, fewer when there is so little work that a pair would

@@ -4,6 +4,7 @@
 #include <cuda.h>
 
 #include "cl_internal.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -143,10 +144,6 @@ __device__ __forceinline__ void umma_commit_pair(unsigned long long *bar) {
                  "h"((unsigned short)3)
                  : "memory");
 }
-
-// ---- programmatic dependent launch ----
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // 32-byte global accesses (32-byte aligned).
 __device__ __forceinline__ void st_global_v8(float *p, const float *v) {
