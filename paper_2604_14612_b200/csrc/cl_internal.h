@@ -288,7 +288,6 @@ cudaError_t cl_launch_attn_wide(const float *q, int ld_q, const void *kcache, co
 cudaError_t cl_launch_wide_silu(const ClWideParts &p, int F, __nv_bfloat16 *A, int lo_row0, int f16, cudaStream_t s);
 
 // tensor-core scoring (bf16 / fp16 LM head): normalise to the 16-bit type, contraction fused with the softmax statistics, finalize
-int cl_score_tc_ranges(int R, int n_sm);
 size_t cl_score_tc_partials(int R, int n_sm);
 cudaError_t cl_launch_rmsnorm_bf16(int in_dtype, const void *x, const float *g, int rows, int d, float eps, void *out,
                                    int f16, cudaStream_t s);

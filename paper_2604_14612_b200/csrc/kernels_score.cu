@@ -11,6 +11,10 @@
 //   warps 2-5 epilogue: thread = one hidden row (one tensor-memory lane); it reads its row of the accumulator
 //            32 columns at a time (tcgen05.ld) and keeps running softmax statistics relative to the running
 //            maximum m: z = sum e^(l-m), s = sum (l-m) e^(l-m), and the argmax (lowest index on ties).
+// Where it pays (see score_plan) the tile is 256 rows by 256 vocabulary entries on a CTA pair (tcgen05 cta_group::2): each CTA
+// holds 128 of the rows and half of the head's tile, 32 KB a stage instead of 48 (6 stages), and the multiply-adds read 64
+// bytes of its shared memory per cycle instead of 96, which held the single-CTA tile at
+// 80 % of the tensor pipe (8 rounds of 2048 rows: 3.66 ms, with pairs 3.56).
 // A CTA owns one block of 128 hidden rows and a contiguous range of vocabulary tiles; CTAs that share the
 // vocabulary range run side by side, so a tile of the LM head is fetched from HBM once and served to the other
 // row blocks from L2.  Per-(row, vocabulary range) statistics are merged in a fixed order by a second kernel,
@@ -18,35 +22,38 @@
 // Every wait is bounded in time; on expiry an error flag is raised and the kernel winds down.
 #include <math.h>
 
+#include <algorithm>
+
 #include "tc_common.cuh"
 
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
-constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int BM = 128, BN = 256, BK = 64;
+constexpr int A_BYTES = BM * BK * 2, RING_BYTES = 196608, MAX_STAGES = 6;   // 192 KB: 4 stages of 48 KB, or 6 of 32 (pair)
 constexpr int NTHREADS = 192;
 struct ScoreSmem {
-    unsigned long long full[STAGES], empty[STAGES], tfull[2], tempty[2];
+    unsigned long long full[MAX_STAGES], empty[MAX_STAGES], tfull[2], tempty[2];
     unsigned tmem_base;
     int abort;
 };
 
 struct ScoreArgs {
-    int R, V, KB, MT, NCG, NT;      // hidden rows, vocabulary, K blocks of 64, row blocks, vocabulary ranges, vocabulary tiles
+    int R, V, KB, MT, NCG, NT;      // hidden rows, vocabulary, K blocks of 64, row blocks of 128 (pair: 256), vocabulary ranges, vocabulary tiles
     ClHeadPartial *partials;        // [MT * BM, NCG]
     int *err;
     int f16;                        // 16-bit type of both operands: 0 bf16, 1 fp16
 };
 
 
+template <bool PAIR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_score(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, ScoreArgs a) {
+    constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES, STAGES = RING_BYTES / STAGE_BYTES;
     extern __shared__ unsigned char smem_dyn[];
     unsigned char *tiles = (unsigned char *)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);   // swizzled tiles: 1 KB aligned
-    ScoreSmem *sm = (ScoreSmem *)(tiles + (size_t)STAGES * STAGE_BYTES);
+    ScoreSmem *sm = (ScoreSmem *)(tiles + RING_BYTES);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int cta = blockIdx.x;
-    if (cta >= a.MT * a.NCG) return;   // whole CTA leaves before anything is set up
+    const int cta = PAIR ? blockIdx.x >> 1 : blockIdx.x, rank = PAIR ? (int)cluster_rank() : 0;
     const int mt = cta % a.MT, cg = cta / a.MT;
     const int nt0 = (int)((long long)a.NT * cg / a.NCG), nt1 = (int)((long long)a.NT * (cg + 1) / a.NCG);
     const int ntiles = nt1 - nt0;
@@ -58,17 +65,23 @@ k_score(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
         }
         for (int i = 0; i < 2; ++i) {
             bar_init(&sm->tfull[i], 1);
-            bar_init(&sm->tempty[i], 128);
+            bar_init(&sm->tempty[i], PAIR ? 8 : 128);   // the epilogue's threads, or its warps in both CTAs
         }
         sm->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s_u32(&sm->tmem_base)) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s_u32(&sm->tmem_base)) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s_u32(&sm->tmem_base)) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (PAIR) cluster_sync();   // the peer's barriers exist before anything signals them
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *(volatile unsigned *)&sm->tmem_base;
     pdl_launch_dependents();
@@ -84,14 +97,23 @@ k_score(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                 for (int kb = 0; kb < a.KB; ++kb) {
                     if (!bar_wait(&sm->empty[stage], par ^ 1u, &sm->abort, a.err)) { ok = false; break; }
                     unsigned char *dst = tiles + (size_t)stage * STAGE_BYTES;
-                    bar_expect(&sm->full[stage], STAGE_BYTES);
-                    tma_load_2d(dst, &mapA, kb * BK, mt * BM, &sm->full[stage]);
-                    tma_load_2d(dst + A_BYTES, &mapB, kb * BK, (nt0 + t) * BN, &sm->full[stage]);
+                    if (PAIR) {
+                        if (rank == 0) bar_expect(&sm->full[stage], 2 * STAGE_BYTES);   // both CTAs' copies count on CTA 0's barrier
+                        tma_load_2d_pair(dst, &mapA, kb * BK, (2 * mt + rank) * BM, &sm->full[stage]);
+                        tma_load_2d_pair(dst + A_BYTES, &mapB, kb * BK, (nt0 + t) * BN + rank * (BN / 2), &sm->full[stage]);
+                    } else {
+                        bar_expect(&sm->full[stage], STAGE_BYTES);
+                        tma_load_2d(dst, &mapA, kb * BK, mt * BM, &sm->full[stage]);
+                        tma_load_2d(dst + A_BYTES, &mapB, kb * BK, (nt0 + t) * BN, &sm->full[stage]);
+                    }
                     issued[stage] = par;
                     if (++stage == STAGES) { stage = 0; par ^= 1u; }
                 }
             }
-            if (!ok) {   // gave up: still let the copies in flight land before the CTA may exit (bounded)
+            if (!ok && PAIR) {   // gave up: let the copies in flight land (they signal CTA 0, so this CTA can only give them time)
+                const unsigned long long t0 = gtime_ns();
+                while (gtime_ns() - t0 < 2000000ull) {}
+            } else if (!ok) {   // still let the copies in flight land before the CTA may exit (bounded)
                 for (int i = 0; i < STAGES; ++i) {
                     if (issued[i] < 2u) {
                         const unsigned long long t0 = gtime_ns();
@@ -103,8 +125,8 @@ k_score(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            const unsigned idesc = umma_idesc(BM, BN, a.f16);
+        if (lane == 0 && rank == 0) {
+            const unsigned idesc = umma_idesc(PAIR ? 2 * BM : BM, BN, a.f16);
             unsigned stage = 0, par = 0;
             bool ok = true;
             for (int t = 0; t < ntiles && ok; ++t) {
@@ -116,13 +138,20 @@ k_score(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const unsigned a_addr = s_u32(tiles + (size_t)stage * STAGE_BYTES), b_addr = a_addr + A_BYTES;
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        umma_bf16(tmem + (unsigned)b * BN, umma_desc(a_addr + k * 32), umma_desc(b_addr + k * 32), idesc,
-                                  (unsigned)(kb | k));
-                    umma_commit(&sm->empty[stage]);   // the stage is free once these multiply-adds have read it
+                    for (int k = 0; k < BK / 16; ++k) {
+                        const unsigned long long da = umma_desc(a_addr + k * 32), db = umma_desc(b_addr + k * 32);
+                        if (PAIR) umma_pair(tmem + (unsigned)b * BN, da, db, idesc, (unsigned)(kb | k));
+                        else umma_bf16(tmem + (unsigned)b * BN, da, db, idesc, (unsigned)(kb | k));
+                    }
+                    // the stage is free once these multiply-adds have read it
+                    if (PAIR) umma_commit_pair(&sm->empty[stage]);
+                    else umma_commit(&sm->empty[stage]);
                     if (++stage == STAGES) { stage = 0; par ^= 1u; }
                 }
-                if (ok) umma_commit(&sm->tfull[b]);   // accumulator b is complete
+                if (ok) {   // accumulator b is complete
+                    if (PAIR) umma_commit_pair(&sm->tfull[b]);
+                    else umma_commit(&sm->tfull[b]);
+                }
             }
         }
     } else {
@@ -177,16 +206,23 @@ k_score(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                 run.s += s;
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            bar_arrive(&sm->tempty[b]);
+            if (PAIR) {
+                __syncwarp();
+                if (lane == 0) bar_arrive_rank0(&sm->tempty[b]);
+            } else {
+                bar_arrive(&sm->tempty[b]);
+            }
         }
-        a.partials[(size_t)(mt * BM + row) * a.NCG + cg] = run;
+        a.partials[(size_t)((PAIR ? 2 * mt + rank : mt) * BM + row) * a.NCG + cg] = run;
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (PAIR) cluster_sync();   // CTA 0's multiply-adds read CTA 1's shared memory, and both signal each other's barriers
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+        if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
 }
 
@@ -270,15 +306,24 @@ __global__ void k_rmsnorm_to_bf16(const ST *x, const float *g, int d, float eps,
 
 }  // namespace
 
-int cl_score_tc_ranges(int R, int n_sm) {
-    const int MT = (R + BM - 1) / BM;
-    int ncg = n_sm / MT;
-    return ncg < 1 ? 1 : ncg;
+// Row blocks and vocabulary ranges of R rows.  A pair's tile counts as two single ones and is finished in about 7 / 8 of the
+// time (measured at 2048 rows); the pair is taken when the longest range of a pair, so weighted, is no longer than that of a
+// single CTA: 256 rows or 2048 go to pairs, 128 rows (half a pair's tile) or 384 do not.
+struct ScorePlan {
+    bool pair;
+    int MT, NCG;
+};
+static ScorePlan score_plan(int R, int V, int n_sm) {
+    const int NT = (V + BN - 1) / BN, MT1 = (R + BM - 1) / BM, MT2 = (MT1 + 1) / 2;
+    const int n1 = std::min(NT, std::max(1, n_sm / MT1)), n2 = std::min(NT, std::max(1, n_sm / 2 / MT2));
+    const long long w1 = ((long long)MT1 * n1 + n_sm - 1) / n_sm, w2 = ((long long)MT2 * n2 + n_sm / 2 - 1) / (n_sm / 2);   // waves
+    const bool pair = (NT + n2 - 1) / n2 * w2 * 7 <= (NT + n1 - 1) / n1 * w1 * 8;
+    return pair ? ScorePlan{true, MT2, n2} : ScorePlan{false, MT1, n1};
 }
 
+// Room for either plan of R rows or fewer, at any vocabulary: a chip's worth of CTAs with 128 rows each, or a range per row.
 size_t cl_score_tc_partials(int R, int n_sm) {
-    const int MT = (R + BM - 1) / BM;
-    return (size_t)MT * BM * cl_score_tc_ranges(R, n_sm);
+    return std::max((size_t)n_sm * BM, (size_t)(R + 2 * BM - 1) / (2 * BM) * 2 * BM);
 }
 
 cudaError_t cl_launch_rmsnorm_bf16(int in_dtype, const void *x, const float *g, int rows, int d, float eps, void *out,
@@ -292,21 +337,21 @@ cudaError_t cl_launch_rmsnorm_bf16(int in_dtype, const void *x, const float *g, 
 // xn: [R, d] bf16 normalised rows; lm_head: [V, d] bf16.  Needs d % 8 == 0 and 16-byte aligned bases.
 cudaError_t cl_launch_score_tc(const void *xn, const void *lm_head, int R, int V, int d, ClHeadPartial *partials, int n_sm,
                                int *err, float *conf, float *pmax, int *arg, int f16, cudaStream_t s) {
+    const ScorePlan plan = score_plan(R, V, n_sm);
     CUtensorMap mapA, mapB;
-    if (!make_map(&mapA, xn, R, d, BM, f16) || !make_map(&mapB, lm_head, V, d, BN, f16)) return cudaErrorInvalidValue;
+    if (!make_map(&mapA, xn, R, d, BM, f16) || !make_map(&mapB, lm_head, V, d, plan.pair ? BN / 2 : BN, f16)) return cudaErrorInvalidValue;
     ScoreArgs a;
     a.f16 = f16;
     a.R = R; a.V = V; a.KB = (d + BK - 1) / BK;
-    a.MT = (R + BM - 1) / BM;
-    a.NCG = cl_score_tc_ranges(R, n_sm);
+    a.MT = plan.MT; a.NCG = plan.NCG;
     a.NT = (V + BN - 1) / BN;
-    if (a.NCG > a.NT) a.NCG = a.NT;
     a.partials = partials; a.err = err;
-    const size_t smem = (size_t)STAGES * STAGE_BYTES + sizeof(ScoreSmem) + 1024;
-    cudaError_t e = cudaFuncSetAttribute(k_score, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = (size_t)RING_BYTES + sizeof(ScoreSmem) + 1024;
+    auto kern = plan.pair ? k_score<true> : k_score<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    // row blocks beyond n_sm CTAs are handled in waves of whole column ranges
-    e = launch_chained(k_score, dim3(a.MT * a.NCG), NTHREADS, smem, 1, s, mapA, mapB, a);
+    // row blocks beyond the chip's CTAs are handled in waves of whole column ranges
+    e = launch_chained(kern, dim3(a.MT * a.NCG * (plan.pair ? 2 : 1)), NTHREADS, smem, plan.pair ? 2 : 1, s, mapA, mapB, a);
     if (e != cudaSuccess) return e;
     return launch_chained(k_score_finalize, dim3((R + 127) / 128), 128, 0, 1, s, partials, a.NCG, R, (float)(1.0 / log((double)V)), conf, pmax, arg);
 }
