@@ -111,8 +111,8 @@ __global__ void __launch_bounds__(256) k_gemv(ClGemvArgs a) {
             W8<WT>::load(w1 + c, wb);
 #pragma unroll
             for (int t = 0; t < T; ++t) {
-                const float4 x0 = __ldg((const float4 *)(a.xin + (size_t)t * cols + c));
-                const float4 x1 = __ldg((const float4 *)(a.xin + (size_t)t * cols + c + 4));
+                const float4 x0 = *(const float4 *)(a.xin + (size_t)t * cols + c);   // (plain: the predecessor wrote it while this kernel lived)
+                const float4 x1 = *(const float4 *)(a.xin + (size_t)t * cols + c + 4);
                 float s0 = acc0[t], s1 = acc1[t];
                 s0 = fmaf(wa[0], x0.x, s0); s1 = fmaf(wb[0], x0.x, s1);
                 s0 = fmaf(wa[1], x0.y, s0); s1 = fmaf(wb[1], x0.y, s1);

@@ -1,0 +1,35 @@
+"""What a kernel that starts while its predecessor is still running may do, read off the sources (no GPU needed).
+
+Launches chained by programmatic dependent launch overlap: until a kernel has waited for its predecessor, and for read-only
+loads even after that, memory that an earlier kernel of the chain writes is not constant.
+"""
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_14612_b200", "csrc")
+
+
+def _kernels():
+    """(name, body) of every __global__ function."""
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        src = re.sub(r"//[^\n]*", "", open(path).read())
+        for m in re.finditer(r"__global__\s+void[^;{]*?\b(k_\w+)\s*\(", src):
+            start = src.index("{", m.end())
+            depth, i = 1, start + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(src[i], 0)
+                i += 1
+            yield m.group(1), src[start:i]
+
+
+def test_chained_kernels_read_only_weights_through_the_read_only_path():
+    """__ldg is for memory that nobody writes while the kernel lives.  In a kernel that overlaps its predecessor that
+    holds for weights (gains) only, not for rows that the predecessor produces."""
+    chained = [(n, b) for n, b in _kernels() if "pdl_wait()" in b]
+    assert {"k_gemv", "k_rmsnorm", "k_wide_norm"} <= {n for n, _ in chained}
+    weights = {"k_wide_norm": {"a.g"}}
+    for name, body in chained:
+        for operand in re.findall(r"__ldg\((?:\(const \w+ \*\)\s*)?\(?([\w.]+)", body):
+            assert operand in weights.get(name, set()), f"{name} reads {operand} through the read-only path"
+        assert "__restrict__" not in body
