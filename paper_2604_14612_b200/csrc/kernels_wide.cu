@@ -182,6 +182,7 @@ k_wide(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtenso
             int s = 0, n = 0;
             unsigned par = 0u;
             bool ok = true;
+            pdl_wait();   // (operand rows cannot arrive earlier, and the time limits below are for this kernel's own work)
             while (ok && walk.next(pc)) {
                 const unsigned b = (unsigned)n & 1u, acc = tmem + b * WN;
                 if (!bar_wait(&sm->tempty[b], ((unsigned)(n >> 1) & 1u) ^ 1u, &sm->abort, a.err)) break;

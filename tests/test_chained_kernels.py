@@ -33,3 +33,18 @@ def test_chained_kernels_read_only_weights_through_the_read_only_path():
         for operand in re.findall(r"__ldg\((?:\(const \w+ \*\)\s*)?\(?([\w.]+)", body):
             assert operand in weights.get(name, set()), f"{name} reads {operand} through the read-only path"
         assert "__restrict__" not in body
+
+
+def test_bounded_waits_of_a_chained_kernel_begin_after_its_predecessor_has_ended():
+    """The time limit of a wait inside a kernel is for this kernel's own work.  A thread that starts such a wait while the
+    predecessor is running counts the predecessor's time, and a healthy kernel behind a slow one reports a timeout."""
+    for name, body in _kernels():
+        if "pdl_wait()" not in body or "bar_wait(" not in body:
+            continue
+        split = re.search(r"\bif \(warp == 0\) \{", body)             # the roles: if (warp == 0) .. else if (warp == 1) .. else ..
+        if "pdl_wait()" in body[:split.start()]:
+            continue
+        roles = re.split(r"\belse if \(warp == 1\) \{|\n    \} else \{", body[split.start():])
+        assert len(roles) == 3, name
+        for role in roles:
+            assert "pdl_wait()" in role and role.index("pdl_wait()") < role.index("bar_wait("), (name, role[:80])
