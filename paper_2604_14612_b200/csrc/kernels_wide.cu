@@ -381,12 +381,19 @@ __global__ void __launch_bounds__(256) k_wide_rope_append(ClWideParts p, int hd,
 // (its own key is already in the cache).  Keys and values are walked 64 at a time through two shared-memory buffers
 // (cp.async, 16-byte pieces permuted by row & 7), with the usual running maximum and sum per row.
 // Both products run on the tensor cores although the queries and the probabilities are fp32: each enters as three parts
-// of the storage type (v = p0 + p1 + p2 holds 24 bits of it; keys and values are of that type already), so the products are
-// as exact as fp32 ones.  A query row is scaled by a power of two to [1, 2) first, so that the parts of fp16 neither
-// overflow nor underflow.  Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile), 2 % of the
-// pass; the register-tiled fp32 products on the CUDA cores that it replaces took 122 us per layer at 512 rows of 32 heads
-// against 393 us of GEMMs and other kernels.  Blocks of late rows see the most keys and are scheduled first.
+// of the storage type (keys and values are of that type already) that hold at least 24 bits of it.  fp16 has the exponents for
+// that only with scaling: a query row is multiplied by a power of two that brings its largest element to [2^14, 2^15) (bf16: to
+// [1, 2)), a probability by 2^14, and of a probability each part is 2^12 times what the parts before it left, so that weights
+// down to 2^-38 of the row's largest keep 24 bits (ATT_STEP).
+// The sums are as exact as fp32 multiply-adds (relative error against 64 bits at 512 rows after 512 / 64 rows after 4032 keys:
+// 6.9e-7 / 1.4e-6 with those, 4.9e-7 / 8.1e-7 here, fp16): the accumulator of the instruction cuts off where an fp32 addition rounds, which
+// over one chain for all keys of a row came to 2.2e-6 / 9.9e-6, so a chain is one tile of 64 keys, the parts have accumulators of their own
+// and everything else is added in fp32.
+// Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile).  At 512 rows of 32 heads it takes 47 us of a
+// layer's 575; the register-tiled fp32 products on the CUDA cores that it replaces took 127.  Blocks of late rows see the most keys and
+// are scheduled first.
 constexpr int AQ = 64, AK = 64;   // rows per CTA, keys per tile
+constexpr int ATT_STEP = 4096;    // fp16: ratio of a probability part's scale to the part before (a rest is below 2^-11 of its value: no overflow)
 
 template <int HD>
 constexpr size_t attn_wide_smem() { return (size_t)(3 * AQ + 4 * AK) * HD * 2 + AQ * 4; }
@@ -406,15 +413,15 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const unsigned (&a)[4], 
         asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// Two values -> three packed pairs of the 16-bit type whose sums are the values to 24 bits.
-template <int F16>
+// Two values -> three packed pairs of the 16-bit type: v = p0 + p1 / STEP + p2 / STEP^2, each the rest so far rounded.
+template <int F16, int STEP>
 __device__ __forceinline__ void split3(float x, float y, unsigned (&o)[3]) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const unsigned short a = f32_to_b16(x, F16), b = f32_to_b16(y, F16);
         o[i] = (unsigned)a | ((unsigned)b << 16);
-        x -= b16_to_f32(a, F16);
-        y -= b16_to_f32(b, F16);
+        x = (x - b16_to_f32(a, F16)) * (float)STEP;
+        y = (y - b16_to_f32(b, F16)) * (float)STEP;
     }
 }
 
@@ -423,6 +430,9 @@ __global__ void __launch_bounds__(128, 2)
 k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsigned short *vcache, __nv_bfloat16 *out_b,
             int lo_row0, int M, int d, int H, int Hkv, int max_seq, const ClDevState *st) {
     constexpr int RB = HD * 2, NC = HD / 8;           // bytes and 16-byte pieces per row
+    constexpr unsigned TOP = F16 ? 14 : 0;            // exponent of the largest element of a scaled query row, and of a weight of 1
+    constexpr int STEP = F16 ? ATT_STEP : 1;
+    constexpr float PSCALE = F16 ? 16384.f : 1.f;
     extern __shared__ __align__(128) unsigned char asm_[];
     unsigned char *Qs = asm_;                          // [3][AQ][RB] parts of the scaled queries
     float *rs = (float *)(asm_ + (3 * AQ + 4 * AK) * RB);   // [AQ] what a row's scores are multiplied by
@@ -448,7 +458,7 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
     };
     load_tile(0);
 
-    // this warp's 16 query rows: scaled to [1, 2) by a power of two, split, stored; nobody else reads them
+    // this warp's 16 query rows: scaled to [2^TOP, 2^(TOP + 1)) by a power of two, split, stored; nobody else reads them
     constexpr int EL = HD / 32;
 #pragma unroll 4
     for (int rr = 0; rr < 16; ++rr) {
@@ -460,18 +470,18 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
         for (int e = 0; e < EL; ++e) amax = fmaxf(amax, fabsf(v[e]));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        const unsigned ex = min(max(__float_as_uint(amax) >> 23, 1u), 253u);
-        const float inv = __uint_as_float((254u - ex) << 23);
+        const unsigned ex = min(max(__float_as_uint(amax) >> 23, 1u + TOP), 253u);
+        const float inv = __uint_as_float((254u + TOP - ex) << 23);
 #pragma unroll
         for (int e = 0; e < EL; e += 2) {
             unsigned s3[3];
-            split3<F16>(v[e] * inv, v[e + 1] * inv, s3);
+            split3<F16, 1>(v[e] * inv, v[e + 1] * inv, s3);
             const int byte = (lane * EL + e) * 2;
 #pragma unroll
             for (int p = 0; p < 3; ++p)
                 *(unsigned *)(Qs + (size_t)(p * AQ + row) * RB + (((byte >> 4) ^ (row & 7)) << 4) + (byte & 15)) = s3[p];
         }
-        if (lane == 0) rs[row] = __uint_as_float(ex << 23) * rsqrtf((float)HD);
+        if (lane == 0) rs[row] = __uint_as_float((ex - TOP) << 23) * rsqrtf((float)HD);
     }
     __syncwarp();
 
@@ -493,9 +503,11 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
         __syncthreads();
         const int k0 = t * AK;
         const unsigned ka = kv_addr + (unsigned)(t & 1) * 2 * AK * RB, va = ka + AK * RB;
-        float s[AK / 8][4];
+        float s[AK / 8][4], u[AK / 8][4];   // products of the queries' first parts and of the two others
 #pragma unroll
-        for (int n = 0; n < AK / 8; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
+        for (int n = 0; n < AK / 8; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[n][e] = u[n][e] = 0.f;
 #pragma unroll
         for (int ks = 0; ks < HD / 16; ++ks) {
             unsigned qa[3][4];
@@ -508,20 +520,19 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
                 const int kr = np * 16 + (mi >> 1) * 8 + mrow, kc = ks * 2 + (mi & 1);
                 ldsm4(kb, ka + kr * RB + ((kc ^ (kr & 7)) << 4));
 #pragma unroll
-                for (int p = 2; p >= 0; --p) {
-                    mma16816<F16>(s[2 * np], qa[p], kb[0], kb[1]);
-                    mma16816<F16>(s[2 * np + 1], qa[p], kb[2], kb[3]);
-                }
+                for (int p = 0; p < 3; ++p)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) mma16816<F16>(p == 1 ? s[2 * np + j] : u[2 * np + j], qa[p == 0 ? 2 : p == 1 ? 0 : 1], kb[2 * j], kb[2 * j + 1]);
             }
         }
         float mx_a = m_a, mx_b = m_b;
 #pragma unroll
         for (int n = 0; n < AK / 8; ++n) {
             const int key = k0 + n * 8 + lc;
-            s[n][0] = key <= pos_a ? s[n][0] * rs_a : -INFINITY;
-            s[n][1] = key + 1 <= pos_a ? s[n][1] * rs_a : -INFINITY;
-            s[n][2] = key <= pos_b ? s[n][2] * rs_b : -INFINITY;
-            s[n][3] = key + 1 <= pos_b ? s[n][3] * rs_b : -INFINITY;
+            s[n][0] = key <= pos_a ? (s[n][0] + u[n][0]) * rs_a : -INFINITY;
+            s[n][1] = key + 1 <= pos_a ? (s[n][1] + u[n][1]) * rs_a : -INFINITY;
+            s[n][2] = key <= pos_b ? (s[n][2] + u[n][2]) * rs_b : -INFINITY;
+            s[n][3] = key + 1 <= pos_b ? (s[n][3] + u[n][3]) * rs_b : -INFINITY;
             mx_a = fmaxf(mx_a, fmaxf(s[n][0], s[n][1]));
             mx_b = fmaxf(mx_b, fmaxf(s[n][2], s[n][3]));
         }
@@ -545,29 +556,38 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
         }
         l_a = fmaf(l_a, ra, sa);   // (this lane's columns; added over the four lanes of a row at the end)
         l_b = fmaf(l_b, rb, sb);
-#pragma unroll
-        for (int n = 0; n < HD / 8; ++n) {
-            o[n][0] *= ra; o[n][1] *= ra;
-            o[n][2] *= rb; o[n][3] *= rb;
-        }
+        unsigned pa[AK / 16][3][4];
 #pragma unroll
         for (int ks = 0; ks < AK / 16; ++ks) {
-            unsigned pa[3][4], s3[3];
+            unsigned s3[3];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                split3<F16>(s[2 * ks + (e >> 1)][(e & 1) * 2], s[2 * ks + (e >> 1)][(e & 1) * 2 + 1], s3);
-                pa[0][e] = s3[0]; pa[1][e] = s3[1]; pa[2][e] = s3[2];
+                const float *w = &s[2 * ks + (e >> 1)][(e & 1) * 2];
+                split3<F16, STEP>(w[0] * PSCALE, w[1] * PSCALE, s3);
+                pa[ks][0][e] = s3[0]; pa[ks][1][e] = s3[1]; pa[ks][2][e] = s3[2];
             }
+        }
 #pragma unroll
-            for (int np = 0; np < HD / 16; ++np) {
+        for (int np = 0; np < HD / 16; ++np) {
+            float c[3][2][4];   // this tile's sums, part by part
+#pragma unroll
+            for (int i = 0; i < 24; ++i) c[i / 8][i / 4 % 2][i % 4] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < AK / 16; ++ks) {
                 unsigned vb[4];
                 const int vr = ks * 16 + (mi & 1) * 8 + mrow, vc = np * 2 + (mi >> 1);
                 ldsm4_t(vb, va + vr * RB + ((vc ^ (vr & 7)) << 4));
 #pragma unroll
-                for (int p = 2; p >= 0; --p) {
-                    mma16816<F16>(o[2 * np], pa[p], vb[0], vb[1]);
-                    mma16816<F16>(o[2 * np + 1], pa[p], vb[2], vb[3]);
+                for (int p = 0; p < 3; ++p) {
+                    mma16816<F16>(c[p][0], pa[ks][p], vb[0], vb[1]);
+                    mma16816<F16>(c[p][1], pa[ks][p], vb[2], vb[3]);
                 }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int j = i / 4, e = i % 4;
+                const float low = fmaf(c[2][j][e], 1.f / STEP, c[1][j][e]), t = fmaf(low, 1.f / STEP, c[0][j][e]);
+                o[2 * np + j][e] = fmaf(o[2 * np + j][e], e < 2 ? ra : rb, t);
             }
         }
         __syncthreads();   // everyone is done with this buffer: the load after next may overwrite it
@@ -577,7 +597,7 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
         l_a += __shfl_xor_sync(0xffffffffu, l_a, w);
         l_b += __shfl_xor_sync(0xffffffffu, l_b, w);
     }
-    const float ia = 1.f / l_a, ib = 1.f / l_b;
+    const float ia = 1.f / (l_a * PSCALE), ib = 1.f / (l_b * PSCALE);   // (exact: a power of two)
 #pragma unroll
     for (int n = 0; n < HD / 8; ++n) {
         const size_t col = (size_t)h * HD + n * 8 + lc;
