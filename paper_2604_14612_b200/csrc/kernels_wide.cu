@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(256) k_wide_rope_append(ClWideParts p, int hd,
 // 6.9e-7 / 1.4e-6 with those, 4.9e-7 / 8.1e-7 here, fp16): the accumulator of the instruction cuts off where an fp32 addition rounds, which
 // over one chain for all keys of a row came to 2.2e-6 / 9.9e-6, so a chain is one tile of 64 keys, the parts have accumulators of their own
 // and everything else is added in fp32.
-// Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile).  At 512 rows of 32 heads it takes 47 us of a
+// Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile).  At 512 rows of 32 heads it takes 48 us of a
 // layer's 575; the register-tiled fp32 products on the CUDA cores that it replaces took 127.  Blocks of late rows see the most keys and
 // are scheduled first.
 constexpr int AQ = 64, AK = 64;   // rows per CTA, keys per tile
@@ -525,14 +525,49 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
                     for (int j = 0; j < 2; ++j) mma16816<F16>(p == 1 ? s[2 * np + j] : u[2 * np + j], qa[p == 0 ? 2 : p == 1 ? 0 : 1], kb[2 * j], kb[2 * j + 1]);
             }
         }
+        float odd = 0.f;
+#pragma unroll
+        for (int n = 0; n < AK / 8; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                s[n][e] = (s[n][e] + u[n][e]) * (e < 2 ? rs_a : rs_b);
+                odd = fmaf(s[n][e], 0.f, odd);   // (not zero once a score is infinite or no number; 3 % of the kernel)
+            }
+        if (__any_sync(0xffffffffu, odd != 0.f)) {
+            // An infinite key or query: parts of it are zeros and infinities of both signs, whose products add up to no number
+            // where the score is infinite or finite.  This tile's scores anew, from whole queries.
+            const float *qa = q + (size_t)min(row_a, M - 1) * ld_q + h * HD, *qb = q + (size_t)min(row_a + 8, M - 1) * ld_q + h * HD;
+            const float scale = rsqrtf((float)HD);
+#pragma unroll
+            for (int n = 0; n < AK / 8; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
+#pragma unroll 1
+            for (int i = 0; i < HD; ++i) {
+                const float xa = __ldcg(qa + i) * scale, xb = __ldcg(qb + i) * scale;
+#pragma unroll
+                for (int n = 0; n < AK / 8; ++n)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int key = n * 8 + lc + e;
+                        unsigned short raw;
+                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(raw) : "r"(ka + key * RB + (((i >> 3) ^ (key & 7)) << 4) + (i & 7) * 2) : "memory");
+                        const float kv = b16_to_f32(raw, F16);
+                        s[n][e] = fmaf(xa, kv, s[n][e]);
+                        s[n][2 + e] = fmaf(xb, kv, s[n][2 + e]);
+                    }
+            }
+#pragma unroll
+            for (int n = 0; n < AK / 8; ++n)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[n][e] = s[n][e] > -INFINITY ? s[n][e] : -INFINITY;   // (no number: no weight)
+        }
         float mx_a = m_a, mx_b = m_b;
 #pragma unroll
         for (int n = 0; n < AK / 8; ++n) {
             const int key = k0 + n * 8 + lc;
-            s[n][0] = key <= pos_a ? (s[n][0] + u[n][0]) * rs_a : -INFINITY;
-            s[n][1] = key + 1 <= pos_a ? (s[n][1] + u[n][1]) * rs_a : -INFINITY;
-            s[n][2] = key <= pos_b ? (s[n][2] + u[n][2]) * rs_b : -INFINITY;
-            s[n][3] = key + 1 <= pos_b ? (s[n][3] + u[n][3]) * rs_b : -INFINITY;
+            s[n][0] = key <= pos_a ? s[n][0] : -INFINITY;
+            s[n][1] = key + 1 <= pos_a ? s[n][1] : -INFINITY;
+            s[n][2] = key <= pos_b ? s[n][2] : -INFINITY;
+            s[n][3] = key + 1 <= pos_b ? s[n][3] : -INFINITY;
             mx_a = fmaxf(mx_a, fmaxf(s[n][0], s[n][1]));
             mx_b = fmaxf(mx_b, fmaxf(s[n][2], s[n][3]));
         }

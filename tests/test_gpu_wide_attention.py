@@ -84,3 +84,19 @@ def test_light_keys_under_a_heavy_one_keep_their_weight(wd):
         e = err[:, head == h]
         assert np.abs(e).max() <= (2e-3 if wd == "fp16" else 1.6e-2), (gaps[h], np.abs(e).max())
         assert abs(e.mean()) <= (1e-5 if wd == "fp16" else 1e-4), (gaps[h], e.mean())
+
+
+def test_keys_that_overflowed_the_cache_and_score_minus_infinity_have_no_weight():
+    """Keys of 1e5 are infinite in an fp16 cache.  Against a negative query they score -inf: their weight is 0 and the first
+    token's value is the whole output of every row."""
+    n = 600
+    g = torch.Generator().manual_seed(6)
+    values, first = (1.0 + torch.rand(256, generator=g)) * 500, 1.0 + torch.rand(256, generator=g)
+    first[:3] = 0.0
+    ctx, emb, _ = _model("fp16", 4, n, [-32.0, -1.0, -3.3, -0.01], values, first_key=0.0, other_key=1e5, first_value=first)
+    tokens = np.concatenate([[0], 1 + np.arange(n - 1) % (V - 1)]).astype(np.int32)
+    got = _hidden(ctx, n, tokens)
+    ctx.close()
+    want = (first / 16.0).half().double().numpy() * 16.0
+    assert np.isfinite(got).all()
+    assert np.abs(got - emb[tokens[n - P:]] - want)[:, 3:].max() <= 2e-3          # half a step of fp16 at 2 is 1e-3
