@@ -38,16 +38,19 @@ namespace {
 // half tile) of which every pair takes an equal contiguous share.  A share may end inside a tile: a tile's product comes in
 // as many parts as pairs touched it, part = pair - first pair of the tile.  Equal shares matter: 4096 x 4096 outputs at
 // M = 512 are 32 tiles for 74 pairs.
-// The accumulator is double-buffered (2 x 256 columns): the store of one piece overlaps the multiply-adds of the next.  A
-// piece is at most `chain` K blocks of one tile (a longer accumulation chain in tensor memory loses accuracy); later pieces
-// of a share are added to the part's memory.
+// The tensor-memory accumulator cuts off where an fp32 addition rounds: a sum loses about 2^-26 of itself per instruction, all in
+// one direction.  So a chain is at most `chain` K blocks of one tile (a piece), and the pieces of a share are added in fp32 in
+// the registers of the store warps.  Error of the sums against 64 bits, 512 rows x 4096 x 11008 fp16, chains of 32 / 16 / 8 / 4 blocks:
+// 4.5e-6 / 2.4e-6 / 1.2e-6 / 6.6e-7; call of 512 tokens at 8 layers, chains of 16 / 8 / 4: 4.70 / 4.68 / 4.79 ms, of 61 tokens 2.10 / 2.11 / 2.17.
+// (Later pieces were added in memory before, chains of 32: 4.83 ms.)  The accumulator is double-buffered (2 x 256 columns):
+// reading one piece overlaps the multiply-adds of the next.
 // Roles per CTA: warp 0 TMA producer (the weights of the first stages are requested before the wait for the previous
-// kernel), warp 1 tensor memory and, in CTA 0, the multiply-adds, warps 2-5 store (thread = operand row, 32 bytes per
-// store instruction).
-constexpr int WN = 256, WTHREADS = 192, W_TILE = 128 * TC_BK * 2;   // 16 KB: 128 rows x 64 elements
+// kernel), warp 1 tensor memory and, in CTA 0, the multiply-adds, warps 2-9 add and store (thread = operand row x 128 columns,
+// 32 bytes per store instruction).
+constexpr int WN = 256, W_STORE_WARPS = 8, WTHREADS = 64 + 32 * W_STORE_WARPS, W_TILE = 128 * TC_BK * 2;   // 16 KB: 128 rows x 64 elements
 constexpr int W_SMEM_TILES = 12;                                     // 192 KB ring: 4 stages of 3 tiles, or 6 of 2 (half tiles only)
 constexpr int W_MAX_STAGES = 6;
-constexpr int W_CHAIN = 32;   // K blocks (of 64 elements) per accumulation chain
+constexpr int W_CHAIN = 8;    // K blocks (of 64 elements) per accumulation chain
 
 struct WSmem {
     unsigned long long full[W_MAX_STAGES], empty[W_MAX_STAGES], tfull[2], tempty[2];
@@ -58,13 +61,12 @@ struct WSmem {
 // The share of a pair, walked piece by piece.
 struct WPiece {
     int nt, mt, kb0, kb1;   // tile and its K blocks
-    bool half, first;       // first piece of this share in the tile: stores, later ones add
+    bool half, last;        // last: the last piece of this share in the tile
 };
 struct WWalk {
     const ClWideParts &p;
     int chain, nt, mt, kb, c, c1;   // next K block; cost of all blocks before it; end of the share
-    bool fresh;
-    __device__ WWalk(const ClWideParts &parts, int pair, int chain_) : p(parts), chain(chain_), fresh(true) {
+    __device__ WWalk(const ClWideParts &parts, int pair, int chain_) : p(parts), chain(chain_) {
         const int T = cl_wide_cost(p), W = cl_wide_col_cost(p), c0 = (int)((long long)T * pair / p.G);
         c1 = (int)((long long)T * (pair + 1) / p.G);
         nt = c0 / W;
@@ -89,10 +91,9 @@ struct WWalk {
         o.kb0 = kb;
         const int left = o.half ? c1 - c : (c1 - c + 1) >> 1;
         o.kb1 = min(min(p.KB, kb + chain), kb + left);
-        o.first = fresh || kb == 0;
-        fresh = false;
         c += (o.kb1 - kb) * (o.half ? 1 : 2);
         kb = o.kb1;
+        o.last = kb == p.KB || c >= c1;
         if (kb == p.KB) step();
         return true;
     }
@@ -114,7 +115,7 @@ k_wide(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtenso
         }
         for (int i = 0; i < 2; ++i) {
             bar_init(&sm->tfull[i], 1);
-            bar_init(&sm->tempty[i], 8);   // the store warps of both CTAs
+            bar_init(&sm->tempty[i], 2 * W_STORE_WARPS);   // the store warps of both CTAs
         }
         sm->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -204,36 +205,41 @@ k_wide(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtenso
             }
         }
     } else {
-        // ---------------- store: one thread per operand row ----------------
-        const int q = warp & 3;                        // the tensor-memory lane quadrant this warp may read
+        // ---------------- add and store: one thread per operand row and half of the columns ----------------
+        constexpr int WC = WN * 4 / W_STORE_WARPS;   // columns of a warp
+        const int q = warp & 3, colw = ((warp - 2) >> 2) * WC;   // q: the tensor-memory lane quadrant this warp may read
+        float sum[WC];   // of the pieces so far of this share's tile
+#pragma unroll
+        for (int i = 0; i < WC; ++i) sum[i] = 0.f;
         pdl_wait();   // the previous kernel may still read the product buffer
         for (int n = 0; walk.next(pc); ++n) {
             const unsigned b = (unsigned)n & 1u;
             if (!bar_wait(&sm->tfull[b], (unsigned)(n >> 1) & 1u, &sm->abort, a.err)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            int part = pair - cl_wide_owner(a.p, pc.nt, pc.mt, 0);
-            int t = pc.mt * 256 + q * 32 + lane;
-            if (pc.half) part = 2 * part + rank;
-            else t += rank * 128;
-            float *dst = a.p.P + ((size_t)part * a.p.M + (size_t)min(t, a.p.M - 1)) * a.p.rows;
-#pragma unroll 1
-            for (int cb = 0; cb < WN / 32; ++cb) {
-                float v[32];
-                tmem_ld32(tmem + b * WN + ((unsigned)(q * 32) << 16) + (unsigned)(cb * 32), v);   // (whole warp, also rows past M)
-                const int col0 = pc.nt * WN + cb * 32;
-                if (t < a.p.M) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        if (col0 + 8 * i + 8 <= a.p.rows) {
-                            if (pc.first) st_global_v8(dst + col0 + 8 * i, v + 8 * i);
-                            else red_add_v8(dst + col0 + 8 * i, v + 8 * i);
-                        }
-                    }
-                }
+            for (int c = 0; c < WC; c += 16) {   // (16 at a time: 128 sums and 32 values loaded do not fit the 168 registers)
+                float v[16];
+                tmem_ld16(tmem + b * WN + ((unsigned)(q * 32) << 16) + (unsigned)(colw + c), v);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) sum[c + i] += v[i];
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) bar_arrive_rank0(&sm->tempty[b]);
+            if (!pc.last) continue;   // (uniform)
+            const int t = pc.mt * 256 + q * 32 + lane + (pc.half ? 0 : rank * 128);
+            if (t < a.p.M) {
+                int part = pair - cl_wide_owner(a.p, pc.nt, pc.mt, 0);
+                if (pc.half) part = 2 * part + rank;
+                const int col0 = pc.nt * WN + colw;
+                float *dst = a.p.P + ((size_t)part * a.p.M + (size_t)t) * a.p.rows + col0;
+#pragma unroll
+                for (int i = 0; i < WC; i += 8)
+                    if (col0 + i + 8 <= a.p.rows) st_global_v8(dst + i, sum + i);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < WC; ++i) sum[i] = 0.f;
         }
     }
 

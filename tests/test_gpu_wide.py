@@ -75,3 +75,35 @@ def test_wide_attention_takes_any_score_range():
     # tie to within a unit: rows with one dominant key agree, so all but a few do
     row = np.abs(got[0] - got[1]).max(axis=2) <= 2 ** -7 * max(1.0, float(np.abs(got[0]).max()))
     assert row.mean() >= 0.9
+
+
+@pytest.mark.parametrize("wd,n", [("fp16", 512), ("fp16", 300), ("bf16", 256)])
+def test_products_of_full_tiles_against_fp64(wd, n):
+    """The FFN half of a layer of width 4096 (sums over 4096 and 11008 elements: several accumulation chains per tile, shares that
+    end inside a tile), every row against fp64.  Each hidden value is the exact one rounded to the storage type, up to what the
+    sums lose: the accumulator of the tensor core cuts off, which makes results smaller, about 2^-26 of them per instruction of a
+    chain of 64 (8 K blocks, hi and lo parts): 1e-6 per matrix, three matrices and the slope of SiLU: 4e-6.  Seen through the
+    storage type's rounding, 2^-11 / sqrt(3) of a value (fp16) over n * 4096 values, 3e-7 (bf16: eight times that)."""
+    d, F, dt = 4096, 11008, {"fp16": torch.float16, "bf16": torch.bfloat16}[wd]
+    g = torch.Generator(device="cuda").manual_seed(n)
+    rnd = lambda r, c, std: (torch.randn((r, c), generator=g, device="cuda") * std).to(dt)
+    zero = torch.zeros((d, d), device="cuda", dtype=dt)
+    V = 2000
+    W = dict(embed=rnd(V, d, 0.5), lm_head=rnd(V, d, 0.02), final_norm=torch.ones(d, device="cuda"), wq=[zero], wk=[zero], wv=[zero], wo=[zero],
+             wg=[rnd(F, d, 0.02)], wu=[rnd(F, d, 0.02)], wd=[rnd(d, F, 0.02)], norm1=[torch.ones(d, device="cuda")],
+             norm2=[1.0 + 0.1 * torch.randn(d, generator=g, device="cuda")])
+    ctx = cl.Context(1, d, 32, F, V, n + 8, wd, tap_positions=n)
+    ctx.cl_load(W)
+    prompt = synth.make_prompt(23, n, V)
+    ctx.cl_prefill(prompt, tap_hidden=True)
+    got = ctx.cl_read_hidden_ring()[0].double().cuda()
+    ctx.close()
+    x = W["embed"][torch.as_tensor(np.asarray(prompt), device="cuda", dtype=torch.long)].double()
+    xn = x * torch.rsqrt((x * x).mean(-1, keepdim=True) + 1e-5) * W["norm2"][0].double()
+    up = torch.nn.functional.silu(xn @ W["wg"][0].double().T) * (xn @ W["wu"][0].double().T)
+    ffn = up @ W["wd"][0].double().T
+    err = got - (x + ffn)
+    half = 2.0 ** (-11 if wd == "fp16" else -8)
+    assert (err.abs() - half * (x + ffn).abs()).max() <= 1e-4 * ffn.abs().max()
+    bias = float((err * ffn).sum() / (ffn * ffn).sum())
+    assert abs(bias) <= (5e-6 if wd == "fp16" else 8e-6), bias
