@@ -38,6 +38,17 @@ __device__ __forceinline__ void fma2(unsigned long long &c, unsigned long long a
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
 }
 
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // Eight consecutive elements of a row as floats; zeros where k >= d (d is a multiple of 8).
 template <typename T>
 struct Raw8;
@@ -70,8 +81,9 @@ __device__ __forceinline__ int tile_at(int k, int c) { return k * 128 + ((((c >>
 template <typename T, int TM>
 __global__ void __launch_bounds__(HT, 2) k_head_rows(HeadRowsArgs a) {
     extern __shared__ __align__(16) float sm[];
-    float *As = sm, *Bs = As + HK * 128, *total = Bs + HK * HN;       // total: [TM * 8][HT], the sums of finished chains
-    ClHeadPartial *run = (ClHeadPartial *)(total + TM * 8 * HT);      // [2][16 * TM], per half of a tile's columns
+    float *As = sm, *Bs = As + HK * 128;
+    unsigned long long *total = (unsigned long long *)(Bs + HK * HN);   // [TM * 4][HT] pairs, the sums of finished chains
+    ClHeadPartial *run = (ClHeadPartial *)(total + TM * 4 * HT);        // [2][16 * TM], per half of a tile's columns
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int mt = blockIdx.x % a.MT, rg = blockIdx.x / a.MT;
     const int row0 = mt * a.rows, nrows = min(a.rows, a.R - row0);
@@ -89,7 +101,7 @@ __global__ void __launch_bounds__(HT, 2) k_head_rows(HeadRowsArgs a) {
     for (int nt = nt0; nt < nt1; ++nt) {
         const int n0 = nt * HN;
 #pragma unroll
-        for (int i = 0; i < TM * 8; ++i) total[i * HT + tid] = 0.f;
+        for (int i = 0; i < TM * 4; ++i) total[i * HT + tid] = 0ull;
         unsigned long long acc[TM][4];
 #pragma unroll
         for (int r = 0; r < TM; ++r)
@@ -156,16 +168,12 @@ __global__ void __launch_bounds__(HT, 2) k_head_rows(HeadRowsArgs a) {
                 for (int r = 0; r < TM; ++r)
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        float u[2];
-                        unpack2(acc[r][c], u[0], u[1]);
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            float &tot = total[(r * 8 + 2 * c + e) * HT + tid];
-                            const float t = tot, sum = t + u[e], b = sum - t;
-                            tot = sum;
-                            u[e] = (t - (sum - b)) + (u[e] - b);   // what the sum lost opens the next chain
-                        }
-                        acc[r][c] = pack2(u[0], u[1]);
+                        unsigned long long &tot = total[(r * 4 + c) * HT + tid];
+                        const unsigned long long t = tot, u = acc[r][c], sum = add2(t, u), b = sub2(sum, t);
+                        float x, y;   // what the two sums lost opens the next chain; no number beside a sum that is not finite: that sum stays
+                        unpack2(add2(sub2(t, sub2(sum, b)), sub2(u, b)), x, y);
+                        tot = sum;
+                        acc[r][c] = pack2(x == x ? x : 0.f, y == y ? y : 0.f);
                     }
             }
         }
@@ -177,8 +185,10 @@ __global__ void __launch_bounds__(HT, 2) k_head_rows(HeadRowsArgs a) {
             float l[8];
             ClHeadPartial p{-INFINITY, 0.f, 0.f, 0x7fffffff};
 #pragma unroll
+            for (int c = 0; c < 4; ++c) unpack2(total[(r * 4 + c) * HT + tid], l[2 * c], l[2 * c + 1]);
+#pragma unroll
             for (int c = 0; c < 8; ++c) {
-                l[c] = fminf(fmaxf(total[(r * 8 + c) * HT + tid], -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP);   // clamp of Section 3.1
+                l[c] = fminf(fmaxf(l[c], -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP);   // clamp of Section 3.1
                 if (col(c) < a.V && l[c] > p.m) { p.m = l[c]; p.idx = col(c); }
             }
             if (p.m == -INFINITY) p.m = 0.f;   // (no valid column: z stays 0 and the partial is ignored)

@@ -36,3 +36,41 @@ def test_tiled_scoring_against_fp64(dtype, V, d, n):
         clear = ((top[:, 0] - top[:, 1]) > 1e-4).cpu().numpy()
         assert np.array_equal(got["argmax"][clear], lg.argmax(-1).cpu().numpy()[clear])
         assert got["argmax"][0] == 0 and abs(got["p_max"][0] - 1 / V) <= 1e-6
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("n", [16, 17, 100])
+def test_logits_beyond_the_clamp_or_infinite(dtype, n):
+    """A logit beyond 1e4 counts as 1e4 (Section 3.1), also where its sum overflows fp32, early in the row or late; the number of
+    rows decides which kernel runs and must not show."""
+    V, d = 300, 512
+    dt = {"bf16": torch.bfloat16, "fp32": torch.float32}[dtype]
+    g = torch.Generator(device="cuda").manual_seed(n)
+    head = (torch.randn((V, d), generator=g, device="cuda") * 2 / d ** 0.5).to(dt)
+    hidden = torch.randn((n, d), generator=g, device="cuda")
+    sign = torch.where(torch.arange(n, device="cuda") % 2 == 0, 1.0, -1.0)
+    hidden[:, [5, 6, 500]] = (hidden[:, [5, 6, 500]].abs() + 0.5) * sign[:, None]
+    hidden[n // 2, [5, 6, 500]] = hidden[n // 2, [5, 6, 500]].abs()
+    hidden = hidden.to(dt)
+    gain = torch.ones(d, device="cuda")
+    special = {7: (5, float("inf")), 9: (6, 3e38), 11: (5, float("-inf")), 13: (500, float("inf")), 15: (6, 3e6)}
+    for pick in ([7], [9], [11], [13], [15], [7, 9, 11, 13, 15]):
+        W = head.clone()
+        for r in pick:
+            W[r, special[r][0]] = special[r][1]
+        if 9 in pick:
+            W[9, 5] = 3e38
+        got = cl.cl_layer_confidences_static(W, gain, hidden, rms_eps=1e-5)
+        x = hidden.double()
+        xn = x * torch.rsqrt((x * x).mean(-1, keepdim=True) + 1e-5)
+        lg = (xn @ W.double().T).clamp(-1e4, 1e4)
+        lp = torch.log_softmax(lg, -1)
+        conf = (1 + (lp.exp() * lp).nan_to_num(0.0).sum(-1) / np.log(V)).cpu().numpy()
+        assert np.abs(got["conf"] - conf).max() <= 2e-5, pick
+        assert np.abs(got["p_max"] - lp.max(-1).values.exp().cpu().numpy()).max() <= 2e-5, pick
+        top = torch.topk(lg, 2).values
+        clear = ((top[:, 0] - top[:, 1]) > 1e-4).cpu().numpy()
+        assert np.array_equal(got["argmax"][clear], lg.argmax(-1).cpu().numpy()[clear]), pick
+        tied = (lg == 1e4).sum(-1) > 1
+        first = (lg == 1e4).int().argmax(-1)
+        assert np.array_equal(got["argmax"][tied.cpu().numpy()], first[tied].cpu().numpy()), pick   # ties: the lowest index
