@@ -306,18 +306,19 @@ __global__ void k_rmsnorm_to_bf16(const ST *x, const float *g, int d, float eps,
 
 }  // namespace
 
-// Row blocks and vocabulary ranges of R rows.  A pair's tile counts as two single ones and is finished in about 7 / 8 of the
-// time (measured at 2048 rows); the pair is taken when the longest range of a pair, so weighted, is no longer than that of a
-// single CTA: 256 rows or 2048 go to pairs, 128 rows (half a pair's tile) or 384 do not.
+// Row blocks and vocabulary ranges of R rows.  A pair's tile counts as two single ones.  It pays where the multiply-adds of a tile
+// take longer than its epilogue (time of pairs / single CTAs with equally long ranges at 512 .. 2560 rows: width 768 to 2048 1.01 to 1.03,
+// 2560 and 3072 0.97 to 1.04, 4096 and 5120 0.89 to 0.95) and where the longest range is not much longer in pairs (at 4096 and 5120, ranges of
+// 42 / 39 tiles 0.98, 13 / 12 0.97, 51 / 46 and 36 / 32 1.02 to 1.03, 14 / 11 1.06).
 struct ScorePlan {
     bool pair;
     int MT, NCG;
 };
-static ScorePlan score_plan(int R, int V, int n_sm) {
+static ScorePlan score_plan(int R, int V, int KB, int n_sm) {
     const int NT = (V + BN - 1) / BN, MT1 = (R + BM - 1) / BM, MT2 = (MT1 + 1) / 2;
     const int n1 = std::min(NT, std::max(1, n_sm / MT1)), n2 = std::min(NT, std::max(1, n_sm / 2 / MT2));
     const long long w1 = ((long long)MT1 * n1 + n_sm - 1) / n_sm, w2 = ((long long)MT2 * n2 + n_sm / 2 - 1) / (n_sm / 2);   // waves
-    const bool pair = (NT + n2 - 1) / n2 * w2 * 7 <= (NT + n1 - 1) / n1 * w1 * 8;
+    const bool pair = KB >= 64 && (NT + n2 - 1) / n2 * w2 * 12 <= (NT + n1 - 1) / n1 * w1 * 13;
     return pair ? ScorePlan{true, MT2, n2} : ScorePlan{false, MT1, n1};
 }
 
@@ -337,7 +338,7 @@ cudaError_t cl_launch_rmsnorm_bf16(int in_dtype, const void *x, const float *g, 
 // xn: [R, d] bf16 normalised rows; lm_head: [V, d] bf16.  Needs d % 8 == 0 and 16-byte aligned bases.
 cudaError_t cl_launch_score_tc(const void *xn, const void *lm_head, int R, int V, int d, ClHeadPartial *partials, int n_sm,
                                int *err, float *conf, float *pmax, int *arg, int f16, cudaStream_t s) {
-    const ScorePlan plan = score_plan(R, V, n_sm);
+    const ScorePlan plan = score_plan(R, V, (d + BK - 1) / BK, n_sm);
     CUtensorMap mapA, mapB;
     if (!make_map(&mapA, xn, R, d, BM, f16) || !make_map(&mapB, lm_head, V, d, plan.pair ? BN / 2 : BN, f16)) return cudaErrorInvalidValue;
     ScoreArgs a;
