@@ -5,13 +5,15 @@
 //
 // Bound: fp32 multiply-adds (the activations stay fp32, so the 16-bit tensor pipe does not apply): 26 GFLOP for 100 rows of
 // the 32000 x 4096 head are 0.35 ms at 74 TFLOP/s.  The eight-row GEMV passes it replaces re-read the head every eight rows and
-// re-read the rows from L1 for every pair of weights, 266 us a pass (100 rows: 3.56 ms for the call, this kernel 1.06).  Shared-
-// memory reads bound it next: 16 wavefronts per 28 packed multiply-adds of a warp at TM = 7.  A CTA takes a tile of 16 * TM rows by 128 weights,
-// 32 elements of K at a time, a thread TM x 8 products as packed pairs (fma.rn.f32x2: two products an instruction, each
-// rounded as fmaf rounds); two CTAs per SM cover each other's barriers.
-// Sums are kept in chains of 64 elements of K, added up in shared memory; what such an addition rounds off opens the next
-// chain (error of the confidences against 64 bits: GEMV 3.6e-7, chains of 64 without that 7e-7, with it 3.1e-7).  Rows are asked for in L2 eight lines ahead: a step of 32 elements is shorter than a trip to
-// HBM.
+// re-read the rows from L1 for every pair of weights, 266 us a pass (100 rows: 3.45 ms for the call, this kernel 1.04).  Shared-
+// memory reads bound it next: 16 wavefronts per 28 packed multiply-adds of a warp at TM = 7.  A CTA takes a tile of 16 * TM rows
+// by 128 weights, 32 elements of K at a time, a thread TM x 8 products as packed pairs (fma.rn.f32x2: two products an
+// instruction, each rounded as fmaf rounds); two CTAs per SM cover each other's barriers.
+// Sums are kept in chains of 64 elements of K, added up in shared memory; what such an addition rounds off opens the next chain.
+// A row's scale and its confidence are worked out in 64 bits.  Error of the confidences against 64 bits, mean over 17 to 400 rows
+// and five inputs, widths 768 / 4096 / 5120: GEMV 3.3e-7 / 3.8e-7 / 4.1e-7, here 2.7e-7 / 2.3e-7 / 2.5e-7 (with scale and confidence
+// in 32 bits 3.5e-7 / 3.3e-7 / 3.3e-7).
+// Rows are asked for in L2 eight lines ahead: a step of 32 elements is shorter than a trip to HBM.
 // The rows of a tile are a matter of balance: R rows are ceil(R / 128) tiles of equal size, rounded up to 16 rows.
 #include <math.h>
 
@@ -212,32 +214,33 @@ __global__ void __launch_bounds__(HT, 2) k_head_rows(HeadRowsArgs a) {
     for (int r = tid; r < nrows; r += HT) a.part[(size_t)(row0 + r) * a.NR + rg] = cl_hp_merge(run[r], run[16 * TM + r]);
 }
 
-// scale[r] = 1 / sqrt(mean x^2 + eps), one CTA per row
+// scale[r] = 1 / sqrt(mean x^2 + eps), one CTA per row.  In 64 bits up to the result: its error moves all logits of a row
+// together, and fp32 sums, quotients and roots made it the largest part of a narrow row's error (see the head of this file).
 template <typename T>
 __global__ void __launch_bounds__(256) k_row_scale(const T *x, int d, float eps, float *scale) {
-    __shared__ float red[8];
-    float ss = 0.f;
+    __shared__ double red[8];
+    double ss = 0.0;
     for (int i = threadIdx.x * 8; i < d; i += 2048) {
         Raw8<T> r;
         float v[8];
         r.load(x + (size_t)blockIdx.x * d + i, true);
         r.get(v);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) ss = fmaf(v[e], v[e], ss);
+        for (int e = 0; e < 8; ++e) ss = fma((double)v[e], (double)v[e], ss);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
     __syncthreads();
     if (threadIdx.x == 0) {
-        float tot = 0.f;
+        double tot = 0.0;
         for (int w = 0; w < 8; ++w) tot += red[w];
-        scale[blockIdx.x] = 1.0f / sqrtf(tot / (float)d + eps);
+        scale[blockIdx.x] = (float)(1.0 / sqrt(tot / d + (double)eps));
     }
 }
 
 // One warp per row: the ranges' statistics in a fixed order, then Eq. 2-4.
-__global__ void __launch_bounds__(128) k_head_rows_merge(const ClHeadPartial *part, int R, int NR, float inv_log_v, float *conf, float *pmax, int *arg) {
+__global__ void __launch_bounds__(128) k_head_rows_merge(const ClHeadPartial *part, int R, int NR, double inv_log_v, float *conf, float *pmax, int *arg) {
     const int r = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= R) return;
     ClHeadPartial f{0.f, 0.f, 0.f, 0x7fffffff};
@@ -248,8 +251,8 @@ __global__ void __launch_bounds__(128) k_head_rows_merge(const ClHeadPartial *pa
         f = (lane & o) == 0 ? cl_hp_merge(f, other) : cl_hp_merge(other, f);
     }
     if (lane == 0) {
-        const float H = logf(f.z) - f.s / f.z;
-        conf[r] = 1.f - H * inv_log_v;
+        const double H = log((double)f.z) - (double)f.s / f.z;   // (64 bits: 1 - H / log V cancels most of a flat row's digits)
+        conf[r] = (float)(1.0 - H * inv_log_v);
         pmax[r] = 1.f / f.z;
         arg[r] = f.idx;
     }
@@ -298,6 +301,6 @@ cudaError_t cl_launch_head_rows(int wdtype, const void *W, const void *x, const 
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = wdtype == 1 ? launch_tm<__nv_bfloat16>(a, s) : launch_tm<float>(a, s);
     if (e != cudaSuccess) return e;
-    k_head_rows_merge<<<(R + 3) / 4, 128, 0, s>>>(part, R, a.NR, (float)(1.0 / log((double)V)), conf, pmax, arg);
+    k_head_rows_merge<<<(R + 3) / 4, 128, 0, s>>>(part, R, a.NR, 1.0 / log((double)V), conf, pmax, arg);
     return cudaGetLastError();
 }

@@ -74,3 +74,25 @@ def test_logits_beyond_the_clamp_or_infinite(dtype, n):
         tied = (lg == 1e4).sum(-1) > 1
         first = (lg == 1e4).int().argmax(-1)
         assert np.array_equal(got["argmax"][tied.cpu().numpy()], first[tied].cpu().numpy()), pick   # ties: the lowest index
+
+
+def test_error_of_narrow_rows_is_that_of_fp32_sums():
+    """4000 rows of width 768 with a leading logit of 10 to 14: the 2-norm of the error of confidence and top-1 probability against
+    fp64.  Eight-row passes of the other kernel leave 1.8e-7 and 2.1e-7 on these inputs, this one 1.5e-7 and 2.1e-7, and with scale
+    and confidence worked out in fp32 1.85e-7 and 2.36e-7 (three seeds, each within 2 %)."""
+    V, d, n = 32000, 768, 4000
+    g = torch.Generator(device="cuda").manual_seed(77)
+    e = torch.randn((V, d), generator=g, device="cuda")
+    head = (torch.roll(e, 1, 0) * (1.28 / d ** 0.5)).bfloat16()
+    gain = 1.0 + 0.1 * torch.randn((d,), generator=g, device="cuda")
+    rho = ((10 + 4 * torch.rand((n, 1), generator=g, device="cuda")) / (1.28 * d ** 0.5)).clamp(max=0.9)
+    x = e[torch.randint(0, V, (n,), generator=g, device="cuda")] * rho + torch.randn((n, d), generator=g, device="cuda") * torch.sqrt(1 - rho * rho)
+    hidden = (3 * x).bfloat16()
+    got = cl.cl_layer_confidences_static(head, gain, hidden, rms_eps=1e-5)
+    h = hidden.double()
+    lg = (h * torch.rsqrt((h * h).mean(-1, keepdim=True) + 1e-5) * gain.double()) @ head.double().T
+    lp = torch.log_softmax(lg, -1)
+    conf = (1 + (lp.exp() * lp).sum(-1) / np.log(V)).cpu().numpy()
+    pm = lp.max(-1).values.exp().cpu().numpy()
+    err = [np.linalg.norm(a - b) / np.linalg.norm(b) for a, b in ((got["conf"], conf), (got["p_max"], pm))]
+    assert err[0] <= 1.8e-7 and err[1] <= 2.2e-7, err
