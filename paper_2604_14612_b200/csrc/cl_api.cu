@@ -40,7 +40,7 @@ struct cl_ctx {
     int head_grid;
     ClDevState *st;
     ClDevState *h_st;             // pinned host mirror
-    float *h_logits;              // pinned staging of the logits that a draft or verify call hands out
+    float *h_logits;              // pinned staging of the logits that a draft or verify call hands out, behind *h_st (null: not to be had)
     int *prompt_dev;              // [max_seq]
     int *out_dev;                 // generated tokens
     int out_cap;
@@ -168,7 +168,16 @@ static int poke(cl_ctx *c, const ClPoke &p) {
 // Logits go to the host through pinned memory, in the same wait as the state: a copy into the caller's pageable buffer
 // is staged by the driver in a second round trip (cycle with 9 rows of 32000 logits 1.86 ms, this way 1.68).
 static int fetch_logits(cl_ctx *c, int rows) {
-    CU(cudaMemcpyAsync(c->h_logits, c->logits, (size_t)rows * c->cfg.vocab * 4, cudaMemcpyDeviceToHost, c->stream));
+    if (c->h_logits)
+        CU(cudaMemcpyAsync(c->h_logits, c->logits, (size_t)rows * c->cfg.vocab * 4, cudaMemcpyDeviceToHost, c->stream));
+    return CL_OK;
+}
+
+// After the wait: into the caller's buffer.
+static int hand_logits(cl_ctx *c, int rows, float *logits) {
+    const size_t bytes = (size_t)rows * c->cfg.vocab * 4;
+    if (c->h_logits) memcpy(logits, c->h_logits, bytes);
+    else CU(cudaMemcpy(logits, c->logits, bytes, cudaMemcpyDeviceToHost));
     return CL_OK;
 }
 
@@ -231,7 +240,6 @@ static void free_all(cl_ctx *c) {
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->h_st) cudaFreeHost(c->h_st);
-    if (c->h_logits) cudaFreeHost(c->h_logits);
 }
 
 extern "C" int cl_destroy(cl_ctx *c) {
@@ -285,7 +293,16 @@ extern "C" int cl_load(cl_ctx *c, const cl_weights *w) {
     CU(cudaMemcpyAsync(c->final_norm, w->final_norm, d * 4, kind, c->stream));
     DM(c->st, sizeof(ClDevState));
     CU(cudaMemsetAsync(c->st, 0, sizeof(ClDevState), c->stream));
-    CU(cudaMallocHost((void **)&c->h_st, sizeof(ClDevState)));
+    // One page-locked block for the state and, where passes can run, the logits they hand out: each block costs milliseconds
+    // (cl_load with a 128256-token vocabulary 16.6 ms with two blocks, 14.5 with one; without the logits 13.1).  Locking the
+    // logits' part only when they are first asked for moves 2 to 3.5 ms into that call (a cycle's first pass 1.75 -> 5.5 ms).
+    const size_t st_bytes = (sizeof(ClDevState) + 255) / 256 * 256, lg_bytes = c->head_only ? 0 : (size_t)CL_MAX_T * V * 4;
+    if (lg_bytes && cudaMallocHost((void **)&c->h_st, st_bytes + lg_bytes) == cudaSuccess) {
+        c->h_logits = (float *)((char *)c->h_st + st_bytes);
+    } else {   // (so much page-locked memory is not to be had: logits are copied into the caller's memory directly)
+        cudaGetLastError();
+        CU(cudaMallocHost((void **)&c->h_st, sizeof(ClDevState)));
+    }
     memset(c->h_st, 0, sizeof(ClDevState));
     DM(c->xn, (size_t)CL_MAX_T * d * 4);
     DM(c->logits, (size_t)CL_MAX_T * V * 4);
@@ -304,7 +321,6 @@ extern "C" int cl_load(cl_ctx *c, const cl_weights *w) {
         DM(c->wbuf, per_layer * L);
         DM(c->norms, 2 * L * d * 4);
         DM(c->embed, V * d * es);
-        CU(cudaMallocHost((void **)&c->h_logits, (size_t)CL_MAX_T * V * 4));
         CU(cudaMemcpyAsync(c->embed, w->embed, V * d * es, kind, c->stream));
         const size_t kv_layer = (size_t)g.max_seq * kvd * es;
         DM(c->kv, 2 * L * kv_layer);
@@ -875,7 +891,7 @@ extern "C" int cl_draft(cl_ctx *c, int K, float stop_p, int32_t *toks, float *p_
     if ((rc = check_device_err(c, "cl_draft"))) return rc;
     if (n < 1 || n > K) return fail(c, CL_ECUDA, "cl_draft: the device reported %d drafted tokens", n);
     c->h_ndraft = n;
-    if (logits) memcpy(logits, c->h_logits, (size_t)n * c->cfg.vocab * 4);
+    if (logits && (rc = hand_logits(c, n, logits))) return rc;
     for (int i = 0; i < n; ++i) {
         if (toks) toks[i] = c->h_st->cyc_tok[1 + i];
         if (p_max) p_max[i] = c->h_st->d_pmax[i];
@@ -915,7 +931,7 @@ extern "C" int cl_verify(cl_ctx *c, int tap_hidden, int32_t *target_toks, float 
     if ((rc = check_device_err(c, "cl_verify"))) return rc;   // target tokens of an aborted pass are never handed out
     if (c->h_ctx + T > c->h_filled) c->h_filled = c->h_ctx + T;
     if (tap_hidden) c->tapped += 1;
-    if (logits) memcpy(logits, c->h_logits, (size_t)T * c->cfg.vocab * 4);
+    if (logits && (rc = hand_logits(c, T, logits))) return rc;
     if (target_toks)
         for (int i = 0; i < T; ++i) target_toks[i] = c->h_st->tgt_tok[i];
     return CL_OK;
