@@ -38,6 +38,12 @@ def test_tiled_scoring_against_fp64(dtype, V, d, n):
         assert got["argmax"][0] == 0 and abs(got["p_max"][0] - 1 / V) <= 1e-6
 
 
+@pytest.mark.parametrize("dtype,V,d,n", [("bf16", 130, 40, 1), ("bf16", 5003, 1024, 8), ("fp32", 301, 72, 9), ("bf16", 4097, 264, 16), ("fp32", 1024, 256, 16)])
+def test_few_rows_against_fp64(dtype, V, d, n):
+    """Up to 16 rows take passes of eight rows of another kernel, with chains of at most d / 32 fp32 additions: the same bounds."""
+    test_tiled_scoring_against_fp64(dtype, V, d, n)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("n", [16, 17, 100])
 def test_logits_beyond_the_clamp_or_infinite(dtype, n):
