@@ -244,8 +244,10 @@ cudaError_t cl_launch_gemv(int wdtype, int T, int epi, const ClGemvArgs &a, int 
 // the process exits.  Layout (bytes): [0, 256) the LM-head kernel's ticket counter; then the normalised rows
 // xn [SC_CHUNK, CL_STATIC_MAX_D] fp32; the softmax partials of either path; the rows' normalisation factors and the three
 // per-row results (confidence, top-1 probability, greedy token) [CL_STATIC_MAX_ROWS] each.
-// Up to SC_GEMV_ROWS rows take passes of the streaming GEMV, more take the tiled kernel of kernels_headrows.cu, whose cost
-// hardly depends on the rows of a tile up to 64 (bf16 heads, whole call, 9 / 16 / 21 / 48 / 100 rows: 32000 x 4096 GEMV
+// Up to SC_GEMV_ROWS rows take one or two passes of the streaming GEMV, more take the tiled kernel of kernels_headrows.cu, whose
+// cost hardly depends on the rows of a tile up to 64.  By the figures the crossing lies between 9 and 16 rows and differs from head
+// to head: at 9 the GEMV is faster for two of three, at 16 the tiled kernel for all (by 5 to 24 %).  The line is at two whole passes,
+// below which no call is slower than it was with passes alone; a line per head between 9 and 16 has not been measured (bf16 heads, whole call, 9 / 16 / 21 / 48 / 100 rows: 32000 x 4096 GEMV
 // 417 / 633 / 761 / 1746 / 3550 us, tiled 479 / 479 / 502 / 564 / 1059; 128256 x 4096 GEMV 1089 / 1752 / 2152 / 5119 / 10622,
 // tiled 1657 / 1662 / 1742 / 2021 / 3773; 5003 x 768 GEMV 114 / 150 / 178 / 331 / 625, tiled 118 / 118 / 121 / 125 / 180).
 namespace {

@@ -395,8 +395,8 @@ __global__ void __launch_bounds__(256) k_wide_rope_append(ClWideParts p, int hd,
 // 6.9e-7 / 1.4e-6 with those, 4.9e-7 / 8.1e-7 here, fp16): the accumulator of the instruction cuts off where an fp32 addition rounds, which
 // over one chain for all keys of a row came to 2.2e-6 / 9.9e-6, so a chain is one tile of 64 keys, the parts have accumulators of their own
 // and everything else is added in fp32.
-// Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile).  At 512 rows of 32 heads it takes 48 us of a
-// layer's 575; the register-tiled fp32 products on the CUDA cores that it replaces took 127.  Blocks of late rows see the most keys and
+// Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile).  At 512 rows of 32 heads it takes 43 us of the
+// 410 that the kernels of a layer take; the register-tiled fp32 products on the CUDA cores that it replaces took 122.  Blocks of late rows see the most keys and
 // are scheduled first.
 constexpr int AQ = 64, AK = 64;   // rows per CTA, keys per tile
 constexpr int ATT_STEP = 4096;    // fp16: ratio of a probability part's scale to the part before (a rest is below 2^-11 of its value: no overflow)
@@ -676,8 +676,8 @@ __global__ void __launch_bounds__(256) k_wide_silu(ClWideParts p, int F, __nv_bf
 
 }  // namespace
 
-// How a GEMM of M operand rows is cut: one CTA pair per two SMs, fewer when there is so little work that a pair would
-// have less than two K blocks, or when the product parts would not fit the workspace.
+// How a GEMM of M operand rows is cut: one CTA pair per two SMs, fewer when there is so little work that a pair's share would
+// cost less than four (two K blocks of a full tile, four of a half tile), or when the product parts would not fit the workspace.
 ClWideParts cl_wide_plan(int M, int rows, int KB, int n_sm, float *P, size_t ws_floats) {
     ClWideParts p;
     p.P = P; p.M = M; p.rows = rows; p.KB = KB;
