@@ -241,28 +241,28 @@ cudaError_t cl_launch_gemv(int wdtype, int T, int epi, const ClGemvArgs &a, int 
 
 // ---- confidence scoring without any allocation ------------------------------------------------------
 // Scratch of cl_layer_confidences_static(): one file-scope array that every GPU loading this library holds until
-// the process exits.  Layout (bytes): [0, 256) the LM-head kernel's ticket counter; then the normalised rows
-// xn [SC_CHUNK, CL_STATIC_MAX_D] fp32; the softmax partials of either path; the rows' normalisation factors and the three
-// per-row results (confidence, top-1 probability, greedy token) [CL_STATIC_MAX_ROWS] each.
-// Up to SC_GEMV_ROWS rows take one or two passes of the streaming GEMV, more take the tiled kernel of kernels_headrows.cu, whose
-// cost hardly depends on the rows of a tile up to 64.  By the figures the crossing lies between 9 and 16 rows and differs from head
-// to head: at 9 the GEMV is faster for two of three, at 16 the tiled kernel for all (by 5 to 24 %).  The line is at two whole passes,
-// below which no call is slower than it was with passes alone; a line per head between 9 and 16 has not been measured (bf16 heads, whole call, 9 / 16 / 21 / 48 / 100 rows: 32000 x 4096 GEMV
-// 417 / 633 / 761 / 1746 / 3550 us, tiled 479 / 479 / 502 / 564 / 1059; 128256 x 4096 GEMV 1089 / 1752 / 2152 / 5119 / 10622,
-// tiled 1657 / 1662 / 1742 / 2021 / 3773; 5003 x 768 GEMV 114 / 150 / 178 / 331 / 625, tiled 118 / 118 / 121 / 125 / 180).
+// the process exits.  Layout (bytes): [0, 256) ticket counters; then the normalised rows
+// xn [SC_CHUNK, CL_STATIC_MAX_D] fp32; the softmax partials of either path; the rows' normalisation factors
+// [CL_STATIC_MAX_ROWS] fp64; two flags and the three per-row results (confidence, top-1 probability, greedy token) [n_rows] each,
+// side by side so that one copy fetches them.
+// Few rows take passes of the streaming GEMV, eight rows each, more take the kernels of kernels_headrows.cu.
+// fp32 heads: the line is at two whole passes (5003 x 768, 16 rows: GEMV 116 us, tiled kernel 101 with 17).
+// bf16 heads: the tensor-core kernel costs the same from 1 to 128 rows and waits for K block after K block, so that it needs a vocabulary
+// that is long against the width.  Whole call, GEMV with 4 / 6 / 8 / 9 / 16 rows against the tensor-core kernel, us:
+//   32000 x 4096  149 / 181 / 304 / 362 / 568  157     128256 x 4096  388 / 497 / 843 / 1029 / 1655  448     32000 x 768  78 / 91 / 127 / 143 / 218  82
+//   32000 x 8192  224 / 275 / 583 / 687 / 1122  236    5003 x 768  63 / 65 / 78 / 92 / 128  62
+//   5003 x 4096  82 / 96 / 121 / 139 / 194  104 .. 111     1000 x 8192  74 / 75 / 100 / 117 / 158  150
+// Hence from 6 rows where V >= 3 d, from 9 where V >= d, else from 17.
 namespace {
 
 constexpr int SC_MAX_GRID = 1024;
 constexpr int SC_CHUNK = 8;   // rows per LM-head pass of the GEMV
-constexpr int SC_GEMV_ROWS = 16;   // most rows that take those passes
 constexpr size_t SC_OFF_XN = 256;
 constexpr size_t SC_OFF_PART = SC_OFF_XN + (size_t)SC_CHUNK * CL_STATIC_MAX_D * sizeof(float);
 constexpr size_t SC_PARTIALS = SC_MAX_GRID * SC_CHUNK > CL_HEAD_ROWS_PARTIALS ? SC_MAX_GRID * SC_CHUNK : CL_HEAD_ROWS_PARTIALS;
 constexpr size_t SC_OFF_SCALE = SC_OFF_PART + SC_PARTIALS * sizeof(ClHeadPartial);
-constexpr size_t SC_OFF_CONF = SC_OFF_SCALE + (size_t)CL_STATIC_MAX_ROWS * sizeof(float);
-constexpr size_t SC_OFF_PMAX = SC_OFF_CONF + (size_t)CL_STATIC_MAX_ROWS * sizeof(float);
-constexpr size_t SC_OFF_ARG = SC_OFF_PMAX + (size_t)CL_STATIC_MAX_ROWS * sizeof(float);
-constexpr size_t SC_BYTES = SC_OFF_ARG + (size_t)CL_STATIC_MAX_ROWS * sizeof(int);
+constexpr size_t SC_OFF_RES = SC_OFF_SCALE + (size_t)CL_STATIC_MAX_ROWS * sizeof(double);
+constexpr size_t SC_BYTES = SC_OFF_RES + (2 + 3 * (size_t)CL_STATIC_MAX_ROWS) * 4;
 
 static __device__ __align__(256) unsigned char g_static_scratch[SC_BYTES];
 
@@ -340,23 +340,44 @@ extern "C" int cl_layer_confidences_static(const void *lm_head, const float *fin
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     float *xn = (float *)(sc + SC_OFF_XN);
-    float *d_conf = (float *)(sc + SC_OFF_CONF), *d_pmax = (float *)(sc + SC_OFF_PMAX);
-    int *d_arg = (int *)(sc + SC_OFF_ARG);
-    cudaError_t e = cudaMemsetAsync(sc, 0, SC_OFF_XN, s);   // the ticket must start at zero whatever the last call left
-    ClGemvArgs a;
-    memset(&a, 0, sizeof(a));
-    a.W = lm_head; a.rows = vocab; a.cols = d_model; a.xin = xn;
-    a.partials = (ClHeadPartial *)(sc + SC_OFF_PART);
-    a.ticket = (unsigned *)sc;
-    a.inv_log_v = (float)(1.0 / log((double)vocab));
-    int grid = ((vocab + 1) / 2 + 7) / 8;
-    if (grid > n_sm * 4) grid = n_sm * 4;
-    if (grid > SC_MAX_GRID) grid = SC_MAX_GRID;
-    if (e == cudaSuccess && n_rows > SC_GEMV_ROWS) {
-        e = cl_launch_head_rows(weight_dtype, lm_head, hidden, final_norm, n_rows, vocab, d_model, rms_eps, n_sm,
-                                (float *)(sc + SC_OFF_SCALE), a.partials, d_conf, d_pmax, d_arg, s);
+    unsigned *flags = (unsigned *)(sc + SC_OFF_RES);
+    float *d_conf = (float *)(flags + 2), *d_pmax = d_conf + n_rows;
+    int *d_arg = (int *)(d_pmax + n_rows);
+    const size_t es = weight_dtype == 1 ? 2 : 4;
+    auto many_rows = [&]() -> cudaError_t {
+        return cl_launch_head_rows(weight_dtype, lm_head, hidden, final_norm, n_rows, vocab, d_model, rms_eps, n_sm, (double *)(sc + SC_OFF_SCALE),
+                                   (ClHeadPartial *)(sc + SC_OFF_PART), d_conf, d_pmax, d_arg, s);
+    };
+    unsigned res[2 + 3 * CL_STATIC_MAX_ROWS];
+    auto fetch = [&]() -> cudaError_t {
+        const cudaError_t e = cudaMemcpyAsync(res, flags, (2 + 3 * (size_t)n_rows) * 4, cudaMemcpyDeviceToHost, s);
+        return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+    };
+    // the tickets and flags must start at zero whatever the last call left
+    cudaError_t e = cudaMemsetAsync(sc, 0, SC_OFF_XN, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 8, s);
+    const bool tc = weight_dtype == 1;
+    const int gemv_rows = !tc || vocab < d_model ? 16 : vocab < 3LL * d_model ? 8 : 5;   // most rows that take those passes
+    if (n_rows > gemv_rows) {
+        if (e == cudaSuccess)
+            e = tc ? cl_launch_head_tc(lm_head, hidden, final_norm, n_rows, vocab, d_model, rms_eps, n_sm, (double *)(sc + SC_OFF_SCALE),
+                                       (ClHeadPartial *)(sc + SC_OFF_PART), (unsigned *)sc, flags, d_conf, d_pmax, d_arg, s)
+                   : many_rows();
+        if (e == cudaSuccess) e = fetch();
+        if (e == cudaSuccess && tc && res[0] && !res[1]) {
+            e = many_rows();
+            if (e == cudaSuccess) e = fetch();
+        }
     } else {
-        const size_t es = weight_dtype == 1 ? 2 : 4;
+        ClGemvArgs a;
+        memset(&a, 0, sizeof(a));
+        a.W = lm_head; a.rows = vocab; a.cols = d_model; a.xin = xn;
+        a.partials = (ClHeadPartial *)(sc + SC_OFF_PART);
+        a.ticket = (unsigned *)sc;
+        a.inv_log_v = (float)(1.0 / log((double)vocab));
+        int grid = ((vocab + 1) / 2 + 7) / 8;
+        if (grid > n_sm * 4) grid = n_sm * 4;
+        if (grid > SC_MAX_GRID) grid = SC_MAX_GRID;
         for (int r0 = 0; r0 < n_rows && e == cudaSuccess; r0 += SC_CHUNK) {
             const int T = n_rows - r0 < SC_CHUNK ? n_rows - r0 : SC_CHUNK;
             e = cl_launch_rmsnorm_rows(weight_dtype, (const char *)hidden + (size_t)r0 * d_model * es, final_norm, T, d_model,
@@ -365,14 +386,18 @@ extern "C" int cl_layer_confidences_static(const void *lm_head, const float *fin
             a.out_tok = d_arg + r0; a.out_pmax = d_pmax + r0; a.out_conf = d_conf + r0;
             e = cl_launch_gemv(weight_dtype, T, CL_EPI_HEAD, a, grid, s);
         }
+        if (e == cudaSuccess) e = fetch();
     }
-    if (e == cudaSuccess && conf) e = cudaMemcpyAsync(conf, d_conf, (size_t)n_rows * 4, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess && p_max) e = cudaMemcpyAsync(p_max, d_pmax, (size_t)n_rows * 4, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess && argmax) e = cudaMemcpyAsync(argmax, d_arg, (size_t)n_rows * 4, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         cl_set_global_error("cl_layer_confidences_static: %s", cudaGetErrorString(e));
         return CL_ECUDA;
     }
+    if (res[1]) {
+        cl_set_global_error("cl_layer_confidences_static: a bounded device-side wait expired; results of this call are invalid");
+        return CL_ETIMEOUT;
+    }
+    if (conf) memcpy(conf, res + 2, (size_t)n_rows * 4);
+    if (p_max) memcpy(p_max, res + 2 + n_rows, (size_t)n_rows * 4);
+    if (argmax) memcpy(argmax, res + 2 + 2 * (size_t)n_rows, (size_t)n_rows * 4);
     return CL_OK;
 }

@@ -1,23 +1,20 @@
-// LM head over many fp32-exact rows on the CUDA cores: the confidence statistics of up to 4096 hidden rows without a copy of
-// the normalised rows and without logits in memory (the allocation-free scoring call).
+// LM head over many fp32-exact rows: the confidence statistics of up to 4096 hidden rows without a copy of the normalised rows and
+// without logits in memory (the allocation-free scoring call).  Two kernels: k_head_rows on the CUDA cores for fp32 heads, and
+// k_head_tc on the tensor cores for bf16 heads (see there).
 //
-//   logits[r, v] = sum_k (x[r, k] * scale[r] * gain[k]) * W[v, k]     x, W: bf16 or fp32; all arithmetic fp32
+//   logits[r, v] = sum_k (x[r, k] * scale[r] * gain[k]) * W[v, k]     x, W: bf16 or fp32, activations and sums fp32 or better
 //
-// Bound: fp32 multiply-adds (the activations stay fp32, so the 16-bit tensor pipe does not apply): 26 GFLOP for 100 rows of
-// the 32000 x 4096 head are 0.35 ms at 74 TFLOP/s.  The eight-row GEMV passes it replaces re-read the head every eight rows and
-// re-read the rows from L1 for every pair of weights, 266 us a pass (100 rows: 3.45 ms for the call, this kernel 1.04).  Shared-
-// memory reads bound it next: 16 wavefronts per 28 packed multiply-adds of a warp at TM = 7.  A CTA takes a tile of 16 * TM rows
-// by 128 weights, 32 elements of K at a time, a thread TM x 8 products as packed pairs (fma.rn.f32x2: two products an
-// instruction, each rounded as fmaf rounds); two CTAs per SM cover each other's barriers.
+// k_head_rows is bound by shared-memory reads (16 wavefronts per 28 packed multiply-adds of a warp at TM = 7; 100 rows of a bf16
+// 32000 x 4096 head 0.99 ms, multiply-adds 0.35).  A CTA takes a tile of 16 * TM rows by 128 weights, 32 elements of K at a time, a
+// thread TM x 8 products as packed pairs (fma.rn.f32x2: two products an instruction, each rounded as fmaf rounds); two CTAs per SM
+// cover each other's barriers.
 // Sums are kept in chains of 64 elements of K, added up in shared memory; what such an addition rounds off opens the next chain.
-// A row's scale and its confidence are worked out in 64 bits.  Error of the confidences against 64 bits, mean over 17 to 400 rows
-// and five inputs, widths 768 / 4096 / 5120: GEMV 3.3e-7 / 3.8e-7 / 4.1e-7, here 2.7e-7 / 2.3e-7 / 2.5e-7 (with scale and confidence
-// in 32 bits 3.5e-7 / 3.3e-7 / 3.3e-7).
+// A row's scale and its confidence are worked out in 64 bits.
 // Rows are asked for in L2 eight lines ahead: a step of 32 elements is shorter than a trip to HBM.
 // The rows of a tile are a matter of balance: R rows are ceil(R / 128) tiles of equal size, rounded up to 16 rows.
 #include <math.h>
 
-#include "cl_internal.h"
+#include "tc_common.cuh"
 
 namespace {
 
@@ -25,7 +22,8 @@ constexpr int HN = 128, HK = 32, HT = 256, CHAIN = 64;
 
 struct HeadRowsArgs {
     const void *W, *x;
-    const float *gain, *scale;       // [d], [R]
+    const float *gain;               // [d]
+    const double *scale;             // [R]
     int R, V, d, MT, rows, NR, NT;   // rows, vocabulary, width, row tiles and their rows, vocabulary ranges, vocabulary tiles
     ClHeadPartial *part;             // [R, NR]
 };
@@ -98,7 +96,7 @@ __global__ void __launch_bounds__(HT, 2) k_head_rows(HeadRowsArgs a) {
     const int so = (tid & 3) * 8, sr = tid >> 2;
     float sc[2];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) sc[j] = sr + 64 * j < nrows ? a.scale[row0 + sr + 64 * j] : 0.f;
+    for (int j = 0; j < 2; ++j) sc[j] = sr + 64 * j < nrows ? (float)a.scale[row0 + sr + 64 * j] : 0.f;
 
     for (int nt = nt0; nt < nt1; ++nt) {
         const int n0 = nt * HN;
@@ -217,7 +215,8 @@ __global__ void __launch_bounds__(HT, 2) k_head_rows(HeadRowsArgs a) {
 // scale[r] = 1 / sqrt(mean x^2 + eps), one CTA per row.  In 64 bits up to the result: its error moves all logits of a row
 // together, and fp32 sums, quotients and roots made it the largest part of a narrow row's error (see the head of this file).
 template <typename T>
-__global__ void __launch_bounds__(256) k_row_scale(const T *x, int d, float eps, float *scale) {
+__global__ void __launch_bounds__(256) k_row_scale(const T *x, int d, float eps, double *scale) {
+    pdl_launch_dependents();
     __shared__ double red[8];
     double ss = 0.0;
     for (int i = threadIdx.x * 8; i < d; i += 2048) {
@@ -235,7 +234,7 @@ __global__ void __launch_bounds__(256) k_row_scale(const T *x, int d, float eps,
     if (threadIdx.x == 0) {
         double tot = 0.0;
         for (int w = 0; w < 8; ++w) tot += red[w];
-        scale[blockIdx.x] = (float)(1.0 / sqrt(tot / d + (double)eps));
+        scale[blockIdx.x] = 1.0 / sqrt(tot / d + (double)eps);
     }
 }
 
@@ -256,6 +255,447 @@ __global__ void __launch_bounds__(128) k_head_rows_merge(const ClHeadPartial *pa
         pmax[r] = 1.f / f.z;
         arg[r] = f.idx;
     }
+}
+
+// ---- bf16 heads: the same products on the tensor cores --------------------------------------------------------------------
+//
+// A weight is one bf16 number, an activation x * gain three of them: hi + mid + lo hold 26 bits of the product, more than fp32.
+// What is left to keep exact are the sums, and the accumulator in tensor memory cuts off where an fp32 addition rounds.  So:
+//   - a chain is one K block: 4 multiply-adds (K 16) of lo, 4 of mid, 4 of hi, in this order, so that only the last four cut
+//     off at the size of the sum; the finished chain is added to the row's fp32 total in registers, and what that addition
+//     rounds off is put back into the accumulator, where the next but one chain starts from it (two accumulators alternate);
+//   - what remains is a loss with a known mean, proportional to the sum: with a significand spread evenly over its logarithm a cut
+//     takes 0.72 * 2^-25 of the value or a little more, and the four cuts of a chain whose products add up evenly meet 1/4, 2/4,
+//     3/4 and all of it.  Measured as the common shrinking of the logits it is HT_SHRINK, within 0.1e-7 at widths 768, 4096 and 5120;
+//     the row's scale makes up for it.  (Chains of 2 and 4 K blocks lose 2.5e-7 and 6.2e-7 and would be 10 us faster.)
+// The scale is applied last, as a pair of floats.  Error of the confidences / of the top-1 probabilities against 64 bits, mean of three
+// inputs at widths 768, 4096 and 5120: 0.72e-7 .. 0.86e-7 / 1.1e-7 .. 1.4e-7 (k_head_rows 1.05e-7 .. 1.5e-7 / 1.6e-7 .. 1.9e-7).
+//
+// Bound: shared memory, then the hand-overs between the roles.  A K block of 128 rows x 224 weights is 12 multiply-adds that read
+// 11 KB each, 108 KB are written and read beside them: 1900 cycles at 128 bytes a cycle against 1344 of multiply-add; measured 2100,
+// and 2700 with the waits of the multiplying thread.  100 rows of the 32000 x 4096 head: 143 us (k_head_rows 987), the call 175
+// (1043); 32000 x 768 50 us, 128256 x 4096 the call 470 (3930).
+// 224 weights a tile: 32000 of them are one tile per SM (143), and the totals of a tile are 112 registers a thread.
+// 16 warps: 0 copies weights, 2 rows (TMA), 1 multiplies, 4-7 split the activations, 8-15 add up chains and keep the softmax
+// statistics.  The head is asked for in L2 eight K blocks ahead.
+constexpr int HTC_THREADS = 512;
+constexpr int HTC_A = 3 * 128 * 128, HTC_X = 128 * 128,   // bytes of a K block's rows, split in three and as they are
+              HTC_AST = 2, HTC_BST = 3, HTC_XST = 2, HTC_AHEAD = 8;   // stages of the rings, K blocks asked for in L2
+constexpr float HT_SHRINK = 0.67e-7f;
+
+struct HeadTcArgs {
+    const __nv_bfloat16 *x;              // [R, d]
+    const float *gain;
+    const double *scale;                 // [R]
+    int R, V, d, KB, MT, rows, NR, NT;   // rows, vocabulary, width, K blocks, row tiles and their rows, vocabulary ranges, vocabulary tiles
+    double inv_log_v;
+    ClHeadPartial *part;                 // [R, NR]
+    unsigned *tickets, *flags;           // [MT], zero at launch; [0] a sum that is not finite was met, [1] a wait ran out
+    float *conf, *pmax;
+    int *arg;
+};
+
+struct HeadTcSmem {
+    unsigned long long afull[HTC_AST], aempty[HTC_AST], bfull[HTC_BST], bempty[HTC_BST], xfull[HTC_XST], xempty[HTC_XST], tfull[2], tempty[2];
+    ClHeadPartial half[128];
+    unsigned tmem_base, last;
+    int abort;
+};
+
+__device__ __forceinline__ void tmem_st16(unsigned taddr, const float (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" ::"f"(v[0]), "f"(v[1]),
+        "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]),
+        "f"(v[13]), "f"(v[14]), "f"(v[15]), "r"(taddr)
+        : "memory");
+}
+// A load whose values may be used after tmem_ld_wait(), which takes them as operands so that nothing moves ahead of it.
+__device__ __forceinline__ void tmem_ld16_async(unsigned taddr, float (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]), "=f"(v[9]), "=f"(v[10]),
+          "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait(float (&v)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]),
+                   "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
+                 :
+                 : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int c0, int c1) {
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(c0), "r"(c1) : "memory");
+}
+__device__ __forceinline__ unsigned cvt_bf16x2(float a, float b) {   // a in the low half
+    unsigned r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    return r;
+}
+__device__ __forceinline__ void bf16x2_get(unsigned u, float &a, float &b) {
+    a = __uint_as_float(u << 16);
+    b = __uint_as_float(u & 0xffff0000u);
+}
+
+template <int N>
+__global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW, HeadTcArgs a) {
+    constexpr int B_BYTES = N * 128, NH = N / 2;
+    extern __shared__ unsigned char smem_dyn[];   // rings of swizzled tiles: 1 KB aligned
+    unsigned char *ringA = (unsigned char *)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023), *ringX = ringA + HTC_AST * HTC_A,
+                  *ringB = ringX + HTC_XST * HTC_X;
+    HeadTcSmem *sm = (HeadTcSmem *)(ringB + HTC_BST * B_BYTES);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int mt = blockIdx.x % a.MT, rg = blockIdx.x / a.MT, KB = a.KB;
+    const int row0 = mt * a.rows, nrows = min(a.rows, a.R - row0);
+    const int nt0 = (int)((long long)a.NT * rg / a.NR), nt1 = (int)((long long)a.NT * (rg + 1) / a.NR), ntiles = nt1 - nt0;
+    int *err = (int *)(a.flags + 1);
+
+    if (tid == 0) {
+        for (int i = 0; i < HTC_AST; ++i) {
+            bar_init(&sm->afull[i], 4);
+            bar_init(&sm->aempty[i], 1);
+        }
+        for (int i = 0; i < HTC_BST; ++i) {
+            bar_init(&sm->bfull[i], 1);
+            bar_init(&sm->bempty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            bar_init(&sm->tfull[i], 1);
+            bar_init(&sm->tempty[i], 8);
+        }
+        for (int i = 0; i < HTC_XST; ++i) {
+            bar_init(&sm->xfull[i], 1);
+            bar_init(&sm->xempty[i], 4);
+        }
+        sm->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s_u32(&sm->tmem_base)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const unsigned tmem = *(volatile unsigned *)&sm->tmem_base;
+    pdl_wait();   // the scales
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        // ---------------- copies: warp 0 weights, warp 2 rows ----------------
+        auto copies = [&](unsigned char *ring, unsigned bytes, int stages, unsigned long long *full, unsigned long long *empty, bool weights) {
+            unsigned st = 0, par = 0, n = 0;
+            bool ok = true;
+            for (int t = 0; t < ntiles && ok; ++t)
+                for (int kb = 0; kb < KB; ++kb, ++n) {
+                    if (weights) {   // asked for in L2 ahead: a few K blocks in shared memory do not cover the trip to HBM
+                        for (int k = kb ? kb + HTC_AHEAD : 0; k < min(kb + HTC_AHEAD + 1, KB); ++k) tma_prefetch_2d(&mapW, k * 64, (nt0 + t) * N);
+                    }
+                    ok = bar_wait(empty + st, par ^ 1u, &sm->abort, err);
+                    if (!ok) break;
+                    bar_expect(full + st, bytes);
+                    if (weights) tma_load_2d(ring + st * bytes, &mapW, kb * 64, (nt0 + t) * N, full + st);
+                    else tma_load_2d(ring + st * bytes, &mapX, kb * 64, row0, full + st);
+                    if (++st == (unsigned)stages) { st = 0; par ^= 1u; }
+                }
+            if (!ok) {   // let the copies in flight land before the CTA may exit (bounded): the last `stages` that were issued
+                const unsigned long long t0 = gtime_ns();
+                for (unsigned i = n > (unsigned)stages ? n - stages : 0; i < n; ++i)
+                    while (!bar_try(full + i % stages, (i / stages) & 1u) && gtime_ns() - t0 < WAIT_NS) {}
+            }
+        };
+        if (warp == 0) {
+            if (lane == 0) copies(ringB, B_BYTES, HTC_BST, sm->bfull, sm->bempty, true);
+        } else if (warp == 2) {
+            if (lane == 0) copies(ringX, HTC_X, HTC_XST, sm->xfull, sm->xempty, false);
+        } else if (warp == 1 && lane == 0) {
+            // ---------------- multiply-adds ----------------
+            const unsigned idesc = umma_idesc(128, N);
+            unsigned sa = 0, pa = 0, sb = 0, pb = 0, g = 0;
+            bool ok = true;
+            for (int t = 0; t < ntiles && ok; ++t)
+                for (int kb = 0; kb < KB; ++kb, ++g) {
+                    const unsigned b = g & 1u;
+                    if (!bar_wait(&sm->tempty[b], (g >> 1) & 1u, &sm->abort, err) || !bar_wait(&sm->bfull[sb], pb, &sm->abort, err) ||
+                        !bar_wait(&sm->afull[sa], pa, &sm->abort, err)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const unsigned a_addr = s_u32(ringA + sa * HTC_A), b_addr = s_u32(ringB + sb * B_BYTES), acc = tmem + b * 256u;
+#pragma unroll
+                    for (int p = 2; p >= 0; --p)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            umma_bf16(acc, umma_desc(a_addr + (unsigned)(p * 16384 + k * 32)), umma_desc(b_addr + (unsigned)(k * 32)), idesc, 1u);
+                    umma_commit(&sm->aempty[sa]);
+                    umma_commit(&sm->bempty[sb]);
+                    umma_commit(&sm->tfull[b]);
+                    if (++sa == HTC_AST) { sa = 0; pa ^= 1u; }
+                    if (++sb == HTC_BST) { sb = 0; pb ^= 1u; }
+                }
+        }
+    } else if (warp < 8) {
+        // ---------------- activations: 8 lanes a row, 16 bytes a lane, 32 rows a warp ----------------
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 112;");
+        const int r0 = (warp - 4) * 32 + (lane >> 3), piece = lane & 7;
+        const bool rows_here = (warp - 4) * 32 < nrows;   // (a row of the product depends on its own row of activations only)
+        float4 g0, g1, n0, n1;
+        auto gains = [&](int kb) {
+            const int k = kb * 64 + piece * 8;
+            n0 = n1 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k < a.d) {
+                n0 = *(const float4 *)(a.gain + k);
+                n1 = *(const float4 *)(a.gain + k + 4);
+            }
+        };
+        gains(0);
+        unsigned sa = 0, pa = 0, sx = 0, px = 0;
+        bool ok = true;
+        for (int t = 0; t < ntiles && ok; ++t)
+            for (int kb = 0; kb < KB; ++kb) {
+                g0 = n0;
+                g1 = n1;
+                gains(kb + 1 < KB ? kb + 1 : 0);
+                ok = __all_sync(0xffffffffu, bar_wait(&sm->xfull[sx], px, &sm->abort, err) && bar_wait(&sm->aempty[sa], pa ^ 1u, &sm->abort, err));
+                if (!ok) break;
+                if (rows_here) {
+                    const unsigned src = s_u32(ringX + sx * HTC_X), dst = s_u32(ringA + sa * HTC_A);
+                    const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+#pragma unroll
+                    for (int jb = 0; jb < 8; jb += 4) {
+                        unsigned w[4][4], off[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int r = r0 + 4 * (jb + j);
+                            off[j] = (unsigned)(r * 128 + ((piece ^ (r & 7)) << 4));
+                            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[j][0]), "=r"(w[j][1]), "=r"(w[j][2]), "=r"(w[j][3]) : "r"(src + off[j]) : "memory");
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            unsigned h[4], m[4], l[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                float x0, x1, h0, h1, m0, m1;
+                                bf16x2_get(w[j][e], x0, x1);
+                                h[e] = cvt_bf16x2(x0 * gg[2 * e], x1 * gg[2 * e + 1]);
+                                bf16x2_get(h[e], h0, h1);
+                                const float q0 = fmaf(x0, gg[2 * e], -h0), q1 = fmaf(x1, gg[2 * e + 1], -h1);   // exact: 32 bits less the leading eight
+                                m[e] = cvt_bf16x2(q0, q1);
+                                bf16x2_get(m[e], m0, m1);
+                                l[e] = cvt_bf16x2(q0 - m0, q1 - m1);
+                            }
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + off[j]), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]));
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + off[j] + 16384u), "r"(m[0]), "r"(m[1]), "r"(m[2]), "r"(m[3]));
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + off[j] + 32768u), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]));
+                        }
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    bar_arrive(&sm->xempty[sx]);
+                    bar_arrive(&sm->afull[sa]);
+                }
+                if (++sx == HTC_XST) { sx = 0; px ^= 1u; }
+                if (++sa == HTC_AST) { sa = 0; pa ^= 1u; }
+            }
+    } else {
+        // ---------------- chains: a thread has half a row of the tile ----------------
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+        const int q = warp & 3, hf = (warp - 8) >> 2, row = q * 32 + lane;
+        const unsigned tl = tmem + ((unsigned)(q * 32) << 16) + (unsigned)(hf * NH);
+        float s_hi = 0.f, s_lo = 0.f;
+        bool ok = true, odd = false;
+        if (row < nrows) {
+            const double f = a.scale[row0 + row] * (1.0 + (double)HT_SHRINK);
+            odd = !(f > 0x1p-60 && f < 0x1p60);   // (parts of very large or very small rows could leave the range of a float)
+            s_hi = (float)f;
+            s_lo = (float)(f - (double)s_hi);
+        }
+        const float zero[16] = {};
+#pragma unroll 1
+        for (int c = 0; c < NH; c += 16) {
+            tmem_st16(tl + c, zero);
+            tmem_st16(tl + 256u + c, zero);
+        }
+        auto release = [&](unsigned b) {
+            if (lane == 0) bar_arrive(&sm->tempty[b]);
+        };
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        release(0);
+        release(1);
+        ClHeadPartial run{0.f, 0.f, 0.f, 0x7fffffff};
+        unsigned g = 0;
+        for (int t = 0; t < ntiles && ok; ++t) {
+            float tot[NH];
+#pragma unroll
+            for (int i = 0; i < NH; ++i) tot[i] = 0.f;
+            for (int ch = 0; ch < KB; ++ch, ++g) {
+                const unsigned b = g & 1u, ta = tl + b * 256u, to = tl + (b ^ 1u) * 256u;
+                ok = __all_sync(0xffffffffu, bar_wait(&sm->tfull[b], (g >> 1) & 1u, &sm->abort, err));
+                if (!ok) break;
+                __syncwarp();
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (ch + 1 < KB) {
+                    float u[2][16];
+                    tmem_ld16_async(ta, u[0]);
+#pragma unroll
+                    for (int c = 0; c < NH; c += 16) {
+                        float(&v)[16] = u[(c >> 4) & 1];
+                        tmem_ld_wait(v);
+                        if (c + 16 < NH) tmem_ld16_async(ta + c + 16, u[((c >> 4) + 1) & 1]);
+#pragma unroll
+                        for (int i = 0; i < 16; i += 2) {   // sum, and what it rounded off (in full where the total is the larger one)
+                            const unsigned long long tt = pack2(tot[c + i], tot[c + i + 1]), uu = pack2(v[i], v[i + 1]), s = add2(tt, uu);
+                            unpack2(sub2(uu, sub2(s, tt)), v[i], v[i + 1]);
+                            unpack2(s, tot[c + i], tot[c + i + 1]);
+                        }
+                        tmem_st16(ta + c, v);
+                    }
+                } else {
+                    // the row's last chain: the logits, with what both accumulators still owe; both start the next tile from zero
+#pragma unroll
+                    for (int c = 0; c < NH; c += 16) {
+                        float u[16], o[16];
+                        tmem_ld16(ta + c, u);
+                        if (KB > 1) tmem_ld16(to + c, o);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const float s = tot[c + i] + u[i], r = (u[i] - (s - tot[c + i])) + (KB > 1 ? o[i] : 0.f);
+                            tot[c + i] = fmaf(s, s_hi, fmaf(s, s_lo, r * s_hi));
+                        }
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) u[i] = tot[c + i];
+                        tmem_st16(ta + c, u);
+                    }
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                if (ch + 1 == KB) {
+                    // softmax statistics of this half row, out of tensor memory again (in registers the 112 logits unroll into
+                    // code that takes longer to fetch than to run); then both accumulators start the next tile from zero
+                    const int c0 = (nt0 + t) * N + hf * NH, nvalid = min(NH, a.V - c0);
+                    ClHeadPartial p{-INFINITY, 0.f, 0.f, 0x7fffffff};
+#pragma unroll 1
+                    for (int c = 0; c < nvalid; c += 16) {
+                        float l[16];
+                        tmem_ld16(ta + c, l);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                        {   // (selections, not branches: a branch per logit costs ten times as much)
+                            const bool in = c + i < nvalid;
+                            odd |= in && !(fabsf(l[i]) < INFINITY);
+                            const float v = in ? fminf(fmaxf(l[i], -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP) : -INFINITY;   // clamp of Section 3.1
+                            p.idx = v > p.m ? c0 + c + i : p.idx;
+                            p.m = fmaxf(p.m, v);
+                        }
+                    }
+#pragma unroll 1
+                    for (int c = 0; c < nvalid; c += 16) {
+                        float l[16], z = 0.f, s = 0.f;
+                        tmem_ld16(ta + c, l);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                        {
+                            const float d = fminf(fmaxf(l[i], -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP) - p.m, e = c + i < nvalid ? expf(d) : 0.f;
+                            z += e;
+                            s = fmaf(d, e, s);
+                        }
+                        p.z += z;
+                        p.s += s;
+                    }
+                    if (nvalid > 0) run = cl_hp_merge(run, p);
+#pragma unroll 1
+                    for (int c = 0; c < NH; c += 16) {
+                        tmem_st16(ta + c, zero);
+                        if (KB > 1) tmem_st16(to + c, zero);
+                    }
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (ch + 1 == KB && KB > 1) release(b ^ 1u);   // (held back so that it could be read once more)
+                if (ch + 2 != KB) release(b);
+            }
+        }
+        if (odd && row < nrows) a.flags[0] = 1u;
+        if (hf) sm->half[row] = run;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (!hf && row < nrows) a.part[(size_t)(row0 + row) * a.NR + rg] = cl_hp_merge(run, sm->half[row]);
+        // the last CTA of a row tile merges its ranges, in a fixed order, eight lanes a row
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (tid == 256) sm->last = ticket_acq_rel(a.tickets + mt) == (unsigned)a.NR - 1u;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (sm->last) {
+            constexpr int PL = 20;   // ranges a lane: 8 * 20 cover the 148 SMs
+            for (int r0 = 0; r0 < nrows; r0 += 32) {
+                const int r = min(r0 + (warp - 8) * 4 + (lane >> 3), nrows - 1);
+                const float4 *pp = (const float4 *)(a.part + (size_t)(row0 + r) * a.NR);
+                float m = -INFINITY;
+                int idx = 0x7fffffff;
+                double z = 0.0, t = 0.0;
+                for (int g0 = lane & 7; g0 < a.NR; g0 += 8 * PL) {
+                    float4 f[PL];
+                    float mn = m;
+#pragma unroll
+                    for (int i = 0; i < PL; ++i) f[i] = g0 + 8 * i < a.NR ? __ldcg(pp + g0 + 8 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < PL; ++i)
+                        if (f[i].y > 0.f && f[i].x > mn) { mn = f[i].x; idx = __float_as_int(f[i].w); }
+                    if (z > 0.0) {
+                        const double e = expf(m - mn);
+                        t = e * (t + (double)(m - mn) * z);
+                        z *= e;
+                    }
+                    m = mn;
+#pragma unroll
+                    for (int i = 0; i < PL; ++i) {
+                        const float dm = f[i].y > 0.f ? f[i].x - m : 0.f, e = f[i].y > 0.f ? expf(dm) : 0.f;
+                        z += (double)(e * f[i].y);
+                        t += (double)(e * fmaf(dm, f[i].y, f[i].z));
+                    }
+                }
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) {
+                    const float om = __shfl_xor_sync(0xffffffffu, m, o), mm = fmaxf(m, om);
+                    const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
+                    const double oz = __shfl_xor_sync(0xffffffffu, z, o), ot = __shfl_xor_sync(0xffffffffu, t, o);
+                    const double e = z > 0.0 ? expf(m - mm) : 0.f, oe = oz > 0.0 ? expf(om - mm) : 0.f;
+                    t = (z > 0.0 ? e * (t + (double)(m - mm) * z) : 0.0) + (oz > 0.0 ? oe * (ot + (double)(om - mm) * oz) : 0.0);
+                    z = e * z + oe * oz;
+                    idx = om > m || (om == m && oi < idx) ? oi : idx;
+                    m = mm;
+                }
+                if ((lane & 7) == 0) {   // (a row may be written more than once, with the same values)
+                    a.conf[row0 + r] = (float)(1.0 - (log(z) - t / z) * a.inv_log_v);   // H = log Z - S / Z (Eq. 2-4)
+                    a.pmax[row0 + r] = (float)(1.0 / z);
+                    a.arg[row0 + r] = idx;
+                }
+            }
+        }
+    }
+
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+    }
+}
+
+template <int N>
+cudaError_t launch_tc(HeadTcArgs a, const void *W, cudaStream_t s) {
+    CUtensorMap mapX, mapW;
+    if (!make_map(&mapX, a.x, a.R, a.d, 128) || !make_map(&mapW, W, a.V, a.d, N)) return cudaErrorInvalidValue;
+    a.NT = (a.V + N - 1) / N;
+    a.NR = a.NR < a.NT ? a.NR : a.NT;
+    const size_t smem = 1024 + HTC_AST * HTC_A + HTC_XST * HTC_X + HTC_BST * N * 128 + sizeof(HeadTcSmem);
+    cudaError_t e = cudaFuncSetAttribute(k_head_tc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_chained(k_head_tc<N>, dim3(a.MT * a.NR), HTC_THREADS, smem, 1, s, mapX, mapW, a);
 }
 
 template <typename T, int TM>
@@ -283,14 +723,19 @@ cudaError_t launch_tm(const HeadRowsArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-// Statistics of R rows; scale: scratch [R]; part: scratch [CL_HEAD_ROWS_PARTIALS].  wdtype 0 fp32, 1 bf16; 16-byte aligned inputs.
+static void row_tiles(int R, int &MT, int &rows) {
+    MT = (R + 127) / 128;
+    rows = (R + MT - 1) / MT;
+    MT = (R + rows - 1) / rows;
+}
+
+// Statistics of R rows on the CUDA cores.  scale: scratch [R]; part: scratch [CL_HEAD_ROWS_PARTIALS].  wdtype 0 fp32, 1 bf16; 16-byte
+// aligned inputs.
 cudaError_t cl_launch_head_rows(int wdtype, const void *W, const void *x, const float *gain, int R, int V, int d, float eps, int n_sm,
-                                float *scale, ClHeadPartial *part, float *conf, float *pmax, int *arg, cudaStream_t s) {
+                                double *scale, ClHeadPartial *part, float *conf, float *pmax, int *arg, cudaStream_t s) {
     HeadRowsArgs a;
     a.W = W; a.x = x; a.gain = gain; a.scale = scale; a.R = R; a.V = V; a.d = d; a.part = part;
-    a.MT = (R + 127) / 128;
-    a.rows = (R + a.MT - 1) / a.MT;
-    a.MT = (R + a.rows - 1) / a.rows;
+    row_tiles(R, a.MT, a.rows);
     a.NT = (V + HN - 1) / HN;
     a.NR = 2 * n_sm / a.MT;   // two CTAs per SM
     while (a.NR > 1 && (size_t)R * a.NR > CL_HEAD_ROWS_PARTIALS) --a.NR;
@@ -303,4 +748,27 @@ cudaError_t cl_launch_head_rows(int wdtype, const void *W, const void *x, const 
     if (e != cudaSuccess) return e;
     k_head_rows_merge<<<(R + 3) / 4, 128, 0, s>>>(part, R, a.NR, 1.0 / log((double)V), conf, pmax, arg);
     return cudaGetLastError();
+}
+
+// The same of bf16 rows and a bf16 head on the tensor cores.  scale: scratch [R].  tickets [32] and flags [2] are zero before it; flags[0] != 0
+// after it: a logit was not finite (an infinite weight meets parts that are zero), the results are to be had from cl_launch_head_rows,
+// where it keeps its sign; flags[1] != 0: a wait ran out.
+cudaError_t cl_launch_head_tc(const void *W, const void *x, const float *gain, int R, int V, int d, float eps, int n_sm, double *scale, ClHeadPartial *part,
+                              unsigned *tickets, unsigned *flags, float *conf, float *pmax, int *arg, cudaStream_t s) {
+    HeadTcArgs t;
+    t.x = (const __nv_bfloat16 *)x; t.gain = gain; t.R = R; t.V = V; t.d = d; t.KB = (d + 63) / 64;
+    t.scale = scale;
+    t.inv_log_v = 1.0 / log((double)V);
+    t.part = part; t.tickets = tickets; t.flags = flags; t.conf = conf; t.pmax = pmax; t.arg = arg;
+    row_tiles(R, t.MT, t.rows);
+    t.NR = n_sm / t.MT;
+    while (t.NR > 1 && (size_t)R * t.NR > CL_HEAD_ROWS_PARTIALS) --t.NR;
+    if (t.NR < 1) t.NR = 1;
+    k_row_scale<<<R, 256, 0, s>>>((const __nv_bfloat16 *)x, d, eps, scale);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    // weights a tile: whichever lets the fullest CTA end first, a K block of N weights taken as 6 N + 500 (by the work of the roles)
+    auto cost = [&](int n) { return (long long)(((V + n - 1) / n + t.NR - 1) / t.NR) * (6 * n + 500); };
+    if (cost(224) <= cost(128) && cost(224) <= cost(64)) return launch_tc<224>(t, W, s);
+    return cost(128) <= cost(64) ? launch_tc<128>(t, W, s) : launch_tc<64>(t, W, s);
 }

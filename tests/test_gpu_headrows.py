@@ -102,3 +102,11 @@ def test_error_of_narrow_rows_is_that_of_fp32_sums():
     pm = lp.max(-1).values.exp().cpu().numpy()
     err = [np.linalg.norm(a - b) / np.linalg.norm(b) for a, b in ((got["conf"], conf), (got["p_max"], pm))]
     assert err[0] <= 1.8e-7 and err[1] <= 2.2e-7, err
+
+
+@pytest.mark.parametrize("V,d,n", [(24, 8, 6), (223, 64, 7), (224, 72, 127), (225, 128, 128), (449, 136, 129), (33153, 64, 130), (33152, 192, 6),
+                                   (9472, 136, 9), (9473, 64, 9), (18944, 72, 100), (4500, 4096, 257)])
+def test_tensor_core_scoring_at_the_edges_of_its_tiles(V, d, n):
+    """Tiles of 64, 128 and 224 weights by 128 rows, one and more of them per CTA, K blocks of 64 elements (one, two, a ragged last one).
+    A chain of a K block loses at most 4 units of 2^-23 of its sum, fewer than the additions behind the bound above."""
+    test_tiled_scoring_against_fp64("bf16", V, d, n)
