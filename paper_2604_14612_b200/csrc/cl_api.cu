@@ -923,8 +923,13 @@ extern "C" int cl_verify(cl_ctx *c, int tap_hidden, int32_t *target_toks, float 
     if (rc) return rc;
     const int T = c->h_ndraft + 1;
     if (c->h_ctx + T > c->cfg.max_seq) return fail(c, CL_ERANGE, "cl_verify: position exceeds max_seq");
-    rc = forward_rows(c, ST_FIELD(c, int, cyc_tok), T, 0, nullptr, tap_hidden, 1, ST_FIELD(c, int, tgt_tok),
-                      ST_FIELD(c, float, v_pmax), ST_FIELD(c, float, v_conf), logits ? c->logits : nullptr);
+    // One row alone is a token step, which streams the weights faster than the T-row pass and keeps fp32 activations (8 layers of width
+    // 4096 after 512 positions 804 us, this way 666; fp32 models save nine launches a layer).  Taps are recorded by the T-row pass only.
+    if (T == 1 && c->use_step && !(tap_hidden && c->ring))
+        rc = run_steps(c, CL_STEP_VERIFY, 1, 0, true, logits ? c->logits : nullptr, nullptr);
+    else
+        rc = forward_rows(c, ST_FIELD(c, int, cyc_tok), T, 0, nullptr, tap_hidden, 1, ST_FIELD(c, int, tgt_tok),
+                          ST_FIELD(c, float, v_pmax), ST_FIELD(c, float, v_conf), logits ? c->logits : nullptr);
     if (rc) return rc;
     if (logits && (rc = fetch_logits(c, T))) return rc;
     if ((rc = sync_state(c))) return rc;

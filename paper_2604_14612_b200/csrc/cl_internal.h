@@ -123,7 +123,7 @@ struct ClLayerDev {
     char *kc, *vc;
 };
 
-enum { CL_STEP_DRAFT = 0, CL_STEP_VANILLA = 1 };
+enum { CL_STEP_DRAFT = 0, CL_STEP_VANILLA = 1, CL_STEP_VERIFY = 2 };   // (VERIFY: one full-model step that commits nothing)
 
 struct ClStepArgs {
     const ClLayerDev *layers;   // device [n_layers]

@@ -1,5 +1,5 @@
-// Persistent single-token decoder step ("token-step kernel"): the skip-masked draft step and the
-// vanilla full-model step at batch 1, one cooperative launch for up to CL_MAX_K (draft) or many
+// Persistent single-token decoder step ("token-step kernel"): the skip-masked draft step, the
+// vanilla full-model step and the verify pass of a cycle without drafts at batch 1, one cooperative launch for up to CL_MAX_K (draft) or many
 // (vanilla) consecutive tokens.
 //
 // One CTA per SM.  The last warp (one elected thread) is the weight producer: it walks the static schedule
@@ -1042,6 +1042,10 @@ __global__ void __launch_bounds__(NCT + 32, 1) k_token_steps(ClStepArgs a) {
                 st->d_pmax[a.row0 + step] = pm;
                 st->d_conf[a.row0 + step] = conf;
                 if (stop || step == a.n_steps - 1) st->n_drafted = a.row0 + step + 1;
+            } else if (a.mode == CL_STEP_VERIFY) {
+                st->tgt_tok[0] = tok;
+                st->v_pmax[0] = pm;
+                st->v_conf[0] = conf;
             } else {
                 // vanilla decoding: the token is emitted at once and becomes the next pending token
                 if (a.out_tokens && st->n_out < st->max_new) a.out_tokens[st->n_out] = tok;

@@ -37,3 +37,33 @@ def test_step_kernel_at_short_row_edges(monkeypatch, wd, d, heads, ffn):
         ctx.close()
     for a, b in zip(*out):
         assert np.isfinite(a).all() and np.abs(a - b).max() <= 5e-3
+
+
+@pytest.mark.parametrize("wd,d,heads,kv,ffn", [("fp32", 256, 4, 4, 688), ("bf16", 768, 12, 4, 2048), ("fp16", 2176, 17, 17, 1000)])
+def test_verify_without_drafts_is_a_full_model_step_that_commits_nothing(monkeypatch, wd, d, heads, kv, ffn):
+    """One row takes the token-step kernel, with the skip set left aside; against the T-row passes, same bounds as above.  The cache row it
+    writes is the one the next pass reads: accepting it and drafting from there gives the same logits on both sides."""
+    sh = dataclasses.replace(synth.WORKLOADS["C2"].shape, n_layers=3, d_model=d, n_heads=heads, n_kv_heads=kv, d_ffn=ffn, vocab=1500, max_seq=64,
+                             weight_dtype=wd)
+    W = synth.make_weights(sh, 43, device="cuda")
+    out = []
+    for off in ("0", "1"):
+        monkeypatch.setenv("CL_DISABLE_STEP_KERNEL", off)
+        ctx = cl.Context.from_shape(sh, tap_positions=8)
+        ctx.cl_load(W)
+        ctx.cl_prefill(synth.make_prompt(43, 21, sh.vocab))
+        ctx.cl_rollback(21, 5)
+        ctx.cl_set_skip_set([0, 3, 0])
+        v = ctx.cl_verify(1, want_logits=True)
+        again = ctx.cl_verify(1, want_logits=True)
+        assert ctx.cl_get_stats().ctx_len == 21 and np.array_equal(v["logits"], again["logits"])
+        assert int(v["logits"][0].argmax()) == int(v["targets"][0])
+        tapped = ctx.cl_verify(1, tap_hidden=True, want_logits=True)["logits"]
+        assert np.abs(tapped - v["logits"]).max() <= 5e-3
+        n, emitted = ctx.cl_accept()
+        assert n == 0 and len(emitted) == 1 and ctx.cl_get_stats().ctx_len == 22
+        ctx.cl_rollback(22, 9)
+        out.append([v["logits"][0], ctx.cl_draft(1, want_logits=True)["logits"][0]])
+        ctx.close()
+    for a, b in zip(*out):
+        assert np.isfinite(a).all() and np.abs(a - b).max() <= 5e-3
