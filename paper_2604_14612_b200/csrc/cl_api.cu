@@ -543,9 +543,10 @@ static char *ring_slot(cl_ctx *c, int l, int which) {
 
 // ---- one pass of T rows through the kept layers ------------------------------------------------
 
-static int gemv(cl_ctx *c, int T, int epi, const void *W, int rows, int cols, const float *xin, float *out, int ld) {
+static int gemv(cl_ctx *c, int T, int epi, const void *W, int rows, int cols, const float *xin, float *out, int ld, const float *g = nullptr) {
     ClGemvArgs a;
     memset(&a, 0, sizeof(a));
+    a.g = g; a.eps = c->cfg.rms_eps;
     a.W = W; a.rows = rows; a.cols = cols; a.xin = xin; a.out = out; a.ld = ld; a.st = c->st;
     const int ngroups = (rows + 1) / 2;
     int grid = (ngroups + 7) / 8;
@@ -555,9 +556,10 @@ static int gemv(cl_ctx *c, int T, int epi, const void *W, int rows, int cols, co
 }
 
 static int head(cl_ctx *c, int T, const float *xin, const ClDevState *st, int *out_tok, float *out_pmax, float *out_conf,
-                float *logits) {
+                float *logits, const float *g = nullptr) {
     ClGemvArgs a;
     memset(&a, 0, sizeof(a));
+    a.g = g; a.eps = c->cfg.rms_eps;
     a.W = c->lm_head; a.rows = c->cfg.vocab; a.cols = c->cfg.d_model; a.xin = xin; a.st = st;
     a.logits = logits; a.partials = c->head_part; a.ticket = c->tickets;
     a.out_tok = out_tok; a.out_pmax = out_pmax; a.out_conf = out_conf;
@@ -602,6 +604,8 @@ static int forward_rows(cl_ctx *c, const int *tok, int T, int row0, const uint8_
     const int d = g.d_model, F = g.d_ffn, wd = g.weight_dtype, qkv_rows = d + 2 * g.n_kv_heads * g.head_dim;
     int rc;
     if (c->use_rows && !mask) return forward_rows_persistent(c, tok, T, row0, tap, want_head, out_tok, out_pmax, out_conf, logits);
+    // rows of short models are normalised by the matrix kernels themselves
+    const bool fused = d <= CL_GEMV_NORM_MAX;
     KL(cl_launch_embed(wd, c->embed, tok, T, d, c->x, c->st, c->stream));
     for (int l = 0; l < g.n_layers; ++l) {
         const int skip_bits = mask ? mask[l] : 0;
@@ -609,8 +613,8 @@ static int forward_rows(cl_ctx *c, const int *tok, int T, int row0, const uint8_
         const ClLayer &y = c->layers[l];
         if (!(skip_bits & 1)) {
         // attention half: RMSNorm -> QKV -> rotary + cache append -> attention over the cache -> output projection + residual
-        KL(cl_launch_rmsnorm(c->x, y.n1, T, d, g.rms_eps, c->xn, c->st, c->stream));
-        if ((rc = gemv(c, T, CL_EPI_STORE, y.wqkv, qkv_rows, d, c->xn, c->qkv, qkv_rows))) return rc;
+        if (!fused) KL(cl_launch_rmsnorm(c->x, y.n1, T, d, g.rms_eps, c->xn, c->st, c->stream));
+        if ((rc = gemv(c, T, CL_EPI_STORE, y.wqkv, qkv_rows, d, fused ? c->x : c->xn, c->qkv, qkv_rows, fused ? y.n1 : nullptr))) return rc;
         KL(cl_launch_rope_append(wd, c->qkv, T, row0, g.n_heads, g.n_kv_heads, g.head_dim, d, c->rope_cs, y.kc, y.vc, g.max_seq, c->st,
                                  c->stream));
         ClAttnArgs a;
@@ -624,16 +628,16 @@ static int forward_rows(cl_ctx *c, const int *tok, int T, int row0, const uint8_
             KL(cl_launch_tap(wd, c->x, T, row0, d, ring_slot(c, l, 0), g.tap_positions, c->st, c->stream));
         if (!(skip_bits & 2)) {
         // FFN half: RMSNorm -> gate/up + SiLU -> down projection + residual
-        KL(cl_launch_rmsnorm(c->x, y.n2, T, d, g.rms_eps, c->xn, c->st, c->stream));
-        if ((rc = gemv(c, T, CL_EPI_SILU, y.wgu, 2 * F, d, c->xn, c->hff, F))) return rc;
+        if (!fused) KL(cl_launch_rmsnorm(c->x, y.n2, T, d, g.rms_eps, c->xn, c->st, c->stream));
+        if ((rc = gemv(c, T, CL_EPI_SILU, y.wgu, 2 * F, d, fused ? c->x : c->xn, c->hff, F, fused ? y.n2 : nullptr))) return rc;
         if ((rc = gemv(c, T, CL_EPI_RESID, y.wd, d, F, c->hff, c->x, d))) return rc;
         }
         if (tap && ring_slot(c, l, 1))
             KL(cl_launch_tap(wd, c->x, T, row0, d, ring_slot(c, l, 1), g.tap_positions, c->st, c->stream));
     }
     if (want_head) {
-        KL(cl_launch_rmsnorm(c->x, c->final_norm, T, d, g.rms_eps, c->xn, c->st, c->stream));
-        if ((rc = head(c, T, c->xn, c->st, out_tok, out_pmax, out_conf, logits))) return rc;
+        if (!fused) KL(cl_launch_rmsnorm(c->x, c->final_norm, T, d, g.rms_eps, c->xn, c->st, c->stream));
+        if ((rc = head(c, T, fused ? c->x : c->xn, c->st, out_tok, out_pmax, out_conf, logits, fused ? c->final_norm : nullptr))) return rc;
     }
     return CL_OK;
 }

@@ -88,6 +88,7 @@ __device__ __forceinline__ ClHeadPartial cl_hp_shfl_xor(const ClHeadPartial &a, 
 
 enum { CL_EPI_STORE = 0, CL_EPI_RESID = 1, CL_EPI_SILU = 2, CL_EPI_HEAD = 3 };
 
+#define CL_GEMV_NORM_MAX 1024   // (rows in shared memory: T * 4 KB at most)
 struct ClGemvArgs {
     const void *W;        // [rows, cols] storage type
     int rows, cols;
@@ -95,6 +96,8 @@ struct ClGemvArgs {
     float *out;           // STORE: out[t*ld + r] = y; RESID: out[t*ld + r] += y; SILU: out[t*ld + r/2] = silu(y_r) * y_{r+1}
     int ld;
     const ClDevState *st;
+    const float *g;             // optional: xin is normalised first (RMSNorm with these gains and eps); rows of up to CL_GEMV_NORM_MAX elements
+    float eps;
     // HEAD epilogue
     float *logits;              // optional [T, rows]
     ClHeadPartial *partials;    // [grid, T]
