@@ -38,6 +38,8 @@
 #include <stddef.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace {
@@ -45,15 +47,16 @@ namespace {
 constexpr int RW = 14;                 // worker warps (16 warps in all: four per scheduler, 128 registers per thread)
 constexpr int RT = RW * 32;            // worker threads
 constexpr int R_THREADS = RT + 64;     // + producer warp + MMA warp
-constexpr int R_RING = 215040;         // ring of tiles in flight per SM, allocated by the byte (multiples of 1 KB): 210 KB,
+constexpr int R_RING = 208896;         // ring of tiles in flight per SM, allocated by the byte (multiples of 1 KB): 204 KB,
                                        // with the control block and the alignment slack all the shared memory a CTA can have
 constexpr int R_NE = 16;               // most ring entries (bulk-copy groups with their own pair of mbarriers) in flight
 constexpr int R_MAXN = 224;            // most rows of a weight tile (an accumulator buffer has 256 columns)
-constexpr int R_CTRL_BYTES = 16384;    // control block behind the ring (at least 16 KB: see the kernel)
+constexpr int R_CTRL_BYTES = 22528;    // control block behind the ring (at least 16 KB: see the kernel)
 constexpr int R_ATT_MAXS = 8;          // most parts the cached keys of a head are cut into
 
 constexpr int R_STAGE_LD = R_MAXN + 1;  // row pitch of the epilogue staging buffer (odd: token rows fall into different banks)
-constexpr int R_STAGE_FLOATS = 2032;   // staging buffer: a GEMM tile's raw products of every token row
+constexpr int R_SC_LD = RW * 16 + 8;    // attention: row pitch of the weights (8 off a multiple of 32: pairs of eight rows in one access)
+constexpr int R_STAGE_FLOATS = CL_MAX_T * R_SC_LD;   // staging buffer: a GEMM tile's raw products of every token row; the weights
 
 struct RSmem {
     unsigned long long full[R_NE], empty[R_NE], tfull[2], tempty[2];
@@ -63,13 +66,16 @@ struct RSmem {
     int abort;
     int is_last;
     float scale[CL_SLOTS];             // RMSNorm scale of every token row for the current phase
-    float red[CL_SLOTS];
+    float qscale[CL_MAX_T], lpart[RW][CL_MAX_T];   // attention: what a row's scores are multiplied by; sums of weights by warp
+    unsigned amax[CL_MAX_T];           // ... a row's largest score so far
+    int vodd;                          // ... an own value of the pass is not finite
     float esum[16][CL_SLOTS];          // embedding phase: per-chunk sums of squares
     ClHeadPartial hpw[RW];             // LM head: per-warp statistics
     float wsum[RW];                    // residual phase: per-warp sums of squares
     // one buffer, used in turn by: the GEMM epilogues (raw products of a tile, [T][R_STAGE_LD]); the residual epilogue
-    // ([T][64] squares); the attention phase (per-warp (max, sum, o[hd]) records, [RW][hd + 2])
+    // ([T][64] squares); the attention phase (weights [T][R_SC_LD], then, over the query parts too, the sums [3][T][hd])
     alignas(16) float stage[R_STAGE_FLOATS];
+    alignas(16) unsigned short qp[3 * CL_MAX_T * 128];   // attention: the rotated queries in three parts (directly behind stage)
     alignas(16) unsigned short knew[CL_MAX_T * 128];   // attention: the pass's own keys (rotated) and values in the storage type
     alignas(16) unsigned short vnew[CL_MAX_T * 128];
     unsigned long long t_prev, ph_ns[8];   // diagnostics: time of thread 0 by phase
@@ -116,7 +122,7 @@ __device__ __forceinline__ unsigned counter_read(const unsigned *c) {
 struct Job {
     const char *W;        // k-block-major weights
     const unsigned short *A;
-    int rows, KB, unit, epi;
+    int rows, KB, unit;
     int dep, dep_shift;   // k-block kb of the activation operand is complete when counter dep + (kb >> dep_shift) ...
     unsigned dep_target;  // ... has reached this value (see "completion counters")
     int split;            // CTAs that share a row block and cut its K range between them (1: every CTA owns rows over all of K)
@@ -129,12 +135,12 @@ __device__ __forceinline__ Job job_of(const ClRowsArgs &a, int ji) {
         const int l = ji >> 2, m = ji & 3;
         const ClRowsLayer &y = a.layers[l];
         const int hs = a.hd == 128 ? 1 : 0;   // k-blocks per head: 2 (hd 128) or 1 (hd 64)
-        if (m == 0) { j.W = y.wqkv; j.A = a.Ax; j.rows = a.d + 2 * a.Hkv * a.hd; j.KB = a.d >> 6; j.unit = 1; j.epi = CL_VEPI_STORE; j.dep = a.c_ax; j.dep_shift = 0; j.dep_target = 64u * (2 * l + 1); j.split = 1; }
-        else if (m == 1) { j.W = y.wo; j.A = a.Aatt; j.rows = a.d; j.KB = a.d >> 6; j.unit = 1; j.epi = CL_VEPI_RESID; j.dep = a.c_att; j.dep_shift = hs; j.dep_target = (unsigned)(l + 1); j.split = a.split; }
-        else if (m == 2) { j.W = y.wgu; j.A = a.Ax; j.rows = 2 * a.F; j.KB = a.d >> 6; j.unit = 2; j.epi = CL_VEPI_SILU; j.dep = a.c_ax; j.dep_shift = 0; j.dep_target = 64u * (2 * l + 2); j.split = 1; }
-        else { j.W = y.wd; j.A = a.Ah; j.rows = a.d; j.KB = a.F >> 6; j.unit = 1; j.epi = CL_VEPI_RESID; j.dep = a.c_ah; j.dep_shift = 0; j.dep_target = 64u * (l + 1); j.split = a.split; }
+        if (m == 0) { j.W = y.wqkv; j.A = a.Ax; j.rows = a.d + 2 * a.Hkv * a.hd; j.KB = a.d >> 6; j.unit = 1; j.dep = a.c_ax; j.dep_shift = 0; j.dep_target = 64u * (2 * l + 1); j.split = 1; }
+        else if (m == 1) { j.W = y.wo; j.A = a.Aatt; j.rows = a.d; j.KB = a.d >> 6; j.unit = 1; j.dep = a.c_att; j.dep_shift = hs; j.dep_target = (unsigned)(l + 1); j.split = a.split; }
+        else if (m == 2) { j.W = y.wgu; j.A = a.Ax; j.rows = 2 * a.F; j.KB = a.d >> 6; j.unit = 2; j.dep = a.c_ax; j.dep_shift = 0; j.dep_target = 64u * (2 * l + 2); j.split = 1; }
+        else { j.W = y.wd; j.A = a.Ah; j.rows = a.d; j.KB = a.F >> 6; j.unit = 1; j.dep = a.c_ah; j.dep_shift = 0; j.dep_target = 64u * (l + 1); j.split = a.split; }
     } else {
-        j.W = a.head; j.A = a.Ax; j.rows = a.V; j.KB = a.d >> 6; j.unit = 1; j.epi = CL_VEPI_HEAD; j.dep = a.c_ax; j.dep_shift = 0; j.dep_target = 64u * (2 * L + 1); j.split = 1;
+        j.W = a.head; j.A = a.Ax; j.rows = a.V; j.KB = a.d >> 6; j.unit = 1; j.dep = a.c_ax; j.dep_shift = 0; j.dep_target = 64u * (2 * L + 1); j.split = 1;
     }
     return j;
 }
@@ -160,7 +166,7 @@ struct Cursor {
     int ji;
     const char *W;
     const unsigned short *A;
-    int rows, KB, unit, epi;
+    int rows, KB, unit;
     int dep, dep_shift;
     unsigned dep_target;
     int kb_begin, kb_end;     // the CTA's k-blocks of the job (all of them unless the job is split over K)
@@ -219,7 +225,7 @@ struct Cursor {
     __device__ void next_job() {
         for (++ji; ji < njobs; ++ji) {
             const Job j = job_of(a, ji);
-            W = j.W; A = j.A; rows = j.rows; KB = j.KB; unit = j.unit; epi = j.epi;
+            W = j.W; A = j.A; rows = j.rows; KB = j.KB; unit = j.unit;
             dep = j.dep; dep_shift = j.dep_shift; dep_target = j.dep_target;
             rows_of(rows, unit, j.split, r0, r1);
             const int member = (int)blockIdx.x % j.split;
@@ -231,6 +237,14 @@ struct Cursor {
             }
         }
         done = true;
+    }
+    // To the start of job j: a worker warp works its cursor out again behind the attention phase, whose registers it would
+    // otherwise take away.  (The place in the ring, which worker warps do not use, is lost.)
+    __device__ void reopen(int j) {
+        ji = j - 1;
+        in_chain = 0;
+        done = false;
+        next_job();
     }
     __device__ __forceinline__ void advance() {
         in_chain = chain_last() ? 0 : in_chain + kbs;
@@ -309,6 +323,15 @@ __device__ __forceinline__ void a_store_split(unsigned short *A, int t, int T, i
     split_b16(v, f16, hi, lo);
     A[a_index(t, k)] = hi;
     A[a_index(T + t, k)] = lo;
+}
+
+// Elements k (even) and k + 1.
+__device__ __forceinline__ void a_store_split2(unsigned short *A, int t, int T, int k, float v0, float v1, int f16) {
+    unsigned short h0, l0, h1, l1;
+    split_b16(v0, f16, h0, l0);
+    split_b16(v1, f16, h1, l1);
+    *(unsigned *)(A + a_index(t, k)) = (unsigned)h0 | ((unsigned)h1 << 16);
+    *(unsigned *)(A + a_index(T + t, k)) = (unsigned)l0 | ((unsigned)l1 << 16);
 }
 
 __device__ __forceinline__ ClHeadPartial rp_merge(const ClHeadPartial &a, const ClHeadPartial &b) { return cl_hp_merge(a, b); }
@@ -492,12 +515,13 @@ struct Group {
 };
 
 // All worker warps call this with the same cursor state.  `run` carries a thread's LM-head statistics across tiles.
+template <int epi>
 __device__ __forceinline__ void gemm_job(const ClRowsArgs &a, RSmem *sm, unsigned tmem, int ji, Cursor &c, unsigned &n, ClHeadPartial &run) {
     if (c.done || c.ji != ji) return;   // this CTA has no part in the job
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool drains = (warp & 3) == 0;
     const int dw = warp >> 2;
-    const int T = a.T, epi = c.epi, rows = c.rows;
+    const int T = a.T, rows = c.rows;
     const int wpt = RW / T;                                  // warps per token row in the epilogue
     const int et = warp / wpt, ej = (warp % wpt) * 32 + lane, estride = wpt * 32;
     bool job_done = false;
@@ -746,14 +770,23 @@ __device__ void embed_phase(const ClRowsArgs &a, RSmem *sm) {
 }
 
 // ---- attention of the T rows over the cache ------------------------------------------------------------------
-// Work item (head h, part s of the cached keys [0, base)) -> one CTA.  Inside the CTA warp w serves token row
-// t = w / nsub and the sub-range sub = w % nsub of the part's keys (nsub = 14 / T warps per row).  A warp walks its
-// keys 32 at a time with an online softmax (scores reduced with warp shuffles).  The rows' own keys and values
-// (positions base .. base + t, causal) come raw from the QKV product: the CTA of the last part first rotates the
-// keys, rounds keys and values to the storage type and keeps them in shared memory (one query head per key/value
-// head also appends them to the cache); the last warp of row t folds them in.  The CTA merges its warps per row and writes one
-// record per (h, s, t); the last CTA of a head to finish (ticket) merges the parts in order and writes the
-// normalised output as the output projection's hi/lo operand rows.
+// Work item (head h, part s of the cached keys [0, base)) -> one CTA.  A part is walked in chunks of 16 keys, 14 chunks at a time:
+//   scores   warp w multiplies the keys of chunk w by all T queries; the rows' maxima, then the weights meet in shared memory
+//   output   warp (key group, 32 elements of the head) adds the weighted values of a third of the chunks; the three sums are
+//            added in shared memory
+// so every key and value row is fetched once per CTA, all of them at once, before the CTA waits for its queries: the phase costs
+// one trip to memory for the queries and none for 224 keys.  Both products run on the tensor cores (mma.sync) with queries
+// and weights in three parts of the storage type, scaled as in k_attn_wide, whose sums are as exact as fp32 multiply-adds; keys and
+// values are the A operand (16 keys or 16 elements of the head), the T rows the columns, so that up to eight rows cost one
+// instruction.  The rows' own keys and values (positions base .. base + t, causal) come raw from the QKV product: the CTA of the
+// last part rotates the keys, rounds both to the storage type and takes them as its last chunk (one query head per
+// key/value head also appends them to the cache).  A CTA writes one (max, sum, output) record per (h, s, t); the last CTA of
+// a head to finish (ticket) merges the parts in order and writes the normalised output as the output projection's hi/lo
+// operand rows.
+// Bound: latency (the queries' trip, the record's, the ticket and the merge).  Before, a warp walked a row's keys 16 at a time, one trip
+// to memory each.  Attention of a layer, mean over CTAs: 640 keys, 5 rows of 32 heads 14.5 -> 8 us; 1003 keys, 9 rows 35 -> 14; verify
+// of 8 layers of width 4096 907 -> 846 and 1141 -> 960 us, 4 layers of width 5120 after 1024 keys (7 rows) 711 -> 643, 12 of width
+// 768 after 200 keys (5 rows) as before.  Nine rows: the values' registers for 14 chunks spill (991 us), 12 chunks 965.
 // Ahead of a layer's QKV job: ask for the cached keys and values this CTA's attention item will read, so that they wait
 // in L2 when the attention phase starts (the worker warps have nothing else to do while the job's weights stream).
 template <int HD>
@@ -769,195 +802,395 @@ __device__ __forceinline__ void attention_prefetch(const ClRowsArgs &a, const Cl
     }
 }
 
-template <typename ST, int HD>
+// Order-preserving map of floats (no NaN) to unsigned, for a maximum by atomics.
+__device__ __forceinline__ unsigned ord_enc(float f) {
+    const unsigned u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float ord_dec(unsigned u) { return __uint_as_float((u & 0x80000000u) ? (u ^ 0x80000000u) : ~u); }
+
+// NT: tiles of eight token rows (one up to T = 8, else two).
+template <typename ST, int HD, int NT>
 __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int layer, int base, RSmem *sm) {
-    constexpr int EPL = 8, LPK = HD / EPL, KPW = 32 / LPK, VPL = HD / 32, WSTRIDE = HD + 2, HALF = HD / 2;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int T = a.T, S = a.att_parts, nsub = RW / T;
-    const int t = warp / nsub, sub = warp % nsub;
-    const bool active = warp < T * nsub;
-    const int li = lane % LPK, ksub = lane / LPK;
+    constexpr int F16 = std::is_same<ST, __half>::value ? 1 : 0;
+    constexpr int HALF = HD / 2, NC = HD / 32, EP = HALF / 32, WSTRIDE = HD + 2;
+    constexpr unsigned TOP = F16 ? 14 : 0;      // exponent of the largest element of a scaled query row, and of a weight of 1
+    constexpr int STEP = F16 ? ATT_STEP : 1;
+    constexpr float PSCALE = F16 ? 16384.f : 1.f;
+    constexpr int CPI = NT == 1 ? RW : 12;      // chunks per iteration (nine rows leave registers for fewer values)
+    constexpr int MAXC = (CPI + 2) / 3;         // most chunks of a key group
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, tig = lane & 3;
+    const int T = a.T, S = a.att_parts;
     const float scale = rsqrtf((float)HD);
     const int group = a.H / a.Hkv, kvd = a.Hkv * HD, ld = a.d + 2 * kvd;
-    ST *Kc = (ST *)y.kc, *Vc = (ST *)y.vc;
-    float *wrec = sm->stage;
+    const int kg = warp / NC, ds = warp % NC;   // this warp's key group and 32 elements of the head
+    const bool pv = warp < 3 * NC;
+    float *sc = sm->stage;                      // [T][R_SC_LD] weights of an iteration; later [3][T][HD] sums of the key groups
     for (int item = blockIdx.x; item < a.H * S; item += gridDim.x) {
         const int h = item % a.H, s = item / a.H, kvh = h / group;
-        // this head's q rows and its key/value head's k and v rows of the QKV product: complete? (three counters, one
-        // lane each)
-        if (warp == 0) {
-            if (lane < 3) {
-                const int b = lane == 0 ? h : (lane == 1 ? a.H + kvh : a.H + a.Hkv + kvh);
-                counter_wait(a.sync + a.c_qkv + b, (unsigned)(HD * (layer + 1)), sm, &a.st->err);
-            }
-            __syncwarp();
+        const bool last_part = s == S - 1;
+        const int k0 = (int)((long long)base * s / S), k1 = (int)((long long)base * (s + 1) / S);
+        const int nk = k1 - k0, nc = (nk + 15) >> 4, nch = nc + (last_part ? 1 : 0);   // cached keys, their chunks, all chunks
+        const unsigned short *Kh = (const unsigned short *)y.kc + ((size_t)kvh * a.max_seq + k0) * HD;
+        const unsigned short *Vh = (const unsigned short *)y.vc + ((size_t)kvh * a.max_seq + k0) * HD;
+        // Fragments: of a key row a lane holds 8 consecutive elements of every 32 (the order of the elements inside an
+        // instruction is free as long as keys and queries agree); of a value row 4 of the warp's 32.
+        uint4 kf[2][NC];
+        uint2 vf[MAXC][4];
+        auto load_keys = [&](int c) {              // cached keys of chunk c: rows g and g + 8
+            const int key = c * 16 + g;
+            const unsigned short *kp = Kh + (size_t)key * HD + tig * 8;
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int q = 0; q < NC; ++q) {
+                    kf[r][q] = make_uint4(0u, 0u, 0u, 0u);
+                    if (key + 8 * r < nk) kf[r][q] = __ldg((const uint4 *)(kp + 8 * r * HD + q * 32));
+                }
+        };
+        auto load_values = [&](int i0, int n) {    // cached values of the key group: rows 2 tig, + 1, + 8, + 9 of a chunk
+            const int v0 = (i0 + n * kg / 3) * 16 + 2 * tig, v1 = pv ? min(nk, (i0 + n * (kg + 1) / 3) * 16) : 0;
+            const unsigned short *vp = Vh + (size_t)v0 * HD + ds * 32 + g * 4;
+#pragma unroll
+            for (int i = 0; i < MAXC; ++i)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int row = i * 16 + (r & 1) + (r & 2) * 4;
+                    vf[i][r] = make_uint2(0u, 0u);
+                    if (v0 + row < v1) vf[i][r] = __ldg((const uint2 *)(vp + row * HD));
+                }
+        };
+        constexpr int NR = NT + 1;                   // rows of a lane: 2 tig, 2 tig + 1 and, where tig = 0, the ninth
+        auto row_of = [&](int r) { return r < 2 ? 2 * tig + r : (tig == 0 ? 8 : CL_MAX_T); };   // (CL_MAX_T: no row)
+        float o[4][NR], m_c[NR], l_c[NR];            // sums of 4 elements; a row's maximum so far, and this lane's sum of its weights
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            m_c[r] = -INFINITY;
+            l_c[r] = o[0][r] = o[1][r] = o[2][r] = o[3][r] = 0.f;
         }
-        phase_clock(a, sm, 7);
-        worker_sync();
-        if (s == S - 1) {
-            // the pass's own keys and values, raw in the QKV product: rotate the keys, round both to the storage type, keep
-            // them for the warps below (one query head per key/value head also appends them to the cache); one thread per
-            // (row, pair of elements i, i + hd / 2), so the whole set costs one memory round trip
-            const bool writer = (h % group) == 0;
-            for (int idx = tid; idx < T * HALF; idx += RT) {
-                const int jn = idx / HALF, i = idx % HALF;
-                const float *kraw = a.qkv + (size_t)jn * ld + a.d + kvh * HD, *vraw = kraw + kvd;
-                const float2 cs = a.rope_cs[(size_t)(base + jn) * HALF + i];
-                const float ka = __ldcg(kraw + i), kb = __ldcg(kraw + i + HALF);
-                const float va = __ldcg(vraw + i), vb = __ldcg(vraw + i + HALF);
-                const unsigned short kk0 = f32_to_b16(ka * cs.x - kb * cs.y, a.f16), kk1 = f32_to_b16(kb * cs.x + ka * cs.y, a.f16);
-                const unsigned short v0 = f32_to_b16(va, a.f16), v1 = f32_to_b16(vb, a.f16);
-                sm->knew[jn * HD + i] = kk0; sm->knew[jn * HD + i + HALF] = kk1;
-                sm->vnew[jn * HD + i] = v0; sm->vnew[jn * HD + i + HALF] = v1;
-                if (writer) {
-                    unsigned short *ck = (unsigned short *)Kc + ((size_t)kvh * a.max_seq + base + jn) * HD;
-                    unsigned short *cv = (unsigned short *)Vc + ((size_t)kvh * a.max_seq + base + jn) * HD;
-                    ck[i] = kk0; ck[i + HALF] = kk1; cv[i] = v0; cv[i + HALF] = v1;
+#pragma unroll 1
+        for (int i0 = 0; i0 == 0 || i0 < nch; i0 += CPI) {
+            const int n = min(CPI, nch - i0);           // the iteration's chunks
+            load_keys(i0 + warp);
+            if (i0 == 0) {
+                if (tid < T) sm->amax[tid] = ord_enc(-INFINITY);
+                if (tid == 0) sm->vodd = 0;
+                // this head's q rows and its key/value head's k and v rows of the QKV product: complete? (three counters, one
+                // lane each)
+                if (warp == 0) {
+                    if (lane < 3) {
+                        const int b = lane == 0 ? h : (lane == 1 ? a.H + kvh : a.H + a.Hkv + kvh);
+                        counter_wait(a.sync + a.c_qkv + b, (unsigned)(HD * (layer + 1)), sm, &a.st->err);
+                    }
+                    __syncwarp();
                 }
-            }
-            worker_sync();
-        }
-        float m_run = -INFINITY, l_run = 0.f, o_run[VPL];
+                phase_clock(a, sm, 7);
+                worker_sync();
+                // warp t: query row t, rotated, scaled to [2^TOP, 2^(TOP + 1)) by a power of two, split
+                float qa[EP], qb[EP];
+                float2 cs[EP];
+                if (warp < T) {
+                    const float *qraw = a.qkv + (size_t)warp * ld + h * HD + lane * EP;
 #pragma unroll
-        for (int e = 0; e < VPL; ++e) o_run[e] = 0.f;
-        if (active) {
-            const int pos = base + t;
-            const float *qraw = a.qkv + (size_t)t * ld + h * HD;
-            float qr[EPL];
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) {
-                const int idx = li * EPL + e;
-                const int i = idx < HALF ? idx : idx - HALF;
-                const float2 cs = a.rope_cs[(size_t)pos * HALF + i];
-                const float qa = __ldcg(qraw + i), qb = __ldcg(qraw + i + HALF);
-                qr[e] = idx < HALF ? qa * cs.x - qb * cs.y : qb * cs.x + qa * cs.y;
-            }
-            const int k0 = (int)((long long)base * s / S), k1 = (int)((long long)base * (s + 1) / S);
-            const int kw0 = k0 + (int)((long long)(k1 - k0) * sub / nsub), kw1 = k0 + (int)((long long)(k1 - k0) * (sub + 1) / nsub);
-            const ST *Kh = Kc + (size_t)kvh * a.max_seq * HD, *Vh = Vc + (size_t)kvh * a.max_seq * HD;
-            // CH keys per iteration: the key rows and the value rows of the iteration are requested together (the values do
-            // not depend on the scores), so an iteration costs one memory round trip; lane j < CH keeps key j's score
-            constexpr int CH = 16, NPASS = CH / KPW;
-            for (int j0 = kw0; j0 < kw1; j0 += CH) {
-                const int n = min(CH, kw1 - j0);
-                uint4 raw[NPASS];
-#pragma unroll
-                for (int p = 0; p < NPASS; ++p) {
-                    const int j = p * KPW + ksub;
-                    raw[p] = make_uint4(0u, 0u, 0u, 0u);
-                    if (j < n) raw[p] = __ldg((const uint4 *)(Kh + (size_t)(j0 + j) * HD + li * EPL));
+                    for (int e = 0; e < EP; ++e) {
+                        qa[e] = __ldcg(qraw + e);
+                        qb[e] = __ldcg(qraw + HALF + e);
+                        cs[e] = a.rope_cs[(size_t)(base + warp) * HALF + lane * EP + e];
+                    }
                 }
-                uint2 vraw[CH];   // the value rows stay in their storage type until they are used
-#pragma unroll
-                for (int j = 0; j < CH; ++j) {
-                    const ST *vp = Vh + (size_t)(j0 + min(j, n - 1)) * HD + lane * VPL;
-                    if (VPL == 4) vraw[j] = __ldg((const uint2 *)vp);
-                    else vraw[j] = make_uint2(__ldg((const unsigned *)vp), 0u);
-                }
-                float my_score = -INFINITY;
-#pragma unroll
-                for (int p = 0; p < NPASS; ++p) {
-                    const int jb = p * KPW;
-                    if (jb < n) {   // uniform
-                        const unsigned u[4] = {raw[p].x, raw[p].y, raw[p].z, raw[p].w};
-                        float sc = 0.f;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            float ka, kb;
-                            ClPair16<ST>::get(u[e], ka, kb);
-                            sc = fmaf(qr[2 * e], ka, sc);
-                            sc = fmaf(qr[2 * e + 1], kb, sc);
-                        }
-#pragma unroll
-                        for (int o = LPK >> 1; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
-                        sc *= scale;
-#pragma unroll
-                        for (int k = 0; k < KPW; ++k) {
-                            const float v = __shfl_sync(0xffffffffu, sc, k * LPK);
-                            if (lane == jb + k && jb + k < n) my_score = v;
+                if (last_part) {
+                    // the pass's own keys and values, raw in the QKV product: rotate the keys, round both to the storage type, keep
+                    // them for the warps below (one query head per key/value head also appends them to the cache); one thread per
+                    // (row, pair of elements i, i + hd / 2), so the whole set costs one memory round trip
+                    const bool writer = (h % group) == 0;
+                    for (int idx = tid; idx < T * HALF; idx += RT) {
+                        const int jn = idx / HALF, i = idx % HALF;
+                        const float *kraw = a.qkv + (size_t)jn * ld + a.d + kvh * HD, *vraw = kraw + kvd;
+                        const float2 cn = a.rope_cs[(size_t)(base + jn) * HALF + i];
+                        const float ka = __ldcg(kraw + i), kb = __ldcg(kraw + i + HALF);
+                        const float va = __ldcg(vraw + i), vb = __ldcg(vraw + i + HALF);
+                        const unsigned short kk0 = f32_to_b16(ka * cn.x - kb * cn.y, F16), kk1 = f32_to_b16(kb * cn.x + ka * cn.y, F16);
+                        const unsigned short v0 = f32_to_b16(va, F16), v1 = f32_to_b16(vb, F16);
+                        sm->knew[jn * HD + i] = kk0; sm->knew[jn * HD + i + HALF] = kk1;
+                        sm->vnew[jn * HD + i] = v0; sm->vnew[jn * HD + i + HALF] = v1;
+                        if (!(fabsf(b16_to_f32(v0, F16)) < INFINITY && fabsf(b16_to_f32(v1, F16)) < INFINITY)) sm->vodd = 1;
+                        if (writer) {
+                            unsigned short *ck = (unsigned short *)y.kc + ((size_t)kvh * a.max_seq + base + jn) * HD;
+                            unsigned short *cv = (unsigned short *)y.vc + ((size_t)kvh * a.max_seq + base + jn) * HD;
+                            ck[i] = kk0; ck[i + HALF] = kk1; cv[i] = v0; cv[i + HALF] = v1;
                         }
                     }
                 }
-                float m_new = my_score;
+                if (warp < T) {
+                    float lo[EP], hi[EP], amax = 0.f;   // elements lane * EP + e of the two halves
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
-                m_new = fmaxf(m_new, m_run);
-                const float p = (lane < n) ? expf(my_score - m_new) : 0.f;
-                const float resc = (l_run > 0.f) ? expf(m_run - m_new) : 0.f;
-                float ps = p;
+                    for (int e = 0; e < EP; ++e) {
+                        lo[e] = qa[e] * cs[e].x - qb[e] * cs[e].y;
+                        hi[e] = qb[e] * cs[e].x + qa[e] * cs[e].y;
+                        amax = fmaxf(amax, fmaxf(fabsf(lo[e]), fabsf(hi[e])));
+                    }
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
-                l_run = fmaf(l_run, resc, ps);
+                    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+                    const unsigned ex = min(max(__float_as_uint(amax) >> 23, 1u + TOP), 253u);
+                    const float inv = __uint_as_float((254u + TOP - ex) << 23);
+                    if (lane == 0) sm->qscale[warp] = __uint_as_float((ex - TOP) << 23) * scale;
+                    unsigned l3[3], h3[3];
+                    split3<F16, 1>(lo[0] * inv, lo[EP - 1] * inv, l3);
+                    split3<F16, 1>(hi[0] * inv, hi[EP - 1] * inv, h3);
 #pragma unroll
-                for (int e = 0; e < VPL; ++e) o_run[e] *= resc;
-                m_run = m_new;
+                    for (int p = 0; p < 3; ++p) {
+                        unsigned short *row = sm->qp + (size_t)(p * CL_MAX_T + warp) * HD;
+                        auto at = [&](int el) { return row + ((((el >> 3) ^ ((warp & 1) << 2)) << 3) | (el & 7)); };
+                        if (EP == 2) {
+                            *(unsigned *)at(lane * 2) = l3[p];
+                            *(unsigned *)at(HALF + lane * 2) = h3[p];
+                        } else {
+                            *at(lane) = (unsigned short)l3[p];
+                            *at(HALF + lane) = (unsigned short)h3[p];
+                        }
+                    }
+                }
+                worker_sync();
+            }
+            // ---- scores: this warp's 16 keys against all rows ----
+            float w[2][NR];   // keys g and g + 8
+            if (warp < n) {
+                const int c = i0 + warp;
+                const bool own = c >= nc;
+                if (own) {
 #pragma unroll
-                for (int j = 0; j < CH; ++j) {
-                    const float pj = __shfl_sync(0xffffffffu, p, j);   // (0 for j >= n: the repeated last row adds nothing)
-                    float v[4];
-                    ClPair16<ST>::get(vraw[j].x, v[0], v[1]);
-                    ClPair16<ST>::get(vraw[j].y, v[2], v[3]);
+                    for (int r = 0; r < 2; ++r)
 #pragma unroll
-                    for (int e = 0; e < VPL; ++e) o_run[e] = fmaf(pj, v[e], o_run[e]);
+                        for (int q = 0; q < NC; ++q) {
+                            kf[r][q] = make_uint4(0u, 0u, 0u, 0u);
+                            if (g + 8 * r < T) kf[r][q] = *(const uint4 *)(sm->knew + (g + 8 * r) * HD + q * 32 + tig * 8);
+                        }
+                }
+                float u[3][4];   // products with the queries' parts
+                float x[4];      // of the ninth row: its parts are the columns
+#pragma unroll
+                for (int e = 0; e < 4; ++e) u[0][e] = u[1][e] = u[2][e] = x[e] = 0.f;
+#pragma unroll
+                for (int q = 0; q < NC; ++q) {
+                    const unsigned a0[4] = {kf[0][q].x, kf[1][q].x, kf[0][q].y, kf[1][q].y}, a1[4] = {kf[0][q].z, kf[1][q].z, kf[0][q].w, kf[1][q].w};
+                    const int tok = min(g, T - 1);
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {
+                        const uint4 b = *(const uint4 *)(sm->qp + (size_t)(p * CL_MAX_T + tok) * HD + (((q * 4 + tig) ^ ((tok & 1) << 2)) << 3));
+                        mma16816<F16>(u[p], a0, b.x, b.y);
+                        mma16816<F16>(u[p], a1, b.z, b.w);
+                    }
+                    if (NT == 2) {
+                        const uint4 b = *(const uint4 *)(sm->qp + (size_t)(min(g, 2) * CL_MAX_T + 8) * HD + ((q * 4 + tig) << 3));
+                        mma16816<F16>(x, a0, b.x, b.y);
+                        mma16816<F16>(x, a1, b.z, b.w);
+                    }
+                }
+                float odd = 0.f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    float &v = w[e >> 1][e & 1];
+                    v = (u[0][e] + (u[1][e] + u[2][e])) * sm->qscale[min(2 * tig + (e & 1), T - 1)];
+                    odd = fmaf(v, 0.f, odd);   // (not zero once a score is infinite or no number)
+                }
+                if (NT == 2) {
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        float &v = w[k][NR - 1];
+                        v = (x[2 * k] + (x[2 * k + 1] + __shfl_xor_sync(0xffffffffu, x[2 * k], 1))) * sm->qscale[8];
+                        if (tig == 0) odd = fmaf(v, 0.f, odd);
+                    }
+                }
+                if (__any_sync(0xffffffffu, odd != 0.f)) {
+                    // An infinite key or query: its parts are zeros and infinities of both signs.  The scores anew, from whole queries.
+                    const unsigned short *kr[2];
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+                        kr[r] = own ? sm->knew + min(g + 8 * r, T - 1) * HD : Kh + (size_t)min(c * 16 + g + 8 * r, nk - 1) * HD;
+#pragma unroll 1
+                    for (int y = 0; y < 2 * NR; ++y) {
+                        const int tok = min(row_of(y >> 1), T - 1);
+                        const float *qr = a.qkv + (size_t)tok * ld + h * HD;
+                        const float2 *rc = a.rope_cs + (size_t)(base + tok) * HALF;
+                        const unsigned short *kp = (y & 1) ? kr[1] : kr[0];
+                        float v = 0.f;
+#pragma unroll 1
+                        for (int i = 0; i < HALF; ++i) {
+                            const float xa = __ldcg(qr + i), xb = __ldcg(qr + i + HALF);
+                            const float2 cn = rc[i];
+                            v = fmaf(xa * cn.x - xb * cn.y, b16_to_f32(kp[i], F16), v);
+                            v = fmaf(xb * cn.x + xa * cn.y, b16_to_f32(kp[i + HALF], F16), v);
+                        }
+                        v *= scale;
+                        v = v > -INFINITY ? v : -INFINITY;   // (no number: no weight)
+#pragma unroll
+                        for (int z = 0; z < 2 * NR; ++z)
+                            if (y == z) w[z & 1][z >> 1] = v;
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    const int tok = row_of(r);
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const int key = g + 8 * k;
+                        if (!(own ? (key < T && key <= tok) : (c * 16 + key < nk))) w[k][r] = -INFINITY;
+                    }
+                    float m = fmaxf(w[0][r], w[1][r]);
+#pragma unroll
+                    for (int x = 4; x <= 16; x <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, x));
+                    if (g == 0 && tok < T) atomicMax(&sm->amax[tok], ord_enc(m));
                 }
             }
-            if (s == S - 1 && sub == nsub - 1) {
-                // the pass's own positions base .. base + t
-                for (int jn = 0; jn <= t; ++jn) {
-                    float kf[EPL], vn[VPL];
-                    const uint4 raw = *(const uint4 *)(sm->knew + jn * HD + li * EPL);
-                    const unsigned u[4] = {raw.x, raw.y, raw.z, raw.w};
+            const int ncl = min(n, nc - i0);       // cached chunks of the iteration
+            load_values(i0, ncl);   // (they arrive while the weights are worked out; with the keys' registers they would not fit)
+            worker_sync();
+            // ---- weights of this warp's keys, now that the rows' maxima are known ----
+            float resc[NR];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) pair16_to_f32(u[e], a.f16, kf[2 * e], kf[2 * e + 1]);
-#pragma unroll
-                    for (int e = 0; e < VPL; ++e) vn[e] = b16_to_f32(sm->vnew[jn * HD + lane * VPL + e], a.f16);
-                    float sc = 0.f;
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) sc = fmaf(qr[e], kf[e], sc);
-#pragma unroll
-                    for (int o = LPK >> 1; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
-                    sc = __shfl_sync(0xffffffffu, sc, 0) * scale;
-                    const float m_new = fmaxf(m_run, sc);
-                    const float resc = (l_run > 0.f) ? expf(m_run - m_new) : 0.f;
-                    const float pn = expf(sc - m_new);
-                    l_run = fmaf(l_run, resc, pn);
-#pragma unroll
-                    for (int e = 0; e < VPL; ++e) o_run[e] = fmaf(o_run[e], resc, pn * vn[e]);
-                    m_run = m_new;
+            for (int r = 0; r < NR; ++r) {
+                const int tok = row_of(r);
+                const float mc = ord_dec(sm->amax[min(tok, T - 1)]), mb = mc > -INFINITY ? mc : 0.f;
+                resc[r] = expf(m_c[r] - mb);   // (0 while the maximum is -inf)
+                m_c[r] = mc;
+                l_c[r] *= resc[r];
+                if (warp < n && tok < T) {
+                    const float p0 = expf(w[0][r] - mb), p1 = expf(w[1][r] - mb);
+                    l_c[r] += p0 + p1;
+                    sc[tok * R_SC_LD + warp * 16 + g] = p0 * PSCALE;
+                    sc[tok * R_SC_LD + warp * 16 + g + 8] = p1 * PSCALE;
                 }
             }
-        }
-        if (lane == 0) {
-            wrec[warp * WSTRIDE] = m_run;
-            wrec[warp * WSTRIDE + 1] = l_run;
-        }
+            worker_sync();
+            // ---- output: a third of the chunks, 32 elements of the head ----
+            if (pv) {
+                const int c0 = ncl * kg / 3, c1 = ncl * (kg + 1) / 3;
+                const bool own = kg == 2 && ncl < n, odd = own && *(volatile int *)&sm->vodd;   // this group takes the pass's own chunk as well
+                auto own_values = [&](uint2(&v)[4]) {
 #pragma unroll
-        for (int e = 0; e < VPL; ++e) wrec[warp * WSTRIDE + 2 + lane * VPL + e] = o_run[e];
+                    for (int r = 0; r < 4; ++r) {
+                        const int key = 2 * tig + (r & 1) + (r & 2) * 4;
+                        v[r] = make_uint2(0u, 0u);
+                        if (key < T && !odd) v[r] = *(const uint2 *)(sm->vnew + key * HD + ds * 32 + g * 4);
+                    }
+                };
+                // a chunk's values as the A operand: 16 elements of the head x 16 keys, twice
+                auto value_operand = [&](const uint2(&v)[4], unsigned(&a0)[4], unsigned(&a1)[4]) {
+                    a0[0] = __byte_perm(v[0].x, v[1].x, 0x5410); a0[1] = __byte_perm(v[0].x, v[1].x, 0x7632);
+                    a0[2] = __byte_perm(v[2].x, v[3].x, 0x5410); a0[3] = __byte_perm(v[2].x, v[3].x, 0x7632);
+                    a1[0] = __byte_perm(v[0].y, v[1].y, 0x5410); a1[1] = __byte_perm(v[0].y, v[1].y, 0x7632);
+                    a1[2] = __byte_perm(v[2].y, v[3].y, 0x5410); a1[3] = __byte_perm(v[2].y, v[3].y, 0x7632);
+                };
+                auto odd_value = [&](int tok, int e) {   // element e of the lane's four: own values that are infinite or no numbers
+                    float v = 0.f;                       // (only rows that give such a value weight may meet it)
+#pragma unroll 1
+                    for (int j = 0; j < T; ++j) {
+                        const float p = sc[min(tok, T - 1) * R_SC_LD + ncl * 16 + j];
+                        const float val = b16_to_f32(sm->vnew[j * HD + ds * 32 + g * 4 + e], F16);
+                        if (p != 0.f) v = fmaf(p, val, v);
+                    }
+                    return v;
+                };
+                {
+                    float c[3][2][4];   // sums by part
+#pragma unroll
+                    for (int e = 0; e < 24; ++e) c[e / 8][e / 4 % 2][e % 4] = 0.f;
+                    const float *row = sc + min(g, T - 1) * R_SC_LD + 2 * tig;
+                    auto chunk = [&](const uint2(&v)[4], int lc) {
+                        unsigned a0[4], a1[4], b0[3], b1[3];
+                        value_operand(v, a0, a1);
+                        const float2 p0 = *(const float2 *)(row + lc * 16), p1 = *(const float2 *)(row + lc * 16 + 8);
+                        split3<F16, STEP>(p0.x, p0.y, b0);
+                        split3<F16, STEP>(p1.x, p1.y, b1);
+#pragma unroll
+                        for (int p = 0; p < 3; ++p) {
+                            mma16816<F16>(c[p][0], a0, b0[p], b1[p]);
+                            mma16816<F16>(c[p][1], a1, b0[p], b1[p]);
+                        }
+                    };
+#pragma unroll
+                    for (int i = 0; i < MAXC; ++i)
+                        if (c0 + i < c1) chunk(vf[i], c0 + i);   // uniform over the warp
+                    if (own) {
+                        uint2 v[4];
+                        own_values(v);
+                        chunk(v, ncl);
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int m = e >> 2, y = e & 3;
+                        const float low = fmaf(c[2][m][y], 1.f / STEP, c[1][m][y]);
+                        float sum = fmaf(low, 1.f / STEP, c[0][m][y]);
+                        if (odd) sum += odd_value(2 * tig + (y & 1), m * 2 + (y >> 1));
+                        float &to = o[m * 2 + (y >> 1)][y & 1];
+                        to = fmaf(to, resc[y & 1], sum);
+                    }
+                }
+                if (NT == 2) {          // the ninth row: the parts of its weights are the columns
+                    float x[2][4];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) x[e / 4][e % 4] = 0.f;
+                    const float *row = sc + 8 * R_SC_LD + 2 * tig;
+                    auto chunk = [&](const uint2(&v)[4], int lc) {
+                        unsigned a0[4], a1[4], b0[3], b1[3];
+                        value_operand(v, a0, a1);
+                        const float2 p0 = *(const float2 *)(row + lc * 16), p1 = *(const float2 *)(row + lc * 16 + 8);
+                        split3<F16, STEP>(p0.x, p0.y, b0);
+                        split3<F16, STEP>(p1.x, p1.y, b1);
+                        const unsigned y0 = g == 0 ? b0[0] : g == 1 ? b0[1] : b0[2], y1 = g == 0 ? b1[0] : g == 1 ? b1[1] : b1[2];
+                        mma16816<F16>(x[0], a0, y0, y1);
+                        mma16816<F16>(x[1], a1, y0, y1);
+                    };
+#pragma unroll
+                    for (int i = 0; i < MAXC; ++i)
+                        if (c0 + i < c1) chunk(vf[i], c0 + i);
+                    if (own) {
+                        uint2 v[4];
+                        own_values(v);
+                        chunk(v, ncl);
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int m = e >> 1, y = (e & 1) * 2;
+                        const float low = fmaf(__shfl_xor_sync(0xffffffffu, x[m][y], 1), 1.f / STEP, x[m][y + 1]);
+                        float sum = fmaf(low, 1.f / STEP, x[m][y]);
+                        if (odd) sum += odd_value(8, e);
+                        o[e][NR - 1] = fmaf(o[e][NR - 1], resc[NR - 1], sum);   // (lanes with tig = 0 hold the row)
+                    }
+                }
+            }
+            worker_sync();   // the weights have been read
+        }
+        // the key groups' sums, added in order; one record per (h, s, t), or the final output if S == 1
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int tok = row_of(r);
+            float l = l_c[r];
+#pragma unroll
+            for (int x = 4; x <= 16; x <<= 1) l += __shfl_xor_sync(0xffffffffu, l, x);
+            if (tok < T) {
+                if (g == 0) sm->lpart[warp][tok] = l;
+                if (pv) *(float4 *)(sc + (size_t)(kg * T + tok) * HD + ds * 32 + g * 4) = make_float4(o[0][r], o[1][r], o[2][r], o[3][r]);
+            }
+        }
         worker_sync();
-        // merge the nsub warps of every row (fixed order); one record per (h, s, t), or the final output if S == 1
         float *part = a.att_part + ((size_t)h * R_ATT_MAXS + s) * CL_MAX_T * WSTRIDE;
-        for (int i = tid; i < T * HD; i += RT) {
-            const int tt = i / HD, e = i % HD;
-            float M = -INFINITY;
-            for (int w = 0; w < nsub; ++w) {
-                const float *r = wrec + (tt * nsub + w) * WSTRIDE;
-                if (r[1] > 0.f) M = fmaxf(M, r[0]);
-            }
-            float Ls = 0.f, O = 0.f;
-            for (int w = 0; w < nsub; ++w) {
-                const float *r = wrec + (tt * nsub + w) * WSTRIDE;
-                if (r[1] > 0.f) {
-                    const float f = expf(r[0] - M);
-                    Ls = fmaf(r[1], f, Ls);
-                    O = fmaf(r[2 + e], f, O);
-                }
+        for (int i = tid; i < T * HALF; i += RT) {
+            const int tt = i / HALF, e = i % HALF * 2;
+            const float *p = sc + (size_t)tt * HD + e;
+            const float2 g0 = *(const float2 *)p, g1 = *(const float2 *)(p + (size_t)T * HD), g2 = *(const float2 *)(p + (size_t)2 * T * HD);
+            const float2 O = make_float2((g0.x + g1.x + g2.x) * (1.f / PSCALE), (g0.y + g1.y + g2.y) * (1.f / PSCALE));
+            float Ls = 0.f;
+            if (S == 1 || e == 0) {
+#pragma unroll
+                for (int x = 0; x < RW; ++x) Ls += sm->lpart[x][tt];
             }
             if (S == 1) {
-                a_store_split(a.Aatt, tt, T, h * HD + e, O / Ls, a.f16);
+                a_store_split2(a.Aatt, tt, T, h * HD + e, O.x / Ls, O.y / Ls, a.f16);
             } else {
                 float *rec = part + (size_t)tt * WSTRIDE;
-                if (e == 0) { rec[0] = M; rec[1] = Ls; }
-                rec[2 + e] = O;
+                if (e == 0) *(float2 *)rec = make_float2(ord_dec(sm->amax[tt]), Ls);
+                *(float2 *)(rec + 2 + e) = O;
             }
         }
         if (S > 1) {
@@ -971,30 +1204,37 @@ __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int l
             worker_sync();
             if (sm->is_last) {
                 const float *p0 = a.att_part + (size_t)h * R_ATT_MAXS * CL_MAX_T * WSTRIDE;
-                for (int i = tid; i < T * HD; i += RT) {
-                    const int tt = i / HD, e = i % HD;
-                    float pm[R_ATT_MAXS], pl[R_ATT_MAXS], po[R_ATT_MAXS];
+                for (int i = tid; i < T * HALF; i += RT) {
+                    const int tt = i / HALF, e = i % HALF * 2;
+                    float2 ml[R_ATT_MAXS], po[R_ATT_MAXS];
 #pragma unroll
-                    for (int s2 = 0; s2 < R_ATT_MAXS; ++s2) {
-                        const float *ps = p0 + ((size_t)min(s2, S - 1) * CL_MAX_T + tt) * WSTRIDE;
-                        pm[s2] = __ldcg(ps);
-                        pl[s2] = (s2 < S) ? __ldcg(ps + 1) : 0.f;
-                        po[s2] = __ldcg(ps + 2 + e);
+                    for (int b = 0; b < R_ATT_MAXS; b += 4) {
+#pragma unroll
+                        for (int s2 = b; s2 < b + 4; ++s2) {
+                            ml[s2] = po[s2] = make_float2(0.f, 0.f);
+                            if (b < S) {   // uniform
+                                const float *ps = p0 + ((size_t)min(s2, S - 1) * CL_MAX_T + tt) * WSTRIDE;
+                                ml[s2] = __ldcg((const float2 *)ps);
+                                po[s2] = __ldcg((const float2 *)(ps + 2 + e));
+                                if (s2 >= S) ml[s2].y = 0.f;
+                            }
+                        }
                     }
                     float M = -INFINITY;
 #pragma unroll
                     for (int s2 = 0; s2 < R_ATT_MAXS; ++s2)
-                        if (pl[s2] > 0.f) M = fmaxf(M, pm[s2]);
-                    float Ls = 0.f, O = 0.f;
+                        if (ml[s2].y > 0.f) M = fmaxf(M, ml[s2].x);
+                    float Ls = 0.f, O0 = 0.f, O1 = 0.f;
 #pragma unroll
                     for (int s2 = 0; s2 < R_ATT_MAXS; ++s2) {   // part order
-                        if (pl[s2] > 0.f) {
-                            const float f = expf(pm[s2] - M);
-                            Ls = fmaf(pl[s2], f, Ls);
-                            O = fmaf(po[s2], f, O);
+                        if (ml[s2].y > 0.f) {
+                            const float f = expf(ml[s2].x - M);
+                            Ls = fmaf(ml[s2].y, f, Ls);
+                            O0 = fmaf(po[s2].x, f, O0);
+                            O1 = fmaf(po[s2].y, f, O1);
                         }
                     }
-                    a_store_split(a.Aatt, tt, T, h * HD + e, O / Ls, a.f16);
+                    a_store_split2(a.Aatt, tt, T, h * HD + e, O0 / Ls, O1 / Ls, a.f16);
                 }
             }
         }
@@ -1055,23 +1295,25 @@ __global__ void __launch_bounds__(R_THREADS, 1) k_rows_pass(const __grid_constan
             const ClRowsLayer &y = a.layers[l];
             attention_prefetch<HD>(a, y, base);
             compute_scales(a, sm, 2 * l + 1);
-            gemm_job(a, sm, tmem, 4 * l, cur, n_acc, run);
+            gemm_job<CL_VEPI_STORE>(a, sm, tmem, 4 * l, cur, n_acc, run);
             phase_clock(a, sm, 1);
-            attention_phase<ST, HD>(a, y, l, base, sm);
+            if (a.T <= 8) attention_phase<ST, HD, 1>(a, y, l, base, sm);
+            else attention_phase<ST, HD, 2>(a, y, l, base, sm);
+            cur.reopen(4 * l + 1);
             phase_clock(a, sm, 2);
-            gemm_job(a, sm, tmem, 4 * l + 1, cur, n_acc, run);
+            gemm_job<CL_VEPI_RESID>(a, sm, tmem, 4 * l + 1, cur, n_acc, run);
             resid_phase(a, 4 * l + 1, base, sm);
             phase_clock(a, sm, 3);
             compute_scales(a, sm, 2 * l + 2);
-            gemm_job(a, sm, tmem, 4 * l + 2, cur, n_acc, run);
+            gemm_job<CL_VEPI_SILU>(a, sm, tmem, 4 * l + 2, cur, n_acc, run);
             phase_clock(a, sm, 4);
-            gemm_job(a, sm, tmem, 4 * l + 3, cur, n_acc, run);
+            gemm_job<CL_VEPI_RESID>(a, sm, tmem, 4 * l + 3, cur, n_acc, run);
             resid_phase(a, 4 * l + 3, base, sm);
             phase_clock(a, sm, 5);
         }
         if (a.want_head) {
             compute_scales(a, sm, 2 * a.L + 1);
-            gemm_job(a, sm, tmem, 4 * a.L, cur, n_acc, run);
+            gemm_job<CL_VEPI_HEAD>(a, sm, tmem, 4 * a.L, cur, n_acc, run);
             head_finish(a, sm, run);
             phase_clock(a, sm, 6);
             grid_barrier(a, bar_target, sm);
@@ -1142,7 +1384,9 @@ cudaError_t cl_launch_tile_layout(const void *src, void *dst, int rows, int K, i
 cudaError_t cl_launch_rows_pass(int wdtype, int head_dim, const ClRowsArgs &a, int grid, cudaStream_t s) {
     static_assert(sizeof(RSmem) <= R_CTRL_BYTES, "control block must fit behind the ring");
     static_assert(R_STAGE_FLOATS >= CL_MAX_T * R_STAGE_LD && R_STAGE_FLOATS % 4 == 0, "staging buffer holds a tile of every token row");
-    static_assert(R_STAGE_FLOATS >= RW * (128 + 2), "staging buffer holds the attention records");
+    static_assert(offsetof(RSmem, qp) == offsetof(RSmem, stage) + R_STAGE_FLOATS * 4 &&
+                  R_STAGE_FLOATS * 4 + sizeof(RSmem::qp) >= 3 * CL_MAX_T * 128 * 4, "staging buffer and query parts hold the sums of three key groups");
+    static_assert(R_RING + R_CTRL_BYTES + 1024 <= 232448, "shared memory of a CTA");
     const void *fn = nullptr;
     if (wdtype == 1 && head_dim == 64) fn = (const void *)k_rows_pass<__nv_bfloat16, 64>;
     else if (wdtype == 1 && head_dim == 128) fn = (const void *)k_rows_pass<__nv_bfloat16, 128>;

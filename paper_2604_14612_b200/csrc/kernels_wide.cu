@@ -399,7 +399,6 @@ __global__ void __launch_bounds__(256) k_wide_rope_append(ClWideParts p, int hd,
 // 410 that the kernels of a layer take; the register-tiled fp32 products on the CUDA cores that it replaces took 122.  Blocks of late rows see the most keys and
 // are scheduled first.
 constexpr int AQ = 64, AK = 64;   // rows per CTA, keys per tile
-constexpr int ATT_STEP = 4096;    // fp16: ratio of a probability part's scale to the part before (a rest is below 2^-11 of its value: no overflow)
 
 template <int HD>
 constexpr size_t attn_wide_smem() { return (size_t)(3 * AQ + 4 * AK) * HD * 2 + AQ * 4; }
@@ -410,27 +409,6 @@ __device__ __forceinline__ void ldsm4(unsigned (&r)[4], unsigned addr) {
 __device__ __forceinline__ void ldsm4_t(unsigned (&r)[4], unsigned addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
-template <int F16>
-__device__ __forceinline__ void mma16816(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-    if (F16)
-        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-    else
-        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// Two values -> three packed pairs of the 16-bit type: v = p0 + p1 / STEP + p2 / STEP^2, each the rest so far rounded.
-template <int F16, int STEP>
-__device__ __forceinline__ void split3(float x, float y, unsigned (&o)[3]) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const unsigned short a = f32_to_b16(x, F16), b = f32_to_b16(y, F16);
-        o[i] = (unsigned)a | ((unsigned)b << 16);
-        x = (x - b16_to_f32(a, F16)) * (float)STEP;
-        y = (y - b16_to_f32(b, F16)) * (float)STEP;
-    }
-}
-
 template <int HD, int F16>
 __global__ void __launch_bounds__(128, 2)
 k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsigned short *vcache, __nv_bfloat16 *out_b,

@@ -243,6 +243,32 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// ---- attention on mma.sync (k_attn_wide says why the queries and the probabilities enter in three parts) ----
+constexpr int ATT_STEP = 4096;    // fp16: ratio of a probability part's scale to the part before (a rest is below 2^-11 of its value: no overflow)
+template <int F16>
+__device__ __forceinline__ void mma16816(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+    if (F16)
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+    else
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Two values -> three packed pairs of the 16-bit type: v = p0 + p1 / STEP + p2 / STEP^2, each the rest so far rounded.
+template <int F16, int STEP>
+__device__ __forceinline__ void split3(float x, float y, unsigned (&o)[3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        // both in one conversion (round to nearest even, as one by one)
+        if (F16) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(o[i]) : "f"(y), "f"(x));
+        else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(o[i]) : "f"(y), "f"(x));
+        float a, b;
+        pair16_to_f32(o[i], F16, a, b);
+        x = (x - a) * (float)STEP;
+        y = (y - b) * (float)STEP;
+    }
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                   const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

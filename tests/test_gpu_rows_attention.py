@@ -1,0 +1,90 @@
+"""Attention of the (K + 1)-row pass at the edges of its chunks of 16 keys and its iterations of 14 (nine rows: 12) of them, for every
+number of rows, and with keys and values that overflowed the cache (run on a B200)."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2604_14612_b200 as cl
+from test_gpu_wide_attention import _model
+
+pytestmark = pytest.mark.gpu
+
+DT = {"bf16": torch.bfloat16, "fp16": torch.float16}
+V = 256
+
+
+def _random_model(wd, heads, kv_heads, hd):
+    d, kvd, F = heads * hd, kv_heads * hd, 128
+    g = torch.Generator(device="cuda").manual_seed(heads * hd)
+    t = lambda r, c, s=0.05: (torch.randn((r, c), generator=g, device="cuda") * s).to(DT[wd])
+    o = lambda: torch.ones(d, device="cuda")
+    return d, F, dict(embed=t(V, d, 1.0), lm_head=t(V, d), final_norm=o(), wq=[t(d, d)], wk=[t(kvd, d)], wv=[t(kvd, d)], wo=[t(d, d)],
+                      wg=[t(F, d)], wu=[t(F, d)], wd=[t(d, F)], norm1=[o()], norm2=[o()])
+
+
+@pytest.mark.parametrize("wd,heads,kv_heads,hd", [("bf16", 2, 2, 64), ("fp16", 4, 2, 128), ("bf16", 40, 40, 64), ("fp16", 37, 37, 64), ("bf16", 8, 1, 128)])
+def test_every_number_of_rows_and_cached_keys(monkeypatch, wd, heads, kv_heads, hd):
+    """Against the CUDA-core pass, on the same cache.  Heads in 8, 8, 3, 4 and 8 parts.  Both passes round the new values to the storage
+    type; an operand of 16 bits (2^-17 off) decides about one bf16 value in 2^8 the other way, by 2^-9: 2^-9 * 2^-4 = 1.2e-4 of the
+    output where one key is all there is, four times that as bound."""
+    d, F, W = _random_model(wd, heads, kv_heads, hd)
+    out = {}
+    for off in ("0", "1"):
+        monkeypatch.setenv("CL_DISABLE_ROWS_KERNEL", off)
+        ctx = cl.Context(1, d, heads, F, V, 2000, wd, 1e-5, 1e4, tap_positions=16, n_kv_heads=kv_heads)
+        ctx.cl_load(W)
+        res = []
+        for n in (17, 18, 31, 33, 127, 129, 447, 448, 449, 895, 897, 1791, 1900):
+            ctx.cl_prefill((np.arange(n) * 7 + n).astype(np.int32) % V)
+            for T in range(1, 10):
+                ctx.cl_rollback(n, n % V)
+                ctx.cl_force_tokens((np.arange(T - 1) * 3 + 1).astype(np.int32))
+                res.append((n, T, ctx.cl_verify(T, tap_hidden=True, want_logits=True)["logits"].copy()))
+        for n in (1, 2, 8):                     # short prompts: chunks of rows behind nothing
+            ctx.cl_prefill((np.arange(n) * 5 + 2).astype(np.int32) % V)
+            ctx.cl_rollback(n, 3)
+            ctx.cl_force_tokens([4, 5])
+            res.append((n, 3, ctx.cl_verify(3, want_logits=True)["logits"].copy()))
+        out[off] = res
+        ctx.close()
+    for (n, T, x), (_, _, y) in zip(out["0"], out["1"]):
+        rel = np.linalg.norm(x - y) / np.linalg.norm(y)
+        assert rel <= 5e-4, (n, T, rel)
+
+
+@pytest.mark.parametrize("T", [1, 5, 9])
+def test_keys_that_score_minus_infinity_have_no_weight(T):
+    """fp16 keys of 1e5 are infinite; against a negative query they score -inf, so the first token's value is the whole output."""
+    n = 600
+    g = torch.Generator().manual_seed(6)
+    values, first = (1.0 + torch.rand(256, generator=g)) * 500, 1.0 + torch.rand(256, generator=g)
+    first[:3] = 0.0
+    ctx, emb, _ = _model("fp16", 4, n + 8, [-32.0, -1.0, -3.3, -0.01], values, first_key=0.0, other_key=1e5, first_value=first)
+    ctx.cl_prefill(np.concatenate([[0], 1 + np.arange(n - 1) % 1000]).astype(np.int32))
+    ctx.cl_rollback(n, 7)
+    ctx.cl_force_tokens(np.arange(1, T).astype(np.int32))
+    ctx.cl_verify(T, tap_hidden=True)
+    ring = ctx.cl_read_hidden_ring().double().numpy()[0]
+    ctx.close()
+    got = ring[[(n + t) % 512 for t in range(T)]]
+    want = (first / 16.0).half().double().numpy() * 16.0
+    assert np.isfinite(got).all()
+    assert np.abs(got - emb[[7] + list(range(1, T))] - want)[:, 3:].max() <= 2e-3          # half a step of fp16 at 2 is 1e-3
+
+
+@pytest.mark.parametrize("T", [5, 9])
+def test_a_candidate_whose_value_overflows_leaves_the_rows_before_it_alone(T):
+    """Token 0 has values of 1e5, infinite in fp16: rows that do not attend to it are the same to the bit, rows that do are not finite."""
+    n = 40
+    ctx, _, _ = _model("fp16", 4, n + 16, [1.0, 2.0, -1.0, 0.5], torch.ones(256), first_value=1e5)
+    rows = {}
+    for third in (0, 5):
+        ctx.cl_prefill((1 + np.arange(n)).astype(np.int32))
+        ctx.cl_rollback(n, 7)
+        ctx.cl_force_tokens(np.array([1, 2, third] + list(range(10, 6 + T)), np.int32))
+        ctx.cl_verify(T, tap_hidden=True)
+        rows[third] = ctx.cl_read_hidden_ring().double().numpy()[0][[(n + t) % 512 for t in range(T)]]
+    ctx.close()
+    assert np.isfinite(rows[5]).all()
+    assert np.array_equal(rows[0][:3], rows[5][:3])
+    assert not np.isfinite(rows[0][3:, 3:]).any()
