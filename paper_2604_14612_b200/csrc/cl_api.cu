@@ -662,7 +662,7 @@ static int forward_wide(cl_ctx *c, const int *tok, int M, int tap) {
     {
         ClWideNormArgs n = nb;
         n.embed = c->embed; n.tok = tok; n.g = L ? c->layers[0].n1 : nullptr;
-        KL(cl_launch_wide_norm(n, c->stream));
+        KL(cl_launch_wide_norm(n, c->n_sm, c->stream));
     }
     int rc;
     ClWideParts p;
@@ -677,14 +677,14 @@ static int forward_wide(cl_ctx *c, const int *tok, int M, int tap) {
         ClWideNormArgs n = nb;
         n.parts = p; n.g = y.n2;
         if (tap) n.tap = ring_slot(c, l, 0);
-        KL(cl_launch_wide_norm(n, c->stream));
+        KL(cl_launch_wide_norm(n, c->n_sm, c->stream));
         if ((rc = gemm(c->map_wx, c->map_gu[l], 2 * F, KBd, &p))) return rc;
         KL(cl_launch_wide_silu(p, F, c->w_ah, lo0, f16, c->stream));
         if ((rc = gemm(c->map_wh, c->map_d[l], d, KBf, &p))) return rc;
         n = nb;
         n.parts = p; n.g = (l + 1 < L) ? c->layers[l + 1].n1 : nullptr;
         if (tap) n.tap = ring_slot(c, l, 1);
-        KL(cl_launch_wide_norm(n, c->stream));
+        KL(cl_launch_wide_norm(n, c->n_sm, c->stream));
     }
     return CL_OK;
 }

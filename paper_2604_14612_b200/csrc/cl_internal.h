@@ -287,7 +287,7 @@ struct ClWideNormArgs {
 ClWideParts cl_wide_plan(int M, int rows, int KB, int n_sm, float *P, size_t ws_floats);
 cudaError_t cl_launch_wide(const ClTensorMap &mapA, const ClTensorMap &mapB, const ClWideParts &p, int lo_row0, int *err, int f16,
                            cudaStream_t s);
-cudaError_t cl_launch_wide_norm(const ClWideNormArgs &a, cudaStream_t s);
+cudaError_t cl_launch_wide_norm(const ClWideNormArgs &a, int n_sm, cudaStream_t s);
 cudaError_t cl_launch_wide_rope_append(const ClWideParts &p, int H, int Hkv, int hd, int d, const float2 *rope_cs, void *kcache,
                                        void *vcache, int max_seq, const ClDevState *st, int f16, cudaStream_t s);
 // causal attention of the M rows of the pass (positions ctx ..) over the cache; q: fp32 rows [M, ld_q], rotary applied;

@@ -4,7 +4,7 @@
 //
 // The pass is bound by HBM weight streaming (at most 9 flop per weight byte), so its shape follows the single-token
 // step kernel: one CTA per SM, every CTA owns a contiguous block of rows of every matrix (single-row granularity, so
-// all SMs stream the same number of bytes), one producer warp walks the static schedule and keeps a 210 KB ring of
+// all SMs stream the same number of bytes), one producer warp walks the static schedule and keeps a 204 KB ring of
 // weight tiles filled straight through the phase boundaries, and the phases of a layer (QKV | attention | O |
 // gate/up | down) follow one another inside the launch, ordered by completion counters per buffer (below), not by
 // launches.  What differs is the arithmetic: 2 T activation

@@ -259,21 +259,28 @@ __device__ __forceinline__ int wide_parts(const ClWideParts &p, int t, int col) 
 }
 
 // One CTA per token row: x[t] = E[token] or x[t] += product parts (added in part order); the optional hidden tap;
-// then the rows of the next GEMM: hi/lo(x * rsqrt(mean x^2 + eps) * g).  A thread's elements stay in registers between
-// the two passes (up to two chunks of 4; the rest is read again).  As many threads as there are chunks of 4, up to 1024: with few
-// rows the loads in flight per SM are what bounds it.
-__global__ void __launch_bounds__(1024) k_wide_norm(ClWideNormArgs a) {
+// then the rows of the next GEMM: hi/lo(x * rsqrt(mean x^2 + eps) * g).  A thread's elements stay in registers between the two
+// passes: KEEP chunks of 4, read side by side, part by part, before anything is written (a store between the loads would order
+// them); of rows longer than KEEP * 4 * THREADS elements the rest is read again.
+// Bound: L2 (parts and stream in, stream and two operand rows out).  Rows that do not all fit on the chip at once cost a second
+// wave, few rows want many loads in flight each, so KEEP is the least of 1, 2, 4 that leaves one wave (cl_launch_wide_norm).
+// us, within a pass, KEEP 1 / 2 / 4: width 4096, 61 rows 6.0 / 7.7 / 11.9, 200 rows 8.5 / 6.2 / 9.5, 512 rows 14.8 / 10.0 / 9.3; width
+// 5120, 400 rows 16.5 / 12.0 / 8.8; width 768, 512 rows 4.7 / 6.5 / 9.0.
+template <int KEEP, int THREADS, int AHEAD>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_wide_norm(ClWideNormArgs a) {
     __shared__ float red[32];
-    constexpr int KEEP = 2;
     pdl_launch_dependents();
     const int t = blockIdx.x, tid = threadIdx.x, d = a.d, span = 4 * blockDim.x;   // columns per round of the CTA
     float *xr = a.x + (size_t)t * d;
-    float4 keep[KEEP], gain[KEEP];
+    float4 gain[KEEP];
+    auto gains = [&]() {   // (weights: they may be read ahead of the wait)
 #pragma unroll
-    for (int k = 0; k < KEEP; ++k) {   // (gains are weights: read ahead of the wait)
-        const int i = tid * 4 + k * span;
-        gain[k] = (a.g && i < d) ? __ldg((const float4 *)(a.g + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+        for (int k = 0; k < KEEP; ++k) {
+            const int i = tid * 4 + k * span;
+            gain[k] = a.g && i < d ? __ldg((const float4 *)(a.g + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    if (KEEP <= 2) gains();
     pdl_wait();
     const unsigned short *er = a.tok ? (const unsigned short *)a.embed + (size_t)a.tok[t] * d : nullptr;
     // only the last tap_P rows of the pass reach the ring: an earlier row of the same slot would be overwritten anyway
@@ -281,41 +288,58 @@ __global__ void __launch_bounds__(1024) k_wide_norm(ClWideNormArgs a) {
     if (a.tap && t >= a.M - a.tap_P) tap = (unsigned short *)a.tap + (size_t)((a.st->ctx + t) % a.tap_P) * d;
     const size_t plane = (size_t)a.M * d;
     float ss = 0.f;
-    auto element = [&](int i) -> float4 {   // the updated stream at columns i .. i + 3
-        float4 v;
-        if (er) {
-            const uint2 u = *(const uint2 *)(er + i);
-            pair16_to_f32(u.x, a.f16, v.x, v.y);
-            pair16_to_f32(u.y, a.f16, v.z, v.w);
-        } else {
-            v = *(const float4 *)(xr + i);
-            const int n = wide_parts(a.parts, t, i);
-            const float *p0 = a.parts.P + (size_t)t * d + i;
-#pragma unroll 4
-            for (int s = 0; s < n; ++s) {
-                const float4 p = __ldcg((const float4 *)(p0 + (size_t)s * plane));
-                v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
+    float4 keep[KEEP];
+    auto read = [&](int i0, int n_chunks) {   // the updated stream at columns i0 + tid * 4 + k * span .. + 3 -> keep[k]
+        int n[KEEP], nmax = 0;
+#pragma unroll
+        for (int k = 0; k < KEEP; ++k) {
+            const int i = i0 + tid * 4 + k * span;
+            const bool in = k < n_chunks && i < d;
+            n[k] = 0;
+            keep[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (in && er) {
+                const uint2 u = *(const uint2 *)(er + i);
+                pair16_to_f32(u.x, a.f16, keep[k].x, keep[k].y);
+                pair16_to_f32(u.y, a.f16, keep[k].z, keep[k].w);
+            } else if (in) {
+                keep[k] = *(const float4 *)(xr + i);
+                n[k] = wide_parts(a.parts, t, i);
+                nmax = max(nmax, n[k]);
             }
         }
-        *(float4 *)(xr + i) = v;
-        if (tap) {
-            const unsigned lo2 = (unsigned)f32_to_b16(v.x, a.f16) | ((unsigned)f32_to_b16(v.y, a.f16) << 16);
-            const unsigned hi2 = (unsigned)f32_to_b16(v.z, a.f16) | ((unsigned)f32_to_b16(v.w, a.f16) << 16);
-            *(uint2 *)(tap + i) = make_uint2(lo2, hi2);
-        }
-        ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
-        return v;
-    };
+        const float *p0 = a.parts.P + (size_t)t * d + i0 + tid * 4;
+#pragma unroll AHEAD
+        for (int s = 0; s < nmax; ++s) {
+            float4 p[KEEP];
 #pragma unroll
-    for (int k = 0; k < KEEP; ++k) {
-        const int i = tid * 4 + k * span;
-        if (i < d) keep[k] = element(i);
-    }
-    for (int i = tid * 4 + KEEP * span; i < d; i += span) element(i);
+            for (int k = 0; k < KEEP; ++k) p[k] = s < n[k] ? __ldcg((const float4 *)(p0 + (size_t)s * plane + k * span)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < KEEP; ++k) {
+                keep[k].x += p[k].x; keep[k].y += p[k].y; keep[k].z += p[k].z; keep[k].w += p[k].w;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < KEEP; ++k) {
+            const int i = i0 + tid * 4 + k * span;
+            const float4 v = keep[k];
+            ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
+            if (k < n_chunks && i < d) {
+                *(float4 *)(xr + i) = v;
+                if (tap) {
+                    const unsigned lo2 = (unsigned)f32_to_b16(v.x, a.f16) | ((unsigned)f32_to_b16(v.y, a.f16) << 16);
+                    const unsigned hi2 = (unsigned)f32_to_b16(v.z, a.f16) | ((unsigned)f32_to_b16(v.w, a.f16) << 16);
+                    *(uint2 *)(tap + i) = make_uint2(lo2, hi2);
+                }
+            }
+        }
+    };
+    for (int i0 = KEEP * span; i0 < d; i0 += span) read(i0, 1);   // (what does not stay in registers first)
+    read(0, KEEP);
     if (!a.g) return;   // uniform
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
     if ((tid & 31) == 0) red[tid >> 5] = ss;
+    if (KEEP > 2) gains();
     __syncthreads();
     float tot = 0.f;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];   // fixed order
@@ -686,10 +710,17 @@ cudaError_t cl_launch_wide(const ClTensorMap &mapA, const ClTensorMap &mapB, con
     return launch_chained(k_wide, dim3(2 * p.G), WTHREADS, smem, 2, s, *(const CUtensorMap *)mapA.bytes, *(const CUtensorMap *)mapB.bytes, a);
 }
 
-cudaError_t cl_launch_wide_norm(const ClWideNormArgs &a, cudaStream_t s) {
+cudaError_t cl_launch_wide_norm(const ClWideNormArgs &a, int n_sm, cudaStream_t s) {
     if (a.d % 4) return cudaErrorInvalidValue;
-    const int chunks = a.d / 4, rounds = (chunks + 1023) / 1024, threads = ((chunks + rounds - 1) / rounds + 31) / 32 * 32;
-    return launch_chained(k_wide_norm, dim3(a.M), threads, 0, 1, s, a);
+    const int chunks = a.d / 4;
+    auto launch = [&](void (*kern)(ClWideNormArgs), int keep, int most) {
+        return launch_chained(kern, dim3(a.M), std::min(most, ((chunks + keep - 1) / keep + 31) / 32 * 32), 0, 1, s, a);
+    };
+    // as few chunks a thread as leave all rows on the chip at once (64 registers: 1024 threads an SM)
+    auto fits = [&](int keep) { return chunks <= keep * 1024 && a.M <= n_sm * (1024 / ((chunks + keep - 1) / keep)); };
+    if (fits(1)) return launch(k_wide_norm<1, 1024, 4>, 1, 1024);
+    if (fits(2)) return launch(k_wide_norm<2, 1024, 2>, 2, 1024);
+    return launch(k_wide_norm<4, 512, 2>, 4, 512);
 }
 
 cudaError_t cl_launch_wide_rope_append(const ClWideParts &p, int H, int Hkv, int hd, int d, const float2 *rope_cs, void *kcache,
