@@ -416,12 +416,15 @@ __global__ void __launch_bounds__(256) k_wide_rope_append(ClWideParts p, int hd,
 // [1, 2)), a probability by 2^14, and of a probability each part is 2^12 times what the parts before it left, so that weights
 // down to 2^-38 of the row's largest keep 24 bits (ATT_STEP).
 // The sums are as exact as fp32 multiply-adds (relative error against 64 bits at 512 rows after 512 / 64 rows after 4032 keys:
-// 6.9e-7 / 1.4e-6 with those, 4.9e-7 / 8.1e-7 here, fp16): the accumulator of the instruction cuts off where an fp32 addition rounds, which
-// over one chain for all keys of a row came to 2.2e-6 / 9.9e-6, so a chain is one tile of 64 keys, the parts have accumulators of their own
-// and everything else is added in fp32.
-// Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile).  At 512 rows of 32 heads it takes 43 us of the
-// 410 that the kernels of a layer take; the register-tiled fp32 products on the CUDA cores that it replaces took 122.  Blocks of late rows see the most keys and
-// are scheduled first.
+// 6.9e-7 / 1.4e-6 with those, 4.0e-7 / 7.5e-7 here, fp16): the accumulator of the instruction cuts off where an fp32 addition rounds, which
+// over one chain for all keys of a row came to 2.2e-6 / 9.9e-6, so a chain is one tile of 64 keys, the parts have accumulators of their own,
+// a score's chain is cut in two (one chain: 4.9e-7 / 8.0e-7) and everything else is added in fp32.
+// Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile, 8.4 cycles each at best) and the ALU work between them, which
+// two warps per scheduler hardly overlap: at 512 rows after 512 of 32 heads 143000 cycles, 68000 of them multiply-adds.  So the
+// instructions beside them count: chains start from a zero operand, masks are applied only where a key may lie ahead, a weight is one
+// multiply-add and one ex2, fragment addresses flip bits of one base.  512 rows of 32 heads 53 -> 40 us, the pass after it 97 -> 78, 333
+// rows 38 -> 29.  Key tiles dealt out evenly over the CTAs, jobs cut where shares end: 41 us (a cut costs more than the balance gains); eight
+// warps of 32 keys: 45.  Blocks of late rows see the most keys and are scheduled first.
 constexpr int AQ = 64, AK = 64;   // rows per CTA, keys per tile
 
 template <int HD>
@@ -433,6 +436,13 @@ __device__ __forceinline__ void ldsm4(unsigned (&r)[4], unsigned addr) {
 __device__ __forceinline__ void ldsm4_t(unsigned (&r)[4], unsigned addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
+constexpr float LOG2E = 1.44269504f;
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 template <int HD, int F16>
 __global__ void __launch_bounds__(128, 2)
 k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsigned short *vcache, __nv_bfloat16 *out_b,
@@ -441,7 +451,7 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
     constexpr unsigned TOP = F16 ? 14 : 0;            // exponent of the largest element of a scaled query row, and of a weight of 1
     constexpr int STEP = F16 ? ATT_STEP : 1;
     constexpr float PSCALE = F16 ? 16384.f : 1.f;
-    extern __shared__ __align__(128) unsigned char asm_[];
+    extern __shared__ __align__(1024) unsigned char asm_[];   // (fragment addresses flip bits 4 .. 8)
     unsigned char *Qs = asm_;                          // [3][AQ][RB] parts of the scaled queries
     float *rs = (float *)(asm_ + (3 * AQ + 4 * AK) * RB);   // [AQ] what a row's scores are multiplied by
     const unsigned q_addr = s_u32(Qs), kv_addr = q_addr + 3 * AQ * RB;   // [2 buffers][keys | values][AK][RB]
@@ -468,28 +478,44 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
 
     // this warp's 16 query rows: scaled to [2^TOP, 2^(TOP + 1)) by a power of two, split, stored; nobody else reads them
     constexpr int EL = HD / 32;
-#pragma unroll 4
-    for (int rr = 0; rr < 16; ++rr) {
-        const int row = warp * 16 + rr;
-        float v[EL], amax = 0.f;
+#pragma unroll 1
+    for (int r8 = 0; r8 < 16; r8 += 8) {
+        float v[8][EL];
 #pragma unroll
-        for (int e = 0; e < EL; ++e) v[e] = r0 + row < M ? __ldcg(q + (size_t)(r0 + row) * ld_q + h * HD + lane * EL + e) : 0.f;
-#pragma unroll
-        for (int e = 0; e < EL; ++e) amax = fmaxf(amax, fabsf(v[e]));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        const unsigned ex = min(max(__float_as_uint(amax) >> 23, 1u + TOP), 253u);
-        const float inv = __uint_as_float((254u + TOP - ex) << 23);
-#pragma unroll
-        for (int e = 0; e < EL; e += 2) {
-            unsigned s3[3];
-            split3<F16, 1>(v[e] * inv, v[e + 1] * inv, s3);
-            const int byte = (lane * EL + e) * 2;
-#pragma unroll
-            for (int p = 0; p < 3; ++p)
-                *(unsigned *)(Qs + (size_t)(p * AQ + row) * RB + (((byte >> 4) ^ (row & 7)) << 4) + (byte & 15)) = s3[p];
+        for (int rr = 0; rr < 8; ++rr) {   // (eight rows' loads at once)
+            const float *src = q + (size_t)min(r0 + warp * 16 + r8 + rr, M - 1) * ld_q + h * HD + lane * EL;
+            if (EL == 4) {
+                const float4 x = __ldcg((const float4 *)src);
+                v[rr][0] = x.x; v[rr][1] = x.y; v[rr][2 % EL] = x.z; v[rr][3 % EL] = x.w;
+            } else {
+                const float2 x = __ldcg((const float2 *)src);
+                v[rr][0] = x.x; v[rr][1] = x.y;
+            }
         }
-        if (lane == 0) rs[row] = __uint_as_float((ex - TOP) << 23) * rsqrtf((float)HD);
+#pragma unroll
+        for (int rr = 0; rr < 8; ++rr) {
+            const int row = warp * 16 + r8 + rr;
+            float amax = 0.f;
+#pragma unroll
+            for (int e = 0; e < EL; ++e) {
+                if (r0 + row >= M) v[rr][e] = 0.f;
+                amax = fmaxf(amax, fabsf(v[rr][e]));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+            const unsigned ex = min(max(__float_as_uint(amax) >> 23, 1u + TOP), 253u);
+            const float inv = __uint_as_float((254u + TOP - ex) << 23);
+#pragma unroll
+            for (int e = 0; e < EL; e += 2) {
+                unsigned s3[3];
+                split3<F16, 1>(v[rr][e] * inv, v[rr][e + 1] * inv, s3);
+                const int byte = (lane * EL + e) * 2;
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+                    *(unsigned *)(Qs + (size_t)(p * AQ + row) * RB + (((byte >> 4) ^ (row & 7)) << 4) + (byte & 15)) = s3[p];
+            }
+            if (lane == 0) rs[row] = __uint_as_float((ex - TOP) << 23) * rsqrtf((float)HD);
+        }
     }
     __syncwarp();
 
@@ -497,6 +523,7 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
     const int mrow = lane & 7, mi = lane >> 3;         // ldmatrix: this lane's row and matrix
     const int row_a = r0 + warp * 16 + lr, pos_a = row_a < M ? ctx + row_a : -1, pos_b = row_a + 8 < M ? ctx + row_a + 8 : -1;
     const float rs_a = rs[warp * 16 + lr], rs_b = rs[warp * 16 + lr + 8];
+    const int pos_first = r0 + warp * 16 + 15 < M ? ctx + r0 + warp * 16 : -1;   // every row of the warp sees the keys up to here
     float o[HD / 8][4], m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
 #pragma unroll
     for (int n = 0; n < HD / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
@@ -511,26 +538,26 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
         __syncthreads();
         const int k0 = t * AK;
         const unsigned ka = kv_addr + (unsigned)(t & 1) * 2 * AK * RB, va = ka + AK * RB;
-        float s[AK / 8][4], u[AK / 8][4];   // products of the queries' first parts and of the two others
-#pragma unroll
-        for (int n = 0; n < AK / 8; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) s[n][e] = u[n][e] = 0.f;
+        float s[AK / 8][4], u[AK / 8][4], w[AK / 8][4];   // products of the queries' first parts (in two chains) and of the two others
+        const unsigned q_lane = q_addr + (warp * 16 + (mi & 1) * 8 + mrow) * RB + (((mi >> 1) ^ mrow) << 4);   // (piece ^ row & 7: ks only flips bits of it)
+        const unsigned k_lane = ka + ((mi >> 1) * 8 + mrow) * RB + (((mi & 1) ^ mrow) << 4);
 #pragma unroll
         for (int ks = 0; ks < HD / 16; ++ks) {
             unsigned qa[3][4];
-            const int qr = warp * 16 + (mi & 1) * 8 + mrow, qc = ks * 2 + (mi >> 1);
 #pragma unroll
-            for (int p = 0; p < 3; ++p) ldsm4(qa[p], q_addr + (p * AQ + qr) * RB + ((qc ^ (qr & 7)) << 4));
+            for (int p = 0; p < 3; ++p) ldsm4(qa[p], (q_lane ^ (ks << 5)) + p * AQ * RB);
 #pragma unroll
             for (int np = 0; np < AK / 16; ++np) {
                 unsigned kb[4];
-                const int kr = np * 16 + (mi >> 1) * 8 + mrow, kc = ks * 2 + (mi & 1);
-                ldsm4(kb, ka + kr * RB + ((kc ^ (kr & 7)) << 4));
+                ldsm4(kb, (k_lane ^ (ks << 5)) + np * 16 * RB);
 #pragma unroll
-                for (int p = 0; p < 3; ++p)
+                for (int p = 2; p >= 0; --p)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) mma16816<F16>(p == 1 ? s[2 * np + j] : u[2 * np + j], qa[p == 0 ? 2 : p == 1 ? 0 : 1], kb[2 * j], kb[2 * j + 1]);
+                    for (int j = 0; j < 2; ++j) {
+                        float(&acc)[4] = p != 0 ? u[2 * np + j] : ks < HD / 32 ? s[2 * np + j] : w[2 * np + j];
+                        if ((ks == 0 && p != 1) || (ks == HD / 32 && p == 0)) mma16816_zero<F16>(acc, qa[p], kb[2 * j], kb[2 * j + 1]);
+                        else mma16816<F16>(acc, qa[p], kb[2 * j], kb[2 * j + 1]);
+                    }
             }
         }
         float odd = 0.f;
@@ -538,7 +565,7 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
         for (int n = 0; n < AK / 8; ++n)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                s[n][e] = (s[n][e] + u[n][e]) * (e < 2 ? rs_a : rs_b);
+                s[n][e] = (s[n][e] + (w[n][e] + u[n][e])) * (e < 2 ? rs_a : rs_b);
                 odd = fmaf(s[n][e], 0.f, odd);   // (not zero once a score is infinite or no number; 3 % of the kernel)
             }
         if (__any_sync(0xffffffffu, odd != 0.f)) {
@@ -569,13 +596,18 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
                 for (int e = 0; e < 4; ++e) s[n][e] = s[n][e] > -INFINITY ? s[n][e] : -INFINITY;   // (no number: no weight)
         }
         float mx_a = m_a, mx_b = m_b;
+        if (k0 + AK - 1 > pos_first) {   // (uniform over the warp; a row past M is behind all keys)
+#pragma unroll
+            for (int n = 0; n < AK / 8; ++n) {
+                const int key = k0 + n * 8 + lc;
+                s[n][0] = key <= pos_a ? s[n][0] : -INFINITY;
+                s[n][1] = key + 1 <= pos_a ? s[n][1] : -INFINITY;
+                s[n][2] = key <= pos_b ? s[n][2] : -INFINITY;
+                s[n][3] = key + 1 <= pos_b ? s[n][3] : -INFINITY;
+            }
+        }
 #pragma unroll
         for (int n = 0; n < AK / 8; ++n) {
-            const int key = k0 + n * 8 + lc;
-            s[n][0] = key <= pos_a ? s[n][0] : -INFINITY;
-            s[n][1] = key + 1 <= pos_a ? s[n][1] : -INFINITY;
-            s[n][2] = key <= pos_b ? s[n][2] : -INFINITY;
-            s[n][3] = key + 1 <= pos_b ? s[n][3] : -INFINITY;
             mx_a = fmaxf(mx_a, fmaxf(s[n][0], s[n][1]));
             mx_b = fmaxf(mx_b, fmaxf(s[n][2], s[n][3]));
         }
@@ -586,14 +618,15 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
         }
         // (a row past M, or one whose scores are all -inf so far, keeps weights of 0)
         const float ba = mx_a > -INFINITY ? mx_a : 0.f, bb = mx_b > -INFINITY ? mx_b : 0.f;
-        const float ra = expf(m_a - ba), rb = expf(m_b - bb);   // (0 while the maximum is -inf)
+        const float ra = ex2((m_a - ba) * LOG2E), rb = ex2((m_b - bb) * LOG2E);   // (0 while the maximum is -inf)
+        const float la = -ba * LOG2E, lb = -bb * LOG2E;   // (rounded once for the whole row, which leaves the weights' ratios alone)
         m_a = mx_a;
         m_b = mx_b;
         float sa = 0.f, sb = 0.f;
 #pragma unroll
         for (int n = 0; n < AK / 8; ++n) {
-            s[n][0] = expf(s[n][0] - ba); s[n][1] = expf(s[n][1] - ba);
-            s[n][2] = expf(s[n][2] - bb); s[n][3] = expf(s[n][3] - bb);
+            s[n][0] = ex2(fmaf(s[n][0], LOG2E, la)); s[n][1] = ex2(fmaf(s[n][1], LOG2E, la));
+            s[n][2] = ex2(fmaf(s[n][2], LOG2E, lb)); s[n][3] = ex2(fmaf(s[n][3], LOG2E, lb));
             sa += s[n][0] + s[n][1];
             sb += s[n][2] + s[n][3];
         }
@@ -610,26 +643,28 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
                 pa[ks][0][e] = s3[0]; pa[ks][1][e] = s3[1]; pa[ks][2][e] = s3[2];
             }
         }
+        const unsigned v_lane = va + ((mi & 1) * 8 + mrow) * RB + (((mi >> 1) ^ mrow) << 4);
 #pragma unroll
         for (int np = 0; np < HD / 16; ++np) {
-            float c[3][2][4];   // this tile's sums, part by part
-#pragma unroll
-            for (int i = 0; i < 24; ++i) c[i / 8][i / 4 % 2][i % 4] = 0.f;
+            float c[3][2][4];   // this tile's sums, part by part (bf16: the two lower parts together, the lowest first)
+            constexpr int LOW = F16 ? 2 : 1;
 #pragma unroll
             for (int ks = 0; ks < AK / 16; ++ks) {
                 unsigned vb[4];
-                const int vr = ks * 16 + (mi & 1) * 8 + mrow, vc = np * 2 + (mi >> 1);
-                ldsm4_t(vb, va + vr * RB + ((vc ^ (vr & 7)) << 4));
+                ldsm4_t(vb, (v_lane ^ (np << 5)) + ks * 16 * RB);
 #pragma unroll
-                for (int p = 0; p < 3; ++p) {
-                    mma16816<F16>(c[p][0], pa[ks][p], vb[0], vb[1]);
-                    mma16816<F16>(c[p][1], pa[ks][p], vb[2], vb[3]);
-                }
+                for (int p = 2; p >= 0; --p)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        float(&acc)[4] = c[p == 2 ? LOW : p][j];
+                        if (ks == 0 && (F16 || p != 1)) mma16816_zero<F16>(acc, pa[ks][p], vb[2 * j], vb[2 * j + 1]);
+                        else mma16816<F16>(acc, pa[ks][p], vb[2 * j], vb[2 * j + 1]);
+                    }
             }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int j = i / 4, e = i % 4;
-                const float low = fmaf(c[2][j][e], 1.f / STEP, c[1][j][e]), t = fmaf(low, 1.f / STEP, c[0][j][e]);
+                const float low = F16 ? fmaf(c[2][j][e], 1.f / STEP, c[1][j][e]) : c[1][j][e], t = fmaf(low, 1.f / STEP, c[0][j][e]);
                 o[2 * np + j][e] = fmaf(o[2 * np + j][e], e < 2 ? ra : rb, t);
             }
         }
