@@ -233,7 +233,7 @@ int cl_read_hidden_ring(cl_ctx *ctx, void *out);
  * pool), or a latency-critical loop in which cudaMalloc's device-wide synchronisation is not acceptable.
  *
  * All working memory (normalised rows, per-block softmax partials, the completion ticket, the result
- * staging) lives in one fixed array compiled into the library: about 0.9 MB that every GPU which loads the
+ * staging) lives in one fixed array compiled into the library: about 17 MB that every GPU which loads the
  * library holds until the process exits.  Hence the fixed limits below; larger sizes return CL_ERANGE.
  *   lm_head    DEVICE [vocab, d_model] row-major, weight_dtype 0 = fp32 / 1 = bf16
  *   final_norm DEVICE float[d_model]

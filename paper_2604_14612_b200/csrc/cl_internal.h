@@ -304,12 +304,13 @@ cudaError_t cl_launch_rmsnorm_bf16(int in_dtype, const void *x, const float *g, 
 cudaError_t cl_launch_score_tc(const void *xn, const void *lm_head, int R, int V, int d, ClHeadPartial *partials, int n_sm,
                                int *err, float *conf, float *pmax, int *arg, int f16, cudaStream_t s);
 // LM head with fp32 activations over many rows (see kernels_headrows.cu)
+#define CL_HEAD_TC_PARTIALS (128 * 148 * 3)     // of k_head_tc: rows of a tile x CTAs x thirds of a tile's columns
 #define CL_HEAD_ROWS_PARTIALS (128 * 296)   // partial statistics: rows of a tile x CTAs of a full chip
 cudaError_t cl_launch_head_rows(int wdtype, const void *W, const void *x, const float *gain, int R, int V, int d, float eps, int n_sm,
                                 double *scale, ClHeadPartial *part, float *conf, float *pmax, int *arg, cudaStream_t s);
 long long cl_head_tc_cost(int V, int n_sm);   // of up to 128 rows, see cl_layer_confidences_static
-cudaError_t cl_launch_head_tc(const void *W, const void *x, const float *gain, int R, int V, int d, float eps, int n_sm, double *scale, ClHeadPartial *part,
-                              unsigned *tickets, unsigned *flags, float *conf, float *pmax, int *arg, cudaStream_t s);
+cudaError_t cl_launch_head_tc(const void *W, const void *x, const float *gain, int R, int V, int d, float eps, int n_sm, double *scale, void *split, size_t split_bytes,
+                              ClHeadPartial *part, unsigned *flags, float *conf, float *pmax, int *arg, cudaStream_t s);
 cudaError_t cl_launch_mean_rows(const float *conf_rows, int rows, int P, float *c_layer, cudaStream_t s);
 cudaError_t cl_launch_select(const cl_select_cfg &cfg, int n_layers, const float *c_layer, uint8_t *mask, double *margins,
                              cudaStream_t s);

@@ -13,6 +13,7 @@
 #include <string.h>
 
 #include <memory>
+#include <algorithm>
 #include <mutex>
 #include <new>
 
@@ -274,7 +275,7 @@ cudaError_t cl_launch_gemv(int wdtype, int T, int epi, const ClGemvArgs &a, int 
 // Scratch of cl_layer_confidences_static(): one file-scope array that every GPU loading this library holds until
 // the process exits.  Layout (bytes): [0, 256) ticket counters; then the normalised rows
 // xn [SC_CHUNK, CL_STATIC_MAX_D] fp32; the softmax partials of either path; the rows' normalisation factors
-// [CL_STATIC_MAX_ROWS] fp64; two flags and the three per-row results (confidence, top-1 probability, greedy token) [n_rows] each,
+// [CL_STATIC_MAX_ROWS] fp64; the rows in three bf16 parts for the tensor cores (15 MB: 512 rows of 5120 elements); two flags and the three per-row results (confidence, top-1 probability, greedy token) [n_rows] each,
 // side by side so that one copy fetches them.
 // Few rows take passes of the streaming GEMV, eight rows each, more take the kernels of kernels_headrows.cu.
 // fp32 heads, from 17 rows.  At 16 rows, two whole passes, it depends on how the tiles share the chip (16 rows, GEMV / tiled kernel, us: 32000 x 4096
@@ -282,19 +283,20 @@ cudaError_t cl_launch_gemv(int wdtype, int T, int epi, const ClGemvArgs &a, int 
 // bf16 heads: the tensor-core kernel costs much the same for 1 to 128 rows (32000 x 4096 with 100 rows 8 % more than with 6, 128256 x 4096 14 %) and waits for K
 // block after K block, so that it needs a vocabulary that is long against the width.  Whole call from idle, GEMV with that many rows / tensor-core kernel, us (under load
 // for some seconds both are up to 10 % faster and the lines hold within 2 %):
-//   V < d         from 14 rows  1000 x 4096 122 / 105 (9 rows 109 / 103), 1000 x 8192 158 / 155 (13: 157 / 164), 2000 x 8192 168 / 163 (12: 160 / 163), 200 x 4096 111 / 102
-//   d <= V < 3 d  from 9        4096 x 4096 111 / 108 (8: 91 / 108), 5003 x 4096 147 / 110 (8: 122 / 112, 7: 104 / 109), 8192 x 8192 221 / 168 (7: 144 / 167)
-//   V >= 3 d      from 8        9000 x 3000 115 / 93, 12288 x 4096 150 / 125, 40000 x 4096 275 / 253, 128256 x 4096 649 / 453; or from 7 or 6 (few_rows_line)
+//   V < d         from 12 rows  1000 x 4096 105 / 101 (10 rows 95 / 99), 2000 x 8192 155 / 150 (10: 142 / 150), 200 x 4096 105 / 101 (10: 93 / 100)
+//   d <= V < 3 d  from 9        4096 x 4096 104 / 101 (8: 88 / 100), 5003 x 4096 130 / 100 (8: 112 / 101, 7: 100 / 101), 8192 x 8192 205 / 152 (7: 138 / 151)
+//   V >= 3 d      from 8        12288 x 4096 150 / 113, 40000 x 4096 274 / 226, 128256 x 4096 647 / 401; or from 7, 6 or 5 (few_rows_line)
 namespace {
 
-// Most rows for the GEMV where V >= 3 d.  Six and seven rows are a matter of the tensor-core kernel's last wave of tiles: both times in us, from fits of
-// heads of 2304 x 768 to 151936 x 3584 (cost: of the fullest CTA, a K block).  Measured, GEMV / tensor cores:
-// 6 rows  28000 x 4096 163 / 153, 32000 x 4096 179 / 167, 64000 x 4096 287 / 253, 151936 x 3584 510 / 490, 32000 x 768 97 / 91, 3000 x 512 62 / 55,
-//         but 12288 x 4096 113 / 124, 40000 x 4096 210 / 251, 50257 x 2560 177 / 189, 100000 x 4096 410 / 441
-// 7 rows  20000 x 4096 164 / 151, 100000 x 4096 461 / 444, 3000 x 512 63 / 56, but 40000 x 4096 236 / 251
+// Most rows for the GEMV where V >= 3 d.  Five to seven rows are a matter of the tensor-core kernel's last wave of tiles: both times in us, from fits of
+// heads of 3000 x 512 to 128256 x 4096 (cost: of the fullest CTA, a K block).  Measured, GEMV / tensor cores:
+// 5 rows  32000 x 4096 177 / 140, 32000 x 5120 187 / 164, 32000 x 768 88 / 76, 3000 x 512 61 / 51, but 12288 x 4096 112 / 113, 40000 x 4096 202 / 226,
+//         50257 x 2560 163 / 166, 100000 x 4096 373 / 400
+// 6 rows  50257 x 2560 177 / 166, 100000 x 4096 403 / 400, 128256 x 4096 498 / 400, but 12288 x 4096 112 / 112, 40000 x 4096 205 / 226
+// 7 rows  12288 x 4096 125 / 114, 40000 x 4096 236 / 226
 int few_rows_line(int V, int d, int n_sm) {
-    const double tc = 53.0 + 8.5e-4 * (double)cl_head_tc_cost(V, n_sm) * ((d + 63) / 64), elems = (double)V * d;
-    return tc <= 70.0 + 8.2e-7 * elems ? 5 : tc <= 81.0 + 9.4e-7 * elems ? 6 : 7;
+    const double tc = 60.0 + 7e-4 * (double)cl_head_tc_cost(V, n_sm) * ((d + 63) / 64), elems = (double)V * d;
+    return tc <= 70.0 + 7.4e-7 * elems ? 4 : tc <= 70.0 + 8.2e-7 * elems ? 5 : tc <= 81.0 + 9.4e-7 * elems ? 6 : 7;
 }
 
 constexpr int SC_MAX_GRID = 1024;
@@ -302,9 +304,12 @@ constexpr int SC_CHUNK = 8;   // rows per LM-head pass of the GEMV
 constexpr int SC_GEMV_ROWS = 2 * SC_CHUNK;   // most rows that take such passes, whatever the head
 constexpr size_t SC_OFF_XN = 256;
 constexpr size_t SC_OFF_PART = SC_OFF_XN + (size_t)SC_CHUNK * CL_STATIC_MAX_D * sizeof(float);
-constexpr size_t SC_PARTIALS = SC_MAX_GRID * SC_CHUNK > CL_HEAD_ROWS_PARTIALS ? SC_MAX_GRID * SC_CHUNK : CL_HEAD_ROWS_PARTIALS;
+constexpr size_t SC_PARTIALS = std::max<size_t>(SC_MAX_GRID * SC_CHUNK, std::max(CL_HEAD_ROWS_PARTIALS, CL_HEAD_TC_PARTIALS));
 constexpr size_t SC_OFF_SCALE = SC_OFF_PART + SC_PARTIALS * sizeof(ClHeadPartial);
-constexpr size_t SC_OFF_RES = SC_OFF_SCALE + (size_t)CL_STATIC_MAX_ROWS * sizeof(double);
+constexpr size_t SC_OFF_SPLIT = SC_OFF_SCALE + (size_t)CL_STATIC_MAX_ROWS * sizeof(double);
+constexpr size_t SC_SPLIT = (size_t)512 * 5120 * 6;   // (128 rows of 8192 elements take 6.3 MB)
+constexpr size_t SC_OFF_RES = SC_OFF_SPLIT + SC_SPLIT;
+static_assert(SC_OFF_SPLIT % 256 == 0 && SC_SPLIT >= (size_t)128 * CL_STATIC_MAX_D * 6, "a row tile's parts");
 constexpr size_t SC_BYTES = SC_OFF_RES + (2 + 3 * (size_t)CL_STATIC_MAX_ROWS) * 4;
 
 static __device__ __align__(256) unsigned char g_static_scratch[SC_BYTES];
@@ -423,15 +428,12 @@ extern "C" int cl_layer_confidences_static(const void *lm_head, const float *fin
         const cudaError_t e = cudaMemcpyAsync(res, flags, (2 + 3 * (size_t)n_rows) * 4, cudaMemcpyDeviceToHost, s);
         return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
     };
-    // the tickets and flags must start at zero whatever the last call left
-    cudaError_t e = cudaMemsetAsync(sc, 0, SC_OFF_XN, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 8, s);
+    cudaError_t e = cudaSuccess;
     const bool tc = weight_dtype == 1;
-    const int gemv_rows = !tc ? SC_GEMV_ROWS : vocab < d_model ? 13 : vocab < 3LL * d_model ? 8 : few_rows_line(vocab, d_model, n_sm);   // most rows that take those passes
+    const int gemv_rows = !tc ? SC_GEMV_ROWS : vocab < d_model ? 11 : vocab < 3LL * d_model ? 8 : few_rows_line(vocab, d_model, n_sm);   // most rows that take those passes
     if (tc && n_rows > gemv_rows) {
-        if (e == cudaSuccess)
-            e = cl_launch_head_tc(lm_head, hidden, final_norm, n_rows, vocab, d_model, rms_eps, n_sm, (double *)(sc + SC_OFF_SCALE),
-                                  (ClHeadPartial *)(sc + SC_OFF_PART), (unsigned *)sc, flags, d_conf, d_pmax, d_arg, s);
+        e = cl_launch_head_tc(lm_head, hidden, final_norm, n_rows, vocab, d_model, rms_eps, n_sm, (double *)(sc + SC_OFF_SCALE), sc + SC_OFF_SPLIT, SC_SPLIT,
+                              (ClHeadPartial *)(sc + SC_OFF_PART), flags, d_conf, d_pmax, d_arg, s);
         if (e == cudaSuccess) e = fetch();
         if (e == cudaSuccess && res[0] && !res[1]) {   // not a call for that kernel: once more as before it (the tickets were used)
             e = cudaMemsetAsync(sc, 0, SC_OFF_XN, s);
@@ -439,6 +441,9 @@ extern "C" int cl_layer_confidences_static(const void *lm_head, const float *fin
             if (e == cudaSuccess) e = fetch();
         }
     } else {
+        // the tickets and flags must start at zero whatever the last call left
+        e = cudaMemsetAsync(sc, 0, SC_OFF_XN, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 8, s);
         if (e == cudaSuccess) e = n_rows > gemv_rows ? many_rows() : few_rows();
         if (e == cudaSuccess) e = fetch();
     }

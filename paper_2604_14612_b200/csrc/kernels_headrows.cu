@@ -14,6 +14,8 @@
 // The rows of a tile are a matter of balance: R rows are ceil(R / 128) tiles of equal size, rounded up to 16 rows.
 #include <math.h>
 
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace {
@@ -213,14 +215,26 @@ __global__ void __launch_bounds__(HT, 2) k_head_rows(HeadRowsArgs a) {
     for (int r = tid; r < nrows; r += HT) a.part[(size_t)(row0 + r) * a.NR + rg] = cl_hp_merge(run[r], run[16 * TM + r]);
 }
 
+__device__ __forceinline__ unsigned cvt_bf16x2(float a, float b) {   // a in the low half
+    unsigned r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    return r;
+}
+__device__ __forceinline__ void bf16x2_get(unsigned u, float &a, float &b) {
+    a = __uint_as_float(u << 16);
+    b = __uint_as_float(u & 0xffff0000u);
+}
+
 // scale[r] = 1 / sqrt(mean x^2 + eps), one CTA per row.  In 64 bits up to the result: its error moves all logits of a row
 // together, and fp32 sums, quotients and roots made it the largest part of a narrow row's error (see the head of this file).
 // With gain: more by what k_head_tc's sums of this row lose (see there).  A cut falls behind each of the four multiply-adds of a K block's highest part
 // that adds anything, at the size of the block's sum so far.  That size is taken from the row's squares, as if the token's weights leaned towards the row,
 // which those of a leading token do.  Eight lanes hold a K block, two of them the 16 elements of a multiply-add.
+// split: the row's three parts for k_head_tc go there, [3][rows][d]; flags [2]: to be cleared.
 template <typename T>
-__global__ void __launch_bounds__(256) k_row_scale(const T *x, const float *gain, int d, float eps, double *scale) {
+__global__ void __launch_bounds__(256) k_row_scale(const T *x, const float *gain, int d, float eps, double *scale, __nv_bfloat16 *split, unsigned *flags) {
     pdl_launch_dependents();
+    if (blockIdx.x == 0 && threadIdx.x < 2 && flags) flags[threadIdx.x] = 0u;
     __shared__ double red[8];
     __shared__ float cuts[8], all[8];
     double ss = 0.0;
@@ -237,6 +251,24 @@ __global__ void __launch_bounds__(256) k_row_scale(const T *x, const float *gain
             float g[8], sq = 0.f;
             g8.load(gain + i, i < d);
             g8.get(g);
+            if (split && i < d) {
+                unsigned h[4], m[4], l[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    float h0, h1, m0, m1;
+                    h[e] = cvt_bf16x2(v[2 * e] * g[2 * e], v[2 * e + 1] * g[2 * e + 1]);
+                    bf16x2_get(h[e], h0, h1);
+                    const float q0 = fmaf(v[2 * e], g[2 * e], -h0), q1 = fmaf(v[2 * e + 1], g[2 * e + 1], -h1);   // exact: 32 bits less the leading eight
+                    m[e] = cvt_bf16x2(q0, q1);
+                    bf16x2_get(m[e], m0, m1);
+                    l[e] = cvt_bf16x2(q0 - m0, q1 - m1);
+                }
+                __nv_bfloat16 *to = split + (size_t)blockIdx.x * d + i;
+                const size_t part = (size_t)gridDim.x * d;
+                *(uint4 *)to = make_uint4(h[0], h[1], h[2], h[3]);
+                *(uint4 *)(to + part) = make_uint4(m[0], m[1], m[2], m[3]);
+                *(uint4 *)(to + 2 * part) = make_uint4(l[0], l[1], l[2], l[3]);
+            }
 #pragma unroll
             for (int e = 0; e < 8; ++e) sq = fmaf(v[e] * g[e], v[e] * g[e], sq);
             sq += __shfl_xor_sync(0xffffffffu, sq, 1);   // a multiply-add's elements
@@ -315,37 +347,36 @@ __global__ void __launch_bounds__(128) k_head_rows_merge(const ClHeadPartial *pa
 // leading logits of 10 to 14, three inputs: width 768 0.87e-7 .. 0.91e-7 / 1.78e-7 .. 1.83e-7 (k_head_rows 1.5e-7 / 2.1e-7), width 4096
 // 0.78e-7 .. 0.84e-7 / 1.47e-7 .. 1.51e-7 (1.2e-7 / 1.7e-7).
 //
-// Bound: shared memory, then the hand-overs between the roles.  A K block of 128 rows x 224 weights is 12 multiply-adds that read
-// 11 KB each, 108 KB are written and read beside them: 1900 cycles at 128 bytes a cycle against 1344 of multiply-add; measured 2100,
-// and 2700 with the waits of the multiplying thread.  100 rows of the 32000 x 4096 head: 143 us (k_head_rows 987), the call 175
-// (1043); 32000 x 768 50 us; 128256 x 4096 the call 503 (3935), 400 rows 1745 (13500); 32000 x 4096, 4096 rows 3845 (29050).
-// 224 weights a tile: 32000 of them are one tile per SM (143), and the totals of a tile are 112 registers a thread.
-// 16 warps: 0 copies weights, 2 rows (TMA), 1 multiplies, 4-7 split the activations, 8-15 add up chains and keep the softmax
-// statistics.  The head is asked for in L2 eight K blocks ahead.
+// Bound: hand-overs between the multiplying thread and the chain warps, then shared memory.  A K block of 128 rows x 224 weights is 12 multiply-adds
+// that read 11 KB each, 76 KB are written beside them: 1630 cycles at 128 bytes a cycle against 1344 of multiply-add; measured 2450, and 2000 where the
+// chain warps only release (every CTA split the rows for itself before, 33 KB more in shared memory and a third of the issue slots: 2600).
+// The parts are written once by k_row_scale.  100 rows of the 32000 x 4096 head: 102 us (137), of them 8 before the first K block and 5 of statistics
+// (11, from two passes over the logits by eight warps); the rows' merge is a kernel of 5 us (13 on one SM by the last CTA).  The call 183 -> 146,
+// 32000 x 768 95 -> 82, 128256 x 4096 513 -> 434, 400 rows of it 1836 -> 1570; 32000 x 4096, 4096 rows 3980 -> 3750.
+// 224 weights a tile: 32000 of them are one tile per SM (143), and the totals of a tile are 80 registers a thread.
+// 16 warps: 0 copies weights, 2 the rows' parts (TMA), 1 multiplies, 4-15 add up chains and keep the softmax statistics, a third of a tile's columns by
+// four warps.  (The columns of a group are constants: with a bound at run time the loop over them took 2.7 us a K block instead of 1.3.)
+// The head is asked for in L2 eight K blocks ahead.
 // A logit that comes out as no finite number may have a sign all the same (an infinite weight times a part that is zero is NaN): the warp that
 // holds it works its token out again for all its rows, from the weights that are not finite (see special_logit): one infinite weight costs 8 to 11
 // us (6 rows of the 32000 x 4096 head 160 -> 168 us, of a second pass on other kernels 650), 300 tokens of infinities side by side 120.  Rows that are NaN throughout (a NaN or an infinity among the
 // activations, or a row of zeros with eps = 0) need nothing: every logit counts as the lower clamp, as in the other kernels.
 constexpr int HTC_THREADS = 512;
-constexpr int HTC_A = 3 * 128 * 128, HTC_X = 128 * 128,   // bytes of a K block's rows, split in three and as they are
-              HTC_AST = 2, HTC_BST = 3, HTC_XST = 2, HTC_AHEAD = 8;   // stages of the rings, K blocks asked for in L2
+constexpr int HTC_A = 3 * 128 * 128,                // bytes of a K block's rows, split in three
+              HTC_AST = 2, HTC_BST = 4, HTC_AHEAD = 8;   // stages of the rings (parts; K blocks of weights), K blocks asked for in L2
 
 struct HeadTcArgs {
-    const __nv_bfloat16 *x, *W;          // [R, d], [V, d]
+    const __nv_bfloat16 *x, *W, *split;  // [R, d], [V, d], [3][R, d]: x * gain in three parts
     const float *gain;
     const double *scale;                 // [R]
     int R, V, d, KB, MT, rows, NR, NT;   // rows, vocabulary, width, K blocks, row tiles and their rows, vocabulary ranges, vocabulary tiles
-    double inv_log_v;
-    ClHeadPartial *part;                 // [R, NR]
-    unsigned *tickets, *flags;           // [MT], zero at launch; [0] results are to be had from the other kernels, [1] a wait ran out
-    float *conf, *pmax;
-    int *arg;
+    ClHeadPartial *part;                 // [R, NR, groups of chain warps]
+    unsigned *flags;                     // zero at launch: [0] results are to be had from the other kernels, [1] a wait ran out
 };
 
 struct HeadTcSmem {
-    unsigned long long afull[HTC_AST], aempty[HTC_AST], bfull[HTC_BST], bempty[HTC_BST], xfull[HTC_XST], xempty[HTC_XST], tfull[2], tempty[2], done;
-    ClHeadPartial half[128];
-    unsigned tmem_base, last;
+    unsigned long long afull[HTC_AST], aempty[HTC_AST], bfull[HTC_BST], bempty[HTC_BST], tfull[2], tempty[2], done;
+    unsigned tmem_base;
     int abort;
 };
 
@@ -421,22 +452,11 @@ __device__ __noinline__ float special_logit(const __nv_bfloat16 *x, const __nv_b
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int c0, int c1) {
     asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(c0), "r"(c1) : "memory");
 }
-__device__ __forceinline__ unsigned cvt_bf16x2(float a, float b) {   // a in the low half
-    unsigned r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
-    return r;
-}
-__device__ __forceinline__ void bf16x2_get(unsigned u, float &a, float &b) {
-    a = __uint_as_float(u << 16);
-    b = __uint_as_float(u & 0xffff0000u);
-}
-
 template <int N>
 __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW, HeadTcArgs a) {
-    constexpr int B_BYTES = N * 128, NH = N / 2;
+    constexpr int B_BYTES = N * 128, NG = (N / 3 + 15) / 16 * 16, NG3 = N - 2 * NG, CHAIN_WARPS = NG3 > 0 ? 12 : 8;   // columns of a group of chain warps, of the third
     extern __shared__ unsigned char smem_dyn[];   // rings of swizzled tiles: 1 KB aligned
-    unsigned char *ringA = (unsigned char *)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023), *ringX = ringA + HTC_AST * HTC_A,
-                  *ringB = ringX + HTC_XST * HTC_X;
+    unsigned char *ringA = (unsigned char *)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023), *ringB = ringA + HTC_AST * HTC_A;
     HeadTcSmem *sm = (HeadTcSmem *)(ringB + HTC_BST * B_BYTES);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int mt = blockIdx.x % a.MT, rg = blockIdx.x / a.MT, KB = a.KB;
@@ -446,7 +466,7 @@ __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constan
 
     if (tid == 0) {
         for (int i = 0; i < HTC_AST; ++i) {
-            bar_init(&sm->afull[i], 4);
+            bar_init(&sm->afull[i], 1);
             bar_init(&sm->aempty[i], 1);
         }
         for (int i = 0; i < HTC_BST; ++i) {
@@ -455,11 +475,7 @@ __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constan
         }
         for (int i = 0; i < 2; ++i) {
             bar_init(&sm->tfull[i], 1);
-            bar_init(&sm->tempty[i], 8);
-        }
-        for (int i = 0; i < HTC_XST; ++i) {
-            bar_init(&sm->xfull[i], 1);
-            bar_init(&sm->xempty[i], 4);
+            bar_init(&sm->tempty[i], CHAIN_WARPS);
         }
         bar_init(&sm->done, 1);
         sm->abort = 0;
@@ -475,6 +491,149 @@ __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constan
     const unsigned tmem = *(volatile unsigned *)&sm->tmem_base;
     pdl_wait();   // the scales
 
+    // ---------------- chains: a thread has a third of a row of the tile, columns [grp * NG, + NC) ----------------
+    auto chains = [&](auto nc, int grp) {
+        constexpr int NC = decltype(nc)::value;
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
+        const int q = warp & 3, row = q * 32 + lane;
+        const unsigned tl = tmem + ((unsigned)(q * 32) << 16) + (unsigned)(grp * NG);
+        float s_hi = 0.f, s_lo = 0.f, scale = 0.f;
+        bool ok = true, odd = false, redo = false;   // redo: a logit of this row that is not finite may be worked out again
+        if (row < nrows) {
+            const double raw = a.scale[row0 + row];
+            const bool number = raw > 0.0 && raw < (double)INFINITY;   // else all logits of the row are NaN, here as in the other kernels
+            odd = number && !(raw > 0x1p-100 && raw < 0x1p90);         // (the lowest parts of such a row, or its sums, could leave the range of a float)
+            redo = number && !odd;
+            scale = (float)raw;
+            s_hi = scale;
+            s_lo = (float)(raw - (double)s_hi);
+        }
+        const float zero[16] = {};
+#pragma unroll 1
+        for (int c = 0; c < NC; c += 16) {
+            tmem_st16(tl + c, zero);
+            tmem_st16(tl + 256u + c, zero);
+        }
+        auto release = [&](unsigned b) {
+            if (lane == 0) bar_arrive(&sm->tempty[b]);
+        };
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        release(0);
+        release(1);
+        ClHeadPartial run{0.f, 0.f, 0.f, 0x7fffffff};   // (a tile's sums by themselves first: added to a leading weight one by one they would lose more)
+        unsigned g = 0;
+        for (int t = 0; t < ntiles && ok; ++t) {
+            float tot[NC];
+#pragma unroll
+            for (int i = 0; i < NC; ++i) tot[i] = 0.f;
+            for (int ch = 0; ch < KB; ++ch, ++g) {
+                const unsigned b = g & 1u, ta = tl + b * 256u, to = tl + (b ^ 1u) * 256u;
+                ok = __all_sync(0xffffffffu, bar_wait(&sm->tfull[b], (g >> 1) & 1u, &sm->abort, err));
+                if (!ok) break;
+                __syncwarp();
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (ch + 1 < KB) {
+#pragma unroll
+                    for (int c = 0; c < NC; c += 16) {
+                        float v[16];
+                        tmem_ld16(ta + c, v);
+#pragma unroll
+                        for (int i = 0; i < 16; i += 2) {   // sum, and what it rounded off (in full where the total is the larger one)
+                            const unsigned long long tt = pack2(tot[c + i], tot[c + i + 1]), uu = pack2(v[i], v[i + 1]), s = add2(tt, uu);
+                            unpack2(sub2(uu, sub2(s, tt)), v[i], v[i + 1]);
+                            unpack2(s, tot[c + i], tot[c + i + 1]);
+                        }
+                        tmem_st16(ta + c, v);
+                    }
+                } else {
+                    // the row's last chain: the logits, with what both accumulators still owe; both start the next tile from zero
+#pragma unroll
+                    for (int c = 0; c < NC; c += 16) {
+                        float u[16], o[16];
+                        tmem_ld16(ta + c, u);
+                        if (KB > 1) tmem_ld16(to + c, o);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const float s = tot[c + i] + u[i], r = (u[i] - (s - tot[c + i])) + (KB > 1 ? o[i] : 0.f);
+                            tot[c + i] = fmaf(s, s_hi, fmaf(s, s_lo, r * s_hi));
+                        }
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) u[i] = tot[c + i];
+                        tmem_st16(ta + c, u);
+                    }
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                if (ch + 1 == KB) {
+                    // softmax statistics of this third of the row, out of tensor memory again (in registers the logits unroll into
+                    // code that takes longer to fetch than to run); then both accumulators start the next tile from zero
+                    const int c0 = (nt0 + t) * N + grp * NG, nvalid = min(NC, a.V - c0);
+                    ClHeadPartial p;
+                    for (bool again = false;; again = true) {
+                        p = ClHeadPartial{-INFINITY, 0.f, 0.f, 0x7fffffff};
+                        bool bad = false;
+#pragma unroll 1
+                        for (int c = 0; c < nvalid; c += 16) {   // sums relative to the largest logit so far
+                            float l[16];
+                            tmem_ld16(ta + c, l);
+                            float big = -INFINITY;
+                            int at = 0;
+#pragma unroll
+                            for (int i = 0; i < 16; ++i)
+                            {   // (selections, not branches: a branch per logit costs ten times as much)
+                                const bool in = c + i < nvalid;
+                                bad |= in && !(fabsf(l[i]) < INFINITY);
+                                l[i] = in ? fminf(fmaxf(l[i], -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP) : -INFINITY;   // clamp of Section 3.1
+                                at = l[i] > big ? i : at;
+                                big = fmaxf(big, l[i]);
+                            }
+                            const float m = fmaxf(p.m, big), back = p.z > 0.f ? p.m - m : 0.f, f = expf(back);
+                            p.idx = big > p.m ? c0 + c + at : p.idx;
+                            p.m = m;
+                            float z = 0.f, s = 0.f;
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                const float d = c + i < nvalid ? l[i] - m : 0.f, e = c + i < nvalid ? expf(d) : 0.f;
+                                z += e;
+                                s = fmaf(d, e, s);
+                            }
+                            p.s = fmaf(f, fmaf(back, p.z, p.s), s);
+                            p.z = fmaf(f, p.z, z);
+                        }
+                        if (again || !__any_sync(0xffffffffu, bad && redo)) break;
+#pragma unroll 1
+                        for (int c = 0; c < nvalid; ++c) {
+                            const float l = tmem_ld1(ta + c);
+                            const bool want = redo && !(fabsf(l) < INFINITY);
+                            if (!__any_sync(0xffffffffu, want)) continue;
+                            bool any;
+                            const float v = special_logit(a.x + (size_t)(row0 + min(row, nrows - 1)) * a.d, a.W + (size_t)(c0 + c) * a.d, a.gain, scale, a.d, want, &any);
+                            odd |= want && !any;   // a sum that overflowed
+                            tmem_st1(ta + c, want && any ? v : l);
+                        }
+                        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    }
+                    if (nvalid > 0) run = cl_hp_merge(run, p);
+                    if (t + 1 < ntiles) {
+#pragma unroll 1
+                        for (int c = 0; c < NC; c += 16) {
+                            tmem_st16(ta + c, zero);
+                            if (KB > 1) tmem_st16(to + c, zero);
+                        }
+                        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (ch + 1 == KB && KB > 1) release(b ^ 1u);   // (held back so that it could be read once more)
+                if (ch + 2 != KB) release(b);
+            }
+        }
+        if (odd) a.flags[0] = 1u;
+        // (each group's statistics go out by themselves: k_head_tc_merge adds them up in 64 bits)
+        if (row < nrows) a.part[((size_t)(row0 + row) * a.NR + rg) * (CHAIN_WARPS / 4) + grp] = run;
+    };
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
         // ---------------- copies: warp 0 weights, warp 2 rows ----------------
@@ -490,7 +649,8 @@ __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constan
                     if (!ok) break;
                     bar_expect(full + st, bytes);
                     if (weights) tma_load_2d(ring + st * bytes, &mapW, kb * 64, (nt0 + t) * N, full + st);
-                    else tma_load_2d(ring + st * bytes, &mapX, kb * 64, row0, full + st);
+                    else
+                        for (int p = 0; p < 3; ++p) tma_load_2d(ring + st * bytes + p * 16384, &mapX, kb * 64, p * a.R + row0, full + st);
                     if (++st == (unsigned)stages) { st = 0; par ^= 1u; }
                 }
             // The CTA may not exit while a copy is in flight, and nobody else waits for it where another role gave up after the last one was
@@ -502,7 +662,7 @@ __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constan
         if (warp == 0) {
             if (lane == 0) copies(ringB, B_BYTES, HTC_BST, sm->bfull, sm->bempty, true);
         } else if (warp == 2) {
-            if (lane == 0) copies(ringX, HTC_X, HTC_XST, sm->xfull, sm->xempty, false);
+            if (lane == 0) copies(ringA, HTC_A, HTC_AST, sm->afull, sm->aempty, false);
         } else if (warp == 1 && lane == 0) {
             // ---------------- multiply-adds ----------------
             const unsigned idesc = umma_idesc(128, N);
@@ -535,264 +695,9 @@ __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constan
             while (!bar_try(&sm->done, 0u) && gtime_ns() - t0 < WAIT_NS) {}
         }
     } else if (warp < 8) {
-        // ---------------- activations: 8 lanes a row, 16 bytes a lane, 32 rows a warp ----------------
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 112;");
-        const int r0 = (warp - 4) * 32 + (lane >> 3), piece = lane & 7;
-        const bool rows_here = (warp - 4) * 32 < nrows;   // (a row of the product depends on its own row of activations only)
-        float4 g0, g1, n0, n1;
-        auto gains = [&](int kb) {
-            const int k = kb * 64 + piece * 8;
-            n0 = n1 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (k < a.d) {
-                n0 = *(const float4 *)(a.gain + k);
-                n1 = *(const float4 *)(a.gain + k + 4);
-            }
-        };
-        gains(0);
-        unsigned sa = 0, pa = 0, sx = 0, px = 0;
-        bool ok = true;
-        for (int t = 0; t < ntiles && ok; ++t)
-            for (int kb = 0; kb < KB; ++kb) {
-                g0 = n0;
-                g1 = n1;
-                gains(kb + 1 < KB ? kb + 1 : 0);
-                ok = __all_sync(0xffffffffu, bar_wait(&sm->xfull[sx], px, &sm->abort, err) && bar_wait(&sm->aempty[sa], pa ^ 1u, &sm->abort, err));
-                if (!ok) break;
-                if (rows_here) {
-                    const unsigned src = s_u32(ringX + sx * HTC_X), dst = s_u32(ringA + sa * HTC_A);
-                    const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-#pragma unroll
-                    for (int jb = 0; jb < 8; jb += 4) {
-                        unsigned w[4][4], off[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int r = r0 + 4 * (jb + j);
-                            off[j] = (unsigned)(r * 128 + ((piece ^ (r & 7)) << 4));
-                            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[j][0]), "=r"(w[j][1]), "=r"(w[j][2]), "=r"(w[j][3]) : "r"(src + off[j]) : "memory");
-                        }
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            unsigned h[4], m[4], l[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                float x0, x1, h0, h1, m0, m1;
-                                bf16x2_get(w[j][e], x0, x1);
-                                h[e] = cvt_bf16x2(x0 * gg[2 * e], x1 * gg[2 * e + 1]);
-                                bf16x2_get(h[e], h0, h1);
-                                const float q0 = fmaf(x0, gg[2 * e], -h0), q1 = fmaf(x1, gg[2 * e + 1], -h1);   // exact: 32 bits less the leading eight
-                                m[e] = cvt_bf16x2(q0, q1);
-                                bf16x2_get(m[e], m0, m1);
-                                l[e] = cvt_bf16x2(q0 - m0, q1 - m1);
-                            }
-                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + off[j]), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]));
-                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + off[j] + 16384u), "r"(m[0]), "r"(m[1]), "r"(m[2]), "r"(m[3]));
-                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + off[j] + 32768u), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]));
-                        }
-                    }
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    bar_arrive(&sm->xempty[sx]);
-                    bar_arrive(&sm->afull[sa]);
-                }
-                if (++sx == HTC_XST) { sx = 0; px ^= 1u; }
-                if (++sa == HTC_AST) { sa = 0; pa ^= 1u; }
-            }
+        if constexpr (NG3 > 0) chains(std::integral_constant<int, NG3>(), 2);
     } else {
-        // ---------------- chains: a thread has half a row of the tile ----------------
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
-        const int q = warp & 3, hf = (warp - 8) >> 2, row = q * 32 + lane;
-        const unsigned tl = tmem + ((unsigned)(q * 32) << 16) + (unsigned)(hf * NH);
-        float s_hi = 0.f, s_lo = 0.f, scale = 0.f;
-        bool ok = true, odd = false, redo = false;   // redo: a logit of this row that is not finite may be worked out again
-        if (row < nrows) {
-            const double raw = a.scale[row0 + row];
-            const bool number = raw > 0.0 && raw < (double)INFINITY;   // else all logits of the row are NaN, here as in the other kernels
-            odd = number && !(raw > 0x1p-100 && raw < 0x1p90);         // (the lowest parts of such a row, or its sums, could leave the range of a float)
-            redo = number && !odd;
-            scale = (float)raw;
-            s_hi = scale;
-            s_lo = (float)(raw - (double)s_hi);
-        }
-        const float zero[16] = {};
-#pragma unroll 1
-        for (int c = 0; c < NH; c += 16) {
-            tmem_st16(tl + c, zero);
-            tmem_st16(tl + 256u + c, zero);
-        }
-        auto release = [&](unsigned b) {
-            if (lane == 0) bar_arrive(&sm->tempty[b]);
-        };
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        release(0);
-        release(1);
-        ClHeadPartial run{0.f, 0.f, 0.f, 0x7fffffff};
-        unsigned g = 0;
-        for (int t = 0; t < ntiles && ok; ++t) {
-            float tot[NH];
-#pragma unroll
-            for (int i = 0; i < NH; ++i) tot[i] = 0.f;
-            for (int ch = 0; ch < KB; ++ch, ++g) {
-                const unsigned b = g & 1u, ta = tl + b * 256u, to = tl + (b ^ 1u) * 256u;
-                ok = __all_sync(0xffffffffu, bar_wait(&sm->tfull[b], (g >> 1) & 1u, &sm->abort, err));
-                if (!ok) break;
-                __syncwarp();
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (ch + 1 < KB) {
-                    float u[2][16];
-                    tmem_ld16_async(ta, u[0]);
-#pragma unroll
-                    for (int c = 0; c < NH; c += 16) {
-                        float(&v)[16] = u[(c >> 4) & 1];
-                        tmem_ld_wait(v);
-                        if (c + 16 < NH) tmem_ld16_async(ta + c + 16, u[((c >> 4) + 1) & 1]);
-#pragma unroll
-                        for (int i = 0; i < 16; i += 2) {   // sum, and what it rounded off (in full where the total is the larger one)
-                            const unsigned long long tt = pack2(tot[c + i], tot[c + i + 1]), uu = pack2(v[i], v[i + 1]), s = add2(tt, uu);
-                            unpack2(sub2(uu, sub2(s, tt)), v[i], v[i + 1]);
-                            unpack2(s, tot[c + i], tot[c + i + 1]);
-                        }
-                        tmem_st16(ta + c, v);
-                    }
-                } else {
-                    // the row's last chain: the logits, with what both accumulators still owe; both start the next tile from zero
-#pragma unroll
-                    for (int c = 0; c < NH; c += 16) {
-                        float u[16], o[16];
-                        tmem_ld16(ta + c, u);
-                        if (KB > 1) tmem_ld16(to + c, o);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const float s = tot[c + i] + u[i], r = (u[i] - (s - tot[c + i])) + (KB > 1 ? o[i] : 0.f);
-                            tot[c + i] = fmaf(s, s_hi, fmaf(s, s_lo, r * s_hi));
-                        }
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) u[i] = tot[c + i];
-                        tmem_st16(ta + c, u);
-                    }
-                }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                if (ch + 1 == KB) {
-                    // softmax statistics of this half row, out of tensor memory again (in registers the 112 logits unroll into
-                    // code that takes longer to fetch than to run); then both accumulators start the next tile from zero
-                    const int c0 = (nt0 + t) * N + hf * NH, nvalid = min(NH, a.V - c0);
-                    ClHeadPartial p;
-                    for (bool again = false;; again = true) {
-                        p = ClHeadPartial{-INFINITY, 0.f, 0.f, 0x7fffffff};
-                        bool bad = false;
-#pragma unroll 1
-                        for (int c = 0; c < nvalid; c += 16) {
-                            float l[16];
-                            tmem_ld16(ta + c, l);
-#pragma unroll
-                            for (int i = 0; i < 16; ++i)
-                            {   // (selections, not branches: a branch per logit costs ten times as much)
-                                const bool in = c + i < nvalid;
-                                bad |= in && !(fabsf(l[i]) < INFINITY);
-                                const float v = in ? fminf(fmaxf(l[i], -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP) : -INFINITY;   // clamp of Section 3.1
-                                p.idx = v > p.m ? c0 + c + i : p.idx;
-                                p.m = fmaxf(p.m, v);
-                            }
-                        }
-                        if (again || !__any_sync(0xffffffffu, bad && redo)) break;
-#pragma unroll 1
-                        for (int c = 0; c < nvalid; ++c) {
-                            const float l = tmem_ld1(ta + c);
-                            const bool want = redo && !(fabsf(l) < INFINITY);
-                            if (!__any_sync(0xffffffffu, want)) continue;
-                            bool any;
-                            const float v = special_logit(a.x + (size_t)(row0 + min(row, nrows - 1)) * a.d, a.W + (size_t)(c0 + c) * a.d, a.gain, scale, a.d, want, &any);
-                            odd |= want && !any;   // a sum that overflowed
-                            tmem_st1(ta + c, want && any ? v : l);
-                        }
-                        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    }
-#pragma unroll 1
-                    for (int c = 0; c < nvalid; c += 16) {
-                        float l[16], z = 0.f, s = 0.f;
-                        tmem_ld16(ta + c, l);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                        {
-                            const float d = fminf(fmaxf(l[i], -CL_LOGIT_CLAMP), CL_LOGIT_CLAMP) - p.m, e = c + i < nvalid ? expf(d) : 0.f;
-                            z += e;
-                            s = fmaf(d, e, s);
-                        }
-                        p.z += z;
-                        p.s += s;
-                    }
-                    if (nvalid > 0) run = cl_hp_merge(run, p);
-#pragma unroll 1
-                    for (int c = 0; c < NH; c += 16) {
-                        tmem_st16(ta + c, zero);
-                        if (KB > 1) tmem_st16(to + c, zero);
-                    }
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (ch + 1 == KB && KB > 1) release(b ^ 1u);   // (held back so that it could be read once more)
-                if (ch + 2 != KB) release(b);
-            }
-        }
-        if (odd) a.flags[0] = 1u;
-        if (hf) sm->half[row] = run;
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (!hf && row < nrows) a.part[(size_t)(row0 + row) * a.NR + rg] = cl_hp_merge(run, sm->half[row]);
-        // the last CTA of a row tile merges its ranges, in a fixed order, eight lanes a row
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (tid == 256) sm->last = ticket_acq_rel(a.tickets + mt) == (unsigned)a.NR - 1u;
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (sm->last) {
-            constexpr int PL = 20;   // ranges a lane: 8 * 20 cover the 148 SMs
-            for (int r0 = 0; r0 < nrows; r0 += 32) {
-                const int r = min(r0 + (warp - 8) * 4 + (lane >> 3), nrows - 1);
-                const float4 *pp = (const float4 *)(a.part + (size_t)(row0 + r) * a.NR);
-                float m = -INFINITY;
-                int idx = 0x7fffffff;
-                double z = 0.0, t = 0.0;
-                for (int g0 = lane & 7; g0 < a.NR; g0 += 8 * PL) {
-                    float4 f[PL];
-                    float mn = m;
-#pragma unroll
-                    for (int i = 0; i < PL; ++i) f[i] = g0 + 8 * i < a.NR ? __ldcg(pp + g0 + 8 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                    for (int i = 0; i < PL; ++i)
-                        if (f[i].y > 0.f && f[i].x > mn) { mn = f[i].x; idx = __float_as_int(f[i].w); }
-                    if (z > 0.0) {
-                        const double e = expf(m - mn);
-                        t = e * (t + (double)(m - mn) * z);
-                        z *= e;
-                    }
-                    m = mn;
-#pragma unroll
-                    for (int i = 0; i < PL; ++i) {
-                        const float dm = f[i].y > 0.f ? f[i].x - m : 0.f, e = f[i].y > 0.f ? expf(dm) : 0.f;
-                        z += (double)(e * f[i].y);
-                        t += (double)(e * fmaf(dm, f[i].y, f[i].z));
-                    }
-                }
-#pragma unroll
-                for (int o = 1; o < 8; o <<= 1) {
-                    const float om = __shfl_xor_sync(0xffffffffu, m, o), mm = fmaxf(m, om);
-                    const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-                    const double oz = __shfl_xor_sync(0xffffffffu, z, o), ot = __shfl_xor_sync(0xffffffffu, t, o);
-                    const double e = z > 0.0 ? expf(m - mm) : 0.f, oe = oz > 0.0 ? expf(om - mm) : 0.f;
-                    t = (z > 0.0 ? e * (t + (double)(m - mm) * z) : 0.0) + (oz > 0.0 ? oe * (ot + (double)(om - mm) * oz) : 0.0);
-                    z = e * z + oe * oz;
-                    idx = om > m || (om == m && oi < idx) ? oi : idx;
-                    m = mm;
-                }
-                if ((lane & 7) == 0) {   // (a row may be written more than once, with the same values)
-                    a.conf[row0 + r] = (float)(1.0 - (log(z) - t / z) * a.inv_log_v);   // H = log Z - S / Z (Eq. 2-4)
-                    a.pmax[row0 + r] = (float)(1.0 / z);
-                    a.arg[row0 + r] = idx;
-                }
-            }
-        }
+        chains(std::integral_constant<int, NG>(), (warp - 8) >> 2);
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -803,16 +708,68 @@ __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constan
     }
 }
 
+// Behind k_head_tc: one warp per row, the ranges' statistics in a fixed order and in 64 bits, then Eq. 2-4.  (By the last CTA of a row tile it
+// took 13 us at 100 rows, all of them on one SM.)
+__global__ void __launch_bounds__(128) k_head_tc_merge(const ClHeadPartial *part, int R, int NR, double inv_log_v, float *conf, float *pmax, int *arg) {
+    constexpr int PL = 7;   // partials a lane at a time: 64 * 7 cover three groups on 148 SMs
+    pdl_wait();
+    const int r = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (r >= R) return;
+    const float4 *pp = (const float4 *)(part + (size_t)r * NR);
+    float m = -INFINITY;
+    int idx = 0x7fffffff;
+    double z = 0.0, t = 0.0;
+    for (int g0 = lane; g0 < NR; g0 += 32 * PL) {
+        float4 f[PL];
+        float mn = m;
+#pragma unroll
+        for (int i = 0; i < PL; ++i) f[i] = g0 + 32 * i < NR ? __ldcg(pp + g0 + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < PL; ++i)
+            if (f[i].y > 0.f && f[i].x > mn) { mn = f[i].x; idx = __float_as_int(f[i].w); }
+        if (z > 0.0) {
+            const double e = expf(m - mn);
+            t = e * (t + (double)(m - mn) * z);
+            z *= e;
+        }
+        m = mn;
+#pragma unroll
+        for (int i = 0; i < PL; ++i) {
+            const float dm = f[i].y > 0.f ? f[i].x - m : 0.f, e = f[i].y > 0.f ? expf(dm) : 0.f;
+            z += (double)(e * f[i].y);
+            t += (double)(e * fmaf(dm, f[i].y, f[i].z));
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float om = __shfl_xor_sync(0xffffffffu, m, o), mm = fmaxf(m, om);
+        const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
+        const double oz = __shfl_xor_sync(0xffffffffu, z, o), ot = __shfl_xor_sync(0xffffffffu, t, o);
+        const double e = z > 0.0 ? expf(m - mm) : 0.f, oe = oz > 0.0 ? expf(om - mm) : 0.f;
+        t = (z > 0.0 ? e * (t + (double)(m - mm) * z) : 0.0) + (oz > 0.0 ? oe * (ot + (double)(om - mm) * oz) : 0.0);
+        z = e * z + oe * oz;
+        idx = om > m || (om == m && oi < idx) ? oi : idx;
+        m = mm;
+    }
+    if (lane == 0) {
+        conf[r] = (float)(1.0 - (log(z) - t / z) * inv_log_v);   // H = log Z - S / Z (Eq. 2-4)
+        pmax[r] = (float)(1.0 / z);
+        arg[r] = idx;
+    }
+}
+
 template <int N>
-cudaError_t launch_tc(HeadTcArgs a, const void *W, cudaStream_t s) {
+cudaError_t launch_tc(HeadTcArgs a, double inv_log_v, float *conf, float *pmax, int *arg, const void *W, cudaStream_t s) {
     CUtensorMap mapX, mapW;
-    if (!make_map(&mapX, a.x, a.R, a.d, 128) || !make_map(&mapW, W, a.V, a.d, N)) return cudaErrorInvalidValue;
+    if (!make_map(&mapX, a.split, 3 * a.R, a.d, 128) || !make_map(&mapW, W, a.V, a.d, N)) return cudaErrorInvalidValue;
     a.NT = (a.V + N - 1) / N;
     a.NR = a.NR < a.NT ? a.NR : a.NT;
-    const size_t smem = 1024 + HTC_AST * HTC_A + HTC_XST * HTC_X + HTC_BST * N * 128 + sizeof(HeadTcSmem);
+    const size_t smem = 1024 + HTC_AST * HTC_A + HTC_BST * N * 128 + sizeof(HeadTcSmem);
     cudaError_t e = cudaFuncSetAttribute(k_head_tc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(k_head_tc<N>, dim3(a.MT * a.NR), HTC_THREADS, smem, 1, s, mapX, mapW, a);
+    e = launch_chained(k_head_tc<N>, dim3(a.MT * a.NR), HTC_THREADS, smem, 1, s, mapX, mapW, a);
+    if (e != cudaSuccess) return e;
+    return launch_chained(k_head_tc_merge, dim3((a.R + 3) / 4), 128, 0, 1, s, (const ClHeadPartial *)a.part, a.R, a.NR * ((N / 3 + 15) / 16 * 32 < N ? 3 : 2), inv_log_v, conf, pmax, arg);
 }
 
 template <typename T, int TM>
@@ -878,8 +835,8 @@ cudaError_t cl_launch_head_rows(int wdtype, const void *W, const void *x, const 
     while (a.NR > 1 && (size_t)R * a.NR > CL_HEAD_ROWS_PARTIALS) --a.NR;
     if (a.NR > a.NT) a.NR = a.NT;
     if (a.NR < 1) a.NR = 1;
-    if (wdtype == 1) k_row_scale<<<R, 256, 0, s>>>((const __nv_bfloat16 *)x, nullptr, d, eps, scale);
-    else k_row_scale<<<R, 256, 0, s>>>((const float *)x, nullptr, d, eps, scale);
+    if (wdtype == 1) k_row_scale<<<R, 256, 0, s>>>((const __nv_bfloat16 *)x, nullptr, d, eps, scale, nullptr, nullptr);
+    else k_row_scale<<<R, 256, 0, s>>>((const float *)x, nullptr, d, eps, scale, nullptr, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = wdtype == 1 ? launch_tm<__nv_bfloat16>(a, s) : launch_tm<float>(a, s);
     if (e != cudaSuccess) return e;
@@ -887,27 +844,37 @@ cudaError_t cl_launch_head_rows(int wdtype, const void *W, const void *x, const 
     return cudaGetLastError();
 }
 
-// The same of bf16 rows and a bf16 head on the tensor cores.  scale: scratch [R].  tickets [32] and flags [2] are zero before it; flags[0] != 0
-// after it: a sum of finite products overflowed, or a row's scale is beyond 2^-100 .. 2^90: the results are to be had from the other kernels;
-// flags[1] != 0: a wait ran out.
-cudaError_t cl_launch_head_tc(const void *W, const void *x, const float *gain, int R, int V, int d, float eps, int n_sm, double *scale, ClHeadPartial *part,
-                              unsigned *tickets, unsigned *flags, float *conf, float *pmax, int *arg, cudaStream_t s) {
-    HeadTcArgs t;
-    t.x = (const __nv_bfloat16 *)x; t.W = (const __nv_bfloat16 *)W; t.gain = gain; t.R = R; t.V = V; t.d = d; t.KB = (d + 63) / 64;
-    t.scale = scale;
-    t.inv_log_v = 1.0 / log((double)V);
-    t.part = part; t.tickets = tickets; t.flags = flags; t.conf = conf; t.pmax = pmax; t.arg = arg;
-    row_tiles(R, t.MT, t.rows);
-    t.NR = n_sm / t.MT;
-    while (t.NR > 1 && (size_t)R * t.NR > CL_HEAD_ROWS_PARTIALS) --t.NR;
-    if (t.NR < 1) t.NR = 1;
-    k_row_scale<<<R, 256, 0, s>>>((const __nv_bfloat16 *)x, gain, d, eps, scale);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    long long cost;
-    switch (head_tc_tile(V, t.NR, cost)) {
-        case 224: return launch_tc<224>(t, W, s);
-        case 128: return launch_tc<128>(t, W, s);
-        default: return launch_tc<64>(t, W, s);
+// The same of bf16 rows and a bf16 head on the tensor cores.  scale: scratch [R]; split: scratch of split_bytes (128 rows of d elements in
+// three parts at least; calls of more rows than fit take several launches).  flags[0] != 0 after it: a sum of finite products overflowed, or
+// a row's scale is beyond 2^-100 .. 2^90: the results are to be had from the other kernels; flags[1] != 0: a wait ran out.  They are
+// cleared here.
+cudaError_t cl_launch_head_tc(const void *W, const void *x, const float *gain, int R, int V, int d, float eps, int n_sm, double *scale, void *split, size_t split_bytes,
+                              ClHeadPartial *part, unsigned *flags, float *conf, float *pmax, int *arg, cudaStream_t s) {
+    const double inv_log_v = 1.0 / log((double)V);
+    const int most = (int)(split_bytes / ((size_t)d * 6)) / 128 * 128;
+    if (most < 128) return cudaErrorInvalidValue;
+    const int chunks = (R + most - 1) / most, per = (R + chunks - 1) / chunks;
+    for (int r0 = 0; r0 < R; r0 += per) {
+        HeadTcArgs t;
+        t.R = R - r0 < per ? R - r0 : per;
+        t.x = (const __nv_bfloat16 *)x + (size_t)r0 * d; t.W = (const __nv_bfloat16 *)W; t.gain = gain; t.V = V; t.d = d; t.KB = (d + 63) / 64;
+        t.split = (__nv_bfloat16 *)split;
+        t.scale = scale;
+        t.part = part; t.flags = flags;
+        row_tiles(t.R, t.MT, t.rows);
+        t.NR = n_sm / t.MT;
+        while (t.NR > 1 && (size_t)t.R * t.NR * 3 > CL_HEAD_TC_PARTIALS) --t.NR;
+        if (t.NR < 1) t.NR = 1;
+        k_row_scale<<<t.R, 256, 0, s>>>(t.x, gain, d, eps, scale, (__nv_bfloat16 *)split, r0 ? nullptr : flags);   // (the flags are the whole call's)
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        long long cost;
+        switch (head_tc_tile(V, t.NR, cost)) {
+            case 224: e = launch_tc<224>(t, inv_log_v, conf + r0, pmax + r0, arg + r0, W, s); break;
+            case 128: e = launch_tc<128>(t, inv_log_v, conf + r0, pmax + r0, arg + r0, W, s); break;
+            default: e = launch_tc<64>(t, inv_log_v, conf + r0, pmax + r0, arg + r0, W, s);
+        }
+        if (e != cudaSuccess) return e;
     }
+    return cudaSuccess;
 }
