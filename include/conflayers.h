@@ -31,7 +31,7 @@
  *     second copy of every matrix in the order that kernel streams it (device memory for weights doubles).  The
  *     confidence scoring of 16-bit models runs on the tensor cores too; fp32 models and the remaining cases use
  *     per-matrix CUDA-core kernels.
- *     A prompt of more than 8 tokens (bf16 / fp16 models) runs through wide tensor-core GEMMs, up to 512 rows at a time;
+ *     A prompt of more than 16 tokens (bf16 / fp16 models) runs through wide tensor-core GEMMs, up to 512 rows at a time;
  *     the LM head then reads its last row only.
  *     Environment switches read by cl_load (diagnostics): CL_DISABLE_STEP_KERNEL=1, CL_DISABLE_ROWS_KERNEL=1,
  *     CL_DISABLE_WIDE_PREFILL=1, CL_DISABLE_ROW_SHARES=1, CL_L2_AHEAD_KB=<n>, CL_ROWS_SPLIT=<1|2|4>, CL_ROWS_CHAIN=<k-blocks

@@ -797,9 +797,7 @@ extern "C" int cl_prefill(cl_ctx *c, const int32_t *tokens, int n, int tap_hidde
     p.ctx = 0; p.n_drafted = 0; p.done = 0;
     if ((rc = poke(c, p))) return rc;
     int c0 = 0;
-    if (c->use_wide && n > CL_PREFILL_CHUNK) {
-        // More than one 8-row pass would stream the weights more than once: 8 rows take 486 us that way and 624 in a wide pass, 9 rows
-        // 876 and 628 (4 layers of width 4096; 6 of width 768 307 / 319 and 547 / 325).
+    if (c->use_wide && n > 2 * CL_PREFILL_CHUNK) {
         // Every prompt row goes through the wide GEMMs, in passes of equal size (a last pass of a row or two would stream all
         // weights for them); then only the last row needs the LM head, whose weights are all that is read again.
         const int n_pass = (n + CL_WIDE_MAX_M - 1) / CL_WIDE_MAX_M;
