@@ -2,7 +2,7 @@
 // vanilla full-model step and the verify pass of a cycle without drafts at batch 1, one cooperative launch for up to CL_MAX_K (draft) or many
 // (vanilla) consecutive tokens.
 //
-// One CTA per SM.  The last warp (one elected thread) is the weight producer: it walks the static schedule
+// One CTA per SM.  The 17th warp (one elected thread) is the weight producer: it walks the static schedule
 // (steps x kept layers x {QKV, O, gate/up, down} + LM head), and for this CTA's contiguous block of
 // rows of each matrix issues bulk asynchronous copies (cp.async.bulk, completion on an mbarrier) into
 // a ring of six 32 KB shared-memory slots (whole rows per slot).  It never waits for activations, so the HBM stream runs ahead
@@ -21,6 +21,12 @@ namespace {
 
 constexpr int NCW = 16;                // consumer warps
 constexpr int NCT = NCW * 32;          // consumer threads
+// Registers: 17 warps leave 96 a thread (five warps on one scheduler), and consumers spilled 200 to 300 bytes into the heads of latency-bound
+// phases.  Launched with 20 warps the producer's group of four gives some back: 512 x 104 + 128 x 64 = 640 x 96, no spills in the consumers.
+// (112 / 32: the producer spills, and a slow producer is a slow stream.  With both cursors of the L2 prefetch alive it spilled at 64 already,
+// and four full steps of 8 layers of width 4096 took 2995 us, 2884 before; as now 2854, 6 steps of 4 layers of width 5120 3590 -> 3396, 12 layers
+// of width 768 991 -> 971.)
+constexpr int NTHREADS = NCT + 128, CONSUMER_REGS = 104, PRODUCER_REGS = 64;
 constexpr int SLOT_BYTES = 32768;      // ring slot: as many whole weight rows as fit (at least one)
 constexpr int NSLOT = 6;               // 192 KB in flight per SM
 constexpr int MAXIT = 4;               // 16-byte chunks per thread per row: rows up to 32 KB (C <= 16384 bf16)
@@ -314,20 +320,20 @@ struct SchedIter {
 // The producer thread.  Two cursors over the same schedule: the fill cursor feeds the shared-memory ring as slots
 // come free; the prefetch cursor only asks L2 to fetch, and only moves while the ring is full (the consumers sit in a
 // grid barrier or the attention phase), up to l2_ahead bytes in front of the fill cursor, so that HBM keeps streaming
-// into L2 during those gaps and the ring is refilled from L2 afterwards.
-template <typename WT>
-__device__ void producer_loop(const ClStepArgs &a, unsigned char *ring, Smem *sm, ClDevState *st) {
+// into L2 during those gaps and the ring is refilled from L2 afterwards.  AHEAD: l2_ahead is not zero.
+template <typename WT, bool AHEAD>
+__device__ __forceinline__ void producer_loop(const ClStepArgs &a, unsigned char *ring, Smem *sm, ClDevState *st) {
     Ring rg{0u, 0u};
     unsigned last_par[NSLOT];
     for (int i = 0; i < NSLOT; ++i) last_par[i] = 2u;
     const unsigned long long policy = policy_evict_first();
-    SchedIter<WT> fill(a), pf(a);
+    SchedIter<WT> fill(a), pf(a);   // (without AHEAD nothing is left of pf)
     unsigned long long filled = 0, fetched = 0;
     const unsigned long long ahead = (unsigned long long)a.l2_ahead;
     const char *src;
     unsigned bytes;
     while (fill.next(src, bytes)) {
-        if (ahead) {
+        if (AHEAD) {
             const char *psrc;
             unsigned pbytes;
             while (fetched < filled + bytes && pf.next(psrc, pbytes)) fetched += pbytes;   // never behind the fill cursor
@@ -922,7 +928,7 @@ __device__ __forceinline__ void load_att_merged(const ClStepArgs &a, float (&xr)
 // ---- the kernel ----------------------------------------------------------------------------------------
 // SHORT: the rows of d_model and of d_ffn elements are short
 template <typename WT, int HD, bool SHORT>
-__global__ void __launch_bounds__(NCT + 32, 1) k_token_steps(ClStepArgs a) {
+__global__ void __launch_bounds__(NTHREADS, 1) k_token_steps(ClStepArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *ring = smem_raw;
     Smem *sm = (Smem *)(smem_raw + (size_t)NSLOT * SLOT_BYTES);
@@ -948,9 +954,14 @@ __global__ void __launch_bounds__(NCT + 32, 1) k_token_steps(ClStepArgs a) {
 
     if (tid >= NCT) {
         // ------------------------------ producer warp ------------------------------
-        if (tid == NCT) producer_loop<WT>(a, ring, sm, st);
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PRODUCER_REGS));
+        if (tid == NCT) {
+            if (a.l2_ahead) producer_loop<WT, true>(a, ring, sm, st);
+            else producer_loop<WT, false>(a, ring, sm, st);
+        }
         return;
     }
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CONSUMER_REGS));
 
     // ------------------------------ consumer warps ------------------------------
     Ring rg{0u, 0u};
@@ -1094,5 +1105,5 @@ cudaError_t cl_launch_token_steps(int wdtype, int head_dim, const ClStepArgs &a,
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void *params[] = {(void *)&a};
-    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(NCT + 32), params, smem, s);
+    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(NTHREADS), params, smem, s);
 }
