@@ -611,13 +611,11 @@ static int forward_rows(cl_ctx *c, const int *tok, int T, int row0, const uint8_
         if (skip_bits == 3) continue;
         const ClLayer &y = c->layers[l];
         if (!(skip_bits & 1)) {
-        // attention half: RMSNorm -> QKV -> rotary + cache append -> attention over the cache -> output projection + residual
+        // attention half: RMSNorm -> QKV -> attention over the cache (rotary, cache append) -> output projection + residual
         if (!fused) KL(cl_launch_rmsnorm(c->x, y.n1, T, d, g.rms_eps, c->xn, c->st, c->stream));
         if ((rc = gemv(c, T, CL_EPI_STORE, y.wqkv, qkv_rows, d, fused ? c->x : c->xn, c->qkv, qkv_rows, fused ? y.n1 : nullptr))) return rc;
-        KL(cl_launch_rope_append(wd, c->qkv, T, row0, g.n_heads, g.n_kv_heads, g.head_dim, d, c->rope_cs, y.kc, y.vc, g.max_seq, c->st,
-                                 c->stream));
         ClAttnArgs a;
-        a.q = c->qkv; a.ld_q = qkv_rows; a.n_kv_heads = g.n_kv_heads; a.kcache = y.kc; a.vcache = y.vc; a.part = c->att_part; a.tickets = c->tickets + 1;
+        a.q = c->qkv; a.ld_q = qkv_rows; a.rope_cs = c->rope_cs; a.n_kv_heads = g.n_kv_heads; a.kcache = y.kc; a.vcache = y.vc; a.part = c->att_part; a.tickets = c->tickets + 1;
         a.out = c->att; a.st = c->st; a.row0 = row0; a.n_heads = g.n_heads; a.head_dim = g.head_dim; a.d_model = d;
         a.nsplit = c->nsplit; a.per_max = c->per_max; a.max_seq = g.max_seq;
         KL(cl_launch_attn(wd, T, a, c->stream));

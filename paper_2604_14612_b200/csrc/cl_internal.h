@@ -115,10 +115,11 @@ struct ClGemvArgs {
 };
 
 struct ClAttnArgs {
-    const float *q;       // [T, ld_q] rotary-embedded queries (fp32)
+    const float *q;       // [T, ld_q] raw QKV product (fp32): [H query heads | Hkv key heads | Hkv value heads]
     int ld_q;
-    const void *kcache;   // this layer's K rows [n_heads, max_seq, head_dim] storage type
-    const void *vcache;
+    const float2 *rope_cs;   // [max_seq, head_dim / 2]
+    void *kcache;         // this layer's K rows [Hkv, max_seq, head_dim] storage type; the pass's own are appended
+    void *vcache;
     float *part;          // [T, H, nsplit, hd + 2] partial (m, l, o[hd])
     unsigned *tickets;    // [T, H]
     float *out;           // [T, d]
@@ -177,8 +178,6 @@ cudaError_t cl_launch_rmsnorm(const float *x, const float *g, int T, int d, floa
                               cudaStream_t s);
 cudaError_t cl_launch_rmsnorm_rows(int in_dtype, const void *x, const float *g, int T, int d, float eps, float *out,
                                    cudaStream_t s);
-cudaError_t cl_launch_rope_append(int wdtype, float *qkv, int T, int row0, int H, int Hkv, int hd, int d, const float2 *rope_cs,
-                                  void *kcache, void *vcache, int max_seq, const ClDevState *st, cudaStream_t s);
 cudaError_t cl_launch_attn(int wdtype, int T, const ClAttnArgs &a, cudaStream_t s);
 cudaError_t cl_launch_tap(int wdtype, const float *x, int T, int row0, int d, void *ring_layer, int P,
                           const ClDevState *st, cudaStream_t s);

@@ -89,41 +89,22 @@ __global__ void __launch_bounds__(1024) k_rmsnorm(const ST *x, const float *g, i
 }
 static int norm_threads(int d) { return d / 4 >= 1024 ? 1024 : (d / 4 + 31) / 32 * 32; }
 
-// ---- rotary embedding of q and k (pairs (i, i + hd/2)), append k, v to the cache -----------
-// qkv: [T, d + 2 kvd] fp32 = [q (H heads) | k (Hkv heads) | v (Hkv heads)]; q is rotated in place; k (rotated) and
-// v go to the cache rows of positions ctx + row0 + t, rounded to the storage type.  grid (T, H): block h rotates
-// query head h and, if h < Hkv, appends key/value head h.
-template <typename ST>
-__global__ void k_rope_append(float *qkv, int row0, int hd, int d, int Hkv, const float2 *rope_cs, ST *kcache, ST *vcache,
-                              int max_seq, const ClDevState *st) {
-    pdl_launch_dependents();
-    pdl_wait();
-    if (st->done) return;
-    const int t = blockIdx.x, h = blockIdx.y, i = threadIdx.x, half = hd >> 1;
-    const int pos = st->ctx + row0 + t;
-    if (pos >= max_seq) return;
-    const int kvd = Hkv * hd;
-    float *row = qkv + (size_t)t * (d + 2 * kvd);
-    float *q = row + h * hd;
-    const float2 cs = rope_cs[(size_t)pos * half + i];
-    const float qa = q[i], qb = q[i + half];
-    q[i] = qa * cs.x - qb * cs.y;
-    q[i + half] = qb * cs.x + qa * cs.y;
-    if (h >= Hkv) return;
-    const float *k = row + d + h * hd, *v = row + d + kvd + h * hd;
-    const float ka = k[i], kb = k[i + half];
-    ST *kc = kcache + ((size_t)h * max_seq + pos) * hd;   // cache layout [head][position][hd]: a head's rows are contiguous
-    ST *vc = vcache + ((size_t)h * max_seq + pos) * hd;
-    kc[i] = from_f32<ST>(ka * cs.x - kb * cs.y);
-    kc[i + half] = from_f32<ST>(kb * cs.x + ka * cs.y);
-    vc[i] = from_f32<ST>(v[i]);
-    vc[i + half] = from_f32<ST>(v[i + half]);
-}
-
 // ---- decode attention over the KV cache -----------------------------------------------------
 // grid (H, T, nsplit); block 128.  Row t attends to cache positions 0 .. ctx + row0 + t; the range
 // is cut into nsplit slices; each block produces (max, sum, unnormalised output) of its slice and
 // the last block of a (t, h) to finish merges the slices in order.
+// The queries and the pass's own keys and values (positions base = ctx + row0 ..) come raw from the QKV product [q | k | v]: every block
+// rotates what it needs, rounding keys and values as the cache does, and never reads the cache there; slice 0 of row t appends its row.
+// (A launch of its own for that was 4 of the 26 of a pass over a 4-layer fp32 model, 4 us each.)
+template <typename ST, int HD>
+__device__ __forceinline__ float rotated(const float *row, const float2 *cs, int idx) {   // element idx of a head's row
+    constexpr int HALF = HD / 2;
+    const int i = idx < HALF ? idx : idx - HALF;
+    const float a = row[i], b = row[i + HALF];
+    const float2 c = cs[i];
+    return idx < HALF ? a * c.x - b * c.y : b * c.x + a * c.y;
+}
+
 template <typename ST, int HD>
 __global__ void __launch_bounds__(128) k_attn(ClAttnArgs a) {
     pdl_launch_dependents();
@@ -143,11 +124,20 @@ __global__ void __launch_bounds__(128) k_attn(ClAttnArgs a) {
     const int n = j1 - j0;
     const int d = a.d_model;
     const int kvh = h / (a.n_heads / a.n_kv_heads);   // grouped-query attention: the key/value head of this query head
-    const ST *K = (const ST *)a.kcache + (size_t)kvh * a.max_seq * HD;
-    const ST *V = (const ST *)a.vcache + (size_t)kvh * a.max_seq * HD;
+    ST *K = (ST *)a.kcache + (size_t)kvh * a.max_seq * HD;
+    ST *V = (ST *)a.vcache + (size_t)kvh * a.max_seq * HD;
+    const int base = a.st->ctx + a.row0;                                        // position of row 0
+    const float *k0 = a.q + a.n_heads * HD + kvh * HD, *v0 = k0 + a.n_kv_heads * HD;   // raw key and value of row 0
+    auto turns = [&](int pos) { return a.rope_cs + (size_t)pos * (HD / 2); };
     const float scale = rsqrtf((float)HD);
 
-    for (int i = tid; i < HD; i += blockDim.x) sq[i] = a.q[(size_t)t * a.ld_q + h * HD + i];
+    for (int i = tid; i < HD; i += blockDim.x) sq[i] = rotated<ST, HD>(a.q + (size_t)t * a.ld_q + h * HD, turns(base + t), i);
+    if (sp == 0 && h % (a.n_heads / a.n_kv_heads) == 0) {
+        for (int i = tid; i < HD; i += blockDim.x) {
+            K[(size_t)(base + t) * HD + i] = from_f32<ST>(rotated<ST, HD>(k0 + (size_t)t * a.ld_q, turns(base + t), i));
+            V[(size_t)(base + t) * HD + i] = from_f32<ST>(v0[(size_t)t * a.ld_q + i]);
+        }
+    }
     __syncthreads();
 
     // scores: LPK lanes per key, 16 bytes of the key row per lane
@@ -162,7 +152,11 @@ __global__ void __launch_bounds__(128) k_attn(ClAttnArgs a) {
     for (int jb = warp * KPW; jb < n; jb += 4 * KPW) {
         const int j = jb + sub;
         float s = 0.f;
-        if (j < n) {
+        if (j < n && j0 + j >= base) {
+            const float *kr = k0 + (size_t)(j0 + j - base) * a.ld_q;
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) s = fmaf(qr[e], to_f32<ST>(from_f32<ST>(rotated<ST, HD>(kr, turns(j0 + j), li * EPL + e))), s);
+        } else if (j < n) {
             const uint4 raw = *(const uint4 *)(K + (size_t)(j0 + j) * HD + li * EPL);
             if (sizeof(ST) == 2) {
                 const unsigned u[4] = {raw.x, raw.y, raw.z, raw.w};
@@ -206,7 +200,10 @@ __global__ void __launch_bounds__(128) k_attn(ClAttnArgs a) {
     constexpr int NS = 128 / HD;   // 2 for HD 64, 1 for HD 128
     const int e = tid % HD, stripe = tid / HD;
     float acc = 0.f;
-    for (int j = stripe; j < n; j += NS) acc = fmaf(sc[j], to_f32<ST>(V[(size_t)(j0 + j) * HD + e]), acc);
+    for (int j = stripe; j < n; j += NS) {
+        const int own = j0 + j - base;
+        acc = fmaf(sc[j], to_f32<ST>(own < 0 ? V[(size_t)(j0 + j) * HD + e] : from_f32<ST>(v0[(size_t)own * a.ld_q + e])), acc);
+    }
     if (NS > 1) {
         red[tid] = acc;
         __syncthreads();
@@ -462,13 +459,6 @@ cudaError_t cl_launch_rmsnorm(const float *x, const float *g, int T, int d, floa
 cudaError_t cl_launch_rmsnorm_rows(int in_dtype, const void *x, const float *g, int T, int d, float eps, float *out,
                                    cudaStream_t s) {
     CL_DISPATCH_ST(in_dtype, return launch_chained(k_rmsnorm<ST>, dim3(T), norm_threads(d), 0, 1, s, (const ST *)x, g, d, eps, out, (const ClDevState *)nullptr));
-}
-
-cudaError_t cl_launch_rope_append(int wdtype, float *qkv, int T, int row0, int H, int Hkv, int hd, int d, const float2 *rope_cs,
-                                  void *kcache, void *vcache, int max_seq, const ClDevState *st, cudaStream_t s) {
-    dim3 grid(T, H);
-    CL_DISPATCH_ST(wdtype, return launch_chained(k_rope_append<ST>, grid, hd / 2, 0, 1, s, qkv, row0, hd, d, Hkv, rope_cs, (ST *)kcache,
-                                                 (ST *)vcache, max_seq, st));
 }
 
 cudaError_t cl_launch_attn(int wdtype, int T, const ClAttnArgs &a, cudaStream_t s) {
