@@ -508,8 +508,7 @@ extern "C" int cl_load(cl_ctx *c, const cl_weights *w) {
                 c->rows_chain = (ch && ch[0]) ? atoi(ch) : 8;
                 if (c->rows_chain < 1) c->rows_chain = 1;
                 const char *en = getenv("CL_ROWS_ENTRY_KB");   // tuning knob
-                c->rows_entry = ((en && en[0]) ? atoi(en) : 68) * 1024;   // (a third of the ring)
-                if (c->rows_entry < 1024) c->rows_entry = 1024;
+                c->rows_entry = (en && en[0]) ? std::max(atoi(en), 1) * 1024 : 0;   // (0: a third of the ring)
                 if (c->rows_entry > 96 * 1024) c->rows_entry = 96 * 1024;   // (two entries must fit the ring of 192 KB)
                 c->use_rows = 1;
             }
@@ -584,7 +583,9 @@ static int forward_rows_persistent(cl_ctx *c, const int *tok, int T, int row0, i
     if (a.att_parts < 1) a.att_parts = 1;
     if (a.att_parts > 8) a.att_parts = 8;
     a.tap = tap && c->ring; a.tap_P = g.tap_positions;
-    a.entry = c->rows_entry; a.chain = c->rows_chain; a.split = c->rows_split; a.ws = c->r_ws;
+    // which of the two builds: by the position as the host last saw it (a batch of cycles may move on; either is right anywhere)
+    const bool walk = c->h_ctx + row0 <= CL_ROWS_WALK_KEYS * a.att_parts;
+    a.entry = c->rows_entry ? c->rows_entry : (walk ? 70 : 68) * 1024; a.chain = c->rows_chain; a.split = c->rows_split; a.ws = c->r_ws;
     a.eps = g.rms_eps; a.inv_d = 1.0f / (float)g.d_model; a.inv_log_v = (float)(1.0 / log((double)g.vocab));
     a.rope_cs = c->rope_cs; a.st = c->st; a.tok = tok;
     a.x = c->x; a.qkv = c->qkv; a.Ax = c->r_ax; a.Aatt = c->r_aatt; a.Ah = c->r_ah;
@@ -593,7 +594,7 @@ static int forward_rows_persistent(cl_ctx *c, const int *tok, int T, int row0, i
     a.sync = c->r_bar; a.bar_arrivals = (unsigned)(c->n_sm + c->bar_extra); a.wait_ns = c->wait_ns; a.phase_ns = c->r_phase_ns;
     a.c_ssq = c->r_c_ssq; a.c_ax = c->r_c_ax; a.c_ah = c->r_c_ah; a.c_att = c->r_c_att; a.c_qkv = c->r_c_qkv;
     CU(cudaMemsetAsync(c->r_bar, 0, (size_t)c->r_sync_words * 4, c->stream));   // every counter starts at zero
-    KL(cl_launch_rows_pass(g.weight_dtype, g.head_dim, a, c->n_sm, c->stream));
+    KL((walk ? cl_launch_rows_pass_walk : cl_launch_rows_pass)(g.weight_dtype, g.head_dim, a, c->n_sm, c->stream));
     return CL_OK;
 }
 
@@ -794,6 +795,7 @@ extern "C" int cl_prefill(cl_ctx *c, const int32_t *tokens, int n, int tap_hidde
     ClPoke p = poke_none();
     p.ctx = 0; p.n_drafted = 0; p.done = 0;
     if ((rc = poke(c, p))) return rc;
+    c->h_ctx = 0;
     int c0 = 0;
     if (c->use_wide && n > 2 * CL_PREFILL_CHUNK) {
         // Every prompt row goes through the wide GEMMs, in passes of equal size (a last pass of a row or two would stream all
@@ -820,6 +822,7 @@ extern "C" int cl_prefill(cl_ctx *c, const int32_t *tokens, int n, int tap_hidde
                           ST_FIELD(c, float, v_pmax), ST_FIELD(c, float, v_conf), nullptr);
         if (rc) return rc;
         KL(cl_launch_advance(c->st, T, last ? T - 1 : -1, c->stream));
+        c->h_ctx += T;
     }
     if ((rc = sync_state(c))) return rc;
     if ((rc = check_device_err(c, "cl_prefill"))) {

@@ -4,7 +4,7 @@
 //
 // The pass is bound by HBM weight streaming (at most 9 flop per weight byte), so its shape follows the single-token
 // step kernel: one CTA per SM, every CTA owns a contiguous block of rows of every matrix (single-row granularity, so
-// all SMs stream the same number of bytes), one producer warp walks the static schedule and keeps a 204 KB ring of
+// all SMs stream the same number of bytes), one producer warp walks the static schedule and keeps a 205 KB ring of
 // weight tiles filled straight through the phase boundaries, and the phases of a layer (QKV | attention | O |
 // gate/up | down) follow one another inside the launch, ordered by completion counters per buffer (below), not by
 // launches.  What differs is the arithmetic: 2 T activation
@@ -47,16 +47,26 @@ namespace {
 constexpr int RW = 14;                 // worker warps (16 warps in all: four per scheduler, 128 registers per thread)
 constexpr int RT = RW * 32;            // worker threads
 constexpr int R_THREADS = RT + 64;     // + producer warp + MMA warp
-constexpr int R_RING = 208896;         // ring of tiles in flight per SM, allocated by the byte (multiples of 1 KB): 204 KB,
-                                       // with the control block and the alignment slack all the shared memory a CTA can have
+// Two builds of this file: as it stands for passes after many cached keys, with CL_ROWS_WALK (kernels_rows_walk.cu) for passes after few, whose
+// attention needs 5 KB less.  A pass is bound by the bytes in flight: those 5 KB are 1 to 2 % of it.
+#ifdef CL_ROWS_WALK
+constexpr int R_RING = 215040;         // ring of tiles in flight per SM, allocated by the byte (multiples of 1 KB): with the control block and
+constexpr int R_CTRL_BYTES = 16384;    // the alignment slack all the shared memory a CTA can have; control block behind the ring (at least 16 KB)
+#else
+constexpr int R_RING = 209920;
+constexpr int R_CTRL_BYTES = 21504;
+#endif
 constexpr int R_NE = 16;               // most ring entries (bulk-copy groups with their own pair of mbarriers) in flight
 constexpr int R_MAXN = 224;            // most rows of a weight tile (an accumulator buffer has 256 columns)
-constexpr int R_CTRL_BYTES = 22528;    // control block behind the ring (at least 16 KB: see the kernel)
 constexpr int R_ATT_MAXS = 8;          // most parts the cached keys of a head are cut into
 
 constexpr int R_STAGE_LD = R_MAXN + 1;  // row pitch of the epilogue staging buffer (odd: token rows fall into different banks)
 constexpr int R_SC_LD = RW * 16 + 8;    // attention: row pitch of the weights (8 off a multiple of 32: pairs of eight rows in one access)
+#ifdef CL_ROWS_WALK
+constexpr int R_STAGE_FLOATS = 2032;
+#else
 constexpr int R_STAGE_FLOATS = CL_MAX_T * R_SC_LD;   // staging buffer: a GEMM tile's raw products of every token row; the weights
+#endif
 
 struct RSmem {
     unsigned long long full[R_NE], empty[R_NE], tfull[2], tempty[2];
@@ -66,16 +76,18 @@ struct RSmem {
     int abort;
     int is_last;
     float scale[CL_SLOTS];             // RMSNorm scale of every token row for the current phase
+#ifndef CL_ROWS_WALK
     float qscale[CL_MAX_T], lpart[RW][CL_MAX_T];   // attention: what a row's scores are multiplied by; sums of weights by warp
     unsigned amax[CL_MAX_T];           // ... a row's largest score so far
     int vodd;                          // ... an own value of the pass is not finite
-    float esum[16][CL_SLOTS];          // embedding phase: per-chunk sums of squares
-    ClHeadPartial hpw[RW];             // LM head: per-warp statistics
+#endif
     float wsum[RW];                    // residual phase: per-warp sums of squares
     // one buffer, used in turn by: the GEMM epilogues (raw products of a tile, [T][R_STAGE_LD]); the residual epilogue
     // ([T][64] squares); the attention phase (weights [T][R_SC_LD], then, over the query parts too, the sums [3][T][hd])
     alignas(16) float stage[R_STAGE_FLOATS];
+#ifndef CL_ROWS_WALK
     alignas(16) unsigned short qp[3 * CL_MAX_T * 128];   // attention: the rotated queries in three parts (directly behind stage)
+#endif
     alignas(16) unsigned short knew[CL_MAX_T * 128];   // attention: the pass's own keys (rotated) and values in the storage type
     alignas(16) unsigned short vnew[CL_MAX_T * 128];
     unsigned long long t_prev, ph_ns[8];   // diagnostics: time of thread 0 by phase
@@ -626,11 +638,12 @@ __device__ void head_finish(const ClRowsArgs &a, RSmem *sm, ClHeadPartial run) {
         const ClHeadPartial other = cl_hp_shfl_xor(run, o);
         run = ((lane & o) == 0) ? rp_merge(run, other) : rp_merge(other, run);
     }
-    if (lane == 0) sm->hpw[warp] = run;
+    ClHeadPartial *hpw = (ClHeadPartial *)sm->stage;   // per-warp statistics (the last tile's products have been read)
+    if (lane == 0) hpw[warp] = run;
     worker_sync();
     if (tid < a.T) {
-        ClHeadPartial r = sm->hpw[tid * wpt];
-        for (int w = 1; w < wpt; ++w) r = rp_merge(r, sm->hpw[tid * wpt + w]);
+        ClHeadPartial r = hpw[tid * wpt];
+        for (int w = 1; w < wpt; ++w) r = rp_merge(r, hpw[tid * wpt + w]);
         a.head_part[(size_t)blockIdx.x * CL_SLOTS + tid] = r;
     }
 }
@@ -731,7 +744,8 @@ __device__ void embed_phase(const ClRowsArgs &a, RSmem *sm) {
     const int T = a.T, nch = a.d >> 3, tid = threadIdx.x;
     const float *g = a.L ? a.layers[0].n1 : a.final_norm;
     const int per = (nch + gridDim.x - 1) / gridDim.x;   // chunks of 8 columns per CTA (at most 16)
-    for (int idx = tid; idx < 16 * CL_SLOTS; idx += RT) sm->esum[idx / CL_SLOTS][idx % CL_SLOTS] = 0.f;
+    float *esum = sm->stage;                             // [16][CL_SLOTS] per-chunk sums of squares
+    for (int idx = tid; idx < 16 * CL_SLOTS; idx += RT) esum[idx] = 0.f;
     worker_sync();
     for (int idx = tid; idx < per * T; idx += RT) {
         const int i = idx / T, t = idx % T, ch = (int)blockIdx.x + i * (int)gridDim.x;
@@ -751,14 +765,14 @@ __device__ void embed_phase(const ClRowsArgs &a, RSmem *sm) {
                 ss = fmaf(v[e], v[e], ss);
                 a_store_split(a.Ax, t, T, ch * 8 + e, v[e] * g[ch * 8 + e], a.f16);
             }
-            sm->esum[i][t] = ss;
+            esum[i * CL_SLOTS + t] = ss;
         }
     }
     proxy_fence_global();   // the operand rows written above are read by other CTAs' bulk copies
     worker_sync();
     if (tid < T) {
         float ss = 0.f;
-        for (int i = 0; i < per; ++i) ss += sm->esum[i][tid];
+        for (int i = 0; i < per; ++i) ss += esum[i * CL_SLOTS + tid];
         a.ssq[(size_t)blockIdx.x * CL_SLOTS + tid] = ss;
     }
     worker_sync();
@@ -809,6 +823,264 @@ __device__ __forceinline__ unsigned ord_enc(float f) {
 }
 __device__ __forceinline__ float ord_dec(unsigned u) { return __uint_as_float((u & 0x80000000u) ? (u ^ 0x80000000u) : ~u); }
 
+// A CTA's records of head h are written (whole: the head's output): the last CTA of the head to come merges its parts in order.
+template <int HD>
+__device__ __forceinline__ void finish_head(const ClRowsArgs &a, int h, int S, bool whole, RSmem *sm) {
+    constexpr int HALF = HD / 2, WSTRIDE = HD + 2;
+    const int tid = threadIdx.x, T = a.T;
+    if (!whole) {
+        worker_sync();
+        if (tid == 0) {
+            const unsigned prev = ticket_acq_rel(a.att_tickets + h);
+            const int last = prev == (unsigned)S - 1;
+            if (last) a.att_tickets[h] = 0u;
+            sm->is_last = last;
+        }
+        worker_sync();
+        if (sm->is_last) {
+            const float *p0 = a.att_part + (size_t)h * R_ATT_MAXS * CL_MAX_T * WSTRIDE;
+            for (int i = tid; i < T * HALF; i += RT) {
+                const int tt = i / HALF, e = i % HALF * 2;
+                float2 ml[R_ATT_MAXS], po[R_ATT_MAXS];
+#pragma unroll
+                for (int b = 0; b < R_ATT_MAXS; b += 4) {
+#pragma unroll
+                    for (int s2 = b; s2 < b + 4; ++s2) {
+                        ml[s2] = po[s2] = make_float2(0.f, 0.f);
+                        if (b < S) {   // uniform
+                            const float *ps = p0 + ((size_t)min(s2, S - 1) * CL_MAX_T + tt) * WSTRIDE;
+                            ml[s2] = __ldcg((const float2 *)ps);
+                            po[s2] = __ldcg((const float2 *)(ps + 2 + e));
+                            if (s2 >= S) ml[s2].y = 0.f;
+                        }
+                    }
+                }
+                float M = -INFINITY;
+#pragma unroll
+                for (int s2 = 0; s2 < R_ATT_MAXS; ++s2)
+                    if (ml[s2].y > 0.f) M = fmaxf(M, ml[s2].x);
+                float Ls = 0.f, O0 = 0.f, O1 = 0.f;
+#pragma unroll
+                for (int s2 = 0; s2 < R_ATT_MAXS; ++s2) {   // part order
+                    if (ml[s2].y > 0.f) {
+                        const float f = expf(ml[s2].x - M);
+                        Ls = fmaf(ml[s2].y, f, Ls);
+                        O0 = fmaf(po[s2].x, f, O0);
+                        O1 = fmaf(po[s2].y, f, O1);
+                    }
+                }
+                a_store_split2(a.Aatt, tt, T, h * HD + e, O0 / Ls, O1 / Ls, a.f16);
+            }
+        }
+    }
+    // the CTA that wrote the head's operand rows says so (its stores are read by other CTAs' bulk copies)
+    const bool wrote = whole || sm->is_last;
+    if (wrote) proxy_fence_global();
+    worker_sync();
+    if (wrote && tid == 0) counter_add(a.sync + a.c_att + h, 1u);
+}
+
+#ifdef CL_ROWS_WALK
+// Few keys: a warp walks the keys of one token row (w / nsub; nsub = 14 / T warps a row share them), 16 at a time with an online softmax on
+// the CUDA cores, a trip to memory each.  With up to CL_ROWS_WALK_KEYS keys a part that is faster than the other form's fixed cost and smaller
+// ring.  us per verify, here / there: 8 layers of width 4096, 9 rows after 100 (25 keys a part) 925 / 953, 3 rows after 54 785 / 799, but 7 rows after
+// 170 (43) 858 / 835, 5 rows after 220 (55) 833 / 820; 12 of width 768, 5 rows after 200 (25) 527 / 542.
+template <typename ST, int HD>
+__device__ void attention_walk(const ClRowsArgs &a, const ClRowsLayer &y, int layer, int base, RSmem *sm) {
+    constexpr int EPL = 8, LPK = HD / EPL, KPW = 32 / LPK, VPL = HD / 32, WSTRIDE = HD + 2, HALF = HD / 2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int T = a.T, S = a.att_parts, nsub = RW / T;
+    const int t = warp / nsub, sub = warp % nsub;
+    const bool active = warp < T * nsub;
+    const int li = lane % LPK, ksub = lane / LPK;
+    const float scale = rsqrtf((float)HD);
+    const int group = a.H / a.Hkv, kvd = a.Hkv * HD, ld = a.d + 2 * kvd;
+    ST *Kc = (ST *)y.kc, *Vc = (ST *)y.vc;
+    float *wrec = sm->stage;
+    for (int item = blockIdx.x; item < a.H * S; item += gridDim.x) {
+        const int h = item % a.H, s = item / a.H, kvh = h / group;
+        // this head's q rows and its key/value head's k and v rows of the QKV product: complete? (three counters, one
+        // lane each)
+        if (warp == 0) {
+            if (lane < 3) {
+                const int b = lane == 0 ? h : (lane == 1 ? a.H + kvh : a.H + a.Hkv + kvh);
+                counter_wait(a.sync + a.c_qkv + b, (unsigned)(HD * (layer + 1)), sm, &a.st->err);
+            }
+            __syncwarp();
+        }
+        phase_clock(a, sm, 7);
+        worker_sync();
+        if (s == S - 1) {
+            // the pass's own keys and values, raw in the QKV product: rotate the keys, round both to the storage type, keep
+            // them for the warps below (one query head per key/value head also appends them to the cache); one thread per
+            // (row, pair of elements i, i + hd / 2), so the whole set costs one memory round trip
+            const bool writer = (h % group) == 0;
+            for (int idx = tid; idx < T * HALF; idx += RT) {
+                const int jn = idx / HALF, i = idx % HALF;
+                const float *kraw = a.qkv + (size_t)jn * ld + a.d + kvh * HD, *vraw = kraw + kvd;
+                const float2 cs = a.rope_cs[(size_t)(base + jn) * HALF + i];
+                const float ka = __ldcg(kraw + i), kb = __ldcg(kraw + i + HALF);
+                const float va = __ldcg(vraw + i), vb = __ldcg(vraw + i + HALF);
+                const unsigned short kk0 = f32_to_b16(ka * cs.x - kb * cs.y, a.f16), kk1 = f32_to_b16(kb * cs.x + ka * cs.y, a.f16);
+                const unsigned short v0 = f32_to_b16(va, a.f16), v1 = f32_to_b16(vb, a.f16);
+                sm->knew[jn * HD + i] = kk0; sm->knew[jn * HD + i + HALF] = kk1;
+                sm->vnew[jn * HD + i] = v0; sm->vnew[jn * HD + i + HALF] = v1;
+                if (writer) {
+                    unsigned short *ck = (unsigned short *)Kc + ((size_t)kvh * a.max_seq + base + jn) * HD;
+                    unsigned short *cv = (unsigned short *)Vc + ((size_t)kvh * a.max_seq + base + jn) * HD;
+                    ck[i] = kk0; ck[i + HALF] = kk1; cv[i] = v0; cv[i + HALF] = v1;
+                }
+            }
+            worker_sync();
+        }
+        float m_run = -INFINITY, l_run = 0.f, o_run[VPL];
+#pragma unroll
+        for (int e = 0; e < VPL; ++e) o_run[e] = 0.f;
+        if (active) {
+            const int pos = base + t;
+            const float *qraw = a.qkv + (size_t)t * ld + h * HD;
+            float qr[EPL];
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) {
+                const int idx = li * EPL + e;
+                const int i = idx < HALF ? idx : idx - HALF;
+                const float2 cs = a.rope_cs[(size_t)pos * HALF + i];
+                const float qa = __ldcg(qraw + i), qb = __ldcg(qraw + i + HALF);
+                qr[e] = idx < HALF ? qa * cs.x - qb * cs.y : qb * cs.x + qa * cs.y;
+            }
+            const int k0 = (int)((long long)base * s / S), k1 = (int)((long long)base * (s + 1) / S);
+            const int kw0 = k0 + (int)((long long)(k1 - k0) * sub / nsub), kw1 = k0 + (int)((long long)(k1 - k0) * (sub + 1) / nsub);
+            const ST *Kh = Kc + (size_t)kvh * a.max_seq * HD, *Vh = Vc + (size_t)kvh * a.max_seq * HD;
+            // CH keys per iteration: the key rows and the value rows of the iteration are requested together (the values do
+            // not depend on the scores), so an iteration costs one memory round trip; lane j < CH keeps key j's score
+            constexpr int CH = 16, NPASS = CH / KPW;
+            for (int j0 = kw0; j0 < kw1; j0 += CH) {
+                const int n = min(CH, kw1 - j0);
+                uint4 raw[NPASS];
+#pragma unroll
+                for (int p = 0; p < NPASS; ++p) {
+                    const int j = p * KPW + ksub;
+                    raw[p] = make_uint4(0u, 0u, 0u, 0u);
+                    if (j < n) raw[p] = __ldg((const uint4 *)(Kh + (size_t)(j0 + j) * HD + li * EPL));
+                }
+                uint2 vraw[CH];   // the value rows stay in their storage type until they are used
+#pragma unroll
+                for (int j = 0; j < CH; ++j) {
+                    const ST *vp = Vh + (size_t)(j0 + min(j, n - 1)) * HD + lane * VPL;
+                    if (VPL == 4) vraw[j] = __ldg((const uint2 *)vp);
+                    else vraw[j] = make_uint2(__ldg((const unsigned *)vp), 0u);
+                }
+                float my_score = -INFINITY;
+#pragma unroll
+                for (int p = 0; p < NPASS; ++p) {
+                    const int jb = p * KPW;
+                    if (jb < n) {   // uniform
+                        const unsigned u[4] = {raw[p].x, raw[p].y, raw[p].z, raw[p].w};
+                        float sc = 0.f;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            float ka, kb;
+                            ClPair16<ST>::get(u[e], ka, kb);
+                            sc = fmaf(qr[2 * e], ka, sc);
+                            sc = fmaf(qr[2 * e + 1], kb, sc);
+                        }
+#pragma unroll
+                        for (int o = LPK >> 1; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
+                        sc *= scale;
+#pragma unroll
+                        for (int k = 0; k < KPW; ++k) {
+                            const float v = __shfl_sync(0xffffffffu, sc, k * LPK);
+                            if (lane == jb + k && jb + k < n) my_score = v;
+                        }
+                    }
+                }
+                float m_new = my_score;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
+                m_new = fmaxf(m_new, m_run);
+                const float p = (lane < n) ? expf(my_score - m_new) : 0.f;
+                const float resc = (l_run > 0.f) ? expf(m_run - m_new) : 0.f;
+                float ps = p;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
+                l_run = fmaf(l_run, resc, ps);
+#pragma unroll
+                for (int e = 0; e < VPL; ++e) o_run[e] *= resc;
+                m_run = m_new;
+#pragma unroll
+                for (int j = 0; j < CH; ++j) {
+                    const float pj = __shfl_sync(0xffffffffu, p, j);   // (0 for j >= n: the repeated last row adds nothing)
+                    float v[4];
+                    ClPair16<ST>::get(vraw[j].x, v[0], v[1]);
+                    ClPair16<ST>::get(vraw[j].y, v[2], v[3]);
+#pragma unroll
+                    for (int e = 0; e < VPL; ++e) o_run[e] = fmaf(pj, v[e], o_run[e]);
+                }
+            }
+            if (s == S - 1 && sub == nsub - 1) {
+                // the pass's own positions base .. base + t
+                for (int jn = 0; jn <= t; ++jn) {
+                    float kf[EPL], vn[VPL];
+                    const uint4 raw = *(const uint4 *)(sm->knew + jn * HD + li * EPL);
+                    const unsigned u[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) pair16_to_f32(u[e], a.f16, kf[2 * e], kf[2 * e + 1]);
+#pragma unroll
+                    for (int e = 0; e < VPL; ++e) vn[e] = b16_to_f32(sm->vnew[jn * HD + lane * VPL + e], a.f16);
+                    float sc = 0.f;
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) sc = fmaf(qr[e], kf[e], sc);
+#pragma unroll
+                    for (int o = LPK >> 1; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
+                    sc = __shfl_sync(0xffffffffu, sc, 0) * scale;
+                    const float m_new = fmaxf(m_run, sc);
+                    const float resc = (l_run > 0.f) ? expf(m_run - m_new) : 0.f;
+                    const float pn = expf(sc - m_new);
+                    l_run = fmaf(l_run, resc, pn);
+#pragma unroll
+                    for (int e = 0; e < VPL; ++e) o_run[e] = fmaf(o_run[e], resc, pn * vn[e]);
+                    m_run = m_new;
+                }
+            }
+        }
+        if (lane == 0) {
+            wrec[warp * WSTRIDE] = m_run;
+            wrec[warp * WSTRIDE + 1] = l_run;
+        }
+#pragma unroll
+        for (int e = 0; e < VPL; ++e) wrec[warp * WSTRIDE + 2 + lane * VPL + e] = o_run[e];
+        worker_sync();
+        // merge the nsub warps of every row (fixed order); one record per (h, s, t), or the final output if S == 1
+        float *part = a.att_part + ((size_t)h * R_ATT_MAXS + s) * CL_MAX_T * WSTRIDE;
+        for (int i = tid; i < T * HD; i += RT) {
+            const int tt = i / HD, e = i % HD;
+            float M = -INFINITY;
+            for (int w = 0; w < nsub; ++w) {
+                const float *r = wrec + (tt * nsub + w) * WSTRIDE;
+                if (r[1] > 0.f) M = fmaxf(M, r[0]);
+            }
+            float Ls = 0.f, O = 0.f;
+            for (int w = 0; w < nsub; ++w) {
+                const float *r = wrec + (tt * nsub + w) * WSTRIDE;
+                if (r[1] > 0.f) {
+                    const float f = expf(r[0] - M);
+                    Ls = fmaf(r[1], f, Ls);
+                    O = fmaf(r[2 + e], f, O);
+                }
+            }
+            if (S == 1) {
+                a_store_split(a.Aatt, tt, T, h * HD + e, O / Ls, a.f16);
+            } else {
+                float *rec = part + (size_t)tt * WSTRIDE;
+                if (e == 0) { rec[0] = M; rec[1] = Ls; }
+                rec[2 + e] = O;
+            }
+        }
+        finish_head<HD>(a, h, S, S == 1, sm);
+    }
+}
+
+#else
 // NT: tiles of eight token rows (one up to T = 8, else two).
 template <typename ST, int HD, int NT>
 __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int layer, int base, RSmem *sm) {
@@ -1193,58 +1465,10 @@ __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int l
                 *(float2 *)(rec + 2 + e) = O;
             }
         }
-        if (S > 1) {
-            worker_sync();
-            if (tid == 0) {
-                const unsigned prev = ticket_acq_rel(a.att_tickets + h);
-                const int last = prev == (unsigned)S - 1;
-                if (last) a.att_tickets[h] = 0u;
-                sm->is_last = last;
-            }
-            worker_sync();
-            if (sm->is_last) {
-                const float *p0 = a.att_part + (size_t)h * R_ATT_MAXS * CL_MAX_T * WSTRIDE;
-                for (int i = tid; i < T * HALF; i += RT) {
-                    const int tt = i / HALF, e = i % HALF * 2;
-                    float2 ml[R_ATT_MAXS], po[R_ATT_MAXS];
-#pragma unroll
-                    for (int b = 0; b < R_ATT_MAXS; b += 4) {
-#pragma unroll
-                        for (int s2 = b; s2 < b + 4; ++s2) {
-                            ml[s2] = po[s2] = make_float2(0.f, 0.f);
-                            if (b < S) {   // uniform
-                                const float *ps = p0 + ((size_t)min(s2, S - 1) * CL_MAX_T + tt) * WSTRIDE;
-                                ml[s2] = __ldcg((const float2 *)ps);
-                                po[s2] = __ldcg((const float2 *)(ps + 2 + e));
-                                if (s2 >= S) ml[s2].y = 0.f;
-                            }
-                        }
-                    }
-                    float M = -INFINITY;
-#pragma unroll
-                    for (int s2 = 0; s2 < R_ATT_MAXS; ++s2)
-                        if (ml[s2].y > 0.f) M = fmaxf(M, ml[s2].x);
-                    float Ls = 0.f, O0 = 0.f, O1 = 0.f;
-#pragma unroll
-                    for (int s2 = 0; s2 < R_ATT_MAXS; ++s2) {   // part order
-                        if (ml[s2].y > 0.f) {
-                            const float f = expf(ml[s2].x - M);
-                            Ls = fmaf(ml[s2].y, f, Ls);
-                            O0 = fmaf(po[s2].x, f, O0);
-                            O1 = fmaf(po[s2].y, f, O1);
-                        }
-                    }
-                    a_store_split2(a.Aatt, tt, T, h * HD + e, O0 / Ls, O1 / Ls, a.f16);
-                }
-            }
-        }
-        // the CTA that wrote the head's operand rows says so (its stores are read by other CTAs' bulk copies)
-        const bool wrote = S == 1 || sm->is_last;
-        if (wrote) proxy_fence_global();
-        worker_sync();
-        if (wrote && tid == 0) counter_add(a.sync + a.c_att + h, 1u);
+        finish_head<HD>(a, h, S, S == 1, sm);
     }
 }
+#endif
 
 // ---- the kernel ---------------------------------------------------------------------------------------------
 template <typename ST, int HD>
@@ -1297,9 +1521,13 @@ __global__ void __launch_bounds__(R_THREADS, 1) k_rows_pass(const __grid_constan
             compute_scales(a, sm, 2 * l + 1);
             gemm_job<CL_VEPI_STORE>(a, sm, tmem, 4 * l, cur, n_acc, run);
             phase_clock(a, sm, 1);
+#ifdef CL_ROWS_WALK
+            attention_walk<ST, HD>(a, y, l, base, sm);
+#else
             if (a.T <= 8) attention_phase<ST, HD, 1>(a, y, l, base, sm);
             else attention_phase<ST, HD, 2>(a, y, l, base, sm);
             cur.reopen(4 * l + 1);
+#endif
             phase_clock(a, sm, 2);
             gemm_job<CL_VEPI_RESID>(a, sm, tmem, 4 * l + 1, cur, n_acc, run);
             resid_phase(a, 4 * l + 1, base, sm);
@@ -1350,6 +1578,7 @@ __global__ void __launch_bounds__(R_THREADS, 1) k_rows_pass(const __grid_constan
     }
 }
 
+#ifndef CL_ROWS_WALK
 // ---- load-time re-layout: row-major [rows, K] -> the streaming order of this kernel: the row block of CTA 0, of
 // CTA 1, ...; inside a block [K / 64][block rows][64] elements with the 16-byte pieces of a row's 128 bytes permuted
 // by (piece ^ (row & 7)) -----------------------------------------------------------------------------------------
@@ -1369,10 +1598,14 @@ __global__ void k_tile_layout(const uint4 *src, uint4 *dst, int rows, int KB, in
         dst[((size_t)r0 * KB + (size_t)kb * (r1 - r0) + (r - r0)) * 8 + (size_t)(c ^ (r & 7))] = src[i];
     }
 }
+#endif
 
 }  // namespace
 
-size_t cl_rows_smem_bytes() { return (size_t)R_RING + R_CTRL_BYTES + 1024; }
+static size_t rows_smem_bytes() { return (size_t)R_RING + R_CTRL_BYTES + 1024; }
+
+#ifndef CL_ROWS_WALK
+size_t cl_rows_smem_bytes() { return rows_smem_bytes(); }
 
 int cl_rows_att_part_floats(int H) { return H * R_ATT_MAXS * CL_MAX_T * (128 + 2); }
 
@@ -1380,12 +1613,20 @@ cudaError_t cl_launch_tile_layout(const void *src, void *dst, int rows, int K, i
     k_tile_layout<<<1184, 256, 0, s>>>((const uint4 *)src, (uint4 *)dst, rows, K / 64, unit, grid);
     return cudaGetLastError();
 }
+#endif
 
+#ifdef CL_ROWS_WALK
+cudaError_t cl_launch_rows_pass_walk(int wdtype, int head_dim, const ClRowsArgs &a, int grid, cudaStream_t s) {
+#else
 cudaError_t cl_launch_rows_pass(int wdtype, int head_dim, const ClRowsArgs &a, int grid, cudaStream_t s) {
+#endif
     static_assert(sizeof(RSmem) <= R_CTRL_BYTES, "control block must fit behind the ring");
     static_assert(R_STAGE_FLOATS >= CL_MAX_T * R_STAGE_LD && R_STAGE_FLOATS % 4 == 0, "staging buffer holds a tile of every token row");
+#ifndef CL_ROWS_WALK
     static_assert(offsetof(RSmem, qp) == offsetof(RSmem, stage) + R_STAGE_FLOATS * 4 &&
                   R_STAGE_FLOATS * 4 + sizeof(RSmem::qp) >= 3 * CL_MAX_T * 128 * 4, "staging buffer and query parts hold the sums of three key groups");
+#endif
+    static_assert(R_STAGE_FLOATS >= RW * (128 + 2), "staging buffer holds the attention records");
     static_assert(R_RING + R_CTRL_BYTES + 1024 <= 232448, "shared memory of a CTA");
     const void *fn = nullptr;
     if (wdtype == 1 && head_dim == 64) fn = (const void *)k_rows_pass<__nv_bfloat16, 64>;
@@ -1393,7 +1634,7 @@ cudaError_t cl_launch_rows_pass(int wdtype, int head_dim, const ClRowsArgs &a, i
     else if (wdtype == 2 && head_dim == 64) fn = (const void *)k_rows_pass<__half, 64>;
     else if (wdtype == 2 && head_dim == 128) fn = (const void *)k_rows_pass<__half, 128>;
     else return cudaErrorInvalidValue;
-    const size_t smem = cl_rows_smem_bytes();
+    const size_t smem = rows_smem_bytes();
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void *params[] = {(void *)&a};
