@@ -416,14 +416,15 @@ __global__ void __launch_bounds__(256) k_wide_rope_append(ClWideParts p, int hd,
 // [1, 2)), a probability by 2^14, and of a probability each part is 2^12 times what the parts before it left, so that weights
 // down to 2^-38 of the row's largest keep 24 bits (ATT_STEP).
 // The sums are as exact as fp32 multiply-adds (relative error against 64 bits at 512 rows after 512 / 64 rows after 4032 keys:
-// 6.9e-7 / 1.4e-6 with those, 4.0e-7 / 7.5e-7 here, fp16): the accumulator of the instruction cuts off where an fp32 addition rounds, which
+// 6.9e-7 / 1.4e-6 with those, 4.0e-7 / 7.4e-7 here, fp16): the accumulator of the instruction cuts off where an fp32 addition rounds, which
 // over one chain for all keys of a row came to 2.2e-6 / 9.9e-6, so a chain is one tile of 64 keys, the parts have accumulators of their own,
 // a score's chain is cut in two (one chain: 4.9e-7 / 8.0e-7) and everything else is added in fp32.
 // Bound: multiply-add issue (384 instructions of 16 x 8 x 16 per warp and key tile, 8.4 cycles each at best) and the ALU work between them, which
 // two warps per scheduler hardly overlap: at 512 rows after 512 of 32 heads 143000 cycles, 68000 of them multiply-adds.  So the
-// instructions beside them count: chains start from a zero operand, masks are applied only where a key may lie ahead, a weight is one
-// multiply-add and one ex2, fragment addresses flip bits of one base.  512 rows of 32 heads 53 -> 40 us, the pass after it 97 -> 78, 333
-// rows 38 -> 29.  Key tiles dealt out evenly over the CTAs, jobs cut where shares end: 41 us (a cut costs more than the balance gains); eight
+// instructions beside them count: chains start from a zero operand, masks are applied only where a key may lie ahead,
+// fragment addresses flip bits of one base.  512 rows of 32 heads 53 -> 40 us, the pass after it 97 -> 78, 333 rows 38 -> 30.
+// (A weight is expf of the exact difference.  ex2 of s * log2(e) less the rounded m * log2(e) takes 37, 73 and 28 us, but that rounding differs
+// from tile to tile as the maximum rises, 2^-25 of the score, and at scores of 2^26 a weight could be 2^7: no number in fp16.)  Key tiles dealt out evenly over the CTAs, jobs cut where shares end: 41 us (a cut costs more than the balance gains); eight
 // warps of 32 keys: 45.  Blocks of late rows see the most keys and are scheduled first.
 constexpr int AQ = 64, AK = 64;   // rows per CTA, keys per tile
 
@@ -436,13 +437,6 @@ __device__ __forceinline__ void ldsm4(unsigned (&r)[4], unsigned addr) {
 __device__ __forceinline__ void ldsm4_t(unsigned (&r)[4], unsigned addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
-constexpr float LOG2E = 1.44269504f;
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 template <int HD, int F16>
 __global__ void __launch_bounds__(128, 2)
 k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsigned short *vcache, __nv_bfloat16 *out_b,
@@ -618,15 +612,14 @@ k_attn_wide(const float *q, int ld_q, const unsigned short *kcache, const unsign
         }
         // (a row past M, or one whose scores are all -inf so far, keeps weights of 0)
         const float ba = mx_a > -INFINITY ? mx_a : 0.f, bb = mx_b > -INFINITY ? mx_b : 0.f;
-        const float ra = ex2((m_a - ba) * LOG2E), rb = ex2((m_b - bb) * LOG2E);   // (0 while the maximum is -inf)
-        const float la = -ba * LOG2E, lb = -bb * LOG2E;   // (rounded once for the whole row, which leaves the weights' ratios alone)
+        const float ra = expf(m_a - ba), rb = expf(m_b - bb);   // (0 while the maximum is -inf)
         m_a = mx_a;
         m_b = mx_b;
         float sa = 0.f, sb = 0.f;
 #pragma unroll
         for (int n = 0; n < AK / 8; ++n) {
-            s[n][0] = ex2(fmaf(s[n][0], LOG2E, la)); s[n][1] = ex2(fmaf(s[n][1], LOG2E, la));
-            s[n][2] = ex2(fmaf(s[n][2], LOG2E, lb)); s[n][3] = ex2(fmaf(s[n][3], LOG2E, lb));
+            s[n][0] = expf(s[n][0] - ba); s[n][1] = expf(s[n][1] - ba);
+            s[n][2] = expf(s[n][2] - bb); s[n][3] = expf(s[n][3] - bb);
             sa += s[n][0] + s[n][1];
             sb += s[n][2] + s[n][3];
         }

@@ -100,3 +100,49 @@ def test_keys_that_overflowed_the_cache_and_score_minus_infinity_have_no_weight(
     want = (first / 16.0).half().double().numpy() * 16.0
     assert np.isfinite(got).all()
     assert np.abs(got - emb[tokens[n - P:]] - want)[:, 3:].max() <= 2e-3          # half a step of fp16 at 2 is 1e-3
+
+
+@pytest.mark.parametrize("wd,steps", [("fp16", [0.5, 1.0, 0.5, 0.0]), ("bf16", [0.5, 1.0, 4.0, 0.0])])
+def test_large_scores_whose_maximum_rises_from_tile_to_tile(wd, steps):
+    """Eight tiles of 64 keys, a score each, then keys without weight.  Scores are exact (the normalised marks are 16, keys and
+    queries have few bits), from 100, 246 and 992 on in steps that the storage type holds; in the last head all are 9.4e7.  Values have alternating signs and
+    cancel up to their own rounding, so that hidden states stay near 1e-3 and their rounding, averaged over rows and columns, near 1e-8.
+    Bound, of the values: a weight is off by 2^-22 at most (two steps of expf), by 2^-24 for each of eight rescalings and two
+    cut-off sums; with signs at random 4 * 2^-24 * sqrt(2^2 + 8 + 2) = 8.9e-7."""
+    heads, d, n = 4, 256, 1024
+    g = torch.Generator().manual_seed(9)
+    starts, queries = [100.0, 246.0, 992.0, 32768.0], [8.0, 8.0, 8.0, 16.0 * 1440.0]
+    emb = (torch.rand((V, d), generator=g) - 0.5) * 1e-3
+    emb[:, :16] = 0.0
+    emb[:, :3] = 256.0
+    tokens = np.concatenate([np.repeat(np.arange(8), 64), np.full(n - 512, 8)]) * 100
+    tokens = (tokens + np.arange(n) % 64).astype(np.int32)
+    for i in range(V):
+        emb[i, 3 + min(i // 100, 8)] = 256.0   # four columns of 256 among 256: normalised 8, with the gain 16
+    emb = emb.to(DT[wd])
+    z = lambda r, c: torch.zeros((r, c), dtype=torch.float32)
+    wq, wk, wv, wo = z(d, d), z(d, d), z(d, d), torch.eye(d)
+    u = 1.0 + torch.rand(64, generator=g)
+    weight = np.zeros((heads, 8))
+    for h in range(heads):
+        score = (starts[h] + steps[h] * np.arange(8)) * queries[h] / 8.0
+        weight[h] = np.exp(score - score.max())
+        wq[64 * h + 31, 0] = queries[h] / 16.0
+        sign = np.array([1.0, -1.0] * 4)
+        sign[7] = -(weight[h] * sign)[:7].sum()
+        for j in range(8):
+            wk[64 * h + 31, 3 + j] = (starts[h] + steps[h] * j) / 16.0
+            wv[64 * h : 64 * h + 64, 3 + j] = u * float(sign[j]) / 16.0
+    wv[:16] = 0.0
+    t = lambda x: x.to(DT[wd]).cuda()
+    ctx = cl.Context(1, d, heads, 64, V, n + 8, wd, 1e-5, 1e20, tap_positions=P)
+    ctx.cl_load(dict(embed=emb.cuda(), lm_head=t(z(V, d)), final_norm=torch.ones(d).cuda(), wq=[t(wq)], wk=[t(wk)], wv=[t(wv)], wo=[t(wo)],
+                     wg=[t(z(64, d))], wu=[t(z(64, d))], wd=[t(z(d, 64))], norm1=[torch.full((d,), 2.0).cuda()], norm2=[torch.ones(d).cuda()]))
+    got = _hidden(ctx, n, tokens) - emb.double().numpy()[tokens[n - P:]]
+    ctx.close()
+    value = (t(wv)[:, 3:11] * 16.0).double().cpu().numpy().reshape(heads, 64, 8)
+    want = (value * weight[:, None]).sum(2) / weight.sum(1)[:, None]
+    err = ((got.reshape(P, heads, 64) - want) / u.double().numpy()).mean(0)
+    for h in range(heads):
+        e = err[h, 16 if h == 0 else 0:].mean()
+        assert abs(e) <= 8.9e-7, (starts[h], e)
