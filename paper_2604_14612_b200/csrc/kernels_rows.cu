@@ -990,7 +990,7 @@ __device__ void attention_walk(const ClRowsArgs &a, const ClRowsLayer &y, int la
 #pragma unroll
                         for (int k = 0; k < KPW; ++k) {
                             const float v = __shfl_sync(0xffffffffu, sc, k * LPK);
-                            if (lane == jb + k && jb + k < n) my_score = v;
+                            if (lane == jb + k && jb + k < n && v > -INFINITY) my_score = v;   // (no number: no weight)
                         }
                     }
                 }
@@ -998,7 +998,7 @@ __device__ void attention_walk(const ClRowsArgs &a, const ClRowsLayer &y, int la
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
                 m_new = fmaxf(m_new, m_run);
-                const float p = (lane < n) ? expf(my_score - m_new) : 0.f;
+                const float p = (lane < n) ? expf(my_score - (m_new > -INFINITY ? m_new : 0.f)) : 0.f;   // (scores may all be -inf so far)
                 const float resc = (l_run > 0.f) ? expf(m_run - m_new) : 0.f;
                 float ps = p;
 #pragma unroll
@@ -1033,9 +1033,10 @@ __device__ void attention_walk(const ClRowsArgs &a, const ClRowsLayer &y, int la
 #pragma unroll
                     for (int o = LPK >> 1; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
                     sc = __shfl_sync(0xffffffffu, sc, 0) * scale;
+                    sc = sc > -INFINITY ? sc : -INFINITY;   // (no number: no weight)
                     const float m_new = fmaxf(m_run, sc);
                     const float resc = (l_run > 0.f) ? expf(m_run - m_new) : 0.f;
-                    const float pn = expf(sc - m_new);
+                    const float pn = expf(sc - (m_new > -INFINITY ? m_new : 0.f));
                     l_run = fmaf(l_run, resc, pn);
 #pragma unroll
                     for (int e = 0; e < VPL; ++e) o_run[e] = fmaf(o_run[e], resc, pn * vn[e]);

@@ -52,10 +52,10 @@ def test_every_number_of_rows_and_cached_keys(monkeypatch, wd, heads, kv_heads, 
         assert rel <= 5e-4, (n, T, rel)
 
 
+@pytest.mark.parametrize("n", [600, 40])   # (many keys a part and few: each build)
 @pytest.mark.parametrize("T", [1, 5, 9])
-def test_keys_that_score_minus_infinity_have_no_weight(T):
+def test_keys_that_score_minus_infinity_have_no_weight(T, n):
     """fp16 keys of 1e5 are infinite; against a negative query they score -inf, so the first token's value is the whole output."""
-    n = 600
     g = torch.Generator().manual_seed(6)
     values, first = (1.0 + torch.rand(256, generator=g)) * 500, 1.0 + torch.rand(256, generator=g)
     first[:3] = 0.0
@@ -70,6 +70,26 @@ def test_keys_that_score_minus_infinity_have_no_weight(T):
     want = (first / 16.0).half().double().numpy() * 16.0
     assert np.isfinite(got).all()
     assert np.abs(got - emb[[7] + list(range(1, T))] - want)[:, 3:].max() <= 2e-3          # half a step of fp16 at 2 is 1e-3
+
+
+@pytest.mark.parametrize("n", [600, 100])
+@pytest.mark.parametrize("T", [1, 5, 9])
+def test_a_key_with_weight_behind_keys_that_score_minus_infinity(T, n):
+    """All cached keys score -inf; the pass's first token, the first to score 0, is the whole output of every row."""
+    g = torch.Generator().manual_seed(6)
+    values, first = (1.0 + torch.rand(256, generator=g)) * 500, 1.0 + torch.rand(256, generator=g)
+    first[:3] = 0.0
+    ctx, emb, _ = _model("fp16", 4, n + 16, [-32.0, -1.0, -3.3, -0.01], values, first_key=0.0, other_key=1e5, first_value=first)
+    ctx.cl_prefill((1 + np.arange(n) % 1000).astype(np.int32))
+    ctx.cl_rollback(n, 0)
+    ctx.cl_force_tokens(np.arange(1, T).astype(np.int32))
+    ctx.cl_verify(T, tap_hidden=True)
+    ring = ctx.cl_read_hidden_ring().double().numpy()[0]
+    ctx.close()
+    got = ring[[(n + t) % 512 for t in range(T)]]
+    want = (first / 16.0).half().double().numpy() * 16.0
+    assert np.isfinite(got).all()
+    assert np.abs(got - emb[[0] + list(range(1, T))] - want)[:, 3:].max() <= 2e-3          # half a step of fp16 at 2 is 1e-3
 
 
 @pytest.mark.parametrize("T", [5, 9])
