@@ -790,9 +790,12 @@ __device__ void embed_phase(const ClRowsArgs &a, RSmem *sm) {
 //            added in shared memory
 // so every key and value row is fetched once per CTA, all of them at once, before the CTA waits for its queries: the phase costs
 // one trip to memory for the queries and none for 224 keys.  Both products run on the tensor cores (mma.sync) with queries
-// and weights in three parts of the storage type, scaled as in k_attn_wide, whose sums are as exact as fp32 multiply-adds; keys and
-// values are the A operand (16 keys or 16 elements of the head), the T rows the columns, so that up to eight rows cost one
-// instruction.  The rows' own keys and values (positions base .. base + t, causal) come raw from the QKV product: the CTA of the
+// and weights in three parts of the storage type, scaled as in k_attn_wide; keys and values are the A operand (16 keys or 16
+// elements of the head), the T rows the columns, so that up to eight rows cost one instruction.  The accumulator cuts off where an
+// fp32 addition rounds, so of the first parts, which carry the sum, every instruction is a chain of its own and the chains are added in
+// fp32.  Error against 64 bits over that of attention_walk, 3 to 9 rows after 300 to 4000 keys, scores of deviation 1 to 8: mean 0.80,
+// largest 1.08 (a chain over the whole score, one over a group's chunks: 1.15 and 2.37; 5 rows after 640 keys, head_dim 128, fp16,
+// deviation 2: 3.4e-7, 6.9e-7 so, 3.7e-7 in attention_walk).  The rows' own keys and values (positions base .. base + t, causal) come raw from the QKV product: the CTA of the
 // last part rotates the keys, rounds both to the storage type and takes them as its last chunk (one query head per
 // key/value head also appends them to the cache).  A CTA writes one (max, sum, output) record per (h, s, t); the last CTA of
 // a head to finish (ticket) merges the parts in order and writes the normalised output as the output projection's hi/lo
@@ -800,7 +803,8 @@ __device__ void embed_phase(const ClRowsArgs &a, RSmem *sm) {
 // Bound: latency (the queries' trip, the record's, the ticket and the merge).  Before, a warp walked a row's keys 16 at a time, one trip
 // to memory each.  Attention of a layer, mean over CTAs: 640 keys, 5 rows of 32 heads 14.5 -> 8 us; 1003 keys, 9 rows 35 -> 14; verify
 // of 8 layers of width 4096 907 -> 846 and 1141 -> 960 us, 4 layers of width 5120 after 1024 keys (7 rows) 711 -> 643, 12 of width
-// 768 after 200 keys (5 rows) as before.  Nine rows: the values' registers for 14 chunks spill (991 us), 12 chunks 965.
+// 768 after 200 keys (5 rows) as before.  Nine rows: the values' registers for 14 chunks spill (991 us), 12 chunks 965.  (With the forms for
+// up to eight and for nine rows in one kernel, 412 to 504 bytes of a thread's registers spill, at head_dim 64 and 128.)
 // Ahead of a layer's QKV job: ask for the cached keys and values this CTA's attention item will read, so that they wait
 // in L2 when the attention phase starts (the worker warps have nothing else to do while the job's weights stream).
 template <int HD>
@@ -1241,8 +1245,20 @@ __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int l
                 }
                 float u[3][4];   // products with the queries' parts
                 float x[4];      // of the ninth row: its parts are the columns
+                float pu[4], px[4];   // of the first parts, an even q's sums until the odd one's are there
 #pragma unroll
                 for (int e = 0; e < 4; ++e) u[0][e] = u[1][e] = u[2][e] = x[e] = 0.f;
+                // first parts: every instruction a chain of its own, the chains added two by two in fp32
+                auto add_first = [&](float(&to)[4], float(&even)[4], const unsigned(&a0)[4], const unsigned(&a1)[4], const uint4 &b, int q) {
+                    float c0[4], c1[4];
+                    mma16816_zero<F16>(c0, a0, b.x, b.y);
+                    mma16816_zero<F16>(c1, a1, b.z, b.w);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (q & 1) to[e] += even[e] + (c0[e] + c1[e]);
+                        else even[e] = c0[e] + c1[e];
+                    }
+                };
 #pragma unroll
                 for (int q = 0; q < NC; ++q) {
                     const unsigned a0[4] = {kf[0][q].x, kf[1][q].x, kf[0][q].y, kf[1][q].y}, a1[4] = {kf[0][q].z, kf[1][q].z, kf[0][q].w, kf[1][q].w};
@@ -1250,13 +1266,16 @@ __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int l
 #pragma unroll
                     for (int p = 0; p < 3; ++p) {
                         const uint4 b = *(const uint4 *)(sm->qp + (size_t)(p * CL_MAX_T + tok) * HD + (((q * 4 + tig) ^ ((tok & 1) << 2)) << 3));
-                        mma16816<F16>(u[p], a0, b.x, b.y);
-                        mma16816<F16>(u[p], a1, b.z, b.w);
+                        if (p == 0) {
+                            add_first(u[0], pu, a0, a1, b, q);
+                        } else {
+                            mma16816<F16>(u[p], a0, b.x, b.y);
+                            mma16816<F16>(u[p], a1, b.z, b.w);
+                        }
                     }
                     if (NT == 2) {
                         const uint4 b = *(const uint4 *)(sm->qp + (size_t)(min(g, 2) * CL_MAX_T + 8) * HD + ((q * 4 + tig) << 3));
-                        mma16816<F16>(x, a0, b.x, b.y);
-                        mma16816<F16>(x, a1, b.z, b.w);
+                        add_first(x, px, a0, a1, b, q);
                     }
                 }
                 float odd = 0.f;
@@ -1354,6 +1373,14 @@ __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int l
                     a1[0] = __byte_perm(v[0].y, v[1].y, 0x5410); a1[1] = __byte_perm(v[0].y, v[1].y, 0x7632);
                     a1[2] = __byte_perm(v[2].y, v[3].y, 0x5410); a1[3] = __byte_perm(v[2].y, v[3].y, 0x7632);
                 };
+                // a chunk's sums by themselves, added in fp32
+                auto add_chunk = [&](float(&to)[2][4], const unsigned(&a0)[4], const unsigned(&a1)[4], unsigned b0, unsigned b1) {
+                    float y[2][4];
+                    mma16816_zero<F16>(y[0], a0, b0, b1);
+                    mma16816_zero<F16>(y[1], a1, b0, b1);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) to[e / 4][e % 4] += y[e / 4][e % 4];
+                };
                 auto odd_value = [&](int tok, int e) {   // element e of the lane's four: own values that are infinite or no numbers
                     float v = 0.f;                       // (only rows that give such a value weight may meet it)
 #pragma unroll 1
@@ -1377,8 +1404,12 @@ __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int l
                         split3<F16, STEP>(p1.x, p1.y, b1);
 #pragma unroll
                         for (int p = 0; p < 3; ++p) {
-                            mma16816<F16>(c[p][0], a0, b0[p], b1[p]);
-                            mma16816<F16>(c[p][1], a1, b0[p], b1[p]);
+                            if (p == 0) {
+                                add_chunk(c[0], a0, a1, b0[0], b1[0]);
+                            } else {
+                                mma16816<F16>(c[p][0], a0, b0[p], b1[p]);
+                                mma16816<F16>(c[p][1], a1, b0[p], b1[p]);
+                            }
                         }
                     };
 #pragma unroll
@@ -1411,8 +1442,7 @@ __device__ void attention_phase(const ClRowsArgs &a, const ClRowsLayer &y, int l
                         split3<F16, STEP>(p0.x, p0.y, b0);
                         split3<F16, STEP>(p1.x, p1.y, b1);
                         const unsigned y0 = g == 0 ? b0[0] : g == 1 ? b0[1] : b0[2], y1 = g == 0 ? b1[0] : g == 1 ? b1[1] : b1[2];
-                        mma16816<F16>(x[0], a0, y0, y1);
-                        mma16816<F16>(x[1], a1, y0, y1);
+                        add_chunk(x, a0, a1, y0, y1);
                     };
 #pragma unroll
                     for (int i = 0; i < MAXC; ++i)

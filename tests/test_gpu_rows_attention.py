@@ -108,3 +108,46 @@ def test_a_candidate_whose_value_overflows_leaves_the_rows_before_it_alone(T):
     assert np.isfinite(rows[5]).all()
     assert np.array_equal(rows[0][:3], rows[5][:3])
     assert not np.isfinite(rows[0][3:, 3:]).any()
+
+
+@pytest.mark.parametrize("wd", ["bf16", "fp16"])
+@pytest.mark.parametrize("T,n", [(3, 1100), (5, 600), (9, 600), (5, 40)])
+def test_small_products_beside_a_large_one_are_not_cut_off(wd, T, n):
+    """Two kinds of keys score 1024 and 1024 + 2.25 * 2^-13; the excess is three products of 0.75 * 2^-13, each in another instruction of
+    the score's contraction.  Products, scores and the scaling by 1/8 are exact (marks are 16 after the norm, numbers have two bits), so
+    a score is off by roundings alone: one step of 2^-13, where an accumulator that cuts off would lose all three products.  The rows of
+    the pass themselves have keys of 0 (no weight); values are u and -u, so the hidden state is -u tanh(excess / 2)."""
+    heads, d, steps = 4, 256, 2.0 ** -13
+    g = torch.Generator().manual_seed(11)
+    emb = (torch.rand((V, d), generator=g) - 0.5) * 1e-3
+    emb[:, :6] = 0.0
+    emb[:, :3] = 256.0
+    for i in range(V):
+        emb[i, 3 + min(i // 100, 2)] = 256.0   # tokens 0 .. 99, 100 .. 199, from 200 on; four columns of 256 among 256: normalised 8, gain 2
+    emb = emb.to(DT[wd])
+    z = lambda r, c: torch.zeros((r, c), dtype=torch.float32)
+    wq, wk, wv = z(d, d), z(d, d), z(d, d)
+    u = (1.0 + torch.rand(d, generator=g)).to(DT[wd]).float()
+    for h in range(heads):
+        # (dimensions 16 .. 31 and their partners 48 .. 63 rotate by less than 1e-6 over all positions; none of these is another's partner)
+        for e, q, k in ((16, 64.0, 128.0), (20, 2.0 ** -5, 0.75 * 2.0 ** -5), (56, 2.0 ** -5, 0.75 * 2.0 ** -5), (60, 2.0 ** -5, 0.75 * 2.0 ** -5)):
+            wq[64 * h + e, 0] = q / 16.0
+            wk[64 * h + e, 4] = k / 16.0
+            if e == 16:
+                wk[64 * h + e, 3] = k / 16.0
+    wv[:, 3], wv[:, 4] = u / 16.0, -u / 16.0
+    wv[:6] = 0.0
+    t = lambda x: x.to(DT[wd]).cuda()
+    ctx = cl.Context(1, d, heads, 64, V, n + 16, wd, 1e-5, 1e20, tap_positions=512)
+    ctx.cl_load(dict(embed=emb.cuda(), lm_head=t(z(V, d)), final_norm=torch.ones(d).cuda(), wq=[t(wq)], wk=[t(wk)], wv=[t(wv)], wo=[t(torch.eye(d))],
+                     wg=[t(z(64, d))], wu=[t(z(64, d))], wd=[t(z(d, 64))], norm1=[torch.full((d,), 2.0).cuda()], norm2=[torch.ones(d).cuda()]))
+    ctx.cl_prefill((np.arange(n) % 2 * 100 + np.arange(n) // 2 % 100).astype(np.int32))
+    rows = 200 + np.arange(T)
+    ctx.cl_rollback(n, int(rows[0]))
+    ctx.cl_force_tokens(rows[1:].astype(np.int32))
+    ctx.cl_verify(T, tap_hidden=True)
+    ring = ctx.cl_read_hidden_ring().double().numpy()[0]
+    ctx.close()
+    att = ring[[(n + i) % 512 for i in range(T)]] - emb.double().numpy()[rows]
+    excess = -2.0 * np.arctanh((att / u.double().numpy())[:, 6:].mean(1))
+    assert np.abs(excess / steps - 2.25).max() <= 1.0, excess / steps
