@@ -1,6 +1,7 @@
 // Host side of libconflayers.so: context, weight arena, and the sequencing of the kernels that make
 // up a draft step, a verify pass, acceptance and the confidence scoring.  All arithmetic of the
 // method runs in the kernels; this file only lays out memory and enqueues launches on one stream.
+#include <limits.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stddef.h>
@@ -570,6 +571,12 @@ static int head(cl_ctx *c, int T, const float *xin, const ClDevState *st, int *o
     return CL_OK;
 }
 
+static int rows_att_parts(const cl_ctx *c) { return std::min(std::max(c->n_sm / c->cfg.n_heads, 1), 8); }
+
+// Which of the two builds of the T-row pass (cl_rows_walk_keys): the one that walks the keys up to this position of its first row.  A matter of
+// T and the position alone, so that a pass comes out the same however its caller got there.
+static long long rows_walk_line(const cl_ctx *c, int T) { return (long long)cl_rows_walk_keys(T) * rows_att_parts(c); }
+
 // The same pass as one persistent launch on the tensor cores (16-bit models): all layers and the LM head.
 static int forward_rows_persistent(cl_ctx *c, const int *tok, int T, int row0, int tap, int want_head, int *out_tok,
                                    float *out_pmax, float *out_conf, float *logits) {
@@ -579,12 +586,9 @@ static int forward_rows_persistent(cl_ctx *c, const int *tok, int T, int row0, i
     a.layers = c->rows_layers_dev; a.L = g.n_layers; a.head = c->head_tile; a.embed = c->embed; a.final_norm = c->final_norm;
     a.d = g.d_model; a.F = g.d_ffn; a.V = g.vocab; a.H = g.n_heads; a.Hkv = g.n_kv_heads; a.hd = g.head_dim; a.max_seq = g.max_seq;
     a.T = T; a.row0 = row0; a.want_head = want_head; a.f16 = g.weight_dtype == 2;
-    a.att_parts = c->n_sm / g.n_heads;
-    if (a.att_parts < 1) a.att_parts = 1;
-    if (a.att_parts > 8) a.att_parts = 8;
+    a.att_parts = rows_att_parts(c);
     a.tap = tap && c->ring; a.tap_P = g.tap_positions;
-    // which of the two builds: by the position as the host last saw it (a batch of cycles may move on; either is right anywhere)
-    const bool walk = c->h_ctx + row0 <= CL_ROWS_WALK_KEYS * a.att_parts;
+    const bool walk = c->h_ctx + row0 <= rows_walk_line(c, T);
     a.entry = c->rows_entry ? c->rows_entry : (walk ? 70 : 68) * 1024; a.chain = c->rows_chain; a.split = c->rows_split; a.ws = c->r_ws;
     a.eps = g.rms_eps; a.inv_d = 1.0f / (float)g.d_model; a.inv_log_v = (float)(1.0 / log((double)g.vocab));
     a.rope_cs = c->rope_cs; a.st = c->st; a.tok = tok;
@@ -990,7 +994,7 @@ extern "C" int cl_step_vanilla(cl_ctx *c, int32_t *tok) {
     return CL_OK;
 }
 
-static int enqueue_cycle(cl_ctx *c, int K, int tap = 0) {
+static int enqueue_cycle(cl_ctx *c, int K, int tap) {
     int rc;
     if (c->use_step && K > 0) {
         if ((rc = run_steps(c, CL_STEP_DRAFT, K, 0, false, nullptr, nullptr))) return rc;
@@ -1006,6 +1010,22 @@ static int enqueue_cycle(cl_ctx *c, int K, int tap = 0) {
                       ST_FIELD(c, float, v_pmax), ST_FIELD(c, float, v_conf), nullptr);
     if (rc) return rc;
     KL(cl_launch_accept(c->st, K, c->out_dev, c->stream));
+    return CL_OK;
+}
+
+// n cycles, the last n_tap of them with taps.  They are enqueued without waiting for one another, except where a cycle could begin on either
+// side of the line between the two builds of the verify pass: a cycle moves on by at most K + 1 positions.
+static int enqueue_cycles(cl_ctx *c, int K, int n, int n_tap = 0) {
+    int rc;
+    const long long line = c->use_rows ? rows_walk_line(c, K + 1) : LLONG_MAX;
+    long long farthest = c->h_ctx;   // the next cycle's position, if the ones enqueued accept everything
+    for (int i = 0; i < n; ++i, farthest += K + 1) {
+        if (c->h_ctx <= line && farthest > line) {
+            if ((rc = sync_state(c))) return rc;
+            farthest = c->h_ctx;
+        }
+        if ((rc = enqueue_cycle(c, K, n - i <= n_tap))) return rc;
+    }
     return CL_OK;
 }
 
@@ -1036,8 +1056,7 @@ extern "C" int cl_generate(cl_ctx *c, int K, int max_new, int32_t *out, int *n_o
     while (remaining > 0) {
         // the fewest cycles that can finish the job; cycles enqueued past the end exit at once on the device
         const int ncyc = (remaining + K) / (K + 1);
-        for (int i = 0; i < ncyc; ++i)
-            if ((rc = enqueue_cycle(c, K))) return rc;
+        if ((rc = enqueue_cycles(c, K, ncyc))) return rc;
         if ((rc = sync_state(c))) return rc;
         remaining = max_new - c->h_st->n_out;
     }
@@ -1102,9 +1121,8 @@ extern "C" int cl_generate_search(cl_ctx *c, const cl_search_cfg *sc, const cl_s
         const int ncyc = r.searching ? sc->interval : (remaining + K) / (K + 1);
         // Taps while searching: every cycle advances by at least one position, so the last P cycles of an interval rewrite
         // every slot of the ring (slot = position mod P); what earlier cycles would record is gone by the search check.
-        for (int i = 0; i < ncyc; ++i)
-            if ((rc = enqueue_cycle(c, K, r.searching && ncyc - i <= P))) return rc;
         const int ctx_before = c->h_ctx;
+        if ((rc = enqueue_cycles(c, K, ncyc, r.searching ? P : 0))) return rc;
         if ((rc = sync_state(c))) return rc;
         if ((rc = check_device_err(c, "cl_generate_search"))) return rc;
         if (r.searching) c->tapped += c->h_ctx - ctx_before;   // every verify pass of the interval recorded its rows

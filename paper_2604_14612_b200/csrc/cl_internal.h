@@ -238,8 +238,8 @@ int cl_rows_att_part_floats(int H);
 // (rows split in units of `unit` rows, exactly as the kernel splits them)
 cudaError_t cl_launch_tile_layout(const void *src, void *dst, int rows, int K, int unit, int grid, cudaStream_t s);
 cudaError_t cl_launch_rows_pass(int wdtype, int head_dim, const ClRowsArgs &a, int grid, cudaStream_t s);
-// the same pass, faster after up to this many cached keys per part of a head (see kernels_rows.cu)
-#define CL_ROWS_WALK_KEYS 32
+// the same pass, faster after up to this many cached keys per part of a head (see attention_walk)
+static inline int cl_rows_walk_keys(int T) { return T <= 2 ? 1 << 20 : T == CL_MAX_T ? 48 : 32 * (14 / T); }
 cudaError_t cl_launch_rows_pass_walk(int wdtype, int head_dim, const ClRowsArgs &a, int grid, cudaStream_t s);
 
 // ---- wide tensor-core GEMM of the prompt pass (bf16 models): up to CL_WIDE_MAX_M prompt rows at a time ----

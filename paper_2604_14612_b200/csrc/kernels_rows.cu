@@ -886,9 +886,15 @@ __device__ __forceinline__ void finish_head(const ClRowsArgs &a, int h, int S, b
 
 #ifdef CL_ROWS_WALK
 // Few keys: a warp walks the keys of one token row (w / nsub; nsub = 14 / T warps a row share them), 16 at a time with an online softmax on
-// the CUDA cores, a trip to memory each.  With up to CL_ROWS_WALK_KEYS keys a part that is faster than the other form's fixed cost and smaller
-// ring.  us per verify, here / there: 8 layers of width 4096, 9 rows after 100 (25 keys a part) 925 / 953, 3 rows after 54 785 / 799, but 7 rows after
-// 170 (43) 858 / 835, 5 rows after 220 (55) 833 / 820; 12 of width 768, 5 rows after 200 (25) 527 / 542.
+// the CUDA cores, a trip to memory each.  Up to two trips that is faster than the other form's fixed cost and smaller ring, hence the line
+// of 32 * (14 / T) keys a part (cl_rows_walk_keys); three trips with nine rows, which cost the other form a second set of columns; and at any
+// length with one or two rows, whose scores leave six or seven of its eight columns idle.  us per verify, here / there, by keys a part:
+//   8 layers of width 4096 (4 parts)  1 row   112 831 / 856   224 823 / 858   640 905 / 971      2 rows  112 843 / 858   224 859 / 883   640 955 / 979
+//     3 rows  64 843 / 860   112 858 / 868   136 880 / 870      4 rows  48 856 / 870   96 870 / 870   136 893 / 881
+//     5 rows  48 870 / 888   64 880 / 882   80 893 / 882        7 rows  32 881 / 904   64 904 / 905   80 917 / 904
+//     8 rows  24 884 / 891   32 892 / 892   40 898 / 884        9 rows  32 953 / 979   48 966 / 979   64 978 / 968
+//   12 of width 768 (8)               2 rows  224 523 / 560   640 605 / 622      3 rows  112 523 / 535   136 535 / 535      5 rows  64 535 / 540
+//   4 of width 5120 (3)               2 rows  224 621 / 639   640 672 / 696      3 rows  112 613 / 634   136 623 / 634      9 rows  48 672 / 684
 template <typename ST, int HD>
 __device__ void attention_walk(const ClRowsArgs &a, const ClRowsLayer &y, int layer, int base, RSmem *sm) {
     constexpr int EPL = 8, LPK = HD / EPL, KPW = 32 / LPK, VPL = HD / 32, WSTRIDE = HD + 2, HALF = HD / 2;

@@ -151,3 +151,38 @@ def test_small_products_beside_a_large_one_are_not_cut_off(wd, T, n):
     att = ring[[(n + i) % 512 for i in range(T)]] - emb.double().numpy()[rows]
     excess = -2.0 * np.arctanh((att / u.double().numpy())[:, 6:].mean(1))
     assert np.abs(excess / steps - 2.25).max() <= 1.0, excess / steps
+
+
+@pytest.mark.parametrize("K,n,gen", [(8, 250, 160), (4, 300, 240)])
+def test_single_cycles_and_one_call_and_several_compute_the_same(K, n, gen):
+    """Generation across the lines between the two builds of the pass (heads in 8 parts: 384 cached keys with nine rows, 512 with five):
+    which one a position takes does not depend on how the cycles are called, so tokens and the logits behind them agree to the bit.
+    (Calls end where a cycle ends: a cycle that begins elsewhere splits the keys differently.)"""
+    d, F, W = _random_model("bf16", 4, 4, 64)
+    W = {k: v * 2 if isinstance(v, list) else v for k, v in W.items()}   # (two layers: the second one's keys depend on the attention)
+    ctx = cl.Context(2, d, 4, F, V, n + gen + 64, "bf16", 1e-5, 1e4, tap_positions=16, n_kv_heads=4)
+    ctx.cl_load(W)
+    prompt = (np.arange(n) * 7 + n).astype(np.int32) % V
+
+    def logits_behind(toks):
+        ctx.cl_force_tokens([4, 5])
+        return toks, ctx.cl_verify(3, want_logits=True)["logits"].copy()
+
+    ctx.cl_prefill(prompt)
+    toks, ends = [], [0]
+    while len(toks) < gen:
+        ctx.cl_draft(K)
+        ctx.cl_verify(K + 1)
+        toks += [int(x) for x in ctx.cl_accept()[1]]
+        ends.append(len(toks))
+    out = [logits_behind(toks)]
+    for cuts in (ends[::len(ends) - 1], [ends[0], ends[len(ends) // 3], ends[2 * len(ends) // 3], ends[-1]]):
+        ctx.cl_prefill(prompt)
+        toks = []
+        for a, b in zip(cuts, cuts[1:]):
+            toks += [int(x) for x in ctx.cl_generate(K, b - a)[0]]
+        out.append(logits_behind(toks))
+    ctx.close()
+    for toks, logits in out[1:]:
+        assert toks == out[0][0]
+        assert np.array_equal(logits, out[0][1])
