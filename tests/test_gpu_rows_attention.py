@@ -1,5 +1,6 @@
-"""Attention of the (K + 1)-row pass at the edges of its chunks of 16 keys and its iterations of 14 (nine rows: 12) of them, for every
-number of rows, and with keys and values that overflowed the cache (run on a B200)."""
+"""Attention of the (K + 1)-row pass: the edges of its chunks of 16 keys and its iterations of 14 (nine rows: 12) of them, for every number of
+rows, on both sides of the line between its two builds; keys and values that overflowed the cache; small products; the same result
+however cycles are called (run on a B200)."""
 import numpy as np
 import pytest
 import torch
@@ -34,7 +35,10 @@ def test_every_number_of_rows_and_cached_keys(monkeypatch, wd, heads, kv_heads, 
         ctx = cl.Context(1, d, heads, F, V, 2000, wd, 1e-5, 1e4, tap_positions=16, n_kv_heads=kv_heads)
         ctx.cl_load(W)
         res = []
-        for n in (17, 18, 31, 33, 127, 129, 447, 448, 449, 895, 897, 1791, 1900):
+        # around the lines between the two builds (8 parts: 8 rows 256, 9 384, 5 to 7 512, 4 768, 3 1024); last parts of 192 and 193 keys, whole
+        # iterations of nine rows, behind which the pass's own chunk stands alone (8 parts 1536, 3 576, 4 768)
+        for n in (17, 18, 31, 33, 127, 129, 256, 257, 273, 384, 385, 401, 447, 448, 449, 512, 513, 529, 576, 579, 768, 769, 772, 895, 897,
+                  1024, 1025, 1536, 1544, 1791, 1900):
             ctx.cl_prefill((np.arange(n) * 7 + n).astype(np.int32) % V)
             for T in range(1, 10):
                 ctx.cl_rollback(n, n % V)
@@ -92,10 +96,10 @@ def test_a_key_with_weight_behind_keys_that_score_minus_infinity(T, n):
     assert np.abs(got - emb[[0] + list(range(1, T))] - want)[:, 3:].max() <= 2e-3          # half a step of fp16 at 2 is 1e-3
 
 
+@pytest.mark.parametrize("n", [40, 600])   # (each build: keys walked, tensor cores)
 @pytest.mark.parametrize("T", [5, 9])
-def test_a_candidate_whose_value_overflows_leaves_the_rows_before_it_alone(T):
+def test_a_candidate_whose_value_overflows_leaves_the_rows_before_it_alone(T, n):
     """Token 0 has values of 1e5, infinite in fp16: rows that do not attend to it are the same to the bit, rows that do are not finite."""
-    n = 40
     ctx, _, _ = _model("fp16", 4, n + 16, [1.0, 2.0, -1.0, 0.5], torch.ones(256), first_value=1e5)
     rows = {}
     for third in (0, 5):
@@ -108,6 +112,25 @@ def test_a_candidate_whose_value_overflows_leaves_the_rows_before_it_alone(T):
     assert np.isfinite(rows[5]).all()
     assert np.array_equal(rows[0][:3], rows[5][:3])
     assert not np.isfinite(rows[0][3:, 3:]).any()
+
+
+@pytest.mark.parametrize("n", [40, 600])
+@pytest.mark.parametrize("T", [5, 9])
+def test_a_candidate_whose_key_overflows_has_no_weight_against_negative_queries(T, n):
+    """Token 0 has keys of 1e5, infinite in fp16, that score -inf; all others score 0 and have the same value: the output of every row."""
+    g = torch.Generator().manual_seed(7)
+    values = 1.0 + torch.rand(256, generator=g)
+    values[:3] = 0.0
+    ctx, emb, v = _model("fp16", 4, n + 16, [-32.0, -1.0, -3.3, -0.01], values, first_key=1e5, first_value=500.0)
+    ctx.cl_prefill((1 + np.arange(n)).astype(np.int32))
+    ctx.cl_rollback(n, 7)
+    tokens = [7, 1, 2, 0] + list(range(10, 6 + T))
+    ctx.cl_force_tokens(np.array(tokens[1:], np.int32))
+    ctx.cl_verify(T, tap_hidden=True)
+    got = ctx.cl_read_hidden_ring().double().numpy()[0][[(n + t) % 512 for t in range(T)]]
+    ctx.close()
+    assert np.isfinite(got).all()
+    assert np.abs(got - emb[tokens] - v)[:, 3:].max() <= 2e-3          # half a step of fp16 at 2 is 1e-3
 
 
 @pytest.mark.parametrize("wd", ["bf16", "fp16"])
