@@ -510,7 +510,7 @@ extern "C" int cl_load(cl_ctx *c, const cl_weights *w) {
                 if (c->rows_chain < 1) c->rows_chain = 1;
                 const char *en = getenv("CL_ROWS_ENTRY_KB");   // tuning knob
                 c->rows_entry = (en && en[0]) ? std::max(atoi(en), 1) * 1024 : 0;   // (0: a third of the ring)
-                if (c->rows_entry > 96 * 1024) c->rows_entry = 96 * 1024;   // (two entries must fit the ring of 192 KB)
+                if (c->rows_entry > 96 * 1024) c->rows_entry = 96 * 1024;   // (two entries must fit the ring, 205 KB in the smaller build)
                 c->use_rows = 1;
             }
         }

@@ -435,7 +435,7 @@ extern "C" int cl_layer_confidences_static(const void *lm_head, const float *fin
         e = cl_launch_head_tc(lm_head, hidden, final_norm, n_rows, vocab, d_model, rms_eps, n_sm, (double *)(sc + SC_OFF_SCALE), sc + SC_OFF_SPLIT, SC_SPLIT,
                               (ClHeadPartial *)(sc + SC_OFF_PART), flags, d_conf, d_pmax, d_arg, s);
         if (e == cudaSuccess) e = fetch();
-        if (e == cudaSuccess && res[0] && !res[1]) {   // not a call for that kernel: once more as before it (the tickets were used)
+        if (e == cudaSuccess && res[0] && !res[1]) {   // not a call for that kernel: once more on the others, whose tickets start at zero
             e = cudaMemsetAsync(sc, 0, SC_OFF_XN, s);
             if (e == cudaSuccess) e = n_rows > SC_GEMV_ROWS ? many_rows() : few_rows();
             if (e == cudaSuccess) e = fetch();

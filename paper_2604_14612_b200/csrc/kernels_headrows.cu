@@ -387,22 +387,6 @@ __device__ __forceinline__ void tmem_st16(unsigned taddr, const float (&v)[16]) 
         "f"(v[13]), "f"(v[14]), "f"(v[15]), "r"(taddr)
         : "memory");
 }
-// A load whose values may be used after tmem_ld_wait(), which takes them as operands so that nothing moves ahead of it.
-__device__ __forceinline__ void tmem_ld16_async(unsigned taddr, float (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]), "=f"(v[9]), "=f"(v[10]),
-          "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait(float (&v)[16]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]),
-                   "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
-                 :
-                 : "memory");
-}
 __device__ __forceinline__ float tmem_ld1(unsigned taddr) {
     float v;
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;" : "=f"(v) : "r"(taddr) : "memory");
@@ -711,7 +695,7 @@ __global__ void __launch_bounds__(HTC_THREADS, 1) k_head_tc(const __grid_constan
 // Behind k_head_tc: one warp per row, the ranges' statistics in a fixed order and in 64 bits, then Eq. 2-4.  (By the last CTA of a row tile it
 // took 13 us at 100 rows, all of them on one SM.)
 __global__ void __launch_bounds__(128) k_head_tc_merge(const ClHeadPartial *part, int R, int NR, double inv_log_v, float *conf, float *pmax, int *arg) {
-    constexpr int PL = 7;   // partials a lane at a time: 64 * 7 cover three groups on 148 SMs
+    constexpr int PL = 7;   // partials a lane at a time: two turns of 32 * 7 cover three groups on 148 SMs
     pdl_wait();
     const int r = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= R) return;

@@ -22,7 +22,8 @@ namespace {
 constexpr int NCW = 16;                // consumer warps
 constexpr int NCT = NCW * 32;          // consumer threads
 // Registers: 17 warps leave 96 a thread (five warps on one scheduler), and consumers spilled 200 to 300 bytes into the heads of latency-bound
-// phases.  Launched with 20 warps the producer's group of four gives some back: 512 x 104 + 128 x 64 = 640 x 96, no spills in the consumers.
+// phases.  Launched with 20 warps the producer's group of four gives some back: 512 x 104 + 128 x 64 = 640 x 96; the consumers spill 40 bytes at
+// 16 bits, head_dim 128 and long rows, else none or 4 (the rest of a build's 128 to 164 is the producer's with both cursors).
 // (112 / 32: the producer spills, and a slow producer is a slow stream.  With both cursors of the L2 prefetch alive it spilled at 64 already,
 // and four full steps of 8 layers of width 4096 took 2995 us, 2884 before; as now 2854, 6 steps of 4 layers of width 5120 3590 -> 3396, 12 layers
 // of width 768 991 -> 971.)

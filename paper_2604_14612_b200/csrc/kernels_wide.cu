@@ -424,8 +424,9 @@ __global__ void __launch_bounds__(256) k_wide_rope_append(ClWideParts p, int hd,
 // instructions beside them count: chains start from a zero operand, masks are applied only where a key may lie ahead,
 // fragment addresses flip bits of one base.  512 rows of 32 heads 53 -> 40 us, the pass after it 97 -> 78, 333 rows 38 -> 30.
 // (A weight is expf of the exact difference.  ex2 of s * log2(e) less the rounded m * log2(e) takes 37, 73 and 28 us, but that rounding differs
-// from tile to tile as the maximum rises, 2^-25 of the score, and at scores of 2^26 a weight could be 2^7: no number in fp16.)  Key tiles dealt out evenly over the CTAs, jobs cut where shares end: 41 us (a cut costs more than the balance gains); eight
-// warps of 32 keys: 45.  Blocks of late rows see the most keys and are scheduled first.
+// from tile to tile as the maximum rises, 2^-25 of the score, and at scores of 2^26 a weight could be 2^7: no number in fp16.)
+// Key tiles dealt out evenly over the CTAs, jobs cut where shares end: 41 us (a cut costs more than the balance gains); eight warps of 32
+// keys: 45.  Blocks of late rows see the most keys and are scheduled first.
 constexpr int AQ = 64, AK = 64;   // rows per CTA, keys per tile
 
 template <int HD>
