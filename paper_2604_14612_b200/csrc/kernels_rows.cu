@@ -1049,7 +1049,7 @@ __device__ void attention_walk(const ClRowsArgs &a, const ClRowsLayer &y, int la
                     const float pn = expf(sc - (m_new > -INFINITY ? m_new : 0.f));
                     l_run = fmaf(l_run, resc, pn);
 #pragma unroll
-                    for (int e = 0; e < VPL; ++e) o_run[e] = fmaf(o_run[e], resc, pn * vn[e]);
+                    for (int e = 0; e < VPL; ++e) o_run[e] = fmaf(o_run[e], resc, pn > 0.f ? pn * vn[e] : 0.f);   // (a value may be infinite)
                     m_run = m_new;
                 }
             }

@@ -114,14 +114,16 @@ def test_a_candidate_whose_value_overflows_leaves_the_rows_before_it_alone(T, n)
     assert not np.isfinite(rows[0][3:, 3:]).any()
 
 
+@pytest.mark.parametrize("value", [500.0, 1e5])
 @pytest.mark.parametrize("n", [40, 600])
 @pytest.mark.parametrize("T", [5, 9])
-def test_a_candidate_whose_key_overflows_has_no_weight_against_negative_queries(T, n):
-    """Token 0 has keys of 1e5, infinite in fp16, that score -inf; all others score 0 and have the same value: the output of every row."""
+def test_a_candidate_whose_key_overflows_has_no_weight_against_negative_queries(T, n, value):
+    """Token 0 has keys of 1e5, infinite in fp16, that score -inf, and values that may be infinite too; all others score 0 and have the same
+    value: the output of every row."""
     g = torch.Generator().manual_seed(7)
     values = 1.0 + torch.rand(256, generator=g)
     values[:3] = 0.0
-    ctx, emb, v = _model("fp16", 4, n + 16, [-32.0, -1.0, -3.3, -0.01], values, first_key=1e5, first_value=500.0)
+    ctx, emb, v = _model("fp16", 4, n + 16, [-32.0, -1.0, -3.3, -0.01], values, first_key=1e5, first_value=value)
     ctx.cl_prefill((1 + np.arange(n)).astype(np.int32))
     ctx.cl_rollback(n, 7)
     tokens = [7, 1, 2, 0] + list(range(10, 6 + T))
