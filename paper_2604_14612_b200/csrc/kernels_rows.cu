@@ -889,7 +889,8 @@ __device__ __forceinline__ void finish_head(const ClRowsArgs &a, int h, int S, b
 // the CUDA cores, a trip to memory each.  Up to two trips that is faster than the other form's fixed cost and smaller ring, hence the line
 // of 32 * (14 / T) keys a part (cl_rows_walk_keys); three trips with nine rows, which cost the other form a second set of columns; and at any
 // length with one or two rows, whose scores leave six or seven of its eight columns idle.  us per verify, here / there, by keys a part:
-//   8 layers of width 4096 (4 parts)  1 row   112 831 / 856   224 823 / 858   640 905 / 971      2 rows  112 843 / 858   224 859 / 883   640 955 / 979
+//   8 layers of width 4096 (4 parts)  1 row   112 831 / 856   224 823 / 858   640 905 / 971   2000 1113 / 1298
+//     2 rows  112 843 / 858   224 859 / 883   640 955 / 979   2000 1261 / 1323
 //     3 rows  64 843 / 860   112 858 / 868   136 880 / 870      4 rows  48 856 / 870   96 870 / 870   136 893 / 881
 //     5 rows  48 870 / 888   64 880 / 882   80 893 / 882        7 rows  32 881 / 904   64 904 / 905   80 917 / 904
 //     8 rows  24 884 / 891   32 892 / 892   40 898 / 884        9 rows  32 953 / 979   48 966 / 979   64 978 / 968
